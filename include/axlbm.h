@@ -335,8 +335,13 @@ AXLBM_API axlbm_status axlbm_load(axlbm_handle* h, const void* buf, size_t bytes
  * axlbm_step call) are replayed from CUDA graphs captured on first use (8
  * and 1 pairs of an even and an odd step, on a stream of the library's own,
  * launched on the handle's stream) when enable != 0, the default, and while
- * kernel timing is off; enable = 0 launches every kernel directly.  The
- * results are the same bit for bit. */
+ * kernel timing is off; enable = 0 launches every kernel directly.  Small
+ * domains with FP32 or FP64 storage (up to 64 MB of populations) take one
+ * graph of a single kernel that runs all the pairs of a call, with device
+ * scratch of the library's own allocated at creation; where that cannot be
+ * allocated, or the domain has wet walls, a Zou-He wall, a node on the axis or
+ * cut faces, the step pairs are replayed.  The results are the same bit for
+ * bit. */
 AXLBM_API axlbm_status axlbm_use_graphs(axlbm_handle* h, int32_t enable);
 
 /* How many times the step graphs were captured and launched since creation

@@ -352,8 +352,17 @@ axlbm_status axlbm_create(const axlbm_grid* grid, double tau, const axlbm_forcin
             cudaFree(fields);
         }
     }
+    if (st == AXLBM_OK && (grid->precision == AXLBM_FP32 || grid->precision == AXLBM_FP64)) {
+        axl::Clock* clk = reinterpret_cast<axl::Clock*>(h->mem + L.off_clock);
+        const axl::ResidentDomain d = {h->mem, h->G, tau, *forcing, *bc, grid->collision == AXLBM_MRT,
+                                       grid->with_temperature, clk->a_z, nullptr};
+        const axl::ResidentOps& ro = grid->precision == AXLBM_FP32 ? axl::resident_fp32 : axl::resident_fp64;
+        e = ro.build(&h->res, &d, 1, grid->with_swirl != 0, grid->with_temperature != 0, h->num_sms, h->stream);
+        if (e != cudaSuccess) st = cuda_fail(h, e, "multi-step launch");
+    }
     if (st != AXLBM_OK) {
         g_create_error = h->err;
+        axl::resident_free(&h->res);
         if (h->owns_mem) cudaFree(h->mem);
         delete h;
         return st;
@@ -370,6 +379,7 @@ void drop_graphs(axlbm_handle* h) {
     if (h->graph_one) cudaGraphExecDestroy(h->graph_one);
     h->graph_many = h->graph_one = nullptr;
     h->graphs_ready = false;
+    axl::resident_drop_graph(&h->res);
 }
 
 // Capture `pairs` plain (even, odd) step pairs and instantiate them; the
@@ -402,9 +412,16 @@ cudaError_t capture_pairs(axlbm_handle* h, const Ops* ops, int pairs, cudaGraphE
 
 // `pairs` plain step pairs from an even level, from the graphs.
 axlbm_status graph_pairs(axlbm_handle* h, const Ops* ops, int64_t pairs) {
+    axl::Clock* clk = reinterpret_cast<axl::Clock*>(h->mem + h->L.off_clock);
     if (!h->graphs_ready) {
-        cudaError_t e = capture_pairs(h, ops, kGraphPairs, &h->graph_many);
-        if (e == cudaSuccess) e = capture_pairs(h, ops, 1, &h->graph_one);
+        cudaError_t e = cudaSuccess;
+        if (h->res.on) {
+            if (!h->cap) e = cudaStreamCreateWithFlags(&h->cap, cudaStreamNonBlocking);
+            if (e == cudaSuccess) e = axl::resident_capture(&h->res, clk, h->cap);
+        } else {
+            e = capture_pairs(h, ops, kGraphPairs, &h->graph_many);
+            if (e == cudaSuccess) e = capture_pairs(h, ops, 1, &h->graph_one);
+        }
         if (e != cudaSuccess) {
             cudaGetLastError();  // the failed capture must not surface in a later call
             drop_graphs(h);
@@ -414,10 +431,18 @@ axlbm_status graph_pairs(axlbm_handle* h, const Ops* ops, int64_t pairs) {
         h->graph_captures += 1;
     }
     for (int64_t p = 0; p < pairs;) {
-        const bool many = pairs - p >= kGraphPairs;
-        const cudaError_t e = cudaGraphLaunch(many ? h->graph_many : h->graph_one, h->stream);
+        cudaError_t e;
+        int64_t done;
+        if (h->res.on) {
+            done = pairs - p < axl::kResMaxSteps / 2 ? pairs - p : axl::kResMaxSteps / 2;
+            e = axl::resident_launch(&h->res, clk, (int)(2 * done), h->t + 2 * p, h->stream);
+        } else {
+            const bool many = pairs - p >= kGraphPairs;
+            done = many ? kGraphPairs : 1;
+            e = cudaGraphLaunch(many ? h->graph_many : h->graph_one, h->stream);
+        }
         if (e != cudaSuccess) return cuda_fail(h, e, "graph launch");
-        p += many ? kGraphPairs : 1;
+        p += done;
         h->graph_launches += 1;
     }
     h->t += 2 * pairs;
@@ -435,11 +460,12 @@ axlbm_status axlbm_step(axlbm_handle* h, int64_t n) {
     // every step but the tail is plain: the tail is the two check steps (lag
     // 1), or a check step, a plain step and a check step (lag 2); with timing
     // off, whole (even, odd) pairs of plain steps replay captured graphs once
-    // the plain bulk kernels have been sized by earlier launches
+    // the plain bulk kernels have been sized by earlier launches (a domain on
+    // the multi-step kernels needs none)
     const int tail = h->residual_lag == 2 ? 3 : 2;
     const bool odd_bulk = h->G.nr > 2 && h->G.nz > 2;
     const bool sized = h->bulk_grid[0][0] > 0 && (h->bulk_grid[1][0] > 0 || !odd_bulk);
-    if (h->use_graphs && !h->timing && sized && n - tail - h->parity >= 2 * kMinGraphPairs) {
+    if (h->use_graphs && !h->timing && (sized || h->res.on) && n - tail - h->parity >= 2 * kMinGraphPairs) {
         if (h->parity == 1) {
             int nl = 0;
             const cudaError_t e = ops->step(h, 0, 0, nullptr, nullptr, &nl);
@@ -743,6 +769,7 @@ axlbm_status axlbm_destroy(axlbm_handle* h) {
     if (!h) return AXLBM_EINVAL;
     cudaError_t e = cudaStreamSynchronize(h->stream);
     drop_graphs(h);
+    axl::resident_free(&h->res);
     if (h->cap) cudaStreamDestroy(h->cap);
     if (h->stage) cudaFree(h->stage);
     for (auto ev : h->ev)

@@ -444,7 +444,7 @@ k_bulk_batch(const __grid_constant__ CUtensorMap map, const BatchArgs<S, R> A) {
     constexpr int NW = batch_nwarps<TK, TJ>();  // computing warps; warp NW is the producer
     constexpr int NP = batch_pairs<TK, TJ>();   // node pairs per computing thread
     constexpr int TPC = TK / (2 * NP);          // computing threads per column
-    using RC = typename std::conditional<std::is_same<R, float>::value, F2, R>::type;
+    using RC = typename PairArith<R>::type;
     static_assert(std::is_same<R, float>::value, "batch arithmetic is FP32");
     static_assert(NW <= kBatchMaxWarps && TPC >= 1 && NW * 32 == TJ * TPC, "NP node pairs of one column per thread");
     static_assert(TK <= kRowAlign && kRowAlign % TK == 0, "a tile row band stays inside one shelf");

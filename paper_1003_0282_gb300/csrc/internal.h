@@ -80,6 +80,50 @@ struct Coef : CoefCore<R> {
     int t_dir[4];   // 1: Dirichlet face
 };
 
+// Multi-step launches of a small domain or batch (resident.cuh): built at
+// creation where the rule takes it, launched from a graph of one kernel node
+// captured on first use, whose step count is set for every launch.
+struct Resident {
+    bool on = false;
+    bool cluster = false;  // one thread-block cluster, else a cooperative grid
+    bool slab = false;     // a grid with the state in shared memory, else in L2
+    int max_tab = 0, max_ghost = 0;
+    bool sw = false, th = false;
+    int grid = 0, threads = 0;
+    size_t smem = 0;
+    const void* kernel = nullptr;
+    void* scratch = nullptr;  // descriptors, CTA map, step counters or words between CTAs
+    size_t off_map = 0, off_flags = 0;
+    unsigned epoch = 0;       // steps launched so far: the step counters' base
+    cudaGraph_t graph = nullptr;
+    cudaGraphNode_t node = nullptr;
+    cudaGraphExec_t exec = nullptr;
+};
+
+// One domain as the rule and the kernels of resident.cuh take it.
+struct ResidentDomain {
+    void* pop;  // population planes (a batch domain's place is in G)
+    Geom G;
+    double tau;
+    axlbm_forcing forcing;
+    axlbm_boundary boundary;
+    int mrt, th;
+    double *az, *az16;
+};
+
+struct ResidentOps {
+    cudaError_t (*build)(Resident* r, const ResidentDomain* d, int n, bool sw, bool th, int num_sms, cudaStream_t stream);
+};
+extern const ResidentOps resident_fp32;
+extern const ResidentOps resident_fp64;
+
+constexpr int64_t kResMaxSteps = 1 << 16;  // steps of one launch, at most (even)
+
+cudaError_t resident_capture(Resident* r, Clock* clock, cudaStream_t cap);
+cudaError_t resident_launch(Resident* r, Clock* clock, int steps, long long t0, cudaStream_t stream);
+void resident_drop_graph(Resident* r);
+void resident_free(Resident* r);
+
 struct Layout {
     int nplanes;      // 9 (+4 g) (+4 h)
     int g_plane;      // first g plane (or -1)
@@ -135,6 +179,7 @@ struct axlbm_handle {
     cudaStream_t cap;
     cudaGraphExec_t graph_many, graph_one;  // kGraphPairs step pairs; one pair
     int64_t graph_captures, graph_launches;
+    axl::Resident res;  // multi-step launches instead of the pair graphs, for small domains
     void* stage;  // device staging buffer of host-side field I/O, kept between calls
     size_t stage_bytes;
     std::string err;

@@ -84,13 +84,20 @@ struct Cell {
         const Sc W0 = Sc(4.0 / 9.0), W1 = Sc(1.0 / 9.0), W2 = Sc(1.0 / 36.0);
         const Sc half = Sc(0.5), one = Sc(1);
         // rates by the sign of e_r (Eq. 13) and their combinations
-        const Sc om0 = C.c0, omp = C.c0 + C.c1 * inv_r, omm = C.c0 - C.c1 * inv_r;
+        const Sc om0 = C.c0, omp = fmaR(C.c1, inv_r, C.c0), omm = fmaR(-C.c1, inv_r, C.c0);
         const Sc inv_r2 = inv_r * inv_r;
 
         // moments (Eqs. 14-17 with the half-force terms)
-        ds0 = ((d[0] + d[1]) + (d[2] + d[3])) + ((d[4] + d[5]) + (d[6] + d[7])) + d[8];
-        const R sr = (d[1] - d[3]) + (d[5] - d[6]) + (d[8] - d[7]);
-        const R sz = (d[2] - d[4]) + (d[5] + d[6]) - (d[7] + d[8]);
+        R sr, sz;
+        if constexpr (std::is_same<R, D1>::value) {  // sums that the MRT collision shares
+            ds0 = (d[0] + ((d[1] + d[3]) + (d[2] + d[4]))) + ((d[5] + d[6]) + (d[7] + d[8]));
+            sr = (d[1] - d[3]) + ((d[5] - d[6]) + (d[8] - d[7]));
+            sz = (d[2] - d[4]) + ((d[5] + d[6]) - (d[7] + d[8]));
+        } else {
+            ds0 = ((d[0] + d[1]) + (d[2] + d[3])) + ((d[4] + d[5]) + (d[6] + d[7])) + d[8];
+            sr = (d[1] - d[3]) + (d[5] - d[6]) + (d[8] - d[7]);
+            sz = (d[2] - d[4]) + (d[5] + d[6]) - (d[7] + d[8]);
+        }
         s0 = ds0 + R(C.rho0);
         R gsum = R(Sc(0)), dtemp = R(Sc(0));
         if (SW) gsum = (g[0] + g[1]) + (g[2] + g[3]);
@@ -110,21 +117,22 @@ struct Cell {
         const R fz = fext_z;
         const R inv_rho = den * inv_s0;
 
+        if (C.mrt) {
+            if constexpr (std::is_same<R, D1>::value) collide_mrt_d1(urr, C, inv_r, drho, fr, fz);
+            else collide_mrt(inv_r, C, drho, fr, fz);
+        } else {
         // equilibrium polynomials P_a
         const R ur2 = ur * ur, uz2 = uz * uz;
         const R A = fmaR(rho * R(Sc(-1.5)), ur2 + uz2, drho);
         const R B = rho * R(Sc(3)), Cq = rho * R(Sc(4.5));
-        const R Bur = B * ur, Buz = B * uz, Cur2 = Cq * ur2, Cuz2 = Cq * uz2;
+        const R Bur = B * ur, Buz = B * uz, Cuz2 = Cq * uz2;
         const R Cx = (Cq + Cq) * (ur * uz);
-        const R Ps = A + Cur2, Pz = A + Cuz2, Q = Ps + Cuz2;
+        const R Ps = mad(Cq, ur2, A), Pz = A + Cuz2, Q = Ps + Cuz2;
         const R Qp = Q + Cx, Qm = Q - Cx, Bs = Bur + Buz, Bd = Bur - Buz;
         const R P[9] = {A, Ps + Bur, Pz + Buz, Ps - Bur, Pz - Buz, Qp + Bs, Qm - Bd, Qp - Bs, Qm + Bd};
         // source factors F_a
-        if (C.mrt) {
-            collide_mrt(inv_r, C, drho, fr, fz);
-        } else {
         const R fr3 = fr * inv_rho * R(Sc(3)), fz3 = fz * inv_rho * R(Sc(3));
-        const R base = fmaR((ur * fr + uz * fz) * R(Sc(-3)), inv_rho, R(Sc(0)) - urr);
+        const R base = fmaR(mad(ur, fr, uz * fz) * R(Sc(-3)), inv_rho, R(Sc(0)) - urr);
         const R F1 = base + fr3, F3 = base - fr3;
         const R F[9] = {base, F1, base + fz3, F3, base - fz3, F1 + fz3, F3 + fz3, F3 - fz3, F1 - fz3};
 #pragma unroll
@@ -143,7 +151,7 @@ struct Cell {
             const R g2r = (g4 + g4) * ur, g2z = (g4 + g4) * uz;
             const R geq[4] = {g4 + g2r, g4 + g2z, g4 - g2r, g4 - g2z};
             const R sg = fmaR(ur, R(Sc(-2) * inv_r), R(-C.nu * inv_r2));
-            const Sc gp = C.g0 + C.g1 * inv_r, gm = C.g0 - C.g1 * inv_r;
+            const Sc gp = fmaR(C.g1, inv_r, C.g0), gm = fmaR(-C.g1, inv_r, C.g0);
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 const int ex = cr4(q);
@@ -156,7 +164,7 @@ struct Cell {
             const R h4 = (dtemp + R(C.t_ref)) * R(Sc(0.25));
             const R h2r = (h4 + h4) * ur, h2z = (h4 + h4) * uz;
             const R heq[4] = {h4 + h2r, h4 + h2z, h4 - h2r, h4 - h2z};
-            const Sc hp = C.h0 + C.h1 * inv_r, hm = C.h0 - C.h1 * inv_r;
+            const Sc hp = fmaR(C.h1, inv_r, C.h0), hm = fmaR(-C.h1, inv_r, C.h0);
             const Sc tref4 = C.t_ref * Sc(0.25);
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
@@ -247,7 +255,99 @@ struct Cell {
         d[7] = ((cd - dr) - dz) + a8;
         d[8] = ((cd + dr) - dz) - a8;
     }
+
+    // The same in FP64, arranged for the fewest FP64 instructions (56 + 25 + 27
+    // for the relaxation, the way back and the moments; they are what bounds
+    // the FP64 kernels): moments share sums, S_4 = -S_3 and S_6 = -S_5, and
+    // the factors 1/|row|^2 ride on the fused multiply-adds of the way back.
+    __device__ __forceinline__ void collide_mrt_d1(R urr, const CoefCore<Sc>& C, Sc inv_r, R drho, R fr, R fz) {
+        const Sc one = Sc(1), half = Sc(0.5);
+        const auto neg = [](R x) { return R(-x.v); };
+        const R s13 = d[1] + d[3], s24 = d[2] + d[4], s56 = d[5] + d[6], s78 = d[7] + d[8];
+        const R ax = s13 + s24, dg = s56 + s78;
+        const R md1 = fmaR(d[0], R(Sc(-4)), fmaR(dg, R(Sc(2)), neg(ax)));
+        const R md2 = fmaR(d[0], R(Sc(4)), fmaR(ax, R(Sc(-2)), dg));
+        const R md4 = fmaR(d[1] - d[3], R(Sc(-2)), (d[5] - d[6]) + (d[8] - d[7]));
+        const R md6 = fmaR(d[2] - d[4], R(Sc(-2)), s56 - s78);
+        const R md7 = s13 - s24;
+        const R md8 = (d[5] + d[7]) - (d[6] + d[8]);
+        const R ru = rho * ur, rz = rho * uz;
+        const R ur2 = ur * ur;
+        const R r3u2 = rho * (fmaR(uz, uz, ur2) * R(Sc(3)));
+        const R pxx_eq = rho * fmaR(neg(uz), uz, ur2), pxy_eq = ru * uz;
+        const R uF6 = fmaR(ur, fr, uz * fz) * R(Sc(6));
+        const R mu = neg(urr);
+        const R S1 = fmaR(mu, fmaR(rho, R(Sc(-2)), r3u2), uF6);
+        const R S2 = fmaR(mu, rho - r3u2, neg(uF6));
+        const R S3 = fmaR(mu, ru, fr), S5 = fmaR(mu, rz, fz);
+        const R dF = fmaR(ur, fr, neg(uz * fz));
+        const R S7 = fmaR(mu, pxx_eq, dF + dF);
+        const R S8 = fmaR(mu, pxy_eq, fmaR(ur, fz, uz * fr));
+        const R q1 = fmaR(drho, R(Sc(2)), neg(r3u2)), q2 = r3u2 - drho;  // m^eq of e and eps, sign reversed
+        const R ne1 = md1 + q1, ne2 = md2 + q2, ne4 = md4 + ru, ne6 = md6 + rz, ne7 = md7 - pxx_eq, ne8 = md8 - pxy_eq;
+        const R p0 = fmaR(mu * rho, R(half), drho);
+        const R p1 = fmaR(ne1, R(one - C.se), fmaR(S1, R(one - half * C.se), neg(q1)));
+        const R p2 = fmaR(ne2, R(one - C.seps), fmaR(S2, R(one - half * C.seps), neg(q2)));
+        const R p4 = fmaR(ne4, R(one - C.sq), fmaR(S3, R(half * C.sq - one), neg(ru)));
+        const R p6 = fmaR(ne6, R(one - C.sq), fmaR(S5, R(half * C.sq - one), neg(rz)));
+        const R p7 = fmaR(ne7, R(one - C.sv), fmaR(S7, R(one - half * C.sv), pxx_eq));
+        const R p8 = fmaR(ne8, R(one - C.sv), fmaR(S8, R(one - half * C.sv), pxy_eq));
+        const Sc gam = C.mrt_gam * inv_r;
+        const R e1 = fmaR(S1, R(half), ne1), pxx1 = fmaR(S7, R(half), ne7), pxy1 = fmaR(S8, R(half), ne8);
+        const R q3 = fmaR(fmaR(e1, R(C.k_e6), pxx1 * R(half)), R(-gam), fmaR(S3, R(half), ru));
+        const R q5 = fmaR(pxy1, R(-gam), fmaR(S5, R(half), rz));
+        const R P0 = p0 * R(Sc(1.0 / 9.0));
+        const R cx = fmaR(p1, R(Sc(-1.0 / 36.0)), fmaR(p2, R(Sc(-1.0 / 18.0)), P0));
+        const R cd = fmaR(p1, R(Sc(1.0 / 18.0)), fmaR(p2, R(Sc(1.0 / 36.0)), P0));
+        const R cxp = fmaR(p7, R(Sc(0.25)), cx), cxm = fmaR(p7, R(Sc(-0.25)), cx);
+        const R cdp = fmaR(p8, R(Sc(0.25)), cd), cdm = fmaR(p8, R(Sc(-0.25)), cd);
+        const R J = q3 - p4, K = q5 - p6;
+        const R M = fmaR(p4, R(half), q3), N = fmaR(p6, R(half), q5);
+        const R MpN = M + N, MmN = M - N;
+        const R sixth = R(Sc(1.0 / 6.0)), nsixth = R(Sc(-1.0 / 6.0));
+        d[0] = fmaR(p2 - p1, R(Sc(1.0 / 9.0)), P0);
+        d[1] = fmaR(J, sixth, cxp);
+        d[2] = fmaR(K, sixth, cxm);
+        d[3] = fmaR(J, nsixth, cxp);
+        d[4] = fmaR(K, nsixth, cxm);
+        d[5] = fmaR(MpN, sixth, cdp);
+        d[6] = fmaR(MmN, nsixth, cdm);
+        d[7] = fmaR(MpN, nsixth, cdp);
+        d[8] = fmaR(MmN, sixth, cdm);
+    }
 };
+
+// The value of one node held in a pair, a wrapped scalar or a plain one.
+__device__ __forceinline__ float scalar_of(F2 x) { return x.v.x; }
+__device__ __forceinline__ float scalar_of(float x) { return x; }
+__device__ __forceinline__ double scalar_of(D1 x) { return x.v; }
+__device__ __forceinline__ double scalar_of(double x) { return x; }
+
+// Collide a node held in R in the arithmetic type A (NodeArith).
+template <class A, class R, bool SW, bool TH>
+__device__ __forceinline__ void collide_as(Cell<R, SW, TH>& c, R inv_r, const CoefCore<R>& C, R az) {
+    Cell<A, SW, TH> w;
+#pragma unroll
+    for (int a = 0; a < 9; ++a) w.d[a] = A(c.d[a]);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        if (SW) w.g[q] = A(c.g[q]);
+        if (TH) w.h[q] = A(c.h[q]);
+    }
+    w.collide(inv_r, C, az);
+#pragma unroll
+    for (int a = 0; a < 9; ++a) c.d[a] = scalar_of(w.d[a]);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        if (SW) c.g[q] = scalar_of(w.g[q]);
+        if (TH) c.h[q] = scalar_of(w.h[q]);
+    }
+    c.rho = scalar_of(w.rho);
+    c.ur = scalar_of(w.ur);
+    c.uz = scalar_of(w.uz);
+    c.s0 = scalar_of(w.s0);
+    c.ds0 = scalar_of(w.ds0);
+}
 
 // ---------------------------------------------------------------------------- boundaries
 
@@ -279,7 +379,7 @@ __device__ __forceinline__ R inv_of(double r) {
 }
 
 // Where the population leaving fluid node (j, k) with velocity (ex, ez) lands.
-__device__ __forceinline__ Site classify(const Geom& G, int j, int k, int ex, int ez) {
+__host__ __device__ __forceinline__ Site classify(const Geom& G, int j, int k, int ex, int ez) {
     Site s{0, -1, j + ex, k + ez, 0, 0};
     if (s.k < 0 || s.k >= G.nz) {
         const int face = s.k < 0 ? AXLBM_FACE_LO : AXLBM_FACE_HI;
@@ -572,7 +672,16 @@ __device__ __forceinline__ R inv_radius(const Geom& G, int j) {
     return inv_of<R>(node_radius(G, j));
 }
 
-// ---------------------------------------------------------------------------- kernels
+// 1/r of column j as the bulk kernels form it.
+template <class R>
+__device__ __forceinline__ R step_inv_radius(const Geom& G, int j) {
+    if (sizeof(R) == 4 && G.rb_exact) {
+        const float r = G.rb + (float)j;
+        return r > 0.0f ? R(rcp(r)) : R(0);
+    }
+    const double r = node_radius(G, j);
+    return r > 0.0 ? rcp(R(r)) : R(0);
+}
 
 // ---------------------------------------------------------------------------- bulk kernel
 
@@ -622,6 +731,13 @@ struct Lanes {
     template <class S>
     __device__ static __forceinline__ R load(const S* p, int /*lane_stride*/) { return Codec<S>::load(p); }
     __device__ static __forceinline__ R get(R v, int) { return v; }
+};
+template <>
+struct Lanes<D1> {
+    static constexpr int n = 1;
+    template <class S>
+    __device__ static __forceinline__ D1 load(const S* p, int /*lane_stride*/) { return D1(Codec<S>::load(p)); }
+    __device__ static __forceinline__ double get(D1 v, int) { return v.v; }
 };
 template <>
 struct Lanes<F2> {
@@ -778,7 +894,7 @@ k_bulk(const __grid_constant__ CUtensorMap map, const KArgs<S, R> A) {
     constexpr int STAGE = stage_elems<S, SW, TH>();
     constexpr int HB = kHalo<S>, BW = kBoxW<S>;
     constexpr int HP = SW ? 13 : 9;  // first h plane
-    using RC = typename std::conditional<std::is_same<R, float>::value, F2, R>::type;  // per-thread arithmetic
+    using RC = typename PairArith<R>::type;  // per-thread arithmetic
     using Sc = R;
     static_assert(kTileK == 4 && kBulkThreads == 2 * kTileJ, "pairing assumes 4-row tiles and 2 threads per column");
     constexpr int kRowsPerThread = kTileK * kTileJ / kBulkThreads;  // 2: rows rr0 and rr0 + 2
@@ -854,14 +970,7 @@ k_bulk(const __grid_constant__ CUtensorMap map, const KArgs<S, R> A) {
             // together below (its lanes meet in __syncwarp)
             const bool ok = mbar_wait_bounded(&full[s], (uint32_t)((it / NS) & 1), kWaitCycles);
             const S* st = sm + s * STAGE;
-            Sc inv_r;
-            if (sizeof(Sc) == 4 && G.rb_exact) {  // FP32: no FP64 instruction in the loop over tiles
-                const float rj = G.rb + (float)j;
-                inv_r = rj > 0.0f ? rcp(Sc(rj)) : Sc(0);
-            } else {
-                const double rj = node_radius(G, j);
-                inv_r = rj > 0.0 ? rcp(Sc(rj)) : Sc(0);
-            }
+            const Sc inv_r = step_inv_radius<Sc>(G, j);  // (FP32: no FP64 instruction in the loop over tiles)
             // warps with a side-column lane load and store with the side-column
             // selections (odd steps); the others without them
             const bool side_lane = PAR == 1 && G.side && (j == 0 || j == G.nr - 1);
@@ -1080,16 +1189,16 @@ template <class S, class R, bool SW, bool TH, bool CHK, bool HALO = false>
 __device__ __forceinline__ void ring_node(const KArgs<S, R>& A, int j, int k, R az, Red& red) {
     Cell<R, SW, TH> c;
     pull_odd<S, R, SW, TH, HALO>(A, j, k, c);
-    const R inv_r = inv_radius<R>(A.G, j);
+    const R inv_r = std::is_same<S, R>::value ? step_inv_radius<R>(A.G, j) : inv_radius<R>(A.G, j);
     if (on_wet_wall(A.G, j, k)) {
         // a wet-wall node holds its post-collision state: stream it as it is
         Cell<R, SW, TH> m = c;
-        m.collide(inv_r, A.C, az);  // moments for the check values
+        collide_as<typename NodeArith<S, R>::type>(m, inv_r, A.C, az);  // moments for the check values
         push_odd<S, R, SW, TH, HALO>(A, j, k, c);
         if (CHK) check_cell(A, j, k, inv_r, m, red);
         return;
     }
-    c.collide(inv_r, A.C, az);
+    collide_as<typename NodeArith<S, R>::type>(c, inv_r, A.C, az);
     push_odd<S, R, SW, TH, HALO>(A, j, k, c);
     if (CHK) check_cell(A, j, k, inv_r, c, red);
 }

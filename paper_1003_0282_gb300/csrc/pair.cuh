@@ -65,6 +65,39 @@ __device__ __forceinline__ F2 rcp(F2 x) {
     return out;
 }
 
+// One FP64 value whose operations round as written: which products are fused
+// is stated in the collision (mad below), so that every kernel rounds a node
+// alike (the compiler fuses plain double expressions differently from kernel
+// to kernel).
+struct D1 {
+    double v;
+    __device__ __forceinline__ D1() {}
+    __device__ __forceinline__ D1(double s) : v(s) {}
+};
+__device__ __forceinline__ D1 operator+(D1 a, D1 b) { return D1(__dadd_rn(a.v, b.v)); }
+__device__ __forceinline__ D1 operator-(D1 a, D1 b) { return D1(__dsub_rn(a.v, b.v)); }
+__device__ __forceinline__ D1 operator*(D1 a, D1 b) { return D1(__dmul_rn(a.v, b.v)); }
+__device__ __forceinline__ D1 fmaR(D1 a, D1 b, D1 c) { return D1(__fma_rn(a.v, b.v, c.v)); }
+// Reciprocal in FP64: the hardware estimate (PTX rcp.approx.ftz.f64, about
+// 20 bits) refined by one step of Halley's third-order iteration for 1/x,
+// r' = r + r (e + e^2) with e = 1 - x r, which cubes the estimate's relative
+// error: three fused multiply-adds, within an ulp for the normal arguments the
+// collision takes, no branch.  A correctly rounded divide costs about three
+// times as many FP64 instructions, and FP64 instructions bound these kernels
+// (GB300 issues one per SM in 16 cycles).
+__device__ __forceinline__ D1 rcp(D1 x) {
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x.v));
+    const double e = __fma_rn(-x.v, r, 1.0);
+    return D1(__fma_rn(r, __fma_rn(e, e, e), r));
+}
+
+// a b + c where the FP32 types round the product (their form is fixed:
+// 16-bit storage would amplify another rounding) and FP64 fuses it.
+template <class R>
+__device__ __forceinline__ R mad(R a, R b, R c) { return a * b + c; }
+__device__ __forceinline__ D1 mad(D1 a, D1 b, D1 c) { return fmaR(a, b, c); }
+
 template <class R>
 struct ScalarOf {
     using type = R;
@@ -72,6 +105,38 @@ struct ScalarOf {
 template <>
 struct ScalarOf<F2> {
     using type = float;
+};
+template <>
+struct ScalarOf<D1> {
+    using type = double;
+};
+
+// Arithmetic of a node in the step kernels: NodeArith for one node (the ring
+// kernels), PairArith for what a thread of the bulk kernels holds.  With FP32
+// storage the ring nodes use a pair with equal lanes, so that every FP32
+// kernel rounds a node alike.  With 16-bit storage they keep the plain float
+// type they have always had: its rounding differs from a lane's in the last
+// FP32 bit, and a 16-bit store would turn that into a whole unit of its last
+// place.
+template <class S, class R>
+struct NodeArith {
+    using type = R;
+};
+template <>
+struct NodeArith<float, float> {
+    using type = F2;
+};
+template <>
+struct NodeArith<double, double> {
+    using type = D1;
+};
+template <class R>
+struct PairArith {
+    using type = F2;
+};
+template <>
+struct PairArith<double> {
+    using type = D1;
 };
 
 }  // namespace axl

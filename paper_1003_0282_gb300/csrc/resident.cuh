@@ -1,0 +1,967 @@
+// resident.cuh -- many lattice steps of a small domain (or of a small batch) in one launch.
+//
+// A domain whose populations fit the L2 cache spends most of a step outside
+// the collision: the launches of a step (an even bulk kernel, an odd bulk
+// kernel, the ring kernels) each cost microseconds and fill few of the 152
+// SMs.  The kernels here advance a whole run of plain steps instead.  Each
+// thread keeps the nodes it owns for the whole launch; a step is "load the
+// node's slots, collide, store the same slots, meet the neighbours".  In the
+// AA pattern a node reads and writes one set of slots per step (its own in
+// even steps, in odd steps the slots it pulls from, which are the ones it
+// pushes to), and no other node touches them in that step, so one meeting per
+// step is enough.  The boundary rules are the addresses of those slots and
+// are worked out once per launch, from classify() as the ring kernels use it.
+//
+// Two forms, chosen by resident_plan():
+//   k_resident_cluster  one thread-block cluster (up to 8 CTAs), one node
+//     pair per thread (FP64: one node), the state in shared memory for the
+//     whole launch; neighbours' slots are reached through distributed shared
+//     memory and a step ends with the cluster barrier.
+//   k_resident_grid     a cooperative grid over the whole chip, the state in
+//     global memory (L2); a CTA owns a contiguous range of node pairs of one
+//     domain and after every step waits only for the CTAs whose nodes its own
+//     exchange populations with (a step counter per CTA, polled with a bound).
+//
+// Arithmetic and storage are those of the step kernels (PairArith, Codec),
+// rounding included: a run here equals the same steps launched one by one.
+#pragma once
+
+#include <cooperative_groups.h>
+
+#include <vector>
+
+#include "ops_impl.cuh"
+
+namespace axl {
+
+constexpr int kResThreads = 256;  // threads of a CTA, at most
+constexpr int kResAz = 256;       // steps whose force a(t) is kept ready (even)
+constexpr int kResPad = 32;       // 32-bit words between two CTAs' step counters (one 128-byte line each)
+constexpr long long kResWait = kWaitCycles;
+__host__ __device__ constexpr int res_up32(int v) { return (v + 31) / 32 * 32; }
+
+// One domain as the resident kernels see it, and the CTAs it has.
+template <class S, class R>
+struct ResDom {
+    S* pop;
+    Geom G;
+    Coef<R> C;
+    double az0, omega_t;
+    double* az;      // a(t) by AA parity: where the step kernels read it (two values)
+    double* az16;    // a batch domain's copy for the bulk kernel, or null
+    void* mail;      // words between CTAs: [plane][lane][pair]
+    int th;
+    int npairs;      // node pairs (FP64: nodes), pair p = (row pair p / nr, column p % nr)
+    int cta0, ncta, chunk;  // CTAs [cta0, cta0 + ncta), `chunk` consecutive pairs each
+};
+
+// The slot that population (er, ez) of node (j, k) is pulled from in an odd
+// step -- and pushed to in the opposite direction: its D2Q9 or D2Q4 plane,
+// its node, and how a value changes on the way: 0 not at all, 1 through the
+// axis (g changes sign), 2 + face off a solid face.
+struct ResSlot {
+    int plane, j, k, how;
+};
+__host__ __device__ __forceinline__ ResSlot res_slot9(const Geom& G, int a, int j, int k) {
+    const Site s = classify(G, j, k, -cr9(a), -cz9(a));
+    if (s.solid) return {a, j, k, 2 + s.face};
+    return {opp9(idx9(s.fr ? -cr9(a) : cr9(a), s.fz ? -cz9(a) : cz9(a))), s.j, s.k, s.fr ? 1 : 0};
+}
+__host__ __device__ __forceinline__ ResSlot res_slot4(const Geom& G, int q, int j, int k) {
+    const Site s = classify(G, j, k, -cr4(q), -cz4(q));
+    if (s.solid) return {q, j, k, 2 + s.face};
+    return {opp4(idx4(s.fr ? -cr4(q) : cr4(q), s.fz ? -cz4(q) : cz4(q))), s.j, s.k, s.fr ? 1 : 0};
+}
+
+// g and h on their way through a slot, as the step kernels' boundary rules
+// round them, without a branch: g' = sg g + cg with sg = 1, -1 (axis, or off a
+// wall: cg = rho0 u_w / 2), h' = (sh h + ch) + ct with sh = -1, ch = -T_ref/2,
+// ct = T_w/2 off a wall of given temperature, else h.  (Zero may lose its sign.)
+template <class R>
+__device__ __forceinline__ void res_through_g(const Geom& G, const Coef<R>& C, int how, int j, R& sg, R& cg) {
+    sg = how == 0 ? R(1) : R(-1);
+    cg = how >= 2 ? mul_rn(R(0.5) * C.rho0, wall_uth(G, C, how - 2, j)) : R(0);
+}
+template <class R>
+__device__ __forceinline__ void res_through_h(const Coef<R>& C, int how, R& sh, R& ch, R& ct) {
+    const bool dirichlet = how >= 2 && pick4(C.t_dir, how - 2);
+    sh = dirichlet ? R(-1) : R(1);
+    ch = dirichlet ? R(-0.5) * C.t_ref : R(0);
+    ct = dirichlet ? R(0.5) * pick4(C.t_w, how - 2) : R(0);
+}
+
+// The slot of plane-ordered population q of node (j, k): plane-ordered slot
+// and lane (ql), pair, and how a value changes on the way.
+template <int NL>
+__host__ __device__ __forceinline__ void res_where(const Geom& G, int q, int j, int k, int& ql, int& p, int& how) {
+    const ResSlot s = q < 9 ? res_slot9(G, q, j, k) : res_slot4(G, (q - 9) & 3, j, k);
+    ql = (q < 9 ? s.plane : 9 + ((q - 9) & ~3) + s.plane) * NL + s.k % NL;
+    p = (s.k / NL) * G.nr + s.j;
+    how = s.how;
+}
+
+// a(t) in R, as the step kernels round it.
+template <class R>
+__device__ __forceinline__ R res_az(double az0, double omega_t, long long t) {
+    return R(az0 * cos(omega_t * (double)t));
+}
+
+// The force and the time level after the last step of a launch (an even
+// level; the odd entry holds the last step's force, as after single steps).
+template <class S, class R>
+__device__ __forceinline__ void res_finish(const ResDom<S, R>& D, long long t1) {
+    const double a0 = D.az0 * cos(D.omega_t * (double)t1), a1 = D.az0 * cos(D.omega_t * (double)(t1 - 1));
+    D.az[0] = a0;
+    D.az[1] = a1;
+    if (D.az16) {
+        D.az16[0] = a0;
+        *reinterpret_cast<float*>(D.az16 + 1) = (float)a0;
+        D.az16[2] = a1;
+        *reinterpret_cast<float*>(D.az16 + 3) = (float)a1;
+    }
+}
+
+template <class RC>
+__device__ __forceinline__ RC res_make(typename ScalarOf<RC>::type a, typename ScalarOf<RC>::type b);
+template <>
+__device__ __forceinline__ F2 res_make<F2>(float a, float b) { return F2(a, b); }
+template <>
+__device__ __forceinline__ D1 res_make<D1>(double a, double) { return D1(a); }
+
+// What one thread holds of its pair for a whole launch: how g and h change on
+// their way through its slots (the slots' addresses are the kernels' own).
+template <class RC, bool SW, bool TH>
+struct ResLinks {
+    RC sg[SW ? 4 : 1], cg[SW ? 4 : 1], sh[TH ? 4 : 1], ch[TH ? 4 : 1], ct[TH ? 4 : 1];
+    __device__ __forceinline__ void set_g(int q, const RC& s, const RC& c) {
+        if (SW) sg[SW ? q : 0] = s, cg[SW ? q : 0] = c;
+    }
+    __device__ __forceinline__ RC g(int q, RC v) const { return SW ? fmaR(v, sg[SW ? q : 0], cg[SW ? q : 0]) : v; }
+    __device__ __forceinline__ RC h(int q, RC v) const {
+        return TH ? fmaR(v, sh[TH ? q : 0], ch[TH ? q : 0]) + ct[TH ? q : 0] : v;
+    }
+};
+
+// Load / store the populations of a pair: at(q, l) is the value of plane-
+// ordered slot q of lane l; in odd steps links change g and h on the way, and
+// slot q takes the opposite population.
+template <class RC, bool SW, bool TH, int PAR, class At, class Links>
+__device__ __forceinline__ void res_load(Cell<RC, SW, TH>& c, const At& at, const Links& L) {
+    constexpr int NL = Lanes<RC>::n, HP = SW ? 13 : 9;
+#pragma unroll
+    for (int a = 0; a < 9; ++a) c.d[a] = res_make<RC>(at(a, 0), at(a, NL - 1));
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        if (SW) c.g[q] = res_make<RC>(at(9 + q, 0), at(9 + q, NL - 1));
+        if (TH) c.h[q] = res_make<RC>(at(HP + q, 0), at(HP + q, NL - 1));
+        if (SW && PAR) c.g[q] = L.g(q, c.g[q]);
+        if (TH && PAR) c.h[q] = L.h(q, c.h[q]);
+    }
+}
+template <class RC, bool SW, bool TH, int PAR, class To, class Links>
+__device__ __forceinline__ void res_store(const Cell<RC, SW, TH>& c, const To& to, const Links& L) {
+    constexpr int NL = Lanes<RC>::n, HP = SW ? 13 : 9;
+#pragma unroll
+    for (int q = 0; q < 9 + (SW ? 4 : 0) + (TH ? 4 : 0); ++q) {
+        const int o = opp4((q - 9) & 3), m = (q - 9) & 3;
+        RC x = q < 9 ? c.d[opp9(q)] : (SW && q < 13 ? c.g[o] : c.h[o]);
+        if (PAR && SW && q >= 9 && q < 13) x = L.g(m, x);
+        if (PAR && TH && q >= HP) x = L.h(m, x);
+#pragma unroll
+        for (int l = 0; l < NL; ++l) to(q, l, Lanes<RC>::get(x, l));
+    }
+}
+
+// Links of the pair in rows k0 and k0 + 1 of column j, and its slots as
+// put(q, l, ql, p) takes them; a lane without a node keeps to itself (p = -1).
+template <class RC, class R, bool SW, bool TH, class Put>
+__device__ __forceinline__ void res_links(const Geom& G, const Coef<R>& C, int j, int k0, ResLinks<RC, SW, TH>& L,
+                                          const Put& put) {
+    constexpr int NL = Lanes<RC>::n, P = 9 + (SW ? 4 : 0) + (TH ? 4 : 0), HP = SW ? 13 : 9;
+#pragma unroll
+    for (int q = 0; q < P; ++q) {
+        R sg[NL], cg[NL], sh[NL], ch[NL], ct[NL];
+#pragma unroll
+        for (int l = 0; l < NL; ++l) {
+            int ql = q * NL + l, p = -1, how = 0;
+            if (k0 + l < G.nz) res_where<NL>(G, q, j, k0 + l, ql, p, how);
+            put(q, l, ql, p);
+            if (SW && q >= 9 && q < 13) res_through_g<R>(G, C, how, j, sg[l], cg[l]);
+            if (TH && q >= HP) res_through_h<R>(C, how, sh[l], ch[l], ct[l]);
+        }
+        const int m = (q - 9) & 3;
+        if (SW && q >= 9 && q < 13) {
+            L.sg[SW ? m : 0] = res_make<RC>(sg[0], sg[NL - 1]);
+            L.cg[SW ? m : 0] = res_make<RC>(cg[0], cg[NL - 1]);
+        }
+        if (TH && q >= HP) {
+            L.sh[TH ? m : 0] = res_make<RC>(sh[0], sh[NL - 1]);
+            L.ch[TH ? m : 0] = res_make<RC>(ch[0], ch[NL - 1]);
+            L.ct[TH ? m : 0] = res_make<RC>(ct[0], ct[NL - 1]);
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------- cluster
+
+__device__ __forceinline__ uint32_t res_mapa(uint32_t addr, uint32_t rank) {
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void res_dst(uint32_t a, float v) {
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
+}
+__device__ __forceinline__ void res_dst(uint32_t a, double v) {
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
+}
+__device__ __forceinline__ void res_dld(uint32_t a, float& v) {
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+}
+__device__ __forceinline__ void res_dld(uint32_t a, double& v) {
+    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(a) : "memory");
+}
+
+// One cluster of D.ncta CTAs, thread i of a CTA owning pair rank * chunk + i.
+// Shared memory: the force table, then the state [plane][lane][chunk].
+//
+// What bounds it: the latency of one step of one thread (slots, the chain of
+// the collision, barrier); the throughput of one scheduler for more pairs.
+// FP64: the FP64 pipe (64.5 cycles per warp instruction and scheduler,
+// whatever its active lanes).
+template <class R, bool SW, bool TH>
+__global__ void __launch_bounds__(kResThreads, 1)
+k_resident_cluster(const ResDom<R, R>* __restrict__ doms, Clock* clock, int nsteps, long long t0) {
+    using RC = typename PairArith<R>::type;
+    constexpr int NL = Lanes<RC>::n, P = nplanes<SW, TH>();
+    extern __shared__ __align__(16) unsigned char res_smem[];
+    const ResDom<R, R>& D = doms[0];
+    const Geom& G = D.G;
+    uint32_t nclust;
+    asm("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(nclust));
+    if ((int)nclust != D.ncta) {  // not launched as one cluster: nothing is touched
+        if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&clock->err, 1u);
+        return;
+    }
+    R* az_tab = reinterpret_cast<R*>(res_smem);
+    R* st = az_tab + kResAz;
+    const int tid = threadIdx.x, chunk = D.chunk, ncta = D.ncta, rank = blockIdx.x;
+    const int p = rank * chunk + tid;
+    const bool on = tid < chunk && p < D.npairs;
+    const int nr = G.nr, kp = on ? p / nr : 0, j = on ? p - kp * nr : 0, k0 = NL * kp;
+    const Coef<R> C = D.C;
+    R* const mine = st + tid;
+    uint32_t at[P][NL];
+    ResLinks<RC, SW, TH> L;
+    if (on) {  // natural-layout state into shared memory; the slots of odd steps
+#pragma unroll
+        for (int q = 0; q < P; ++q)
+#pragma unroll
+            for (int l = 0; l < NL; ++l) mine[(q * NL + l) * chunk] = k0 + l < G.nz ? *slot(D.pop, G, q, j, k0 + l) : R(0);
+        res_links<RC, R, SW, TH>(G, C, j, k0, L, [&](int q, int l, int ql, int sp) {
+            if (sp < 0) sp = p;
+            const int sr = sp / chunk, si = sp - sr * chunk;
+            at[q][l] = res_mapa(smem_u32(st) + (uint32_t)((ql * chunk + si) * sizeof(R)), sr);
+        });
+    }
+    const R inv_r = step_inv_radius<R>(G, j);
+    auto meet = [&]() {
+        if (ncta == 1) {
+            __syncthreads();
+        } else {
+            asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+        }
+    };
+    for (int s = 0; s < nsteps; ++s) {
+        if (s % kResAz == 0) {  // (the meeting that ended the last step has everybody past the old entries)
+            for (int i = tid; i < kResAz && s + i < nsteps; i += blockDim.x)
+                az_tab[i] = res_az<R>(D.az0, D.omega_t, t0 + s + i);
+            if (s == 0) meet();  // and the state of every CTA is in place
+            else __syncthreads();
+        }
+        if (on) {
+            const R az = az_tab[s % kResAz];
+            Cell<RC, SW, TH> c;
+            if ((s & 1) == 0) {  // even step: own slots, back into the opposite ones
+                res_load<RC, SW, TH, 0>(c, [&](int q, int l) { return mine[(q * NL + l) * chunk]; }, L);
+                c.collide(inv_r, C, az);
+                res_store<RC, SW, TH, 0>(c, [&](int q, int l, R v) { mine[(q * NL + l) * chunk] = v; }, L);
+            } else {
+                R v[P][NL];
+#pragma unroll
+                for (int q = 0; q < P; ++q)
+#pragma unroll
+                    for (int l = 0; l < NL; ++l) res_dld(at[q][l], v[q][l]);
+                res_load<RC, SW, TH, 1>(c, [&](int q, int l) { return v[q][l]; }, L);
+                c.collide(inv_r, C, az);
+                res_store<RC, SW, TH, 1>(c, [&](int q, int l, R x) { res_dst(at[q][l], x); }, L);
+            }
+        }
+        meet();
+    }
+    if (on) {
+#pragma unroll
+        for (int l = 0; l < NL; ++l) {
+            if (k0 + l >= G.nz) continue;
+#pragma unroll
+            for (int q = 0; q < P; ++q) *slot(D.pop, G, q, j, k0 + l) = mine[(q * NL + l) * chunk];
+        }
+    }
+    if (rank == 0 && tid == 0) {
+        res_finish(D, t0 + nsteps);
+        clock->t = t0 + nsteps;
+    }
+}
+
+// ---------------------------------------------------------------------------- grid, state in shared memory
+
+// A population on its way between two CTAs: the value and the step it is for
+// in one 8-byte word (FP64: two halves, each with the step), written and read
+// with relaxed 8-byte accesses.  The reader polls the word itself, so a hop
+// costs one store and one load of L2 (470-850 cycles one way on GB300, the
+// larger figure between the dies) where a flag behind a release costs 2600.
+// One word serves a slot in both directions: its owner and the node that uses
+// it in odd steps take turns.
+template <class R>
+struct ResWord;
+template <>
+struct ResWord<float> {
+    using type = unsigned long long;
+    __device__ static __forceinline__ void store(type* p, float v, unsigned step) {
+        const type w = ((type)step << 32) | __float_as_uint(v);
+        asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(w) : "memory");
+    }
+    __device__ static __forceinline__ type load(const type* p) {
+        type w;
+        asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(w) : "l"(p) : "memory");
+        return w;
+    }
+    __device__ static __forceinline__ bool is(type w, unsigned step) { return (unsigned)(w >> 32) == step; }
+    __device__ static __forceinline__ float value(type w) { return __uint_as_float((unsigned)w); }
+};
+template <>
+struct ResWord<double> {
+    using type = ulonglong2;
+    __device__ static __forceinline__ void store(type* p, double v, unsigned step) {
+        const unsigned long long b = (unsigned long long)__double_as_longlong(v), t = (unsigned long long)step << 32;
+        asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(p), "l"(t | (b & 0xffffffffull)),
+                     "l"(t | (b >> 32))
+                     : "memory");
+    }
+    __device__ static __forceinline__ type load(const type* p) {
+        type w;
+        asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(w.x), "=l"(w.y) : "l"(p) : "memory");
+        return w;
+    }
+    __device__ static __forceinline__ bool is(const type& w, unsigned step) {
+        return (unsigned)(w.x >> 32) == step && (unsigned)(w.y >> 32) == step;
+    }
+    __device__ static __forceinline__ double value(const type& w) {
+        return __longlong_as_double((long long)((w.y << 32) | (w.x & 0xffffffffull)));
+    }
+};
+
+// Shared memory of a CTA whose state sits there: the force table; the values
+// (its own slots [plane][lane][chunk], then copies of other CTAs' slots that
+// its nodes use in odd steps, the "ghosts"); per ghost this CTA's own slot
+// that the same neighbour uses, and the words of the two.
+template <class R>
+struct ResSlab {
+    R *az, *st;
+    int *own, *even, *odd;  // [max_ghost]
+    unsigned char* rest;
+    __device__ ResSlab(unsigned char* smem, int values, int max_ghost) {
+        az = reinterpret_cast<R*>(smem);
+        st = az + kResAz;
+        own = reinterpret_cast<int*>(st + values + max_ghost);
+        even = own + max_ghost;
+        odd = even + max_ghost;
+        rest = reinterpret_cast<unsigned char*>(odd + max_ghost);
+    }
+};
+template <class R, bool SW, bool TH>
+__host__ __device__ constexpr size_t res_slab_smem(int chunk, int max_ghost) {
+    return (kResAz + (size_t)nplanes<SW, TH>() * Lanes<typename PairArith<R>::type>::n * chunk + max_ghost) * sizeof(R) +
+           (size_t)max_ghost * 3 * sizeof(int);
+}
+
+// Words of a step into shared memory (PAR 0: the CTA's own slots, 1: the
+// ghosts), a thread's polls all in flight together; a poll gives up after
+// kResWait cycles, or when another CTA has.
+template <class R, int PAR>
+__device__ __forceinline__ void res_gather(const ResSlab<R>& S, const typename ResWord<R>::type* mail, int gbase, int ng,
+                                           unsigned want, Clock* clock, int* bad) {
+    using W = ResWord<R>;
+    constexpr int U = sizeof(R) == 4 ? 8 : 4;
+    const int T = blockDim.x;
+    for (int g0 = threadIdx.x; g0 < ng; g0 += U * T) {
+        typename W::type w[U];
+        int from[U];
+        unsigned miss = 0;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            from[u] = 0;
+            if (g0 + u * T < ng) {
+                from[u] = (PAR ? S.odd : S.even)[g0 + u * T];
+                miss |= 1u << u;
+            }
+        }
+        const long long w0 = clock64();
+        for (int tries = 0; miss; ++tries) {
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if ((miss >> u) & 1u) w[u] = W::load(mail + from[u]);
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (((miss >> u) & 1u) && W::is(w[u], want)) {
+                    S.st[PAR ? gbase + g0 + u * T : S.own[g0 + u * T]] = W::value(w[u]);
+                    miss &= ~(1u << u);
+                }
+            if ((tries & 255) == 255) {
+                const bool late = clock64() - w0 > kResWait;
+                if (late || *reinterpret_cast<volatile int*>(bad) || *reinterpret_cast<volatile unsigned*>(&clock->err)) {
+                    if (late) atomicOr(&clock->err, 1u);
+                    *bad = 1;
+                    break;
+                }
+            }
+        }
+    }
+}
+// The step's results that belong to other CTAs (odd) or that they use next (even).
+template <class R, int PAR>
+__device__ __forceinline__ void res_scatter(const ResSlab<R>& S, typename ResWord<R>::type* mail, int gbase, int ng,
+                                            unsigned step) {
+    for (int g = threadIdx.x; g < ng; g += blockDim.x)
+        ResWord<R>::store(mail + (PAR ? S.odd : S.even)[g], S.st[PAR ? gbase + g : S.own[g]], step);
+}
+
+// A lane's slot in another CTA becomes a ghost: its number (consecutive within
+// the warp, so that copies and words lie side by side), or -1.
+__device__ __forceinline__ int res_new_ghost(bool remote, int* count) {
+    const unsigned act = __activemask(), m = __ballot_sync(act, remote);
+    const int lane = threadIdx.x & 31, first = __ffs(m) - 1;
+    int g = 0;
+    if (remote && lane == first) g = atomicAdd(count, __popc(m));
+    if (m) g = __shfl_sync(act, g, first);
+    return remote ? g + __popc(m & ((1u << lane) - 1u)) : -1;
+}
+
+// The common part of the kernels that keep the state in shared memory: loads
+// it, runs nsteps steps of update(par, force), each between the words of its
+// neighbours coming in and going out, and writes it back.
+template <class R, bool SW, bool TH, class Update>
+__device__ __forceinline__ void res_slab_run(const ResDom<R, R>& D, const ResSlab<R>& S, Clock* clock, int nsteps,
+                                             unsigned epoch, long long t0, int ng, int* bad, const Update& update) {
+    constexpr int NL = Lanes<typename PairArith<R>::type>::n, PL = nplanes<SW, TH>() * NL;
+    const Geom& G = D.G;
+    const int tid = threadIdx.x, T = blockDim.x, chunk = D.chunk, nr = G.nr;
+    const int rank = blockIdx.x - D.cta0, p0 = rank * chunk, n = min(chunk, D.npairs - p0), gbase = PL * chunk;
+    auto* mail = static_cast<typename ResWord<R>::type*>(D.mail);
+    auto step = [&](auto par_tag, int s) {
+        constexpr int PAR = decltype(par_tag)::value;
+        if (s > 0 && ng > 0) {
+            res_gather<R, PAR>(S, mail, gbase, ng, epoch + (unsigned)s, clock, bad);
+            __syncthreads();
+        }
+        update(par_tag, S.az[s % kResAz]);
+        __syncthreads();
+        if (ng > 0) res_scatter<R, PAR>(S, mail, gbase, ng, epoch + (unsigned)s + 1u);
+    };
+    int stop = __syncthreads_or(*bad);
+    for (int s = 0; s < nsteps && !stop; s += 2) {
+        if (s % kResAz == 0) {
+            for (int i = tid; i < kResAz && s + i < nsteps; i += T) S.az[i] = res_az<R>(D.az0, D.omega_t, t0 + s + i);
+            __syncthreads();
+        }
+        step(std::integral_constant<int, 0>{}, s);
+        step(std::integral_constant<int, 1>{}, s + 1);
+        // (a wait that gives up ends the loop for the whole CTA: looked at rarely, and after the last step)
+        if ((s & 62) == 62) stop = __syncthreads_or(*bad);
+    }
+    if (!stop && ng > 0) res_gather<R, 0>(S, mail, gbase, ng, epoch + (unsigned)nsteps, clock, bad);
+    if (__syncthreads_or(*bad)) {
+        if (tid == 0) atomicOr(&clock->err, 1u);
+        return;
+    }
+    for (int m = tid; m < PL * n; m += T) {
+        const int ql = m / n, i = m - ql * n, p = p0 + i, kp = p / nr, j = p - kp * nr, k = NL * kp + ql % NL;
+        if (k < G.nz) *slot(D.pop, G, ql / NL, j, k) = S.st[ql * chunk + i];
+    }
+    if (rank == 0 && tid == 0) res_finish(D, t0 + nsteps);
+    if (blockIdx.x == 0 && tid == 0) clock->t = t0 + nsteps;
+}
+
+// One pair per thread: addresses and links stay in registers.
+template <class R, bool SW, bool TH>
+__device__ __forceinline__ void res_one_cta(const ResDom<R, R>& D, Clock* clock, int nsteps, unsigned epoch, long long t0,
+                                            int max_ghost, unsigned char* smem) {
+    using RC = typename PairArith<R>::type;
+    constexpr int NL = Lanes<RC>::n, P = nplanes<SW, TH>();
+    __shared__ int ghosts, bad;
+    const Geom& G = D.G;
+    const Coef<R> C = D.C;
+    const int tid = threadIdx.x, chunk = D.chunk, nr = G.nr, np = D.npairs;
+    const int p0 = (blockIdx.x - D.cta0) * chunk, n = min(chunk, np - p0), gbase = P * NL * chunk;
+    const ResSlab<R> S(smem, gbase, max_ghost);
+    if (tid == 0) ghosts = bad = 0;
+    __syncthreads();
+    const bool on = tid < n;
+    const int p = p0 + (on ? tid : 0), kp = p / nr, j = p - kp * nr, k0 = NL * kp;
+    R* const mine = S.st + tid;
+    int at[P][NL];
+    ResLinks<RC, SW, TH> L;
+    if (tid < res_up32(n)) {  // whole warps
+        res_links<RC, R, SW, TH>(G, C, j, k0, L, [&](int q, int l, int ql, int sp) {
+            const bool local = sp >= p0 && sp < p0 + n;
+            const int g = res_new_ghost(on && sp >= 0 && !local, &ghosts);
+            at[q][l] = sp < 0 ? (q * NL + l) * chunk + tid : (g < 0 ? ql * chunk + (local ? sp - p0 : 0) : gbase + g);
+            if (g >= max_ghost) {
+                bad = 2;
+                at[q][l] = gbase;
+            } else if (g >= 0) {
+                S.own[g] = (q * NL + l) * chunk + tid;
+                S.even[g] = (q * NL + l) * np + p;
+                S.odd[g] = ql * np + sp;
+            }
+            if (on) mine[(q * NL + l) * chunk] = k0 + l < G.nz ? *slot(D.pop, G, q, j, k0 + l) : R(0);
+        });
+    }
+    __syncthreads();
+    const R inv_r = step_inv_radius<R>(G, j);
+    res_slab_run<R, SW, TH>(D, S, clock, nsteps, epoch, t0, min(ghosts, max_ghost), &bad, [&](auto par_tag, R az) {
+        constexpr int PAR = decltype(par_tag)::value;
+        if (!on) return;
+        Cell<RC, SW, TH> c;
+        if (PAR == 0) {
+            res_load<RC, SW, TH, 0>(c, [&](int q, int l) { return mine[(q * NL + l) * chunk]; }, L);
+            c.collide(inv_r, C, az);
+            res_store<RC, SW, TH, 0>(c, [&](int q, int l, R v) { mine[(q * NL + l) * chunk] = v; }, L);
+        } else {
+            res_load<RC, SW, TH, 1>(c, [&](int q, int l) { return S.st[at[q][l]]; }, L);
+            c.collide(inv_r, C, az);
+            res_store<RC, SW, TH, 1>(c, [&](int q, int l, R v) { S.st[at[q][l]] = v; }, L);
+        }
+    });
+}
+
+// Cooperative grid, one CTA per SM, one pair per thread; CTA b works for
+// domain cta_dom[b].
+//
+// What bounds it: the latency of a step -- the neighbours' words (a store and
+// a polled load of L2), one node's chain, two barriers.
+template <class R, bool SW, bool TH>
+__global__ void __launch_bounds__(kResThreads, 1)
+k_resident_one(const ResDom<R, R>* __restrict__ doms, const int* __restrict__ cta_dom, Clock* clock, int nsteps,
+               unsigned epoch, long long t0, int max_ghost, int) {
+    extern __shared__ __align__(16) unsigned char res_smem[];
+    const ResDom<R, R>& D = doms[cta_dom[blockIdx.x]];
+    if (TH && D.th) res_one_cta<R, SW, TH>(D, clock, nsteps, epoch, t0, max_ghost, res_smem);
+    else res_one_cta<R, SW, false>(D, clock, nsteps, epoch, t0, max_ghost, res_smem);
+}
+
+constexpr int kResSlabThreads = 384;
+
+// A pair of the kernel below: bit 30 of i: the second lane is empty; tab: its
+// row of the slot table, or -1 where every slot is the CTA's own and away
+// from the outline.
+template <class R>
+struct ResPair {
+    R inv_r;
+    int i, tab;
+};
+// A row of the slot table: where population (q, l) is pulled from in an odd
+// step (index into the values), then the links.
+template <class R, bool SW, bool TH>
+__host__ __device__ constexpr size_t res_row_bytes() {
+    return Lanes<typename PairArith<R>::type>::n *
+           (nplanes<SW, TH>() * sizeof(int) + ((SW ? 8 : 0) + (TH ? 12 : 0)) * sizeof(R));
+}
+
+// Several pairs per thread.
+template <class R, bool SW, bool TH>
+__device__ __forceinline__ void res_slab_cta(const ResDom<R, R>& D, Clock* clock, int nsteps, unsigned epoch, long long t0,
+                                             int max_ghost, int max_tab, unsigned char* smem) {
+    using RC = typename PairArith<R>::type;
+    constexpr int NL = Lanes<RC>::n, P = nplanes<SW, TH>(), PL = P * NL, NF = (SW ? 8 : 0) + (TH ? 12 : 0);
+    __shared__ int ghosts, bad, rows;
+    const Geom& G = D.G;
+    const Coef<R> C = D.C;
+    const int tid = threadIdx.x, T = blockDim.x, chunk = D.chunk, nr = G.nr, np = D.npairs;
+    const int p0 = (blockIdx.x - D.cta0) * chunk, n = min(chunk, np - p0), gbase = PL * chunk;
+    const ResSlab<R> S(smem, gbase, max_ghost);
+    ResPair<R>* pairs = reinterpret_cast<ResPair<R>*>(S.rest + (sizeof(R) == 8 ? (max_ghost & 1) * 4 : 0));
+    R* tf = reinterpret_cast<R*>(pairs + chunk);  // [NF][NL][max_tab]: sg, cg, then sh, ch, ct, four each
+    int* tab = reinterpret_cast<int*>(tf + NF * NL * max_tab);  // [P][NL][max_tab]
+    if (tid == 0) ghosts = bad = 0;
+    __syncthreads();
+    // pairs in order, those with a row of the table last (a warp's slots and words then lie side by side)
+    if (tid < 32) {
+        int plain = 0;
+        for (int pass = 0; pass < 2; ++pass) {
+            int at0 = 0, at1 = plain;
+            for (int i0 = 0; i0 < n; i0 += 32) {
+                const int i = i0 + tid, p = p0 + i, kp = p / nr, j = p - kp * nr;
+                const bool two = NL == 2 && NL * kp + 1 < G.nz;
+                const bool ring = j == 0 || j == nr - 1 || kp == 0 || NL * kp + (two ? 1 : 0) == G.nz - 1;
+                const bool row = ring || i < nr + 1 || i + nr + 1 >= n;
+                const unsigned m0 = __ballot_sync(0xffffffffu, i < n && !row), m1 = __ballot_sync(0xffffffffu, i < n && row);
+                if (pass && i < n) {
+                    ResPair<R> r;
+                    r.inv_r = step_inv_radius<R>(G, j);
+                    r.i = i;
+                    const int to = row ? at1 + __popc(m1 & ((1u << tid) - 1u)) : at0 + __popc(m0 & ((1u << tid) - 1u));
+                    r.tab = row ? to - plain : -1;
+                    pairs[to] = r;
+                }
+                at0 += __popc(m0);
+                at1 += __popc(m1);
+            }
+            if (!pass) plain = at0;
+        }
+        if (tid == 0) {
+            rows = n - plain;
+            if (rows > max_tab) bad = 2;
+        }
+    }
+    __syncthreads();
+    const int nt = rows, n0 = n - nt;
+    if (!bad) {
+        const int blocks = (nt + 31) / 32, lane = tid & 31;
+        for (int w = tid >> 5; w < blocks * PL; w += T >> 5) {  // 32 pairs of one population and lane
+            const int x = w / blocks, t = (w - x * blocks) * 32 + lane, q = x / NL, l = x - q * NL;
+            const bool on = t < nt;
+            const int i = pairs[n0 + (on ? t : 0)].i, p = p0 + i, kp = p / nr, j = p - kp * nr, k = NL * kp + l;
+            int ql = x, sp = p, how = 0;  // (a lane without a node keeps to itself)
+            if (k < G.nz) res_where<NL>(G, q, j, k, ql, sp, how);
+            const bool local = sp >= p0 && sp < p0 + n;
+            const int g = res_new_ghost(on && !local, &ghosts);
+            int e = local ? ql * chunk + (sp - p0) : gbase + g;
+            if (g >= max_ghost) {
+                bad = 2;
+                e = gbase;
+            } else if (g >= 0) {
+                S.own[g] = x * chunk + i;
+                S.even[g] = x * np + p;
+                S.odd[g] = ql * np + sp;
+            }
+            if (on) {
+                tab[x * max_tab + t] = e;
+                const int m = (q - 9) & 3;
+                R* f = tf + l * max_tab + t;
+                
+                if (SW && q >= 9 && q < 13) {
+                    R sg, cg;
+                    res_through_g<R>(G, C, how, j, sg, cg);
+                    f[m * NL * max_tab] = sg;
+                    f[(4 + m) * NL * max_tab] = cg;
+                }
+                if (TH && q >= (SW ? 13 : 9)) {
+                    R sh, ch, ct;
+                    res_through_h<R>(C, how, sh, ch, ct);
+                    constexpr int B = SW ? 8 : 0;
+                    f[(B + m) * NL * max_tab] = sh;
+                    f[(B + 4 + m) * NL * max_tab] = ch;
+                    f[(B + 8 + m) * NL * max_tab] = ct;
+                }
+            }
+        }
+    }
+    for (int m = tid; m < PL * n; m += T) {  // the state, natural layout
+        const int ql = m / n, i = m - ql * n, p = p0 + i, kp = p / nr, j = p - kp * nr, k = NL * kp + ql % NL;
+        S.st[ql * chunk + i] = k < G.nz ? *slot(D.pop, G, ql / NL, j, k) : R(0);
+    }
+    __syncthreads();
+    // links read from the table where they are used
+    struct TabLinks {
+        const R* f;
+        int stride;
+        __device__ __forceinline__ RC of(int x) const {
+            return res_make<RC>(f[x * NL * stride], f[(x * NL + NL - 1) * stride]);
+        }
+        __device__ __forceinline__ RC g(int q, RC v) const { return fmaR(v, of(q), of(4 + q)); }
+        __device__ __forceinline__ RC h(int q, RC v) const {
+            constexpr int B = SW ? 8 : 0;
+            return fmaR(v, of(B + q), of(B + 4 + q)) + of(B + 8 + q);
+        }
+    };
+    res_slab_run<R, SW, TH>(D, S, clock, nsteps, epoch, t0, min(ghosts, max_ghost), &bad, [&](auto par_tag, R az) {
+        constexpr int PAR = decltype(par_tag)::value;
+        for (int m = tid; m < n; m += T) {
+            const ResPair<R> r = pairs[m];
+            R* const mine = S.st + r.i;
+            // index (from `mine`) of the slot of population q, lane l, in an odd step without a table row
+            auto inside = [&](int q, int l) {
+                const int er = q < 9 ? cr9(q) : cr4((q - 9) & 3), ez = q < 9 ? cz9(q) : cz4((q - 9) & 3);
+                const int pl = q < 9 ? opp9(q) : 9 + ((q - 9) & ~3) + opp4((q - 9) & 3);
+                if (NL == 1) return pl * chunk - ez * nr - er;
+                const int row = l - ez;  // -1, 0, 1, 2: of the pair below, this pair, this pair, the pair above
+                return (pl * NL + (row & 1)) * chunk + (row < 0 ? -nr : (row > 1 ? nr : 0)) - er;
+            };
+            const TabLinks tl{tf + r.tab, max_tab};
+            struct NoLinks {
+                __device__ __forceinline__ RC g(int, RC v) const { return v; }
+                __device__ __forceinline__ RC h(int, RC v) const { return v; }
+            } none;
+            const int* e = tab + r.tab;
+            Cell<RC, SW, TH> c;
+            if (PAR == 0) res_load<RC, SW, TH, 0>(c, [&](int q, int l) { return mine[(q * NL + l) * chunk]; }, none);
+            else if (r.tab < 0) res_load<RC, SW, TH, 1>(c, [&](int q, int l) { return mine[inside(q, l)]; }, none);
+            else res_load<RC, SW, TH, 1>(c, [&](int q, int l) { return S.st[e[(q * NL + l) * max_tab]]; }, tl);
+            c.collide(r.inv_r, C, az);
+            if (PAR == 0) res_store<RC, SW, TH, 0>(c, [&](int q, int l, R v) { mine[(q * NL + l) * chunk] = v; }, none);
+            else if (r.tab < 0) res_store<RC, SW, TH, 1>(c, [&](int q, int l, R v) { mine[inside(q, l)] = v; }, none);
+            else res_store<RC, SW, TH, 1>(c, [&](int q, int l, R v) { S.st[e[(q * NL + l) * max_tab]] = v; }, tl);
+        }
+    });
+}
+
+// Cooperative grid, one CTA per SM, several pairs per thread.
+//
+// What bounds it: instruction issue (FP32) or the FP64 pipe.
+template <class R, bool SW, bool TH>
+__global__ void __launch_bounds__(kResSlabThreads, 1)
+k_resident_slab(const ResDom<R, R>* __restrict__ doms, const int* __restrict__ cta_dom, Clock* clock, int nsteps,
+                unsigned epoch, long long t0, int max_ghost, int max_tab) {
+    extern __shared__ __align__(16) unsigned char res_smem[];
+    const ResDom<R, R>& D = doms[cta_dom[blockIdx.x]];
+    if (TH && D.th) res_slab_cta<R, SW, TH>(D, clock, nsteps, epoch, t0, max_ghost, max_tab, res_smem);
+    else res_slab_cta<R, SW, false>(D, clock, nsteps, epoch, t0, max_ghost, max_tab, res_smem);
+}
+
+// ---------------------------------------------------------------------------- grid, state in L2
+
+// Shared memory of a grid CTA: the force table, a record per pair, and for
+// the pairs with a node on the domain's outline the slots of odd steps.
+template <class R>
+struct ResRec {
+    R inv_r;
+    int x;     // offset of the pair's first node in a plane; bit 30: the second lane is empty
+    int ring;  // entry of the outline table, or -1
+};
+constexpr int kResHowShift = 28;   // an outline entry: offset below, ResSlot::how above
+constexpr int kResOff = (1 << kResHowShift) - 1;
+
+template <class R, bool SW, bool TH>
+__host__ __device__ constexpr size_t res_ring_bytes() {
+    return Lanes<typename PairArith<R>::type>::n * (nplanes<SW, TH>() * sizeof(int) + (SW ? 4 * sizeof(R) : 0));
+}
+template <class R, bool SW, bool TH>
+__host__ __device__ constexpr size_t res_grid_smem(int chunk, int max_ring) {
+    return kResAz * sizeof(R) + (size_t)chunk * sizeof(ResRec<R>) + (size_t)max_ring * res_ring_bytes<R, SW, TH>();
+}
+
+__device__ __forceinline__ unsigned res_ld_acquire(const unsigned* p) {
+    unsigned v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void res_st_release(unsigned* p, unsigned v) {
+    asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+
+template <class R>
+__device__ __forceinline__ R res_ring_g(R v, int how, R cg) {
+    return how == 0 ? v : (how == 1 ? -v : cg - v);
+}
+template <class R>
+__device__ __forceinline__ R res_ring_h(R v, int how, const Coef<R>& C) {
+    return how < 2 ? v : bounce_h(C, how - 2, v);
+}
+
+// One step of the CTA's pairs.  PAR 1: an odd step (neighbours' slots).
+template <class S, class R, bool SW, bool TH, int PAR>
+__device__ __forceinline__ void res_grid_step(const ResDom<S, R>& D, const Coef<R>& C, const ResRec<R>* rec, int n,
+                                              const int* ring_at, const R* ring_cg, R az) {
+    using RC = typename PairArith<R>::type;
+    constexpr int NL = Lanes<RC>::n, P = nplanes<SW, TH>(), HP = SW ? 13 : 9;
+    const int plane = (int)D.G.plane, pitch = (int)D.G.pitch;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        const ResRec<R> r = rec[i];
+        const bool two = NL == 2 && !(r.x & (1 << 30));
+        S* const base = D.pop + (r.x & ~(1 << 30));
+        const int row1 = two ? pitch : 0;  // an empty lane repeats the first one's node (never stored)
+        const bool ring = PAR == 1 && r.ring >= 0;
+        const int* at = ring_at + r.ring * (P * NL);
+        const R* cg = ring_cg + r.ring * (4 * NL);
+        // offset from `base` of the slot of plane-ordered population q in an odd step, away from the outline
+        auto inside = [&](int q) {
+            const int er = q < 9 ? cr9(q) : cr4((q - 9) & 3), ez = q < 9 ? cz9(q) : cz4((q - 9) & 3);
+            const int pl = q < 9 ? opp9(q) : 9 + ((q - 9) & ~3) + opp4((q - 9) & 3);
+            return pl * plane - ez * pitch - er;
+        };
+        R v[P][NL];
+        if (PAR == 0) {
+#pragma unroll
+            for (int q = 0; q < P; ++q)
+#pragma unroll
+                for (int l = 0; l < NL; ++l) v[q][l] = __ldcg(base + (q * plane + l * row1));
+        } else if (!ring) {
+#pragma unroll
+            for (int q = 0; q < P; ++q)
+#pragma unroll
+                for (int l = 0; l < NL; ++l) v[q][l] = __ldcg(base + (inside(q) + l * row1));
+        } else {
+#pragma unroll
+            for (int q = 0; q < P; ++q)
+#pragma unroll
+                for (int l = 0; l < NL; ++l) v[q][l] = __ldcg(D.pop + (at[q * NL + l] & kResOff));
+#pragma unroll
+            for (int q = 9; q < P; ++q)
+#pragma unroll
+                for (int l = 0; l < NL; ++l) {
+                    const int how = (unsigned)at[q * NL + l] >> kResHowShift;
+                    v[q][l] = SW && q < 13 ? res_ring_g<R>(v[q][l], how, cg[(q - 9) * NL + l])
+                                           : res_ring_h<R>(v[q][l], how, C);
+                }
+        }
+        Cell<RC, SW, TH> c;
+#pragma unroll
+        for (int a = 0; a < 9; ++a) c.d[a] = res_make<RC>(v[a][0], v[a][NL - 1]);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            if (SW) c.g[q] = res_make<RC>(v[9 + q][0], v[9 + q][NL - 1]);
+            if (TH) c.h[q] = res_make<RC>(v[HP + q][0], v[HP + q][NL - 1]);
+        }
+        c.collide(r.inv_r, C, az);
+        // slot q takes the opposite population (even steps: of the node itself)
+#pragma unroll
+        for (int l = 0; l < NL; ++l) {
+            if (l && !two) continue;
+            if (!ring) {
+#pragma unroll
+                for (int q = 0; q < P; ++q) {
+                    const RC x = q < 9 ? c.d[opp9(q)] : (SW && q < 13 ? c.g[opp4((q - 9) & 3)] : c.h[opp4((q - 9) & 3)]);
+                    S* to = base + ((PAR ? inside(q) : q * plane) + l * row1);
+                    *to = (S)Lanes<RC>::get(x, l);
+                }
+            } else {
+#pragma unroll
+                for (int q = 0; q < P; ++q) {
+                    const int e = at[q * NL + l], how = (unsigned)e >> kResHowShift;
+                    const RC x = q < 9 ? c.d[opp9(q)] : (SW && q < 13 ? c.g[opp4((q - 9) & 3)] : c.h[opp4((q - 9) & 3)]);
+                    R y = Lanes<RC>::get(x, l);
+                    if (SW && q >= 9 && q < 13) y = res_ring_g<R>(y, how, cg[(q - 9) * NL + l]);
+                    if (TH && q >= HP) y = res_ring_h<R>(y, how, C);
+                    D.pop[e & kResOff] = (S)y;
+                }
+            }
+        }
+    }
+}
+
+// The work of one CTA: a contiguous range of pairs of domain D.
+template <class S, class R, bool SW, bool TH>
+__device__ __forceinline__ void res_grid_cta(const ResDom<S, R>& D, unsigned* flags, Clock* clock, int nsteps,
+                                             unsigned epoch, long long t0, unsigned char* smem) {
+    using RC = typename PairArith<R>::type;
+    constexpr int NL = Lanes<RC>::n, P = nplanes<SW, TH>();
+    __shared__ int n_ring, abort_flag;
+    const Geom& G = D.G;
+    const Coef<R> C = D.C;
+    const int tid = threadIdx.x, chunk = D.chunk, nr = G.nr;
+    const int rank = blockIdx.x - D.cta0;
+    const int p0 = rank * chunk, n = min(chunk, D.npairs - p0);
+    R* az_tab = reinterpret_cast<R*>(smem);
+    ResRec<R>* rec = reinterpret_cast<ResRec<R>*>(az_tab + kResAz);
+    if (tid == 0) n_ring = abort_flag = 0;
+    __syncthreads();
+    for (int i = tid; i < n; i += blockDim.x) {
+        const int p = p0 + i, kp = p / nr, j = p - kp * nr, k = NL * kp;
+        const bool two = NL == 2 && k + 1 < G.nz;
+        ResRec<R> r;
+        r.inv_r = step_inv_radius<R>(G, j);
+        r.x = (int)((long long)(G.row0 + k) * G.pitch + G.col0 + j) | (NL == 2 && !two ? 1 << 30 : 0);
+        r.ring = j == 0 || j == nr - 1 || k == 0 || k + (two ? 1 : 0) == G.nz - 1 ? atomicAdd(&n_ring, 1) : -1;
+        rec[i] = r;
+    }
+    __syncthreads();
+    // outline table: the slots, and rho0 u_w / 2 where a g population meets a wall
+    R* ring_cg = reinterpret_cast<R*>(rec + chunk);
+    int* ring_at = reinterpret_cast<int*>(ring_cg + (SW ? n_ring * 4 * NL : 0));
+    for (int i = tid; i < n; i += blockDim.x) {
+        const int e = rec[i].ring;
+        if (e < 0) continue;
+        const int p = p0 + i, kp = p / nr, j = p - kp * nr;
+        for (int l = 0; l < NL; ++l) {
+            const int k = NL * kp + l < G.nz ? NL * kp + l : NL * kp;
+            for (int q = 0; q < P; ++q) {
+                const ResSlot s = q < 9 ? res_slot9(G, q, j, k) : res_slot4(G, (q - 9) & 3, j, k);
+                const int plane = q < 9 ? s.plane : 9 + ((q - 9) & ~3) + s.plane;
+                ring_at[(e * P + q) * NL + l] = (int)(slot(D.pop, G, plane, s.j, s.k) - D.pop) | (s.how << kResHowShift);
+                if (SW && q >= 9 && q < 13)
+                    ring_cg[(e * 4 + (q - 9)) * NL + l] =
+                        s.how >= 2 ? mul_rn(R(0.5) * C.rho0, wall_uth(G, C, s.how - 2, j)) : R(0);
+            }
+        }
+    }
+    // the CTAs this one meets: owners of pairs within one node of its range,
+    // and across periodic ends
+    const int last = D.npairs - 1;
+    const int a0 = max(p0 - nr - 1, 0) / chunk, a1 = min(p0 + n + nr, last) / chunk;
+    int b0 = 0, b1 = -1, c0 = 0, c1 = -1;
+    if (G.z_lo == AXLBM_Z_PERIODIC) {
+        if (p0 <= nr) b0 = max(last - 2 * nr, 0) / chunk, b1 = last / chunk;
+        if (p0 + n - 1 >= last - nr) c0 = 0, c1 = min(2 * nr, last) / chunk;
+    }
+    const int na = a1 - a0 + 1, nb = b1 - b0 + 1, nc = c1 - c0 + 1, nmeet = na + nb + nc;
+    const unsigned* dom_flags = flags + (long long)D.cta0 * kResPad;
+    unsigned* my_flag = flags + (long long)blockIdx.x * kResPad;
+    for (int s = 0; s < nsteps; ++s) {
+        if (s % kResAz == 0) {
+            __syncthreads();
+            for (int i = tid; i < kResAz && s + i < nsteps; i += blockDim.x)
+                az_tab[i] = res_az<R>(D.az0, D.omega_t, t0 + s + i);
+        }
+        if (s > 0 && tid < 32) {
+            const unsigned want = epoch + (unsigned)s;
+            for (int m = tid; m < nmeet; m += 32) {
+                const int c = m < na ? a0 + m : (m < na + nb ? b0 + (m - na) : c0 + (m - na - nb));
+                if (c == rank) continue;
+                const unsigned* f = dom_flags + (long long)c * kResPad;
+                if ((int)(res_ld_acquire(f) - want) >= 0) continue;
+                const long long w0 = clock64();
+                int tries = 0;
+                while ((int)(res_ld_acquire(f) - want) < 0) {
+                    if (clock64() - w0 > kResWait ||
+                        ((++tries & 1023) == 0 && *reinterpret_cast<volatile unsigned*>(&clock->err) != 0u)) {
+                        abort_flag = 1;
+                        break;
+                    }
+                }
+            }
+        }
+        __syncthreads();
+        if (abort_flag) break;
+        const R az = az_tab[s % kResAz];
+        if ((s & 1) == 0) res_grid_step<S, R, SW, TH, 0>(D, C, rec, n, ring_at, ring_cg, az);
+        else res_grid_step<S, R, SW, TH, 1>(D, C, rec, n, ring_at, ring_cg, az);
+        __syncthreads();
+        if (tid == 0) {
+            res_st_release(my_flag, epoch + (unsigned)s + 1u);
+        }
+    }
+    if (abort_flag) {
+        if (tid == 0) atomicOr(&clock->err, 1u);
+        return;
+    }
+    if (rank == 0 && tid == 0) res_finish(D, t0 + nsteps);
+    if (blockIdx.x == 0 && tid == 0) clock->t = t0 + nsteps;
+}
+
+// Cooperative grid; CTA b works for domain cta_dom[b].
+//
+// What bounds it: for few pairs per CTA the latency of a step -- the slots
+// from L2, the collision's chain, a fence, a release store and the
+// neighbours' polls; for many, instruction issue (FP32) or the FP64 pipe.
+template <class S, class R, bool SW, bool TH>
+__global__ void __launch_bounds__(kResThreads, 2)
+k_resident_grid(const ResDom<S, R>* __restrict__ doms, const int* __restrict__ cta_dom, unsigned* flags, Clock* clock,
+                int nsteps, unsigned epoch, long long t0) {
+    extern __shared__ __align__(16) unsigned char res_smem[];
+    const ResDom<S, R>& D = doms[cta_dom[blockIdx.x]];
+    if (TH && D.th) res_grid_cta<S, R, SW, true>(D, flags, clock, nsteps, epoch, t0, res_smem);
+    else res_grid_cta<S, R, SW, false>(D, flags, clock, nsteps, epoch, t0, res_smem);
+}
+
+}  // namespace axl

@@ -1,0 +1,250 @@
+// resident_ops.cuh -- which domains run on the multi-step kernels, and their launches.
+#pragma once
+
+#include <algorithm>
+
+#include "resident.cuh"
+
+namespace axl {
+
+// Populations that a grid keeps in L2 between steps: beyond this the step
+// kernels, which stream them through shared memory by TMA, are faster.
+constexpr size_t kResMaxBytes = 64u << 20;
+constexpr int kResSmemMax = 224 << 10;  // dynamic shared memory of a CTA (half of it with two CTAs per SM)
+constexpr int kResClusterMax = 8;  // CTAs of a portable cluster
+
+// Pairs of CTA [p0, p1) with a node on the outline of an nr x nz domain (nl nodes per pair).
+inline int res_ring_pairs(int p0, int p1, int nr, int nz, int nl) {
+    const int last = (nz - 1) / nl;
+    int count = 0;
+    for (int kp = p0 / nr; kp * (long long)nr < p1; ++kp) {
+        const int ja = std::max(p0 - kp * nr, 0), jb = std::min(p1 - kp * nr, nr) - 1;
+        if (kp == 0 || kp == last) count += jb - ja + 1;
+        else count += (ja == 0) + (jb == nr - 1 && nr > 1);
+    }
+    return count;
+}
+
+// The slab form's tables for CTA [p0, p1): pairs on the outline or within a row of the CTA's ends, and at most
+// how many of their slots other CTAs own (outline pairs counted on the safe side: a link may be mirrored or wrapped).
+inline void res_slab_tables(int p0, int p1, int nr, int nz, int nl, bool sw, bool th, int* pairs, int* ghosts) {
+    const int n = p1 - p0, planes = 9 + (sw ? 4 : 0) + (th ? 4 : 0);
+    *pairs = *ghosts = 0;
+    for (int i = 0; i < n; ++i) {
+        const int p = p0 + i, kp = p / nr, j = p - kp * nr;
+        const bool two = nl == 2 && nl * kp + 1 < nz;
+        const bool ring = j == 0 || j == nr - 1 || kp == 0 || nl * kp + (two ? 1 : 0) == nz - 1;
+        if (!ring && i >= nr + 1 && i + nr + 1 < n) continue;
+        *pairs += 1;
+        for (int q = 1; q < planes; ++q) {
+            const int er = q < 9 ? cr9(q) : cr4((q - 9) & 3), ez = q < 9 ? cz9(q) : cz4((q - 9) & 3);
+            for (int l = 0; l < (two ? 2 : 1); ++l) {
+                const int row = l - ez;
+                const int at = i + (nl == 1 ? -ez * nr : (row < 0 ? -nr : (row > 1 ? nr : 0)));
+                bool out = at - er < 0 || at - er >= n;
+                if (ring) out = out || at - 1 < 0 || at + 1 >= n || (nl == 2 && !two && ez < 0);
+                *ghosts += out;
+            }
+        }
+    }
+}
+
+template <class R>
+int res_lanes() { return std::is_same<R, float>::value ? 2 : 1; }
+
+template <class S, bool SW, bool TH>
+cudaError_t res_build(Resident* r, const ResidentDomain* d, int n, int num_sms, cudaStream_t stream) {
+    using R = S;
+    const int nl = res_lanes<R>();
+    size_t state = 0;
+    long long pairs = 0;
+    std::vector<ResDom<S, R>> doms(n);
+    for (int i = 0; i < n; ++i) {
+        const ResidentDomain& x = d[i];
+        const Geom& G = x.G;
+        // grids whose steps end with passes of their own (wet walls, Zou-He walls, the mirror column) and
+        // cut domains keep the step kernels
+        if (G.inner == AXLBM_INNER_AXIS_NODE || G.outer != AXLBM_OUTER_BB || G.z_lo == AXLBM_Z_NEE ||
+            G.z_hi == AXLBM_Z_NEE || G.z_lo == AXLBM_Z_HALO || G.z_hi == AXLBM_Z_HALO)
+            return cudaSuccess;
+        const int planes = 9 + (SW ? 4 : 0) + (TH ? 4 : 0);
+        if (planes * G.plane >= (1ll << kResHowShift)) return cudaSuccess;  // offsets of the outline table
+        state += (size_t)G.nr * G.nz * (9 + (SW ? 4 : 0) + (x.th ? 4 : 0)) * sizeof(S);
+        const long long np = (long long)((G.nz + nl - 1) / nl) * G.nr;
+        if (state > kResMaxBytes) return cudaSuccess;
+        pairs += np;
+        ResDom<S, R>& y = doms[i];
+        y.pop = static_cast<S*>(x.pop);
+        y.G = G;
+        y.C = make_coef<R>(x.tau, x.forcing, x.boundary);
+        y.C.mrt = x.mrt;
+        y.az0 = x.forcing.az0;
+        y.omega_t = x.forcing.omega_t;
+        y.az = x.az;
+        y.az16 = x.az16;
+        y.mail = nullptr;
+        y.th = x.th;
+        y.npairs = (int)np;
+    }
+    r->sw = SW;
+    r->th = TH;
+    cudaError_t e;
+    std::vector<int> cta_dom;
+    // One domain of up to 8 x 256 pairs: a cluster.  A warp of FP32 pairs per
+    // scheduler of an SM keeps a step at the latency of one thread, so an SM
+    // takes 128 pairs before the next CTA is added; FP64 nodes are spread at a
+    // warp per SM, whose FP64 pipe one warp already fills.
+    if (n == 1 && pairs <= kResClusterMax * kResThreads) {
+        const int full = nl == 2 ? 128 : 32;
+        int c = 1;
+        while (c < kResClusterMax && pairs > (long long)c * full) c *= 2;
+        const int chunk = (int)((pairs + c - 1) / c);
+        doms[0].cta0 = 0;
+        doms[0].ncta = c;
+        doms[0].chunk = chunk;
+        r->cluster = true;
+        r->grid = c;
+        r->threads = res_up32(chunk);
+        r->smem = kResAz * sizeof(R) + (size_t)nplanes<SW, TH>() * nl * chunk * sizeof(S);
+        auto kern = k_resident_cluster<R, SW, TH>;
+        // the attribute belongs to the kernel, not to this handle: always the largest a handle can ask for
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kResSmemMax);
+        if (e != cudaSuccess) return e;
+        r->kernel = reinterpret_cast<const void*>(kern);
+        cta_dom.assign(c, 0);
+    } else {
+        bool fits = false;
+        auto place = [&](int chunk) {  // every domain has CTAs of its own
+            int cta = 0;
+            cta_dom.clear();
+            for (int i = 0; i < n; ++i) {
+                ResDom<S, R>& y = doms[i];
+                y.cta0 = cta;
+                y.chunk = chunk;
+                y.ncta = (y.npairs + chunk - 1) / chunk;
+                cta += y.ncta;
+                cta_dom.insert(cta_dom.end(), y.ncta, i);
+            }
+            r->grid = cta;
+        };
+        auto chunk_for = [&](int most, int least, int unit) {
+            int chunk = std::max<int>(least, ((int)((pairs + most - 1) / most) + unit - 1) / unit * unit);
+            for (;; chunk += std::max(unit, chunk / 64)) {
+                long long ctas = 0;
+                for (int i = 0; i < n; ++i) ctas += (doms[i].npairs + chunk - 1) / chunk;
+                if (ctas <= most) return chunk;
+            }
+        };
+        r->cluster = false;
+        // the state in shared memory, one CTA per SM
+        const int slab = n > num_sms ? 0 : chunk_for(num_sms, 32, 1);
+        if (slab && (size_t)nplanes<SW, TH>() * nl * slab * sizeof(R) < (size_t)kResSmemMax) {
+            place(slab);
+            const bool one = slab <= kResThreads;
+            int tab = 1, ghost = 1;
+            for (const ResDom<S, R>& y : doms)
+                for (int c = 0; c < y.ncta; ++c) {
+                    int t, g;
+                    res_slab_tables(c * slab, std::min((c + 1) * slab, y.npairs), y.G.nr, y.G.nz, nl, SW, TH && y.th, &t, &g);
+                    tab = std::max(tab, t);
+                    ghost = std::max(ghost, g);
+                }
+            r->smem = res_slab_smem<R, SW, TH>(slab, ghost);
+            if (!one) r->smem += 8 + (size_t)slab * sizeof(ResPair<R>) + tab * res_row_bytes<R, SW, TH>();
+            if (r->smem <= (size_t)kResSmemMax) {
+                const int iters = (slab + kResSlabThreads - 1) / kResSlabThreads;
+                r->threads = one ? kResThreads : std::max(kResThreads, res_up32((slab + iters - 1) / iters));
+                const auto k1 = k_resident_one<R, SW, TH>;
+                const auto k2 = k_resident_slab<R, SW, TH>;
+                r->kernel = one ? reinterpret_cast<const void*>(k1) : reinterpret_cast<const void*>(k2);
+                e = cudaFuncSetAttribute(r->kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kResSmemMax);
+                if (e != cudaSuccess) return e;
+                int got = 0;
+                e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&got, r->kernel, r->threads, r->smem);
+                if (e != cudaSuccess) return e;
+                fits = (long long)got * num_sms >= r->grid;
+                r->slab = true;
+                r->max_tab = tab;
+                r->max_ghost = ghost;
+            }
+        }
+        auto kern = k_resident_grid<S, R, SW, TH>;
+        for (int per_sm = 2; per_sm >= 1 && !fits; --per_sm) {
+            const int most = per_sm * num_sms;
+            if (n > most) return cudaSuccess;
+            const int chunk = chunk_for(most, 32, 32);
+            place(chunk);
+            int ring = 0;
+            for (const ResDom<S, R>& y : doms)
+                for (int c = 0; c < y.ncta; ++c)
+                    ring = std::max(ring, res_ring_pairs(c * chunk, std::min((c + 1) * chunk, y.npairs), y.G.nr, y.G.nz, nl));
+            const int iters = (chunk + kResThreads - 1) / kResThreads;
+            r->slab = false;
+            r->kernel = reinterpret_cast<const void*>(kern);
+            r->threads = res_up32((chunk + iters - 1) / iters);
+            r->smem = res_grid_smem<R, SW, TH>(chunk, ring);
+            if (r->smem > (size_t)(per_sm == 2 ? kResSmemMax / 2 : kResSmemMax)) continue;
+            e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kResSmemMax);
+            if (e != cudaSuccess) return e;
+            int got = 0;
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&got, kern, r->threads, r->smem);
+            if (e != cudaSuccess) return e;
+            fits = (long long)got * num_sms >= r->grid;
+        }
+        if (!fits) return cudaSuccess;
+    }
+    // descriptors, CTA map, step counters: one allocation of the library's own
+    const size_t b_doms = (n * sizeof(ResDom<S, R>) + 255) / 256 * 256;
+    const size_t b_map = (cta_dom.size() * sizeof(int) + 255) / 256 * 256;
+    size_t b_flags = (size_t)r->grid * kResPad * sizeof(unsigned);
+    if (r->slab) {
+        b_flags = 0;
+        for (const ResDom<S, R>& y : doms) b_flags += (size_t)y.npairs * nl * nplanes<SW, TH>() * sizeof(typename ResWord<R>::type);
+    }
+    if (cudaMalloc(&r->scratch, b_doms + b_map + b_flags) != cudaSuccess) {
+        cudaGetLastError();
+        r->scratch = nullptr;
+        return cudaSuccess;  // no room for it: the step kernels run
+    }
+    r->off_map = b_doms;
+    r->off_flags = b_doms + b_map;
+    char* m = static_cast<char*>(r->scratch);
+    if (r->slab) {
+        size_t off = r->off_flags;
+        for (ResDom<S, R>& y : doms) {
+            y.mail = m + off;
+            off += (size_t)y.npairs * nl * nplanes<SW, TH>() * sizeof(typename ResWord<R>::type);
+        }
+    }
+    e = cudaMemcpyAsync(m, doms.data(), n * sizeof(ResDom<S, R>), cudaMemcpyHostToDevice, stream);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(m + r->off_map, cta_dom.data(), cta_dom.size() * sizeof(int), cudaMemcpyHostToDevice, stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(m + r->off_flags, 0, b_flags, stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(stream);  // the lists live on this stack
+    r->epoch = 0;
+    r->on = e == cudaSuccess;
+    return e;
+}
+
+template <class S>
+cudaError_t res_build_any(Resident* r, const ResidentDomain* d, int n, bool sw, bool th, int num_sms, cudaStream_t st) {
+    if (sw && th) return res_build<S, true, true>(r, d, n, num_sms, st);
+    if (sw) return res_build<S, true, false>(r, d, n, num_sms, st);
+    if (th) return res_build<S, false, true>(r, d, n, num_sms, st);
+    return res_build<S, false, false>(r, d, n, num_sms, st);
+}
+
+// Batches carry g in every domain.
+template <class S>
+cudaError_t res_build_swirl(Resident* r, const ResidentDomain* d, int n, bool, bool th, int num_sms, cudaStream_t st) {
+    return th ? res_build<S, true, true>(r, d, n, num_sms, st) : res_build<S, true, false>(r, d, n, num_sms, st);
+}
+
+template <class S>
+ResidentOps make_resident_ops() {
+    ResidentOps o;
+    o.build = &res_build_any<S>;
+    return o;
+}
+
+}  // namespace axl

@@ -1,0 +1,76 @@
+"""Runs of plain steps on the multi-step kernels.
+
+A small domain's plain steps run in one launch (a thread-block cluster, or a
+grid whose CTAs keep the state in shared memory or in L2).  Whatever its form,
+the populations, the check values and the clock must equal those of the same
+steps launched kernel by kernel, bit for bit (the arithmetic is the same), at
+the sizes where the forms and their work split change: one pair of nodes,
+empty second lanes (odd nz), one and several CTAs, one and several pairs per
+thread, the state in L2, and links that wrap or mirror across CTAs.
+"""
+import numpy as np
+import pytest
+
+from parity_util import problem, seeded_state
+
+pytestmark = pytest.mark.gpu
+
+SHAPES = [
+    (1, 1), (3, 2), (64, 4), (9, 255),   # one CTA or a few of a cluster
+    (64, 64), (65, 64), (64, 65),        # the largest cluster (FP32 pairs), the smallest grids
+    (4099, 3), (3, 1999),                # rows longer than a CTA's range, columns across many CTAs
+    (199, 391),                          # several pairs per thread
+]
+
+
+@pytest.fixture(scope="module")
+def B():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1003_0282_gb300 import build
+    build.build()
+    from paper_1003_0282_gb300 import axlbm
+    return axlbm
+
+
+def both_ways(B, pb, precision, calls, seed=3):
+    st = seeded_state(pb, seed)
+    out = []
+    for graphs in (True, False):
+        dom = B.Domain(pb, precision)
+        dom.use_graphs(graphs)
+        dom.set_populations(st.f, st.g if pb.swirl else None, st.h if pb.temperature else None, time=6)
+        for n in calls:
+            dom.step(n)
+        assert dom.time == 6 + sum(calls)
+        out.append((dom.get_populations(), dom.residual()))
+        dom.close()
+    (p0, r0), (p1, r1) = out
+    assert r0 == r1
+    for x, y in zip(p0, p1):
+        assert (x is None and y is None) or np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("shape", SHAPES)
+@pytest.mark.parametrize("mix", ["pipe", "crystal", "annulus-mixed"])
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_equals_single_steps(B, shape, mix, precision):
+    both_ways(B, problem(*shape, mix), precision, [11, 12])
+
+
+@pytest.mark.parametrize("swirl,temp,collision", [(False, False, "bgk"), (True, False, "mrt"), (False, True, "mrt")])
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_distributions_and_collisions(B, swirl, temp, collision, precision):
+    for shape in ((37, 23), (130, 97)):
+        both_ways(B, problem(*shape, "closed", swirl=swirl, temperature=temp, collision=collision), precision, [21])
+
+
+def test_state_in_l2(B):
+    both_ways(B, problem(701, 809, "crystal", temperature=False), "fp32", [12])
+
+
+def test_long_runs_refresh_the_force(B):
+    """An oscillating force over more steps than a launch keeps ready, from an odd level."""
+    pb = problem(40, 11, "pipe", swirl=False, temperature=False)
+    both_ways(B, pb, "fp64", [1, 600, 301])
