@@ -535,8 +535,10 @@ AXLBM_API axlbm_status axlbm_batch_tile_shape(const axlbm_batch* b, int32_t* row
  * axlbm_batch_step call) are replayed from CUDA graphs captured on first use
  * (8 and 1 pairs of an even and an odd step; recaptured after a tile shape
  * change) when enable != 0, the default, and while kernel timing is off;
- * enable = 0 launches every kernel directly.  The results are the same bit
- * for bit.  The first capture synchronises nothing but takes a few ms. */
+ * enable = 0 launches every kernel directly.  Small FP32 batches (up to 64 MB
+ * of populations, domains as axlbm_use_graphs lists them) take one graph of a
+ * single kernel that runs all the pairs of a call.  The results are the same
+ * bit for bit.  The first capture synchronises nothing but takes a few ms. */
 AXLBM_API axlbm_status axlbm_batch_use_graphs(axlbm_batch* b, int32_t enable);
 
 /* How many times the step graphs were captured and launched since creation

@@ -420,6 +420,29 @@ cudaError_t batch_capture_pairs(axlbm_batch* b, const BatchOps* ops, int pairs, 
 // `pairs` plain step pairs from an even level, from the graphs (captured on
 // first use for the pair of tile shapes in use).
 axlbm_status batch_graph_pairs(axlbm_batch* b, const BatchOps* ops, int64_t pairs) {
+    if (b->res.on) {
+        axl::Clock* clk = reinterpret_cast<axl::Clock*>(b->mem + b->L.off_clock);
+        cudaError_t e = cudaSuccess;
+        if (!b->res.exec) {
+            if (!b->cap) e = cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking);
+            if (e == cudaSuccess) e = axl::resident_capture(&b->res, clk, b->cap);
+            if (e != cudaSuccess) {
+                cudaGetLastError();  // the failed capture must not surface in a later call
+                return bcuda(b, e, "graph capture");
+            }
+            b->graph_captures += 1;
+        }
+        for (int64_t p = 0; p < pairs;) {
+            const int64_t done = std::min(pairs - p, axl::kResMaxSteps / 2);
+            e = axl::resident_launch(&b->res, clk, (int)(2 * done), b->t + 2 * p, b->stream);
+            if (e != cudaSuccess) return bcuda(b, e, "graph launch");
+            p += done;
+            b->graph_launches += 1;
+        }
+        b->t += 2 * pairs;
+        b->speed_valid = false;
+        return AXLBM_OK;
+    }
     const int key = 4 * b->shape[0] + b->shape[1];
     if (b->graph_shape != key) {
         batch_drop_graphs(b);
@@ -451,10 +474,11 @@ axlbm_status batch_step_n(axlbm_batch* b, int64_t n) {
     // every step but the tail is plain: the tail is the two check steps (lag
     // 1), or a check step, a plain step and a check step (lag 2); with timing
     // off, whole (even, odd) pairs of plain steps replay captured graphs once
-    // the plain kernels of the shapes in use have been sized by earlier launches
+    // the plain kernels of the shapes in use have been sized by earlier
+    // launches (a batch on the multi-step kernels needs none)
     const int tail = b->residual_lag == 2 ? 3 : 2;
     const bool sized = b->grid[b->shape[0]][0][0] > 0 && b->grid[b->shape[1]][1][0] > 0;
-    if (b->use_graphs && !b->timing && sized && n - tail - b->parity >= 2 * kMinGraphPairs) {
+    if (b->use_graphs && !b->timing && (sized || b->res.on) && n - tail - b->parity >= 2 * kMinGraphPairs) {
         if (b->parity == 1) {
             int nl = 0;
             const cudaError_t e = ops->step(b, 0, 0, nullptr, nullptr, &nl);
@@ -728,12 +752,40 @@ axlbm_status axlbm_batch_create(const axlbm_domain* domains, int32_t n, int32_t 
     if (st == AXLBM_OK) st = reset_rest(b);
     if (st == AXLBM_OK) st = tune(b);
     if (st == AXLBM_OK) st = reset_rest(b);
+    if (st == AXLBM_OK && precision == AXLBM_FP32) {
+        double* az = reinterpret_cast<double*>(b->mem + L.off_az);
+        std::vector<axl::ResidentDomain> rd(n);
+        for (int d = 0; d < n; ++d) {
+            const axlbm_domain& D = domains[d];
+            const axl::DomDesc& x = dd[d];
+            axl::Geom G = {};
+            G.nr = x.nr;
+            G.nz = x.nz;
+            G.pitch = L.pitch;
+            G.plane = L.plane;
+            G.r0 = x.r0;
+            G.inner = x.inner;
+            G.outer = x.outer;
+            G.z_lo = x.z_lo;
+            G.z_hi = x.z_hi;
+            G.r_split = x.r_split;
+            G.col0 = x.col0;
+            G.row0 = x.row0;
+            G.rb = x.rb;
+            G.rb_exact = x.rb_exact;
+            rd[d] = {b->mem, G, D.tau, D.forcing, D.boundary, D.grid.collision == AXLBM_MRT, D.grid.with_temperature,
+                     az + 2 * d, az + 2 * n + 4 * d};
+        }
+        const cudaError_t e = axl::resident_fp32.build(&b->res, rd.data(), n, true, b->thmax != 0, b->num_sms, b->stream);
+        if (e != cudaSuccess) st = bcuda(b, e, "multi-step launch");
+    }
     if (st == AXLBM_OK) {
         cudaError_t e = cudaStreamSynchronize(b->stream);
         if (e != cudaSuccess) st = bcuda(b, e, "create");
     }
     if (st != AXLBM_OK) {
         g_batch_error = b->err;
+        axl::resident_free(&b->res);
         if (b->owns_mem) cudaFree(b->mem);
         if (b->fork) cudaEventDestroy(b->fork);
         if (b->join) cudaEventDestroy(b->join);
@@ -1266,6 +1318,7 @@ axlbm_status axlbm_batch_destroy(axlbm_batch* b) {
         cudaStreamDestroy(b->side);
     }
     batch_drop_graphs(b);
+    axl::resident_free(&b->res);
     if (b->cap) cudaStreamDestroy(b->cap);
     if (b->stage) cudaFree(b->stage);
     if (b->io_back) {

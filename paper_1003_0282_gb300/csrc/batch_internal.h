@@ -85,6 +85,7 @@ struct axlbm_batch {
     cudaGraphExec_t graph_many;     // kGraphPairs (even, odd) step pairs
     cudaGraphExec_t graph_one;      // one pair
     int64_t graph_captures, graph_launches;
+    axl::Resident res;  // multi-step launches instead of the pair graphs, for small batches
     void* stage;  // device staging buffer of host-side field I/O, kept between calls
     size_t stage_bytes;
     // asynchronous all-domain host I/O (axlbm_batch_*_all_async): a copy

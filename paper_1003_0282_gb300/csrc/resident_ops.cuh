@@ -234,12 +234,6 @@ cudaError_t res_build_any(Resident* r, const ResidentDomain* d, int n, bool sw, 
     return res_build<S, false, false>(r, d, n, num_sms, st);
 }
 
-// Batches carry g in every domain.
-template <class S>
-cudaError_t res_build_swirl(Resident* r, const ResidentDomain* d, int n, bool, bool th, int num_sms, cudaStream_t st) {
-    return th ? res_build<S, true, true>(r, d, n, num_sms, st) : res_build<S, true, false>(r, d, n, num_sms, st);
-}
-
 template <class S>
 ResidentOps make_resident_ops() {
     ResidentOps o;

@@ -74,3 +74,30 @@ def test_long_runs_refresh_the_force(B):
     """An oscillating force over more steps than a launch keeps ready, from an odd level."""
     pb = problem(40, 11, "pipe", swirl=False, temperature=False)
     both_ways(B, pb, "fp64", [1, 600, 301])
+
+
+@pytest.mark.parametrize("scale", [1, 4])
+def test_small_batches(B, scale):
+    """Domains of uneven size, with and without temperature, in one multi-step launch."""
+    probs = [problem(17 * scale, 29 * scale, "crystal"), problem(43 * scale, 8 * scale, "pipe", temperature=False),
+             problem(50 * scale, 63, "annulus-mixed", collision="mrt", tau=0.55), problem(1, 1, "closed"),
+             problem(64, 33 * scale, "free-top", temperature=False)]
+    out = []
+    for graphs in (True, False):
+        batch = B.Batch(probs, "fp32")
+        batch.use_graphs(graphs)
+        for d, pb in enumerate(probs):
+            st = seeded_state(pb, 40 + d)
+            batch.set_populations(d, st.f, st.g, st.h if pb.temperature else None)
+        batch.step(1)
+        batch.step(24)
+        batch.step(13)
+        caps, launches = batch.graph_stats()
+        assert (caps, launches) == ((1, 2) if graphs else (0, 0))
+        out.append(([batch.get_populations(d) for d in range(len(probs))], batch.residuals(), batch.time))
+        batch.close()
+    (p0, r0, t0), (p1, r1, t1) = out
+    assert t0 == t1 == 38 and np.array_equal(r0, r1)
+    for d in range(len(probs)):
+        for x, y in zip(p0[d], p1[d]):
+            assert (x is None and y is None) or np.array_equal(x, y), d
