@@ -87,7 +87,6 @@ struct Resident {
     bool on = false;
     bool cluster = false;  // one thread-block cluster, else a cooperative grid
     bool slab = false;     // a grid with the state in shared memory, else in L2
-    int max_tab = 0, max_ghost = 0;
     bool sw = false, th = false;
     int grid = 0, threads = 0;
     size_t smem = 0;

@@ -14,8 +14,7 @@ struct ResArgs {
     int steps;
     unsigned epoch;
     long long t0;
-    int max_tab, max_ghost;
-    void* args[8];
+    void* args[7];
     ResArgs(const Resident& r, Clock* clk, int steps_, long long t0_) {
         char* m = static_cast<char*>(r.scratch);
         doms = m;
@@ -25,8 +24,6 @@ struct ResArgs {
         steps = steps_;
         epoch = r.epoch;
         t0 = t0_;
-        max_tab = r.max_tab;
-        max_ghost = r.max_ghost;
         int n = 0;
         args[n++] = &doms;
         if (!r.cluster) args[n++] = &map;
@@ -35,10 +32,6 @@ struct ResArgs {
         args[n++] = &steps;
         if (!r.cluster) args[n++] = &epoch;
         args[n++] = &t0;
-        if (r.slab) {
-            args[n++] = &max_ghost;
-            args[n++] = &max_tab;
-        }
     }
 };
 

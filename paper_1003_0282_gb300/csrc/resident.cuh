@@ -49,10 +49,31 @@ struct ResDom {
     double az0, omega_t;
     double* az;      // a(t) by AA parity: where the step kernels read it (two values)
     double* az16;    // a batch domain's copy for the bulk kernel, or null
-    void* mail;      // words between CTAs: [plane][lane][pair]
+    void* mail;      // words between CTAs: [CTA][plane][lane][place on the tile's outline]
     int th;
     int npairs;      // node pairs (FP64: nodes), pair p = (row pair p / nr, column p % nr)
-    int cta0, ncta, chunk;  // CTAs [cta0, cta0 + ncta), `chunk` consecutive pairs each
+    int cta0, ncta;  // CTAs [cta0, cta0 + ncta)
+    int chunk;       // cluster, grid in L2: consecutive pairs of a CTA; else the most pairs of a CTA
+    int tx, w, h;    // state in shared memory: tiles of w columns x h row pairs, tx in a row
+    int max_tab, max_ghost;  // rows of a CTA's slot table, slots of other CTAs, at most
+};
+
+// The rectangle of pairs that CTA `rank` of domain D keeps in shared memory.
+struct ResTile {
+    int j0, k0, w, h;
+    template <class D>
+    __host__ __device__ ResTile(const D& d, int nkp, int rank)
+        : j0((rank % d.tx) * d.w), k0((rank / d.tx) * d.h), w(d.G.nr - j0 < d.w ? d.G.nr - j0 : d.w),
+          h(nkp - k0 < d.h ? nkp - k0 : d.h) {}
+    // place of a pair of the tile's outline along it: first row, last row, first column, last column
+    __host__ __device__ int outline(int j, int kp) const {
+        const int jl = j - j0, kl = kp - k0;
+        return kl == 0 ? jl : (kl == h - 1 ? w + jl : (jl == 0 ? 2 * w + kl : 2 * w + h + kl));
+    }
+    // index of pair (j, kp) in the tile, or -1
+    __host__ __device__ int index(int j, int kp) const {
+        return j >= j0 && j < j0 + w && kp >= k0 && kp < k0 + h ? (kp - k0) * w + (j - j0) : -1;
+    }
 };
 
 // The slot that population (er, ez) of node (j, k) is pulled from in an odd
@@ -392,7 +413,7 @@ template <class R, int PAR>
 __device__ __forceinline__ void res_gather(const ResSlab<R>& S, const typename ResWord<R>::type* mail, int gbase, int ng,
                                            unsigned want, Clock* clock, int* bad) {
     using W = ResWord<R>;
-    constexpr int U = sizeof(R) == 4 ? 8 : 4;
+    constexpr int U = 2;  // a tile's outline rarely has more than two words per thread
     const int T = blockDim.x;
     for (int g0 = threadIdx.x; g0 < ng; g0 += U * T) {
         typename W::type w[U];
@@ -436,6 +457,14 @@ __device__ __forceinline__ void res_scatter(const ResSlab<R>& S, typename ResWor
         ResWord<R>::store(mail + (PAR ? S.odd : S.even)[g], S.st[PAR ? gbase + g : S.own[g]], step);
 }
 
+// The word of slot ql of pair (j, kp), which lies on the outline of its tile:
+// words of one side of a tile lie side by side, apart from other tiles'.
+template <int PL, class D>
+__host__ __device__ __forceinline__ int res_word(const D& d, int nkp, int ql, int j, int kp) {
+    const int rank = (kp / d.h) * d.tx + j / d.w;
+    return (rank * PL + ql) * (2 * (d.w + d.h)) + ResTile(d, nkp, rank).outline(j, kp);
+}
+
 // A lane's slot in another CTA becomes a ghost: its number (consecutive within
 // the warp, so that copies and words lie side by side), or -1.
 __device__ __forceinline__ int res_new_ghost(bool remote, int* count) {
@@ -455,8 +484,9 @@ __device__ __forceinline__ void res_slab_run(const ResDom<R, R>& D, const ResSla
                                              unsigned epoch, long long t0, int ng, int* bad, const Update& update) {
     constexpr int NL = Lanes<typename PairArith<R>::type>::n, PL = nplanes<SW, TH>() * NL;
     const Geom& G = D.G;
-    const int tid = threadIdx.x, T = blockDim.x, chunk = D.chunk, nr = G.nr;
-    const int rank = blockIdx.x - D.cta0, p0 = rank * chunk, n = min(chunk, D.npairs - p0), gbase = PL * chunk;
+    const int tid = threadIdx.x, T = blockDim.x, chunk = D.chunk;
+    const int rank = blockIdx.x - D.cta0, gbase = PL * chunk;
+    const ResTile tile(D, (G.nz + NL - 1) / NL, rank);
     auto* mail = static_cast<typename ResWord<R>::type*>(D.mail);
     auto step = [&](auto par_tag, int s) {
         constexpr int PAR = decltype(par_tag)::value;
@@ -484,8 +514,9 @@ __device__ __forceinline__ void res_slab_run(const ResDom<R, R>& D, const ResSla
         if (tid == 0) atomicOr(&clock->err, 1u);
         return;
     }
+    const int n = tile.w * tile.h;
     for (int m = tid; m < PL * n; m += T) {
-        const int ql = m / n, i = m - ql * n, p = p0 + i, kp = p / nr, j = p - kp * nr, k = NL * kp + ql % NL;
+        const int ql = m / n, i = m - ql * n, kl = i / tile.w, j = tile.j0 + i - kl * tile.w, k = NL * (tile.k0 + kl) + ql % NL;
         if (k < G.nz) *slot(D.pop, G, ql / NL, j, k) = S.st[ql * chunk + i];
     }
     if (rank == 0 && tid == 0) res_finish(D, t0 + nsteps);
@@ -495,34 +526,36 @@ __device__ __forceinline__ void res_slab_run(const ResDom<R, R>& D, const ResSla
 // One pair per thread: addresses and links stay in registers.
 template <class R, bool SW, bool TH>
 __device__ __forceinline__ void res_one_cta(const ResDom<R, R>& D, Clock* clock, int nsteps, unsigned epoch, long long t0,
-                                            int max_ghost, unsigned char* smem) {
+                                            unsigned char* smem) {
     using RC = typename PairArith<R>::type;
     constexpr int NL = Lanes<RC>::n, P = nplanes<SW, TH>();
     __shared__ int ghosts, bad;
     const Geom& G = D.G;
     const Coef<R> C = D.C;
-    const int tid = threadIdx.x, chunk = D.chunk, nr = G.nr, np = D.npairs;
-    const int p0 = (blockIdx.x - D.cta0) * chunk, n = min(chunk, np - p0), gbase = P * NL * chunk;
+    const int tid = threadIdx.x, chunk = D.chunk, nr = G.nr, nkp = (G.nz + NL - 1) / NL;
+    const int gbase = P * NL * chunk, max_ghost = D.max_ghost;
+    const ResTile tile(D, nkp, blockIdx.x - D.cta0);
+    const int n = tile.w * tile.h;
     const ResSlab<R> S(smem, gbase, max_ghost);
     if (tid == 0) ghosts = bad = 0;
     __syncthreads();
     const bool on = tid < n;
-    const int p = p0 + (on ? tid : 0), kp = p / nr, j = p - kp * nr, k0 = NL * kp;
+    const int kl = (on ? tid : 0) / tile.w, j = tile.j0 + (on ? tid : 0) - kl * tile.w, kp = tile.k0 + kl, k0 = NL * kp;
     R* const mine = S.st + tid;
     int at[P][NL];
     ResLinks<RC, SW, TH> L;
     if (tid < res_up32(n)) {  // whole warps
         res_links<RC, R, SW, TH>(G, C, j, k0, L, [&](int q, int l, int ql, int sp) {
-            const bool local = sp >= p0 && sp < p0 + n;
-            const int g = res_new_ghost(on && sp >= 0 && !local, &ghosts);
-            at[q][l] = sp < 0 ? (q * NL + l) * chunk + tid : (g < 0 ? ql * chunk + (local ? sp - p0 : 0) : gbase + g);
+            const int here = sp < 0 ? tid : tile.index(sp % nr, sp / nr);
+            const int g = res_new_ghost(on && here < 0, &ghosts);
+            at[q][l] = g < 0 ? ql * chunk + max(here, 0) : gbase + g;
             if (g >= max_ghost) {
                 bad = 2;
                 at[q][l] = gbase;
             } else if (g >= 0) {
                 S.own[g] = (q * NL + l) * chunk + tid;
-                S.even[g] = (q * NL + l) * np + p;
-                S.odd[g] = ql * np + sp;
+                S.even[g] = res_word<P * NL>(D, nkp, q * NL + l, j, kp);
+                S.odd[g] = res_word<P * NL>(D, nkp, ql, sp % nr, sp / nr);
             }
             if (on) mine[(q * NL + l) * chunk] = k0 + l < G.nz ? *slot(D.pop, G, q, j, k0 + l) : R(0);
         });
@@ -553,18 +586,17 @@ __device__ __forceinline__ void res_one_cta(const ResDom<R, R>& D, Clock* clock,
 template <class R, bool SW, bool TH>
 __global__ void __launch_bounds__(kResThreads, 1)
 k_resident_one(const ResDom<R, R>* __restrict__ doms, const int* __restrict__ cta_dom, Clock* clock, int nsteps,
-               unsigned epoch, long long t0, int max_ghost, int) {
+               unsigned epoch, long long t0) {
     extern __shared__ __align__(16) unsigned char res_smem[];
     const ResDom<R, R>& D = doms[cta_dom[blockIdx.x]];
-    if (TH && D.th) res_one_cta<R, SW, TH>(D, clock, nsteps, epoch, t0, max_ghost, res_smem);
-    else res_one_cta<R, SW, false>(D, clock, nsteps, epoch, t0, max_ghost, res_smem);
+    if (TH && D.th) res_one_cta<R, SW, TH>(D, clock, nsteps, epoch, t0, res_smem);
+    else res_one_cta<R, SW, false>(D, clock, nsteps, epoch, t0, res_smem);
 }
 
 constexpr int kResSlabThreads = 384;
 
-// A pair of the kernel below: bit 30 of i: the second lane is empty; tab: its
-// row of the slot table, or -1 where every slot is the CTA's own and away
-// from the outline.
+// A pair of the kernel below: its index in the tile; tab: its row of the slot
+// table, or -1 away from the tile's outline, where every slot is the CTA's own.
 template <class R>
 struct ResPair {
     R inv_r;
@@ -581,14 +613,16 @@ __host__ __device__ constexpr size_t res_row_bytes() {
 // Several pairs per thread.
 template <class R, bool SW, bool TH>
 __device__ __forceinline__ void res_slab_cta(const ResDom<R, R>& D, Clock* clock, int nsteps, unsigned epoch, long long t0,
-                                             int max_ghost, int max_tab, unsigned char* smem) {
+                                             unsigned char* smem) {
     using RC = typename PairArith<R>::type;
     constexpr int NL = Lanes<RC>::n, P = nplanes<SW, TH>(), PL = P * NL, NF = (SW ? 8 : 0) + (TH ? 12 : 0);
     __shared__ int ghosts, bad, rows;
     const Geom& G = D.G;
     const Coef<R> C = D.C;
-    const int tid = threadIdx.x, T = blockDim.x, chunk = D.chunk, nr = G.nr, np = D.npairs;
-    const int p0 = (blockIdx.x - D.cta0) * chunk, n = min(chunk, np - p0), gbase = PL * chunk;
+    const int tid = threadIdx.x, T = blockDim.x, chunk = D.chunk, nr = G.nr, nkp = (G.nz + NL - 1) / NL;
+    const int gbase = PL * chunk, max_ghost = D.max_ghost, max_tab = D.max_tab;
+    const ResTile tile(D, nkp, blockIdx.x - D.cta0);
+    const int tw = tile.w, n = tw * tile.h;
     const ResSlab<R> S(smem, gbase, max_ghost);
     ResPair<R>* pairs = reinterpret_cast<ResPair<R>*>(S.rest + (sizeof(R) == 8 ? (max_ghost & 1) * 4 : 0));
     R* tf = reinterpret_cast<R*>(pairs + chunk);  // [NF][NL][max_tab]: sg, cg, then sh, ch, ct, four each
@@ -601,14 +635,12 @@ __device__ __forceinline__ void res_slab_cta(const ResDom<R, R>& D, Clock* clock
         for (int pass = 0; pass < 2; ++pass) {
             int at0 = 0, at1 = plain;
             for (int i0 = 0; i0 < n; i0 += 32) {
-                const int i = i0 + tid, p = p0 + i, kp = p / nr, j = p - kp * nr;
-                const bool two = NL == 2 && NL * kp + 1 < G.nz;
-                const bool ring = j == 0 || j == nr - 1 || kp == 0 || NL * kp + (two ? 1 : 0) == G.nz - 1;
-                const bool row = ring || i < nr + 1 || i + nr + 1 >= n;
+                const int i = i0 + tid, kl = i / tw, jl = i - kl * tw;
+                const bool row = jl == 0 || jl == tw - 1 || kl == 0 || kl == tile.h - 1;  // the tile's outline
                 const unsigned m0 = __ballot_sync(0xffffffffu, i < n && !row), m1 = __ballot_sync(0xffffffffu, i < n && row);
                 if (pass && i < n) {
                     ResPair<R> r;
-                    r.inv_r = step_inv_radius<R>(G, j);
+                    r.inv_r = step_inv_radius<R>(G, tile.j0 + jl);
                     r.i = i;
                     const int to = row ? at1 + __popc(m1 & ((1u << tid) - 1u)) : at0 + __popc(m0 & ((1u << tid) - 1u));
                     r.tab = row ? to - plain : -1;
@@ -631,19 +663,19 @@ __device__ __forceinline__ void res_slab_cta(const ResDom<R, R>& D, Clock* clock
         for (int w = tid >> 5; w < blocks * PL; w += T >> 5) {  // 32 pairs of one population and lane
             const int x = w / blocks, t = (w - x * blocks) * 32 + lane, q = x / NL, l = x - q * NL;
             const bool on = t < nt;
-            const int i = pairs[n0 + (on ? t : 0)].i, p = p0 + i, kp = p / nr, j = p - kp * nr, k = NL * kp + l;
-            int ql = x, sp = p, how = 0;  // (a lane without a node keeps to itself)
+            const int i = pairs[n0 + (on ? t : 0)].i, kl = i / tw, j = tile.j0 + i - kl * tw, kp = tile.k0 + kl, k = NL * kp + l;
+            int ql = x, sp = kp * nr + j, how = 0;  // (a lane without a node keeps to itself)
             if (k < G.nz) res_where<NL>(G, q, j, k, ql, sp, how);
-            const bool local = sp >= p0 && sp < p0 + n;
-            const int g = res_new_ghost(on && !local, &ghosts);
-            int e = local ? ql * chunk + (sp - p0) : gbase + g;
+            const int here = tile.index(sp % nr, sp / nr);
+            const int g = res_new_ghost(on && here < 0, &ghosts);
+            int e = here >= 0 ? ql * chunk + here : gbase + g;
             if (g >= max_ghost) {
                 bad = 2;
                 e = gbase;
             } else if (g >= 0) {
                 S.own[g] = x * chunk + i;
-                S.even[g] = x * np + p;
-                S.odd[g] = ql * np + sp;
+                S.even[g] = res_word<PL>(D, nkp, x, j, kp);
+                S.odd[g] = res_word<PL>(D, nkp, ql, sp % nr, sp / nr);
             }
             if (on) {
                 tab[x * max_tab + t] = e;
@@ -668,7 +700,7 @@ __device__ __forceinline__ void res_slab_cta(const ResDom<R, R>& D, Clock* clock
         }
     }
     for (int m = tid; m < PL * n; m += T) {  // the state, natural layout
-        const int ql = m / n, i = m - ql * n, p = p0 + i, kp = p / nr, j = p - kp * nr, k = NL * kp + ql % NL;
+        const int ql = m / n, i = m - ql * n, kl = i / tw, j = tile.j0 + i - kl * tw, k = NL * (tile.k0 + kl) + ql % NL;
         S.st[ql * chunk + i] = k < G.nz ? *slot(D.pop, G, ql / NL, j, k) : R(0);
     }
     __syncthreads();
@@ -694,9 +726,9 @@ __device__ __forceinline__ void res_slab_cta(const ResDom<R, R>& D, Clock* clock
             auto inside = [&](int q, int l) {
                 const int er = q < 9 ? cr9(q) : cr4((q - 9) & 3), ez = q < 9 ? cz9(q) : cz4((q - 9) & 3);
                 const int pl = q < 9 ? opp9(q) : 9 + ((q - 9) & ~3) + opp4((q - 9) & 3);
-                if (NL == 1) return pl * chunk - ez * nr - er;
+                if (NL == 1) return pl * chunk - ez * tw - er;
                 const int row = l - ez;  // -1, 0, 1, 2: of the pair below, this pair, this pair, the pair above
-                return (pl * NL + (row & 1)) * chunk + (row < 0 ? -nr : (row > 1 ? nr : 0)) - er;
+                return (pl * NL + (row & 1)) * chunk + (row < 0 ? -tw : (row > 1 ? tw : 0)) - er;
             };
             const TabLinks tl{tf + r.tab, max_tab};
             struct NoLinks {
@@ -722,11 +754,11 @@ __device__ __forceinline__ void res_slab_cta(const ResDom<R, R>& D, Clock* clock
 template <class R, bool SW, bool TH>
 __global__ void __launch_bounds__(kResSlabThreads, 1)
 k_resident_slab(const ResDom<R, R>* __restrict__ doms, const int* __restrict__ cta_dom, Clock* clock, int nsteps,
-                unsigned epoch, long long t0, int max_ghost, int max_tab) {
+                unsigned epoch, long long t0) {
     extern __shared__ __align__(16) unsigned char res_smem[];
     const ResDom<R, R>& D = doms[cta_dom[blockIdx.x]];
-    if (TH && D.th) res_slab_cta<R, SW, TH>(D, clock, nsteps, epoch, t0, max_ghost, max_tab, res_smem);
-    else res_slab_cta<R, SW, false>(D, clock, nsteps, epoch, t0, max_ghost, max_tab, res_smem);
+    if (TH && D.th) res_slab_cta<R, SW, TH>(D, clock, nsteps, epoch, t0, res_smem);
+    else res_slab_cta<R, SW, false>(D, clock, nsteps, epoch, t0, res_smem);
 }
 
 // ---------------------------------------------------------------------------- grid, state in L2

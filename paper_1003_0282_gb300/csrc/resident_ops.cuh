@@ -25,28 +25,57 @@ inline int res_ring_pairs(int p0, int p1, int nr, int nz, int nl) {
     return count;
 }
 
-// The slab form's tables for CTA [p0, p1): pairs on the outline or within a row of the CTA's ends, and at most
-// how many of their slots other CTAs own (outline pairs counted on the safe side: a link may be mirrored or wrapped).
-inline void res_slab_tables(int p0, int p1, int nr, int nz, int nl, bool sw, bool th, int* pairs, int* ghosts) {
-    const int n = p1 - p0, planes = 9 + (sw ? 4 : 0) + (th ? 4 : 0);
+// Tables of CTA `rank` of domain y: pairs on its tile's outline, and how many
+// of their slots other CTAs own.
+template <int NL, class Dom>
+void res_tile_tables(const Dom& y, int rank, bool sw, bool th, int* pairs, int* ghosts) {
+    const int nr = y.G.nr, nz = y.G.nz, planes = 9 + (sw ? 4 : 0) + (th ? 4 : 0);
+    const ResTile t(y, (nz + NL - 1) / NL, rank);
     *pairs = *ghosts = 0;
-    for (int i = 0; i < n; ++i) {
-        const int p = p0 + i, kp = p / nr, j = p - kp * nr;
-        const bool two = nl == 2 && nl * kp + 1 < nz;
-        const bool ring = j == 0 || j == nr - 1 || kp == 0 || nl * kp + (two ? 1 : 0) == nz - 1;
-        if (!ring && i >= nr + 1 && i + nr + 1 < n) continue;
-        *pairs += 1;
-        for (int q = 1; q < planes; ++q) {
-            const int er = q < 9 ? cr9(q) : cr4((q - 9) & 3), ez = q < 9 ? cz9(q) : cz4((q - 9) & 3);
-            for (int l = 0; l < (two ? 2 : 1); ++l) {
-                const int row = l - ez;
-                const int at = i + (nl == 1 ? -ez * nr : (row < 0 ? -nr : (row > 1 ? nr : 0)));
-                bool out = at - er < 0 || at - er >= n;
-                if (ring) out = out || at - 1 < 0 || at + 1 >= n || (nl == 2 && !two && ez < 0);
-                *ghosts += out;
+    for (int kl = 0; kl < t.h; ++kl)
+        for (int jl = 0; jl < t.w; jl += (kl == 0 || kl == t.h - 1 || t.w < 3) ? 1 : t.w - 1) {
+            const int j = t.j0 + jl, kp = t.k0 + kl;
+            const bool two = NL == 2 && NL * kp + 1 < nz;
+            const bool ring = j == 0 || j == nr - 1 || kp == 0 || NL * kp + (two ? 1 : 0) == nz - 1;
+            *pairs += 1;
+            for (int q = 1; q < planes; ++q) {
+                const int er = q < 9 ? cr9(q) : cr4((q - 9) & 3), ez = q < 9 ? cz9(q) : cz4((q - 9) & 3);
+                for (int l = 0; l < (two ? 2 : 1); ++l) {
+                    if (ring) {  // the link may be wrapped, mirrored or bounced back
+                        int ql, p, how;
+                        res_where<NL>(y.G, q, j, NL * kp + l, ql, p, how);
+                        *ghosts += t.index(p % nr, p / nr) < 0;
+                        continue;
+                    }
+                    const int row = NL == 1 ? -2 * ez : l - ez;  // below 0 or above 1: another row of pairs
+                    const int kq = kl + (row < 0 ? -1 : (row > 1 ? 1 : 0));
+                    *ghosts += kq < 0 || kq >= t.h || jl - er < 0 || jl - er >= t.w;
+                }
             }
         }
-    }
+}
+
+// Splits a domain of nr x nkp pairs (nl nodes each) into the fewest tiles of
+// at most `most` pairs that are no longer than three times their width where
+// the domain lets them; the words a tile exchanges grow with its outline.
+inline int res_tiling(int nr, int nkp, int nl, int most, int* w, int* h) {
+    int best = 0x7fffffff, edge = 0;
+    for (int square = 1; square >= 0 && best == 0x7fffffff; --square)
+        for (int tx = 1; tx <= nr; ++tx) {
+            const int tw = (nr + tx - 1) / tx;
+            if (tx > 1 && tw == (nr + tx - 2) / (tx - 1)) continue;  // the same width in fewer tiles
+            if (tw > most) continue;
+            const int ty = (nkp + most / tw - 1) / (most / tw), th = (nkp + ty - 1) / ty;
+            if (square && ((tw > 3 * nl * th && th < nkp) || (nl * th > 3 * tw && tw < nr))) continue;
+            const int tiles = ((nr + tw - 1) / tw) * ((nkp + th - 1) / th);
+            if (tiles < best || (tiles == best && tw + nl * th < edge)) {
+                best = tiles;
+                edge = tw + nl * th;
+                *w = tw;
+                *h = th;
+            }
+        }
+    return best;
 }
 
 template <class R>
@@ -127,52 +156,76 @@ cudaError_t res_build(Resident* r, const ResidentDomain* d, int n, int num_sms, 
             }
             r->grid = cta;
         };
-        auto chunk_for = [&](int most, int least, int unit) {
-            int chunk = std::max<int>(least, ((int)((pairs + most - 1) / most) + unit - 1) / unit * unit);
-            for (;; chunk += std::max(unit, chunk / 64)) {
+        auto chunk_for = [&](int most) {
+            int chunk = std::max(32, res_up32((int)((pairs + most - 1) / most)));
+            for (;; chunk += 32) {
                 long long ctas = 0;
                 for (int i = 0; i < n; ++i) ctas += (doms[i].npairs + chunk - 1) / chunk;
                 if (ctas <= most) return chunk;
             }
         };
         r->cluster = false;
-        // the state in shared memory, one CTA per SM
-        const int slab = n > num_sms ? 0 : chunk_for(num_sms, 32, 1);
-        if (slab && (size_t)nplanes<SW, TH>() * nl * slab * sizeof(R) < (size_t)kResSmemMax) {
-            place(slab);
-            const bool one = slab <= kResThreads;
-            int tab = 1, ghost = 1;
-            for (const ResDom<S, R>& y : doms)
+        // the state in shared memory, one CTA per SM: the smallest tiles that give no more CTAs than SMs
+        const int room = (int)(kResSmemMax / (nplanes<SW, TH>() * nl * sizeof(R)));
+        int most = std::max<int>(32, (int)((pairs + num_sms - 1) / num_sms));
+        for (; n <= num_sms && most < room; most += std::max(1, most / 64)) {
+            long long ctas = 0;
+            for (int i = 0; i < n; ++i) {
+                ResDom<S, R>& y = doms[i];
+                ctas += y.ncta = res_tiling(y.G.nr, (y.G.nz + nl - 1) / nl, nl, most, &y.w, &y.h);
+            }
+            if (ctas > num_sms) continue;
+            r->grid = (int)ctas;
+            int cta = 0, chunk = 0;
+            cta_dom.clear();
+            for (int i = 0; i < n; ++i) {
+                ResDom<S, R>& y = doms[i];
+                y.tx = (y.G.nr + y.w - 1) / y.w;
+                y.cta0 = cta;
+                y.chunk = y.w * y.h;
+                cta += y.ncta;
+                cta_dom.insert(cta_dom.end(), y.ncta, i);
+                chunk = std::max(chunk, y.chunk);
+            }
+            const bool one = chunk <= kResThreads;
+            size_t smem = 0;
+            for (ResDom<S, R>& y : doms) {
+                const bool h = TH && y.th;
+                y.max_tab = y.max_ghost = 1;
                 for (int c = 0; c < y.ncta; ++c) {
                     int t, g;
-                    res_slab_tables(c * slab, std::min((c + 1) * slab, y.npairs), y.G.nr, y.G.nz, nl, SW, TH && y.th, &t, &g);
-                    tab = std::max(tab, t);
-                    ghost = std::max(ghost, g);
+                    res_tile_tables<Lanes<typename PairArith<R>::type>::n>(y, c, SW, h, &t, &g);
+                    y.max_tab = std::max(y.max_tab, t);
+                    y.max_ghost = std::max(y.max_ghost, g);
                 }
-            r->smem = res_slab_smem<R, SW, TH>(slab, ghost);
-            if (!one) r->smem += 8 + (size_t)slab * sizeof(ResPair<R>) + tab * res_row_bytes<R, SW, TH>();
-            if (r->smem <= (size_t)kResSmemMax) {
-                const int iters = (slab + kResSlabThreads - 1) / kResSlabThreads;
-                r->threads = one ? kResThreads : std::max(kResThreads, res_up32((slab + iters - 1) / iters));
-                const auto k1 = k_resident_one<R, SW, TH>;
-                const auto k2 = k_resident_slab<R, SW, TH>;
-                r->kernel = one ? reinterpret_cast<const void*>(k1) : reinterpret_cast<const void*>(k2);
-                e = cudaFuncSetAttribute(r->kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kResSmemMax);
-                if (e != cudaSuccess) return e;
-                int got = 0;
-                e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&got, r->kernel, r->threads, r->smem);
-                if (e != cudaSuccess) return e;
-                fits = (long long)got * num_sms >= r->grid;
-                r->slab = true;
-                r->max_tab = tab;
-                r->max_ghost = ghost;
+                // (a domain without h in a batch with it has fewer planes)
+                size_t need = h ? res_slab_smem<R, SW, TH>(y.chunk, y.max_ghost) : res_slab_smem<R, SW, false>(y.chunk, y.max_ghost);
+                if (!one)
+                    need += 8 + (size_t)y.chunk * sizeof(ResPair<R>) +
+                            y.max_tab * (h ? res_row_bytes<R, SW, TH>() : res_row_bytes<R, SW, false>());
+                smem = std::max(smem, need);
             }
+            if (smem > (size_t)kResSmemMax) break;
+            r->smem = smem;
+            const int iters = (chunk + kResSlabThreads - 1) / kResSlabThreads;
+            r->threads = one ? kResThreads : std::max(kResThreads, res_up32((chunk + iters - 1) / iters));
+            const auto k1 = k_resident_one<R, SW, TH>;
+            const auto k2 = k_resident_slab<R, SW, TH>;
+            r->kernel = one ? reinterpret_cast<const void*>(k1) : reinterpret_cast<const void*>(k2);
+            e = cudaFuncSetAttribute(r->kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kResSmemMax);
+            if (e != cudaSuccess) return e;
+            int got = 0;
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&got, r->kernel, r->threads, r->smem);
+            if (e != cudaSuccess) return e;
+            fits = (long long)got * num_sms >= r->grid;
+            r->slab = true;
+            break;
         }
         auto kern = k_resident_grid<S, R, SW, TH>;
         for (int per_sm = 2; per_sm >= 1 && !fits; --per_sm) {
             const int most = per_sm * num_sms;
             if (n > most) return cudaSuccess;
-            const int chunk = chunk_for(most, 32, 32);
+            const int chunk = chunk_for(most);
             place(chunk);
             int ring = 0;
             for (const ResDom<S, R>& y : doms)
@@ -196,10 +249,14 @@ cudaError_t res_build(Resident* r, const ResidentDomain* d, int n, int num_sms, 
     // descriptors, CTA map, step counters: one allocation of the library's own
     const size_t b_doms = (n * sizeof(ResDom<S, R>) + 255) / 256 * 256;
     const size_t b_map = (cta_dom.size() * sizeof(int) + 255) / 256 * 256;
+    auto words = [&](const ResDom<S, R>& y) {  // (whole 128-byte lines per domain)
+        const size_t b = (size_t)y.ncta * nplanes<SW, TH>() * nl * 2 * (y.w + y.h) * sizeof(typename ResWord<R>::type);
+        return (b + 127) / 128 * 128;
+    };
     size_t b_flags = (size_t)r->grid * kResPad * sizeof(unsigned);
     if (r->slab) {
         b_flags = 0;
-        for (const ResDom<S, R>& y : doms) b_flags += (size_t)y.npairs * nl * nplanes<SW, TH>() * sizeof(typename ResWord<R>::type);
+        for (const ResDom<S, R>& y : doms) b_flags += words(y);
     }
     if (cudaMalloc(&r->scratch, b_doms + b_map + b_flags) != cudaSuccess) {
         cudaGetLastError();
@@ -213,7 +270,7 @@ cudaError_t res_build(Resident* r, const ResidentDomain* d, int n, int num_sms, 
         size_t off = r->off_flags;
         for (ResDom<S, R>& y : doms) {
             y.mail = m + off;
-            off += (size_t)y.npairs * nl * nplanes<SW, TH>() * sizeof(typename ResWord<R>::type);
+            off += words(y);
         }
     }
     e = cudaMemcpyAsync(m, doms.data(), n * sizeof(ResDom<S, R>), cudaMemcpyHostToDevice, stream);
