@@ -17,13 +17,16 @@
 // two convolutions per level (224 -> 96 -> 96, 160 -> 64 -> 64,
 // 96 -> 32 -> 32), and a 1x1 head 32 -> 4 without activation: 0.91 M weights.
 // Activations are NHWC in BF16.  Every 3x3 convolution -- forward, and in
-// training the input and weight gradients -- is an implicit GEMM of this
-// library on the tensor cores (ws_conv.cuh: mma.sync BF16 with FP32
-// accumulation, operands gathered straight from the activations); no im2col
-// matrix is formed and no GEMM library is called.
+// training the input and weight gradients -- is a kernel of this library on
+// the tensor cores (ws_conv.cuh: mma.sync BF16 with FP32 accumulation); no
+// im2col matrix is formed and no GEMM library is called.  The pools come out
+// of the epilogue of the convolution before them, the upsampled and
+// concatenated input of a decoder level is read from its two sources by the
+// convolution itself.
 #include <cuda_bf16.h>
 #include <math.h>
 
+#include <algorithm>
 #include <mutex>
 #include <new>
 #include <string>
@@ -42,12 +45,11 @@ constexpr int kCh[kLevels] = {32, 64, 96, 128};
 
 // The activations of one pass over n canvases: x0 the input canvas; per
 // encoder level the outputs of its two convolutions (a, e) and the pooled e
-// (p); per decoder level the upsampled deeper output concatenated with the
-// skip (u) and the outputs of its two convolutions (b, d).
+// (p); per decoder level the outputs of its two convolutions (b, d).
 struct Acts {
     __nv_bfloat16 *x0 = nullptr;
     __nv_bfloat16 *a[kLevels] = {}, *e[kLevels] = {}, *p[kLevels - 1] = {};
-    __nv_bfloat16 *u[kLevels - 1] = {}, *b[kLevels - 1] = {}, *d[kLevels - 1] = {};
+    __nv_bfloat16 *b[kLevels - 1] = {}, *d[kLevels - 1] = {};
 };
 
 }  // namespace
@@ -56,8 +58,8 @@ struct axlbm_ws {
     cudaStream_t stream;
     __nv_bfloat16* w;  // all layers, packed as in include/axlbm.h
     std::vector<size_t> woff, boff;
-    int chunk;
-    Acts act;  // one chunk of canvases
+    int chunk;  // canvases that `act` holds
+    Acts act;
     axlbm_ws_train* train;  // allocated by the first training call
     std::string err;
 };
@@ -102,47 +104,42 @@ __global__ void k_ws_input(const float* feat, int n, bf16* x) {
     const long long total = (long long)n * kH * kW;
     if (i >= total) return;
     const int c = int(i % kW), r = int((i / kW) % kH), b = int(i / ((long long)kH * kW));
-    bf16* o = x + i * 8;
+    __align__(16) bf16 o[8];
+#pragma unroll
     for (int f = 0; f < kFeat; ++f) o[f] = __float2bfloat16(feat[b * kFeat + f]);
     o[6] = __float2bfloat16((c + 0.5f) / kW);
     o[7] = __float2bfloat16((r + 0.5f) / kH);
+    *reinterpret_cast<uint4*>(x + i * 8) = *reinterpret_cast<const uint4*>(o);
 }
 
-// 2x2 average pool, NHWC.
-__global__ void k_ws_pool(const bf16* x, int n, int h, int w, int c, bf16* out) {
-    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    const int h2 = h / 2, w2 = w / 2;
-    if (i >= (long long)n * h2 * w2 * c) return;
-    const int ch = int(i % c);
-    const long long p = i / c;
-    const int xw = int(p % w2), yh = int((p / w2) % h2), b = int(p / ((long long)h2 * w2));
-    auto at = [&](int yy, int xx) { return __bfloat162float(x[(((long long)b * h + yy) * w + xx) * c + ch]); };
-    const float s = at(2 * yh, 2 * xw) + at(2 * yh, 2 * xw + 1) + at(2 * yh + 1, 2 * xw) + at(2 * yh + 1, 2 * xw + 1);
-    out[i] = __float2bfloat16(0.25f * s);
-}
-
-// Nearest 2x upsampling of `deep` (h/2 x w/2 x cd) concatenated with `skip`
-// (h x w x cs): out (h x w x (cd + cs)), deep channels first.
-__global__ void k_ws_up_concat(const bf16* deep, const bf16* skip, int n, int h, int w, int cd, int cs, bf16* out) {
-    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    const int c = cd + cs;
-    if (i >= (long long)n * h * w * c) return;
-    const int ch = int(i % c);
-    const long long p = i / c;
-    const int xw = int(p % w), yh = int((p / w) % h), b = int(p / ((long long)h * w));
-    out[i] = ch < cd ? deep[(((long long)b * (h / 2) + yh / 2) * (w / 2) + xw / 2) * cd + ch]
-                     : skip[p * cs + (ch - cd)];
-}
-
-// 1x1 head 32 -> 4 (no activation), to FP32 canvases [n][4][kH][kW].
-__global__ void k_ws_head(const bf16* x, const bf16* wt, const bf16* bias, int n, float* out) {
+// 1x1 head 32 -> 4 (no activation), to FP32 canvases [n][4][kH][kW]: one
+// pixel per thread, its 64 bytes in four loads, the weights in shared memory.
+__global__ void __launch_bounds__(256) k_ws_head(const bf16* x, const bf16* wt, const bf16* bias, int n, float* out) {
+    __shared__ float ws[4 * 32], bs[4];
+    if (threadIdx.x < 128) ws[threadIdx.x] = __bfloat162float(wt[threadIdx.x]);
+    if (threadIdx.x < 4) bs[threadIdx.x] = __bfloat162float(bias[threadIdx.x]);
+    __syncthreads();
     const long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (p >= (long long)n * kH * kW) return;
     const int b = int(p / ((long long)kH * kW));
     const long long pix = p % ((long long)kH * kW);
+    float v[32];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const uint4 u = reinterpret_cast<const uint4*>(x + p * 32)[q];
+        const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&u);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const float2 f = __bfloat1622float2(h[e]);
+            v[8 * q + 2 * e] = f.x;
+            v[8 * q + 2 * e + 1] = f.y;
+        }
+    }
+#pragma unroll
     for (int o = 0; o < 4; ++o) {
-        float s = __bfloat162float(bias[o]);
-        for (int c = 0; c < 32; ++c) s += __bfloat162float(wt[o * 32 + c]) * __bfloat162float(x[p * 32 + c]);
+        float s = bs[o];
+#pragma unroll
+        for (int c = 0; c < 32; ++c) s = fmaf(ws[o * 32 + c], v[c], s);
         out[((long long)b * 4 + o) * kH * kW + pix] = s;
     }
 }
@@ -197,23 +194,52 @@ __global__ void k_ws_to_canvas(const float* m, axlbm_ws_domain D, float* canvas)
 
 unsigned blocks_for(long long n) { return (unsigned)((n + 255) / 256); }
 
-// Output channels per block column of the implicit GEMM: 64 where they
-// divide, else 32 (every channel count here is a multiple of 32).
-int conv_bn(int cout) { return cout % 64 == 0 ? 64 : 32; }
-
-// 3x3 convolution of layer `layer` over n canvases of h x wd, with bias,
-// ReLU and BF16 output (the forward pass).
-cudaError_t conv3(axlbm_ws* w, int layer, const bf16* in, int n, int h, int wd, bf16* out) {
+// Launches a 3x3 convolution (ws_conv.cuh) over n images: cout in block columns
+// of 32 WN channels, tiles of 16 x 16 pixels where those still give every SM
+// two blocks, else of 8 x 16 (the deep levels; wide outputs of the gradients).
+template <int MODE>
+cudaError_t launch_conv(cudaStream_t st, const axl::wsconv::ConvIn& in, int n, const bf16* wt, int cout, const bf16* bias,
+                        const axl::wsconv::ConvOut& to) {
     using namespace axl::wsconv;
-    const Layer& L = kNet[layer];
-    const long long pixels = (long long)n * h * wd;
-    const int bn = conv_bn(L.cout);
-    const dim3 grid((unsigned)((pixels + kBM - 1) / kBM), (unsigned)(L.cout / bn));
-    const bf16* wt = w->w + w->woff[layer];
-    const bf16* bias = w->w + w->boff[layer];
-    if (bn == 64) k_conv_igemm<64, 0><<<grid, kThreads, 0, w->stream>>>(in, n, h, wd, L.cin, 0, wt, L.cout, bias, out);
-    else k_conv_igemm<32, 0><<<grid, kThreads, 0, w->stream>>>(in, n, h, wd, L.cin, 0, wt, L.cout, bias, out);
-    return cudaGetLastError();
+    const int wn = cout % 96 == 0 ? 3 : (cout % 64 == 0 ? 2 : (cout % 160 == 0 ? 5 : (cout % 224 == 0 ? 7 : 1)));
+    const long long px = (long long)n * in.h * in.w;
+    const bool tall = wn <= 3 && px / 256 * (cout / (32 * wn)) >= 2 * 148;
+    auto go = [&](auto wn_tag, auto th_tag) -> cudaError_t {
+        constexpr int WN = decltype(wn_tag)::value, TH = decltype(th_tag)::value;
+        auto kern = k_conv3<WN, TH, MODE>;
+        const size_t smem = conv_smem<WN, TH>(in.c0 + in.c1);
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)conv_smem<WN, TH>(224));
+        if (e != cudaSuccess) return e;
+        kern<<<dim3((unsigned)(px / (TH * kTW)), (unsigned)(cout / (32 * WN))), 8 * WN * TH, smem, st>>>(in, wt, cout, bias, to);
+        return cudaGetLastError();
+    };
+    using std::integral_constant;
+    const integral_constant<int, 8> low;
+    const integral_constant<int, 16> high;
+    switch (wn) {
+        case 1: return tall ? go(integral_constant<int, 1>{}, high) : go(integral_constant<int, 1>{}, low);
+        case 2: return tall ? go(integral_constant<int, 2>{}, high) : go(integral_constant<int, 2>{}, low);
+        case 3: return tall ? go(integral_constant<int, 3>{}, high) : go(integral_constant<int, 3>{}, low);
+    }
+    if constexpr (MODE == 1) {  // the inputs of the decoder's first convolutions
+        if (wn == 5) return go(integral_constant<int, 5>{}, low);
+        if (wn == 7) return go(integral_constant<int, 7>{}, low);
+    }
+    return cudaErrorInvalidValue;
+}
+
+// 3x3 convolution of layer `layer` over n canvases, with bias, ReLU and BF16
+// output, and the output's 2x2 average in `pool` unless null (the forward pass).
+cudaError_t conv3(axlbm_ws* w, int layer, const axl::wsconv::ConvIn& in, int n, bf16* out, bf16* pool = nullptr) {
+    return launch_conv<0>(w->stream, in, n, w->w + w->woff[layer], kNet[layer].cout, w->w + w->boff[layer],
+                          {out, pool, nullptr, nullptr, 0, nullptr});
+}
+
+// Input of an encoder level's first convolution, of any level's second, and of
+// a decoder level's first.
+axl::wsconv::ConvIn plain_in(const bf16* x, int c, int l) { return {x, nullptr, c, 0, 0, kH >> l, kW >> l}; }
+axl::wsconv::ConvIn decoder_in(const Acts& A, int l) {
+    return {l + 2 < kLevels ? A.d[l + 1] : A.e[kLevels - 1], A.e[l], kCh[l + 1], kCh[l], 1, kH >> l, kW >> l};
 }
 
 // Forward pass of n canvases through the network into the activations A,
@@ -222,27 +248,15 @@ cudaError_t forward_acts(axlbm_ws* w, const float* feat_dev, int n, Acts& A, flo
     cudaError_t e;
     k_ws_input<<<blocks_for((long long)n * kH * kW), 256, 0, w->stream>>>(feat_dev, n, A.x0);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    const bf16* in = A.x0;
     for (int l = 0; l < kLevels; ++l) {  // encoder
-        const int h = kH >> l, wd = kW >> l;
-        if ((e = conv3(w, enc_layer(l), in, n, h, wd, A.a[l])) != cudaSuccess) return e;
-        if ((e = conv3(w, enc_layer(l) + 1, A.a[l], n, h, wd, A.e[l])) != cudaSuccess) return e;
-        if (l + 1 < kLevels) {
-            k_ws_pool<<<blocks_for((long long)n * (h / 2) * (wd / 2) * kCh[l]), 256, 0, w->stream>>>(
-                A.e[l], n, h, wd, kCh[l], A.p[l]);
-            if ((e = cudaGetLastError()) != cudaSuccess) return e;
-            in = A.p[l];
-        }
+        e = conv3(w, enc_layer(l), l ? plain_in(A.p[l - 1], kCh[l - 1], l) : plain_in(A.x0, 8, 0), n, A.a[l]);
+        if (e != cudaSuccess) return e;
+        e = conv3(w, enc_layer(l) + 1, plain_in(A.a[l], kCh[l], l), n, A.e[l], l + 1 < kLevels ? A.p[l] : nullptr);
+        if (e != cudaSuccess) return e;
     }
-    const bf16* deep = A.e[kLevels - 1];
     for (int l = kLevels - 2; l >= 0; --l) {  // decoder
-        const int h = kH >> l, wd = kW >> l, cd = kCh[l + 1], cs = kCh[l];
-        k_ws_up_concat<<<blocks_for((long long)n * h * wd * (cd + cs)), 256, 0, w->stream>>>(deep, A.e[l], n, h, wd, cd,
-                                                                                           cs, A.u[l]);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        if ((e = conv3(w, dec_layer(l), A.u[l], n, h, wd, A.b[l])) != cudaSuccess) return e;
-        if ((e = conv3(w, dec_layer(l) + 1, A.b[l], n, h, wd, A.d[l])) != cudaSuccess) return e;
-        deep = A.d[l];
+        if ((e = conv3(w, dec_layer(l), decoder_in(A, l), n, A.b[l])) != cudaSuccess) return e;
+        if ((e = conv3(w, dec_layer(l) + 1, plain_in(A.b[l], kCh[l], l), n, A.d[l])) != cudaSuccess) return e;
     }
     k_ws_head<<<blocks_for((long long)n * kH * kW), 256, 0, w->stream>>>(A.d[0], w->w + w->woff[kHead],
                                                                           w->w + w->boff[kHead], n, canvas);
@@ -262,7 +276,6 @@ std::vector<size_t> acts_sizes(int n) {
     }
     for (int l = 0; l + 1 < kLevels; ++l) {
         const size_t P = P0 >> (2 * l);
-        v.push_back(P * (kCh[l] + kCh[l + 1]));    // u
         v.push_back(P * kCh[l]);                   // b
         v.push_back(P * kCh[l]);                   // d
     }
@@ -277,7 +290,6 @@ std::vector<bf16**> acts_ptrs(Acts& A) {
         if (l + 1 < kLevels) v.push_back(&A.p[l]);
     }
     for (int l = 0; l + 1 < kLevels; ++l) {
-        v.push_back(&A.u[l]);
         v.push_back(&A.b[l]);
         v.push_back(&A.d[l]);
     }
@@ -308,15 +320,15 @@ void acts_free(Acts& A) {
 // layer's output; the loss is the mean squared error over the canvases; the
 // backward pass runs through the head, the ReLU masks, the convolutions (the
 // weight gradient dW[o][k] = sum_p dY[p][o] A[p][k] and the input gradient,
-// a convolution of dY with the mirrored taps, both implicit GEMMs of
-// ws_conv.cuh with FP32 accumulation), the concatenations and the pools; Adam
+// a convolution of dY with the mirrored taps, both kernels of ws_conv.cuh
+// with FP32 accumulation), the concatenations and the pools; Adam
 // then updates FP32 master weights and rewrites the BF16 weights the forward
 // pass uses.  Reductions (loss, biases, head, weight gradients over pixel
 // ranges) go through partials summed in a fixed order, so a step is
 // deterministic.
 
-constexpr int kTrainMax = 16;      // canvases per training step
-constexpr int kRowsPerBlock = 2048;  // rows of one reduction block
+constexpr int kTrainMax = 16;    // canvases per training step
+constexpr int kPredictMax = 32;  // canvases per inference pass
 
 // Mean-squared-error gradient 2 (out - target) / count, and per-block sums of
 // (out - target)^2.
@@ -339,111 +351,144 @@ __global__ void k_ws_loss_grad(const float* out, const float* target, long long 
     if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
 }
 
-__global__ void k_ws_sum_double(const double* part, int n, double* out) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        double s = 0.0;
-        for (int i = 0; i < n; ++i) s += part[i];
-        *out = s;
-    }
-}
-
-// Column sums of x [rows][cols] (cols <= 256): per-block partials
-// part[block][cols] over rows [block * kRowsPerBlock, ...).
-__global__ void k_ws_colsum(const bf16* x, long long rows, int cols, float* part) {
-    __shared__ float sh[256];
-    const int nph = blockDim.x / cols;
-    const int c = threadIdx.x % cols, ph = threadIdx.x / cols;
-    const long long r0 = (long long)blockIdx.x * kRowsPerBlock;
-    const long long r1 = r0 + kRowsPerBlock < rows ? r0 + kRowsPerBlock : rows;
-    float s = 0.0f;
-    if (ph < nph)
-        for (long long r = r0 + ph; r < r1; r += nph) s += __bfloat162float(x[r * cols + c]);
+// Sum of n doubles in a fixed order (n a multiple of 256, one block of 256).
+__global__ void __launch_bounds__(256) k_ws_sum_double(const double* part, int n, double* out) {
+    __shared__ double sh[256];
+    double s = 0.0;
+    for (int i = threadIdx.x; i < n; i += 256) s += part[i];
     sh[threadIdx.x] = s;
     __syncthreads();
-    if (ph == 0) {
-        for (int k = 1; k < nph; ++k) s += sh[k * cols + c];
-        part[(long long)blockIdx.x * cols + c] = s;
+    for (int k = 128; k > 0; k >>= 1) {
+        if (threadIdx.x < k) sh[threadIdx.x] += sh[threadIdx.x + k];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) *out = sh[0];
+}
+
+// out[c] = sum over blocks of part[block][c], in a fixed order: eight
+// interleaved runs of blocks per value, then the runs.
+__global__ void __launch_bounds__(256) k_ws_fold(const float* part, int nblocks, int cols, float* out) {
+    __shared__ float sh[8][32];
+    const int v = threadIdx.x & 31, run = threadIdx.x >> 5, c = blockIdx.x * 32 + v;
+    float s = 0.0f;
+    if (c < cols)
+        for (int b = run; b < nblocks; b += 8) s += part[(long long)b * cols + c];
+    sh[run][v] = s;
+    __syncthreads();
+    if (run == 0 && c < cols) {
+        for (int g = 1; g < 8; ++g) s += sh[g][v];
+        out[c] = s;
     }
 }
 
-// out[c] = sum over blocks of part[block][c], in block order.
-__global__ void k_ws_fold(const float* part, int nblocks, int cols, float* out) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= cols) return;
-    float s = 0.0f;
-    for (int b = 0; b < nblocks; ++b) s += part[(long long)b * cols + c];
-    out[c] = s;
-}
-
-// Head (1x1, 32 -> 4) gradients: per-block partials of dW[o][c] =
-// sum_p dout[o](p) x[p][c] (threads 0..127) and db[o] (threads 128..131).
-__global__ void k_ws_head_wgrad(const float* dout, const bf16* x, int n, float* part) {
-    const long long pixels = (long long)n * kH * kW;
-    const long long r0 = (long long)blockIdx.x * kRowsPerBlock;
-    const long long r1 = r0 + kRowsPerBlock < pixels ? r0 + kRowsPerBlock : pixels;
-    const int t = threadIdx.x;
-    if (t >= 132) return;
-    const int o = t < 128 ? t >> 5 : t - 128, c = t & 31;
-    float s = 0.0f;
-    for (long long p = r0; p < r1; ++p) {
-        const long long b = p / ((long long)kH * kW), pix = p % ((long long)kH * kW);
-        const float g = dout[(b * 4 + o) * kH * kW + pix];
-        s += t < 128 ? g * __bfloat162float(x[p * 32 + c]) : g;
+// Head (1x1, 32 -> 4) gradients: per-block partials [132] of dW[o][c] =
+// sum_p dout[o](p) x[p][c], then db[o].  A warp reads one pixel's 32 channels
+// at a time, lane = channel; blocks of kHeadRows pixels of one canvas.
+constexpr int kHeadRows = 512;
+__global__ void __launch_bounds__(256) k_ws_head_wgrad(const float* dout, const bf16* x, float* part) {
+    __shared__ float sh[8][132];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const long long p0 = (long long)blockIdx.x * kHeadRows, b = p0 / ((long long)kH * kW), pix0 = p0 % ((long long)kH * kW);
+    const float* d = dout + b * 4 * kH * kW + pix0;
+    float s[4] = {0.0f, 0.0f, 0.0f, 0.0f}, sb[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    for (int r = wid; r < kHeadRows; r += 8) {
+        const float v = __bfloat162float(x[(p0 + r) * 32 + lane]);
+#pragma unroll
+        for (int o = 0; o < 4; ++o) {
+            const float g = d[(long long)o * kH * kW + r];
+            s[o] = fmaf(g, v, s[o]);
+            sb[o] += g;
+        }
     }
-    part[(long long)blockIdx.x * 132 + t] = s;
+#pragma unroll
+    for (int o = 0; o < 4; ++o) {
+        sh[wid][o * 32 + lane] = s[o];
+        if (lane == 0) sh[wid][128 + o] = sb[o];
+    }
+    __syncthreads();
+    for (int t = threadIdx.x; t < 132; t += blockDim.x) {
+        float v = sh[0][t];
+        for (int g = 1; g < 8; ++g) v += sh[g][t];
+        part[(long long)blockIdx.x * 132 + t] = v;
+    }
 }
 
-// Head input gradient through the ReLU of its input x:
-// dy[p][c] = (sum_o dout[o](p) W[o][c]) [x[p][c] > 0].
-__global__ void k_ws_head_dx(const float* dout, const bf16* wt, const bf16* x, int n, bf16* dy) {
-    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    const long long pixels = (long long)n * kH * kW;
-    if (i >= pixels * 32) return;
-    const int c = int(i & 31);
-    const long long p = i >> 5, b = p / ((long long)kH * kW), pix = p % ((long long)kH * kW);
-    float g = 0.0f;
-    for (int o = 0; o < 4; ++o) g += dout[(b * 4 + o) * kH * kW + pix] * __bfloat162float(wt[o * 32 + c]);
-    dy[i] = __float2bfloat16(__bfloat162float(x[i]) > 0.0f ? g : 0.0f);
+// Eight BF16 values of v where the activations are positive, else zero.
+__device__ __forceinline__ uint4 ws_masked8(const float (&v)[8], const bf16* act) {
+    const uint4 u = *reinterpret_cast<const uint4*>(act);
+    const __nv_bfloat162* a = reinterpret_cast<const __nv_bfloat162*>(&u);
+    uint4 out;
+    __nv_bfloat162* o = reinterpret_cast<__nv_bfloat162*>(&out);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        o[e].x = __float2bfloat16(__bfloat162float(a[e].x) > 0.0f ? v[2 * e] : 0.0f);
+        o[e].y = __float2bfloat16(__bfloat162float(a[e].y) > 0.0f ? v[2 * e + 1] : 0.0f);
+    }
+    return out;
+}
+__device__ __forceinline__ void ws_load8(const float* p, float (&v)[8]) {
+    const float4 a = reinterpret_cast<const float4*>(p)[0], b = reinterpret_cast<const float4*>(p)[1];
+    v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w, v[4] = b.x, v[5] = b.y, v[6] = b.z, v[7] = b.w;
 }
 
-// Gradient of a layer's output through its ReLU: dy = (g + g2) [act > 0].
-__global__ void k_ws_mask(const float* g, const float* g2, const bf16* act, long long count, bf16* dy) {
+// Head input gradient through the ReLU of its input x, eight channels per
+// thread: dy[p][c] = (sum_o dout[o](p) W[o][c]) [x[p][c] > 0].
+__global__ void __launch_bounds__(256) k_ws_head_dx(const float* dout, const bf16* wt, const bf16* x, int n, bf16* dy) {
+    __shared__ float ws[4 * 32];
+    if (threadIdx.x < 128) ws[threadIdx.x] = __bfloat162float(wt[threadIdx.x]);
+    __syncthreads();
     const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (i >= count) return;
-    const float v = g[i] + (g2 ? g2[i] : 0.0f);
-    dy[i] = __float2bfloat16(__bfloat162float(act[i]) > 0.0f ? v : 0.0f);
+    if (i >= (long long)n * kH * kW * 4) return;
+    const int c = int(i & 3) * 8;
+    const long long p = i >> 2, b = p / ((long long)kH * kW), pix = p % ((long long)kH * kW);
+    float g[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+    for (int o = 0; o < 4; ++o) {
+        const float d = dout[(b * 4 + o) * kH * kW + pix];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) g[e] = fmaf(d, ws[o * 32 + c + e], g[e]);
+    }
+    *reinterpret_cast<uint4*>(dy + p * 32 + c) = ws_masked8(g, x + p * 32 + c);
 }
 
-// Backward of the nearest upsampling + concatenation (h x w output, deep
-// channels first): gdeep (h/2 x w/2 x cd) sums its four copies, gskip
-// (h x w x cs) takes the skip channels.
-__global__ void k_ws_upcat_bwd_deep(const float* gu, int n, int h, int w, int cd, int cs, float* gdeep) {
+// Gradient of a decoder level's deep input (h x w, c channels, FP32, at the
+// level's resolution) at the deeper level's: the sum of the four copies the
+// upsampling made, through the ReLU of `act`; eight channels per thread.
+__global__ void __launch_bounds__(256) k_ws_up_bwd(const float* g, int n, int h, int w, int c, const bf16* act, bf16* dy) {
     const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    const int h2 = h / 2, w2 = w / 2, c = cd + cs;
-    if (i >= (long long)n * h2 * w2 * cd) return;
-    const int ch = int(i % cd);
-    const long long p = i / cd;
+    const int h2 = h / 2, w2 = w / 2, nch = c / 8;
+    if (i >= (long long)n * h2 * w2 * nch) return;
+    const int ch = int(i % nch) * 8;
+    const long long p = i / nch;
     const int x2 = int(p % w2), y2 = int((p / w2) % h2), b = int(p / ((long long)h2 * w2));
-    float s = 0.0f;
-    for (int dy = 0; dy < 2; ++dy)
-        for (int dx = 0; dx < 2; ++dx) s += gu[(((long long)b * h + 2 * y2 + dy) * w + 2 * x2 + dx) * c + ch];
-    gdeep[i] = s;
-}
-__global__ void k_ws_upcat_bwd_skip(const float* gu, long long pixels, int cd, int cs, float* gskip) {
-    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (i >= pixels * cs) return;
-    gskip[i] = gu[(i / cs) * (cd + cs) + cd + i % cs];
+    float s[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+    for (int d = 0; d < 4; ++d) {
+        float v[8];
+        ws_load8(g + (((long long)b * h + 2 * y2 + (d >> 1)) * w + 2 * x2 + (d & 1)) * c + ch, v);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) s[e] += v[e];
+    }
+    *reinterpret_cast<uint4*>(dy + p * c + ch) = ws_masked8(s, act + p * c + ch);
 }
 
-// Backward of the 2x2 average pool (h x w input): gx = gp / 4 at each of the
-// four inputs of a pooled pixel.
-__global__ void k_ws_pool_bwd(const float* gp, int n, int h, int w, int c, float* gx) {
+// Gradient of an encoder level's output (h x w, c channels), which feeds the
+// 2x2 average pool (gradient gp) and the skip (gradient gs), through its ReLU;
+// eight channels per thread.
+__global__ void __launch_bounds__(256) k_ws_pool_bwd(const float* gp, const float* gs, int n, int h, int w, int c,
+                                                     const bf16* act, bf16* dy) {
     const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (i >= (long long)n * h * w * c) return;
-    const int ch = int(i % c);
-    const long long p = i / c;
+    const int nch = c / 8;
+    if (i >= (long long)n * h * w * nch) return;
+    const int ch = int(i % nch) * 8;
+    const long long p = i / nch;
     const int xw = int(p % w), yh = int((p / w) % h), b = int(p / ((long long)h * w));
-    gx[i] = 0.25f * gp[(((long long)b * (h / 2) + yh / 2) * (w / 2) + xw / 2) * c + ch];
+    float v[8], s[8];
+    ws_load8(gp + (((long long)b * (h / 2) + yh / 2) * (w / 2) + xw / 2) * c + ch, v);
+    ws_load8(gs + p * c + ch, s);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) v[e] = 0.25f * v[e] + s[e];
+    *reinterpret_cast<uint4*>(dy + p * c + ch) = ws_masked8(v, act + p * c + ch);
 }
 
 // Adam on FP32 master weights (bias corrections c1 = 1 - beta1^t, c2 =
@@ -475,9 +520,9 @@ struct axlbm_ws_train {
     float *master = nullptr, *grad = nullptr, *m = nullptr, *v = nullptr;
     int64_t step = 0;
     Acts act;            // every activation of the kept forward pass
-    bf16* dy = nullptr;  // gradient of a layer's pre-activation output (BF16, the GEMM operand)
+    bf16 *dy = nullptr, *dy2 = nullptr;  // gradients of two layers' pre-activation outputs (BF16, the GEMM operands)
     bf16* wtt = nullptr; // the mirrored-tap weights of the input gradient of one layer
-    float *out = nullptr, *dout = nullptr, *gx = nullptr, *gx2 = nullptr, *part = nullptr, *wpart = nullptr;
+    float *out = nullptr, *dout = nullptr, *gx = nullptr, *part = nullptr, *wpart = nullptr, *bpart = nullptr;
     float* gs[kLevels - 1] = {};  // gradients reaching the skips
     double *dpart = nullptr, *loss = nullptr;
 };
@@ -485,28 +530,45 @@ struct axlbm_ws_train {
 namespace {
 
 constexpr int kLossBlocks = 1024;
-constexpr int kSplitPixels = 2048;  // pixels per partial of a weight gradient
+constexpr int kWgradBlocks = 4 * 148;  // blocks of a weight gradient, about (two waves of two blocks per SM)
+
+// Splits of layer l's weight gradient over n canvases, and the pixel tiles of one.
+void wgrad_splits(int l, int n, int* nsplit, int* per, int* tiles);
 
 void train_free(axlbm_ws_train* t) {
     if (!t) return;
     acts_free(t->act);
-    void* ps[] = {t->master, t->grad, t->m, t->v, t->dy, t->wtt, t->out, t->dout, t->gx, t->gx2, t->part, t->wpart,
-                  t->gs[0], t->gs[1], t->gs[2], t->dpart, t->loss};
+    void* ps[] = {t->master, t->grad, t->m, t->v, t->dy, t->dy2, t->wtt, t->out, t->dout, t->gx, t->part, t->wpart,
+                  t->bpart, t->gs[0], t->gs[1], t->gs[2], t->dpart, t->loss};
     for (void* p : ps)
         if (p) cudaFree(p);
     delete t;
 }
 
+int layer_level(int l) { return l < 8 ? l / 2 : 2 - (l - 8) / 2; }
+int wgrad_nc(int l) { return kNet[l].cin == 8 ? 8 : 32; }
+
+void wgrad_splits(int l, int n, int* nsplit, int* per, int* tiles) {
+    const int lev = layer_level(l);
+    *tiles = n * (kH >> lev) * (kW >> lev) / (axl::wsconv::kWgTH * axl::wsconv::kTW);
+    const int cols = kNet[l].cin / wgrad_nc(l) * (kNet[l].cout / 32);
+    int s = kWgradBlocks / cols;
+    s = s < 1 ? 1 : (s > *tiles ? *tiles : s);
+    *per = (*tiles + s - 1) / s;
+    *nsplit = (*tiles + *per - 1) / *per;
+}
+
 // Values of the largest weight-gradient partial buffer of a training step.
-size_t wpart_values() {
+size_t wpart_values(size_t* bias) {
     size_t best = 0;
-    for (int l = 0; l < kHead; ++l) {
-        const int lev = l < 8 ? l / 2 : 2 - (l - 8) / 2;  // level of layer l
-        const size_t P = (size_t)kTrainMax * (kH >> lev) * (kW >> lev);
-        const size_t nsplit = (P + kSplitPixels - 1) / kSplitPixels;
-        const size_t v = nsplit * kNet[l].cout * 9 * kNet[l].cin;
-        if (v > best) best = v;
-    }
+    *bias = 0;
+    for (int l = 0; l < kHead; ++l)
+        for (int n = 1; n <= kTrainMax; ++n) {
+            int nsplit, per, tiles;
+            wgrad_splits(l, n, &nsplit, &per, &tiles);
+            best = std::max(best, (size_t)nsplit * kNet[l].cout * 9 * kNet[l].cin);
+            *bias = std::max(*bias, (size_t)nsplit * kNet[l].cout);
+        }
     return best;
 }
 
@@ -519,13 +581,15 @@ axlbm_status train_ensure(axlbm_ws* w) {
     const size_t P = (size_t)kTrainMax * kH * kW;  // level-0 pixels
     size_t wtt = 0;
     for (int l = 0; l < kHead; ++l) wtt = std::max(wtt, (size_t)9 * kNet[l].cin * kNet[l].cout);
+    size_t bvals = 0;
+    const size_t wvals = wpart_values(&bvals);
     struct Buf { void** p; size_t bytes; };
     const Buf bufs[] = {
         {(void**)&t->master, count * 4}, {(void**)&t->grad, count * 4}, {(void**)&t->m, count * 4},
-        {(void**)&t->v, count * 4},      {(void**)&t->dy, P * 32 * 2},  {(void**)&t->wtt, wtt * 2},
-        {(void**)&t->out, P * 4 * 4},    {(void**)&t->dout, P * 4 * 4}, {(void**)&t->gx, P * 96 * 4},
-        {(void**)&t->gx2, P * 32 * 4},   {(void**)&t->part, (P / kRowsPerBlock + 1) * 132 * 4},
-        {(void**)&t->wpart, wpart_values() * 4},
+        {(void**)&t->v, count * 4},      {(void**)&t->dy, P * 32 * 2},  {(void**)&t->dy2, P * 32 * 2},
+        {(void**)&t->wtt, wtt * 2},      {(void**)&t->out, P * 4 * 4},  {(void**)&t->dout, P * 4 * 4},
+        {(void**)&t->gx, P * 64 * 4},    {(void**)&t->part, P / kHeadRows * 132 * 4},
+        {(void**)&t->wpart, wvals * 4},  {(void**)&t->bpart, bvals * 4},
         {(void**)&t->gs[0], P * kCh[0] * 4}, {(void**)&t->gs[1], P / 4 * kCh[1] * 4},
         {(void**)&t->gs[2], P / 16 * kCh[2] * 4}, {(void**)&t->dpart, kLossBlocks * 8}, {(void**)&t->loss, 8}};
     for (const Buf& b : bufs) {
@@ -566,40 +630,49 @@ cudaError_t train_loss(axlbm_ws* w, const float* target, int n, bool grad) {
     axlbm_ws_train* t = w->train;
     const long long count = (long long)n * 4 * kH * kW;
     k_ws_loss_grad<<<kLossBlocks, 256, 0, w->stream>>>(t->out, target, count, grad ? t->dout : nullptr, t->dpart);
-    k_ws_sum_double<<<1, 32, 0, w->stream>>>(t->dpart, kLossBlocks, t->loss);
+    k_ws_sum_double<<<1, 256, 0, w->stream>>>(t->dpart, kLossBlocks, t->loss);
     return cudaGetLastError();
 }
 
-// Backward of 3x3 layer l (input `in`, n canvases of h x wd) from the
-// gradient of its pre-activation output in t->dy: bias and weight gradients
-// into t->grad, and the input gradient into gx (FP32) unless gx is null.
-cudaError_t conv_bwd(axlbm_ws* w, int l, const bf16* in, int n, int h, int wd, float* gx) {
+// Bias and weight gradients of 3x3 layer l (input `in`, n canvases) into
+// t->grad, from the gradient dy of its pre-activation output.
+cudaError_t conv_wgrad(axlbm_ws* w, int l, const axl::wsconv::ConvIn& in, int n, const bf16* dy) {
     using namespace axl::wsconv;
     axlbm_ws_train* t = w->train;
     const Layer& L = kNet[l];
-    cudaStream_t st = w->stream;
-    const long long P = (long long)n * h * wd;
-    const int K = 9 * L.cin;
-    const int nb = (int)((P + kRowsPerBlock - 1) / kRowsPerBlock);
-    k_ws_colsum<<<nb, 256, 0, st>>>(t->dy, P, L.cout, t->part);
-    k_ws_fold<<<1, 128, 0, st>>>(t->part, nb, L.cout, t->grad + w->boff[l]);
-    const int nsplit = (int)((P + kSplitPixels - 1) / kSplitPixels);
-    const dim3 gw((unsigned)((K + kWgN - 1) / kWgN), (unsigned)(L.cout / 32), (unsigned)nsplit);
-    k_conv_wgrad<<<gw, kThreads, 0, st>>>(t->dy, in, n, h, wd, L.cin, L.cout, kSplitPixels, t->wpart);
-    const long long cnt = (long long)L.cout * K;
-    k_fold_splits<<<blocks_for(cnt), 256, 0, st>>>(t->wpart, nsplit, cnt, t->grad + w->woff[l]);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess || !gx) return e;
-    // the input gradient: dy convolved with the mirrored taps of Wt[c][tap][o]
-    k_transpose_taps<<<blocks_for(cnt), 256, 0, st>>>(w->w + w->woff[l], L.cout, L.cin, t->wtt);
-    const int bn = conv_bn(L.cin);
-    const dim3 gi((unsigned)((P + kBM - 1) / kBM), (unsigned)(L.cin / bn));
-    if (bn == 64) k_conv_igemm<64, 1><<<gi, kThreads, 0, st>>>(t->dy, n, h, wd, L.cout, 1, t->wtt, L.cin, nullptr, gx);
-    else k_conv_igemm<32, 1><<<gi, kThreads, 0, st>>>(t->dy, n, h, wd, L.cout, 1, t->wtt, L.cin, nullptr, gx);
+    int nsplit, per, tiles;
+    wgrad_splits(l, n, &nsplit, &per, &tiles);
+    auto go = [&](auto nc_tag) -> cudaError_t {
+        constexpr int NC = decltype(nc_tag)::value;
+        auto kern = k_conv_wgrad<NC>;
+        constexpr size_t smem = 2 * wgrad_stage<NC>();
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        kern<<<dim3((unsigned)(L.cin / NC), (unsigned)(L.cout / 32), (unsigned)nsplit), 288, smem, w->stream>>>(
+            dy, in, L.cout, tiles, per, t->wpart, t->bpart);
+        return cudaGetLastError();
+    };
+    const cudaError_t e = wgrad_nc(l) == 8 ? go(std::integral_constant<int, 8>{}) : go(std::integral_constant<int, 32>{});
+    if (e != cudaSuccess) return e;
+    const long long cnt = (long long)L.cout * 9 * L.cin;
+    k_fold_splits<<<(unsigned)((cnt + L.cout + kFoldVals - 1) / kFoldVals), kFoldRuns * kFoldVals, 0, w->stream>>>(
+        t->wpart, t->bpart, nsplit, cnt, L.cout, t->grad + w->woff[l], t->grad + w->boff[l]);
     return cudaGetLastError();
 }
 
+// Input gradient of 3x3 layer l: dy convolved with the mirrored taps of Wt[c][tap][o].
+template <int MODE>
+cudaError_t conv_dgrad(axlbm_ws* w, int l, int n, const bf16* dy, const axl::wsconv::ConvOut& to) {
+    using namespace axl::wsconv;
+    axlbm_ws_train* t = w->train;
+    const Layer& L = kNet[l];
+    k_transpose_taps<<<blocks_for((long long)L.cout * 9 * L.cin), 256, 0, w->stream>>>(w->w + w->woff[l], L.cout, L.cin, t->wtt);
+    return launch_conv<MODE>(w->stream, plain_in(dy, L.cout, layer_level(l)), n, t->wtt, L.cin, nullptr, to);
+}
+
 // Backward pass of the kept forward pass from t->dout, gradients into t->grad.
+// A level's second convolution passes its gradient through the ReLU of the
+// first one's output within its own input gradient (dy -> dy2).
 cudaError_t train_backward(axlbm_ws* w, int n) {
     axlbm_ws_train* t = w->train;
     Acts& A = t->act;
@@ -607,35 +680,37 @@ cudaError_t train_backward(axlbm_ws* w, int n) {
     cudaError_t e;
     const long long P0 = (long long)n * kH * kW;
     // head (packed kernel then bias: 132 contiguous values)
-    const int nb = (int)((P0 + kRowsPerBlock - 1) / kRowsPerBlock);
-    k_ws_head_wgrad<<<nb, 160, 0, st>>>(t->dout, A.d[0], n, t->part);
-    k_ws_fold<<<1, 160, 0, st>>>(t->part, nb, 132, t->grad + w->woff[kHead]);
-    k_ws_head_dx<<<blocks_for(P0 * 32), 256, 0, st>>>(t->dout, w->w + w->woff[kHead], A.d[0], n, t->dy);
+    const int nb = (int)(P0 / kHeadRows);
+    k_ws_head_wgrad<<<nb, 256, 0, st>>>(t->dout, A.d[0], t->part);
+    k_ws_fold<<<(132 + 31) / 32, 256, 0, st>>>(t->part, nb, 132, t->grad + w->woff[kHead]);
+    k_ws_head_dx<<<blocks_for(P0 * 4), 256, 0, st>>>(t->dout, w->w + w->woff[kHead], A.d[0], n, t->dy);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     // decoder levels 0, 1, 2; t->dy holds the gradient of the level's second convolution
     for (int l = 0; l + 1 < kLevels; ++l) {
         const int h = kH >> l, wd = kW >> l, cd = kCh[l + 1], cs = kCh[l];
-        const long long P = P0 >> (2 * l);
-        if ((e = conv_bwd(w, dec_layer(l) + 1, A.b[l], n, h, wd, t->gx)) != cudaSuccess) return e;
-        k_ws_mask<<<blocks_for(P * cs), 256, 0, st>>>(t->gx, nullptr, A.b[l], P * cs, t->dy);
-        if ((e = conv_bwd(w, dec_layer(l), A.u[l], n, h, wd, t->gx)) != cudaSuccess) return e;
-        k_ws_upcat_bwd_deep<<<blocks_for(P / 4 * cd), 256, 0, st>>>(t->gx, n, h, wd, cd, cs, t->gx2);
-        k_ws_upcat_bwd_skip<<<blocks_for(P * cs), 256, 0, st>>>(t->gx, P, cd, cs, t->gs[l]);
-        const bf16* deep = l + 2 < kLevels ? A.d[l + 1] : A.e[kLevels - 1];
-        k_ws_mask<<<blocks_for(P / 4 * cd), 256, 0, st>>>(t->gx2, nullptr, deep, P / 4 * cd, t->dy);
+        if ((e = conv_wgrad(w, dec_layer(l) + 1, plain_in(A.b[l], cs, l), n, t->dy)) != cudaSuccess) return e;
+        if ((e = conv_dgrad<2>(w, dec_layer(l) + 1, n, t->dy, {t->dy2, nullptr, nullptr, nullptr, 0, A.b[l]})) != cudaSuccess)
+            return e;
+        if ((e = conv_wgrad(w, dec_layer(l), decoder_in(A, l), n, t->dy2)) != cudaSuccess) return e;
+        if ((e = conv_dgrad<1>(w, dec_layer(l), n, t->dy2, {nullptr, nullptr, t->gx, t->gs[l], cd, nullptr})) != cudaSuccess)
+            return e;
+        k_ws_up_bwd<<<blocks_for((P0 >> (2 * l)) / 4 * (cd / 8)), 256, 0, st>>>(t->gx, n, h, wd, cd,
+                                                                               decoder_in(A, l).x0, t->dy);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     // encoder levels 3 .. 0; t->gx holds the gradient of the pooled output of the level
     for (int l = kLevels - 1; l >= 0; --l) {
         const int h = kH >> l, wd = kW >> l, c = kCh[l];
-        const long long P = P0 >> (2 * l);
         if (l + 1 < kLevels) {  // e[l] feeds the pool and the skip
-            k_ws_pool_bwd<<<blocks_for(P * c), 256, 0, st>>>(t->gx, n, h, wd, c, t->gx2);
-            k_ws_mask<<<blocks_for(P * c), 256, 0, st>>>(t->gx2, t->gs[l], A.e[l], P * c, t->dy);
+            k_ws_pool_bwd<<<blocks_for((P0 >> (2 * l)) * (c / 8)), 256, 0, st>>>(t->gx, t->gs[l], n, h, wd, c, A.e[l], t->dy);
+            if ((e = cudaGetLastError()) != cudaSuccess) return e;
         }
-        if ((e = conv_bwd(w, enc_layer(l) + 1, A.a[l], n, h, wd, t->gx)) != cudaSuccess) return e;
-        k_ws_mask<<<blocks_for(P * c), 256, 0, st>>>(t->gx, nullptr, A.a[l], P * c, t->dy);
-        if ((e = conv_bwd(w, enc_layer(l), l ? A.p[l - 1] : A.x0, n, h, wd, l ? t->gx : nullptr)) != cudaSuccess)
+        if ((e = conv_wgrad(w, enc_layer(l) + 1, plain_in(A.a[l], c, l), n, t->dy)) != cudaSuccess) return e;
+        if ((e = conv_dgrad<2>(w, enc_layer(l) + 1, n, t->dy, {t->dy2, nullptr, nullptr, nullptr, 0, A.a[l]})) != cudaSuccess)
+            return e;
+        const axl::wsconv::ConvIn in = l ? plain_in(A.p[l - 1], kCh[l - 1], l) : plain_in(A.x0, 8, 0);
+        if ((e = conv_wgrad(w, enc_layer(l), in, n, t->dy2)) != cudaSuccess) return e;
+        if (l && (e = conv_dgrad<1>(w, enc_layer(l), n, t->dy2, {nullptr, nullptr, t->gx, t->gx, in.c0, nullptr})) != cudaSuccess)
             return e;
     }
     return cudaGetLastError();
@@ -657,7 +732,7 @@ axlbm_status axlbm_ws_create(const uint16_t* weights, size_t count, void* cuda_s
     }
     if (!w) return wfail(nullptr, AXLBM_ENOMEM, "host allocation failed");
     w->stream = static_cast<cudaStream_t>(cuda_stream);
-    w->chunk = 8;
+    w->chunk = 8;  // (axlbm_ws_predict grows it)
     size_t off = 0;
     for (const Layer& l : kNet) {
         w->woff.push_back(off);
@@ -689,7 +764,22 @@ axlbm_status axlbm_ws_predict(axlbm_ws* w, const float* features, int32_t n, flo
         cudaGetLastError();
         return wfail(w, AXLBM_ENOMEM, "feature buffer");
     }
-    e = cudaMemcpyAsync(fd, features, (size_t)n * kFeat * sizeof(float), cudaMemcpyHostToDevice, w->stream);
+    // more canvases per pass fill the SMs at the deep levels (level 3 of 8 canvases is 32 tiles); without
+    // room for them the pass stays as it was
+    if (n > w->chunk && w->chunk < kPredictMax) {
+        Acts more;
+        const int want = n < kPredictMax ? n : kPredictMax;
+        e = cudaStreamSynchronize(w->stream);
+        if (e == cudaSuccess && acts_alloc(more, want)) {
+            acts_free(w->act);
+            w->act = more;
+            w->chunk = want;
+        } else {
+            acts_free(more);
+        }
+    }
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(fd, features, (size_t)n * kFeat * sizeof(float), cudaMemcpyHostToDevice, w->stream);
     for (int b0 = 0; b0 < n && e == cudaSuccess; b0 += w->chunk) {
         const int m = n - b0 < w->chunk ? n - b0 : w->chunk;
         e = forward_acts(w, fd + (size_t)b0 * kFeat, m, w->act, canvas + (size_t)b0 * 4 * kH * kW);

@@ -1,19 +1,17 @@
-// ws_conv.cuh -- BF16 implicit-GEMM 3x3 convolutions of the warm-start
-// network on the tensor cores (mma.sync m16n8k16, FP32 accumulation).
+// ws_conv.cuh -- BF16 3x3 convolutions of the warm-start network on the
+// tensor cores (mma.sync m16n8k16, FP32 accumulation).
 //
 // Activations are NHWC BF16; a layer's weights are packed [cout][tap][cin]
 // with tap = 3 ky + kx (the layout of the weight blob in include/axlbm.h), so
-// the K index of the GEMM is k = tap * cin + c.  Nothing is materialised:
-// each thread block gathers its A tile (pixels x k) straight from the input
-// image with 16-byte cp.async copies (zero-filled outside the image and past
-// K), double-buffered in shared memory, and feeds the tensor cores from
-// shared memory with ldmatrix.
+// the K index of the GEMM is k = tap * cin + c.  No im2col matrix is formed:
+// a block keeps a tile of pixels with its border in shared memory and takes
+// the operands of every tap from it at a shifted address, by ldmatrix.
 //
 //   forward:       y[p][o]  = sum_k  A[p][k] W[o][k],  A[p][(tap, c)] = x[p + d(tap)][c]
 //   input grad:    gx[q][c] = sum_k' B[q][k'] Wt[c][k'], B[q][(tap, o)] = dy[q - d(tap)][o]
 //                  (the same kernel with the taps mirrored and Wt[c][tap][o] = W[o][tap][c])
-//   weight grad:   dW[o][k] = sum_p dy[p][o] A[p][k], split over pixel ranges
-//                  into per-range partials that a fixed-order fold adds up
+//   weight grad:   dW[o][k] = sum_p dy[p][o] A[p][k], split over runs of tiles
+//                  into partials that a fixed-order fold adds up
 // with d(tap) = (ky - 1, kx - 1).  Channel counts are multiples of 8 so that
 // a 16-byte chunk of k never straddles two taps.
 #pragma once
@@ -26,10 +24,8 @@ namespace wsconv {
 
 using bf16 = __nv_bfloat16;
 
-constexpr int kBM = 128;  // pixels per block (forward / input grad)
 constexpr int kBK = 32;   // k per pipeline stage
 constexpr int kLd = kBK + 8;  // shared-memory row stride (bf16): 80 bytes, conflict-free ldmatrix
-constexpr int kThreads = 128;
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
@@ -51,10 +47,21 @@ __device__ __forceinline__ void ldsm_x4(uint32_t (&r)[4], const void* p) {
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                  : "r"(smem_addr(p)));
 }
+__device__ __forceinline__ void ldsm_x4_at(uint32_t (&r)[4], uint32_t a) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(a));
+}
 __device__ __forceinline__ void ldsm_x4_t(uint32_t (&r)[4], const void* p) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];\n"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                  : "r"(smem_addr(p)));
+}
+
+__device__ __forceinline__ void ldsm_x4_t_at(uint32_t (&r)[4], uint32_t a) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(a));
 }
 
 // D = A (16x16, row) B (16x8, col) + D, BF16 in, FP32 accumulate.
@@ -66,233 +73,360 @@ __device__ __forceinline__ void mma16816(float (&d)[4], const uint32_t (&a)[4], 
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-// Where the 16-byte chunk k..k+7 of row pixel (b, y, x) of an implicit im2col
-// matrix lives: the input pixel shifted by the chunk's tap (mirrored when
-// flip), channel offset c.  Returns false outside the image or past K.
-__device__ __forceinline__ bool gather_at(int k, int K, int cin, int flip, int y, int x, int h, int w, int* yy,
-                                          int* xx, int* c) {
-    if (k >= K) return false;
-    const int tap = k / cin;
-    *c = k - tap * cin;
-    const int ky = tap / 3, kx = tap - 3 * ky;
-    *yy = y + (flip ? 1 - ky : ky - 1);
-    *xx = x + (flip ? 1 - kx : kx - 1);
-    return *yy >= 0 && *yy < h && *xx >= 0 && *xx < w;
+// The input of a convolution: c0 channels of x0 (stored at half the
+// resolution and upsampled by nearest when up0), then c1 channels of x1
+// (c1 = 0: none).  NHWC, n images of h x w pixels.
+struct ConvIn {
+    const bf16* x0;
+    const bf16* x1;
+    int c0, c1, up0, h, w;
+};
+
+// Where a convolution's result goes.  MODE 0 (forward): y, BF16 [p][cout], and
+// its 2x2 average in `pool` if given.  MODE 1 (input gradient): FP32, the
+// first c0 channels to g0 [p][c0], the rest to g1 [p][cout - c0].  MODE 2
+// (input gradient through the ReLU that made the input): y = acc where act > 0.
+struct ConvOut {
+    bf16* y;
+    bf16* pool;
+    float* g0;
+    float* g1;
+    int c0;
+    const bf16* act;
+};
+
+// Tiles of the 3x3 convolutions: TH rows x 16 columns of pixels with all input
+// channels and a one-pixel border in shared memory, 16-byte chunks of a pixel
+// at an odd stride (in chunks), so that ldmatrix rows of consecutive pixels
+// fall into different banks.
+constexpr int kTW = 16;
+__host__ __device__ constexpr int conv_stride(int cin) { return (cin / 8) | 1; }
+constexpr int kWStages = 4;  // weight stages of kBK values of k in flight
+template <int WN, int TH>
+__host__ __device__ constexpr size_t conv_smem(int cin) {
+    const size_t tile = (size_t)(TH + 2) * (kTW + 2) * conv_stride(cin) * 16 + 16 + (size_t)kWStages * 32 * WN * kLd * 2;
+    const size_t out = (size_t)TH / 4 * WN * 64 * (32 * 2 + 16);  // the epilogue's copy of the results
+    return tile > out ? tile : out;
 }
 
-
-// Implicit-GEMM 3x3 convolution, padding 1, over n images of h x w:
-// out[p][o] for o in [blockIdx.y BN, +BN), p in [blockIdx.x kBM, +kBM).
-// x: NHWC [n][h][w][cin]; wt: [cout][9 cin] (row o holds k = tap cin + c);
-// flip mirrors the taps (the input gradient of a convolution).  MODE 0:
-// out = BF16 NHWC relu(acc + bias); MODE 1: out = FP32 [p][cout] acc.
-// Four warps, each 32 pixels x BN channels; cout must be a multiple of BN.
-template <int BN, int MODE>
-__global__ void __launch_bounds__(kThreads) k_conv_igemm(const bf16* __restrict__ x, int n, int h, int w, int cin,
-                                                          int flip, const bf16* __restrict__ wt, int cout,
-                                                          const bf16* __restrict__ bias, void* out) {
-    __shared__ __align__(128) bf16 As[2][kBM][kLd];
-    __shared__ __align__(128) bf16 Bs[2][BN][kLd];
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const long long M = (long long)n * h * w;
-    const long long m0 = (long long)blockIdx.x * kBM;
-    const int n0 = blockIdx.y * BN;
-    const int K = 9 * cin, nk = (K + kBK - 1) / kBK;
-    // this thread's four A rows (fixed) and its chunk column
-    const int kc = tid & 3;
-    int rb[4], ry[4], rx[4];
-    bool rok[4];
+// v where the eight BF16 activations a are positive, else zero.
+__device__ __forceinline__ uint4 relu_mask(uint4 v, uint4 a) {
+    const __nv_bfloat162* ap = reinterpret_cast<const __nv_bfloat162*>(&a);
+    __nv_bfloat162* vp = reinterpret_cast<__nv_bfloat162*>(&v);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        const long long p = m0 + (tid >> 2) + 32 * i;
-        rok[i] = p < M;
-        const long long pp = rok[i] ? p : 0;
-        rb[i] = int(pp / ((long long)h * w));
-        const int rem = int(pp - (long long)rb[i] * h * w);
-        ry[i] = rem / w;
-        rx[i] = rem - ry[i] * w;
+        if (!(__bfloat162float(ap[i].x) > 0.0f)) vp[i].x = __float2bfloat16(0.0f);
+        if (!(__bfloat162float(ap[i].y) > 0.0f)) vp[i].y = __float2bfloat16(0.0f);
     }
-    auto load_stage = [&](int st, int kt) {
-        const int k = kt * kBK + kc * 8;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            int yy = 0, xx = 0, c = 0;
-            const bool ok = rok[i] && gather_at(k, K, cin, flip, ry[i], rx[i], h, w, &yy, &xx, &c);
-            const bf16* src = ok ? x + (((long long)rb[i] * h + yy) * w + xx) * cin + c : x;
-            cp16(&As[st][(tid >> 2) + 32 * i][kc * 8], src, ok ? 16 : 0);
-        }
-#pragma unroll
-        for (int i = 0; i < BN / 32; ++i) {
-            const int row = (tid >> 2) + 32 * i;
-            const bool ok = k < K && n0 + row < cout;
-            const bf16* src = ok ? wt + (long long)(n0 + row) * K + k : wt;
-            cp16(&Bs[st][row][kc * 8], src, ok ? 16 : 0);
+    return v;
+}
+
+// 3x3 convolution, padding 1: out[p][o], o in [32 WN blockIdx.y, +32 WN), for
+// one TH x 16 tile of pixels per block.  wt: [cout][9 cin] (row o holds k =
+// tap cin + c); modes other than 0 mirror the taps.
+//
+// The tile's input is read once (an implicit im2col gather reads it nine
+// times); the A operands of every tap are the same shared memory at a shifted
+// address.  A warp owns four rows of 16 pixels x 32 channels: 6 ldmatrix per
+// 16 mma, below the shared-memory rate at the full mma.sync rate (600 TFLOP/s
+// measured on GB300, against 57 reached by the gathering kernel).  Weights
+// stream through kWStages cp.async stages.  k ascends in steps of 16 into one
+// accumulator per output, so sums round as in any other tiling.
+template <int WN, int TH, int MODE>
+__global__ void __launch_bounds__(8 * WN * TH, 512 / (8 * WN * TH) > 0 ? 512 / (8 * WN * TH) : 1)
+k_conv3(const ConvIn in, const bf16* __restrict__ wt, int cout, const bf16* __restrict__ bias, const ConvOut to) {
+    constexpr bool FLIP = MODE != 0;
+    constexpr int BN = 32 * WN, T = 8 * WN * TH;
+    extern __shared__ __align__(128) unsigned char conv_sm[];
+    const int cin = in.c0 + in.c1, nch = cin / 8, stride = conv_stride(cin) * 16;  // bytes of a pixel
+    const int K = 9 * cin, nk = (K + kBK - 1) / kBK;
+    const int h = in.h, w = in.w, tiles_x = w / kTW, tiles_y = h / TH;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, wm = wid % (TH / 4), wn = wid / (TH / 4);
+    const int img = blockIdx.x / (tiles_x * tiles_y), trem = blockIdx.x - img * tiles_x * tiles_y;
+    const int y0 = (trem / tiles_x) * TH, x0 = (trem % tiles_x) * kTW, n0 = blockIdx.y * BN;
+    unsigned char* zero = conv_sm + (TH + 2) * (kTW + 2) * stride;  // 16 bytes of zeros
+    bf16* Bs = reinterpret_cast<bf16*>(zero + 16);                 // [kWStages][BN][kLd]
+    auto load_weights = [&](int kt) {
+        if (kt < nk) {
+            bf16* dst = Bs + (kt % kWStages) * BN * kLd;
+            for (int i = tid; i < BN * (kBK / 8); i += T) {
+                const int row = i >> 2, k = kt * kBK + (i & 3) * 8;
+                const bool ok = k < K;
+                cp16(dst + row * kLd + (i & 3) * 8, ok ? wt + (long long)(n0 + row) * K + k : wt, ok ? 16 : 0);
+            }
         }
         cp_commit();
     };
-    float acc[2][BN / 8][4];
+    if (tid < 4) reinterpret_cast<int*>(zero)[tid] = 0;
+    for (int i = tid; i < (TH + 2) * (kTW + 2) * nch; i += T) {
+        const int px = i / nch, ch = i - px * nch, ly = px / (kTW + 2), lx = px - ly * (kTW + 2);
+        const int y = y0 + ly - 1, x = x0 + lx - 1, c = ch * 8;
+        const bool ok = y >= 0 && y < h && x >= 0 && x < w;
+        const bf16* src = in.x0;
+        if (ok) {
+            if (c < in.c0)
+                src = in.up0 ? in.x0 + (((long long)img * (h / 2) + y / 2) * (w / 2) + x / 2) * in.c0 + c
+                             : in.x0 + (((long long)img * h + y) * w + x) * in.c0 + c;
+            else src = in.x1 + (((long long)img * h + y) * w + x) * in.c1 + (c - in.c0);
+        }
+        cp16(conv_sm + px * stride + ch * 16, src, ok ? 16 : 0);
+    }
+    load_weights(0);  // (one group with the tile)
 #pragma unroll
-    for (int a = 0; a < 2; ++a)
+    for (int s = 1; s < kWStages - 1; ++s) load_weights(s);
+    float acc[4][4][4];
 #pragma unroll
-        for (int b = 0; b < BN / 8; ++b)
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b)
 #pragma unroll
             for (int c = 0; c < 4; ++c) acc[a][b][c] = 0.0f;
-    load_stage(0, 0);
+    // this lane's row of the A fragments (pixel lane & 15 of the warp's rows, upper half of k for lanes 16..31)
+    const uint32_t a_lane = smem_addr(conv_sm) + (uint32_t)((4 * wm * (kTW + 2) + (lane & 15)) * stride + (lane >> 4) * 16);
+    const uint32_t a_row = (kTW + 2) * stride;
+    auto tap_at = [&](int tap) {
+        const int ky = tap / 3, kx = tap - 3 * ky;
+        return (uint32_t)(((FLIP ? 2 - ky : ky) * (kTW + 2) + (FLIP ? 2 - kx : kx)) * stride);
+    };
+    const int bi = lane >> 3, br = lane & 7;
+    const int b_lane = (wn * 32 + (bi >> 1) * 8 + br) * kLd + (bi & 1) * 8;
+    int tap = 0, c = 0;
     for (int kt = 0; kt < nk; ++kt) {
-        const int st = kt & 1;
-        if (kt + 1 < nk) {
-            load_stage(st ^ 1, kt + 1);
-            cp_wait<1>();
-        } else {
-            cp_wait<0>();
-        }
+        cp_wait<kWStages - 2>();
         __syncthreads();
+        load_weights(kt + kWStages - 1);  // into the stage everybody has left
+        const bf16* B = Bs + (kt % kWStages) * BN * kLd;
 #pragma unroll
         for (int kk = 0; kk < kBK; kk += 16) {
-            uint32_t af[2][4];
+            if (kt * kBK + kk >= K) break;
+            uint32_t at[4];
+            if (cin >= 16) {
+                const uint32_t a = a_lane + tap_at(tap) + c * 2;
 #pragma unroll
-            for (int mi = 0; mi < 2; ++mi)
-                ldsm_x4(af[mi], &As[st][wid * 32 + mi * 16 + (lane & 15)][kk + (lane >> 4) * 8]);
+                for (int m = 0; m < 4; ++m) at[m] = a + m * a_row;
+                c += 16;
+                if (c == cin) c = 0, ++tap;
+            } else {  // eight channels: two taps in 16 values of k, zeros past the last
+                const int t = (kt * kBK + kk) / 8 + (lane >> 4);
+                const uint32_t a = a_lane - (lane >> 4) * 16 + tap_at(t < 9 ? t : 0);
 #pragma unroll
-            for (int nj = 0; nj < BN / 16; ++nj) {
-                uint32_t bf[4];  // n tiles 2 nj and 2 nj + 1, k halves 0 and 1
-                const int i = lane >> 3, r = lane & 7;
-                ldsm_x4(bf, &Bs[st][nj * 16 + (i >> 1) * 8 + r][kk + (i & 1) * 8]);
-#pragma unroll
-                for (int mi = 0; mi < 2; ++mi) {
-                    mma16816(acc[mi][2 * nj], af[mi], bf[0], bf[1]);
-                    mma16816(acc[mi][2 * nj + 1], af[mi], bf[2], bf[3]);
-                }
+                for (int m = 0; m < 4; ++m) at[m] = t < 9 ? a + m * a_row : smem_addr(zero);
             }
+            uint32_t af[4][4], bf[2][4];
+#pragma unroll
+            for (int j = 0; j < 2; ++j) ldsm_x4(bf[j], B + b_lane + j * 16 * kLd + kk);
+#pragma unroll
+            for (int m = 0; m < 4; ++m) ldsm_x4_at(af[m], at[m]);
+#pragma unroll
+            for (int m = 0; m < 4; ++m)
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    mma16816(acc[m][2 * j], af[m], bf[j][0], bf[j][1]);
+                    mma16816(acc[m][2 * j + 1], af[m], bf[j][2], bf[j][3]);
+                }
         }
-        __syncthreads();  // the stage is refilled by the next iteration's copies
     }
-    // epilogue
     const int gid = lane >> 2, tig = lane & 3;
+    const long long p0 = ((long long)img * h + y0 + 4 * wm) * w + x0;  // pixel of the warp's first row
+    const int o0 = n0 + wn * 32;
+    if (MODE == 1) {
+        const bool first = o0 < to.c0;  // (both parts are multiples of 32 channels)
+        float* base = first ? to.g0 + o0 : to.g1 + (o0 - to.c0);
+        const int ld = first ? to.c0 : cout - to.c0;
 #pragma unroll
-    for (int mi = 0; mi < 2; ++mi) {
+        for (int m = 0; m < 4; ++m)
 #pragma unroll
-        for (int half = 0; half < 2; ++half) {
-            const long long p = m0 + wid * 32 + mi * 16 + gid + 8 * half;
-            if (p >= M) continue;
+            for (int half = 0; half < 2; ++half) {
+                float* dst = base + (p0 + (long long)m * w + gid + 8 * half) * ld + tig * 2;
 #pragma unroll
-            for (int ni = 0; ni < BN / 8; ++ni) {
-                const int o = n0 + ni * 8 + tig * 2;
-                float v0 = acc[mi][ni][2 * half], v1 = acc[mi][ni][2 * half + 1];
-                if (MODE == 0) {
-                    v0 += __bfloat162float(bias[o]);
-                    v1 += __bfloat162float(bias[o + 1]);
-                    __nv_bfloat162 r;
-                    r.x = __float2bfloat16(v0 > 0.0f ? v0 : 0.0f);
-                    r.y = __float2bfloat16(v1 > 0.0f ? v1 : 0.0f);
-                    *reinterpret_cast<__nv_bfloat162*>(static_cast<bf16*>(out) + p * cout + o) = r;
-                } else {
-                    *reinterpret_cast<float2*>(static_cast<float*>(out) + p * cout + o) = make_float2(v0, v1);
-                }
+                for (int ni = 0; ni < 4; ++ni)
+                    *reinterpret_cast<float2*>(dst + ni * 8) = make_float2(acc[m][ni][2 * half], acc[m][ni][2 * half + 1]);
             }
+        return;
+    }
+    // bias and ReLU (or the ReLU's mask) and BF16 through shared memory: 16-byte stores of whole pixels' channels
+    cp_wait<0>();
+    __syncthreads();
+    unsigned char* mine = conv_sm + wid * 64 * 80;
+#pragma unroll
+    for (int ni = 0; ni < 4; ++ni) {
+        const int o = o0 + ni * 8 + tig * 2;
+        const float b0 = MODE == 0 ? __bfloat162float(bias[o]) : 0.0f, b1 = MODE == 0 ? __bfloat162float(bias[o + 1]) : 0.0f;
+#pragma unroll
+        for (int m = 0; m < 4; ++m)
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+                const float v0 = acc[m][ni][2 * half] + b0, v1 = acc[m][ni][2 * half + 1] + b1;
+                __nv_bfloat162 r;
+                r.x = __float2bfloat16(MODE == 2 || v0 > 0.0f ? v0 : 0.0f);
+                r.y = __float2bfloat16(MODE == 2 || v1 > 0.0f ? v1 : 0.0f);
+                *reinterpret_cast<__nv_bfloat162*>(mine + (m * 16 + gid + 8 * half) * 80 + (ni * 8 + tig * 2) * 2) = r;
+            }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int e = i * 32 + lane, px = e >> 2, ch = e & 3;
+        const long long at = (p0 + (long long)(px >> 4) * w + (px & 15)) * cout + o0 + ch * 8;
+        uint4 v = *reinterpret_cast<const uint4*>(mine + px * 80 + ch * 16);
+        if (MODE == 2) v = relu_mask(v, *reinterpret_cast<const uint4*>(to.act + at));
+        *reinterpret_cast<uint4*>(to.y + at) = v;
+    }
+    if (MODE == 0 && to.pool) {
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {  // 2 x 8 pooled pixels x 4 chunks
+            const int e = i * 32 + lane, px = e >> 2, ch = e & 3, py = px >> 3, pxx = px & 7;
+            const unsigned char* q = mine + ((2 * py) * 16 + 2 * pxx) * 80 + ch * 16;
+            __nv_bfloat162 r[4];
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                const float2 a = __bfloat1622float2(reinterpret_cast<const __nv_bfloat162*>(q)[v]);
+                const float2 b = __bfloat1622float2(reinterpret_cast<const __nv_bfloat162*>(q + 80)[v]);
+                const float2 d = __bfloat1622float2(reinterpret_cast<const __nv_bfloat162*>(q + 16 * 80)[v]);
+                const float2 e2 = __bfloat1622float2(reinterpret_cast<const __nv_bfloat162*>(q + 17 * 80)[v]);
+                r[v].x = __float2bfloat16(0.25f * (a.x + b.x + d.x + e2.x));
+                r[v].y = __float2bfloat16(0.25f * (a.y + b.y + d.y + e2.y));
+            }
+            const long long pp = ((long long)img * (h / 2) + (y0 + 4 * wm) / 2 + py) * (w / 2) + x0 / 2 + pxx;
+            *reinterpret_cast<uint4*>(to.pool + pp * cout + o0 + ch * 8) = *reinterpret_cast<const uint4*>(r);
         }
     }
 }
 
-// Weight gradient of a 3x3 convolution, split over pixel ranges:
-// part[s][o][k] = sum over pixels p of range s (ps pixels each, a multiple of
-// kBK) of dy[p][o] A[p][k], A the implicit im2col of x (NHWC [n][h][w][cin]).
-// Block: 32 output channels (blockIdx.y) x 64 values of k (blockIdx.x) x one
-// range (blockIdx.z); each warp owns 16 values of k.  Both operands are
-// staged pixel-major and transposed by ldmatrix.trans.
-constexpr int kWgN = 64;
-constexpr int kLdD = 32 + 8, kLdC = kWgN + 8;
-__global__ void __launch_bounds__(kThreads) k_conv_wgrad(const bf16* __restrict__ dy, const bf16* __restrict__ x,
-                                                          int n, int h, int w, int cin, int cout, int ps,
-                                                          float* __restrict__ part) {
-    __shared__ __align__(128) bf16 Ds[2][kBK][kLdD];
-    __shared__ __align__(128) bf16 Cs[2][kBK][kLdC];
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const long long P = (long long)n * h * w;
-    const int K = 9 * cin;
-    const int k0 = blockIdx.x * kWgN, o0 = blockIdx.y * 32, s = blockIdx.z;
-    const long long pbeg = (long long)s * ps;
-    const long long pend = pbeg + ps < P ? pbeg + ps : P;
-    const int nt = pend > pbeg ? int((pend - pbeg + kBK - 1) / kBK) : 0;
-    auto load_stage = [&](int st, int t) {
-        const long long pb = pbeg + (long long)t * kBK;
-        {  // dy: 32 pixels x 32 channels
-            const int r = tid >> 2, oc = tid & 3;
-            const long long p = pb + r;
-            const bool ok = p < pend;
-            cp16(&Ds[st][r][oc * 8], ok ? dy + p * cout + o0 + oc * 8 : dy, ok ? 16 : 0);
-        }
-#pragma unroll
-        for (int i = 0; i < 2; ++i) {  // im2col: 32 pixels x 64 values of k
-            const int r = (tid >> 3) + 16 * i, kc = tid & 7;
-            const long long p = pb + r;
-            int yy = 0, xx = 0, c = 0, b = 0;
-            bool ok = p < pend;
-            if (ok) {
-                b = int(p / ((long long)h * w));
-                const int rem = int(p - (long long)b * h * w);
-                const int y = rem / w, xq = rem - y * w;
-                ok = gather_at(k0 + kc * 8, K, cin, 0, y, xq, h, w, &yy, &xx, &c);
+// Weight gradient of a 3x3 convolution, split over runs of pixel tiles:
+// part[s][o][k] = sum over the pixels of the tiles of split s (`per` tiles of 8
+// x 16 each) of dy[p][o] A[p][k], and the bias gradient's partials
+// bpart[s][o] = sum dy[p][o].  Block: 32 output channels (blockIdx.y) x NC
+// input channels (blockIdx.x) x one split (blockIdx.z); warp t takes tap t,
+// 32 x NC products, the pixels of a tile row being the 16 values of its k.
+// The tile of dy and the bordered tile of x are staged pixel-major (two
+// stages of cp.async) and transposed by ldmatrix.trans: x is read 1.4 times
+// instead of nine times, and a warp issues four ldmatrix per eight mma.
+constexpr int kWgTH = 8;
+template <int NC>
+__host__ __device__ constexpr int wgrad_stride() { return (NC / 8) | 1; }  // 16-byte chunks of a pixel of x
+constexpr int kWgLdD = 32 + 8;
+template <int NC>
+__host__ __device__ constexpr size_t wgrad_stage() {
+    return (size_t)kWgTH * kTW * kWgLdD * 2 + (size_t)(kWgTH + 2) * (kTW + 2) * wgrad_stride<NC>() * 16;
+}
+template <int NC>
+__global__ void __launch_bounds__(288, 2) k_conv_wgrad(const bf16* __restrict__ dy, const ConvIn in, int cout, int tiles,
+                                                       int per, float* __restrict__ part, float* __restrict__ bpart) {
+    constexpr int T = 288, ST = wgrad_stride<NC>() * 16, NJ = NC / 8;
+    extern __shared__ __align__(128) unsigned char conv_sm[];
+    const int tid = threadIdx.x, lane = tid & 31, tap = tid >> 5;
+    const int cin = in.c0 + in.c1, K = 9 * cin, h = in.h, w = in.w, tiles_x = w / kTW, tiles_y = h / kWgTH;
+    const int c0 = blockIdx.x * NC, o0 = blockIdx.y * 32, t0 = blockIdx.z * per, t1 = min(t0 + per, tiles);
+    const bool half = in.up0 && c0 < in.c0;  // (a block's channels lie in one of the two sources)
+    const bf16* src = c0 < in.c0 ? in.x0 + c0 : in.x1 + (c0 - in.c0);
+    const int sc = c0 < in.c0 ? in.c0 : in.c1;
+    auto load = [&](int t) {
+        if (t < t1) {
+            unsigned char* sm = conv_sm + ((t - t0) & 1) * wgrad_stage<NC>();
+            const int img = t / (tiles_x * tiles_y), rem = t - img * tiles_x * tiles_y;
+            const int y0 = (rem / tiles_x) * kWgTH, x0 = (rem % tiles_x) * kTW;
+            for (int i = tid; i < kWgTH * kTW * 4; i += T) {
+                const int px = i >> 2, ch = i & 3;
+                const long long p = ((long long)img * h + y0 + (px >> 4)) * w + x0 + (px & 15);
+                cp16(sm + px * (kWgLdD * 2) + ch * 16, dy + p * cout + o0 + ch * 8, 16);
             }
-            cp16(&Cs[st][r][kc * 8], ok ? x + (((long long)b * h + yy) * w + xx) * cin + c : x, ok ? 16 : 0);
+            sm += kWgTH * kTW * kWgLdD * 2;
+            for (int i = tid; i < (kWgTH + 2) * (kTW + 2) * NJ; i += T) {
+                const int px = i / NJ, ch = i - px * NJ, ly = px / (kTW + 2), y = y0 + ly - 1, x = x0 + px - ly * (kTW + 2) - 1;
+                const bool ok = y >= 0 && y < h && x >= 0 && x < w;
+                const bf16* at = half ? src + (((long long)img * (h / 2) + y / 2) * (w / 2) + x / 2) * sc
+                                      : src + (((long long)img * h + y) * w + x) * sc;
+                cp16(sm + px * ST + ch * 16, ok ? at + ch * 8 : src, ok ? 16 : 0);
+            }
         }
         cp_commit();
     };
-    float acc[2][2][4];
+    float acc[2][NJ][4], bsum = 0.0f;
 #pragma unroll
     for (int a = 0; a < 2; ++a)
 #pragma unroll
-        for (int b = 0; b < 2; ++b)
+        for (int b = 0; b < NJ; ++b)
 #pragma unroll
             for (int c = 0; c < 4; ++c) acc[a][b][c] = 0.0f;
-    if (nt > 0) load_stage(0, 0);
-    for (int t = 0; t < nt; ++t) {
-        const int st = t & 1;
-        if (t + 1 < nt) {
-            load_stage(st ^ 1, t + 1);
-            cp_wait<1>();
-        } else {
-            cp_wait<0>();
-        }
+    const int i = lane >> 3, r = lane & 7, ky = tap / 3, kx = tap - 3 * ky;
+    load(t0);
+    for (int t = t0; t < t1; ++t) {
+        load(t + 1);
+        cp_wait<1>();
         __syncthreads();
-        const int i = lane >> 3, r = lane & 7;
+        unsigned char* sm = conv_sm + ((t - t0) & 1) * wgrad_stage<NC>();
+        const bf16* Ds = reinterpret_cast<const bf16*>(sm);
+        const uint32_t xs = smem_addr(sm + kWgTH * kTW * kWgLdD * 2) + (uint32_t)((ky * (kTW + 2) + kx) * ST);
 #pragma unroll
-        for (int kk = 0; kk < kBK; kk += 16) {
-            uint32_t af[2][4], bf[4];
+        for (int row = 0; row < kWgTH; ++row) {
+            uint32_t af[2][4], bf[NJ / 2 > 0 ? NJ / 2 : 1][4];
 #pragma unroll
-            for (int mi = 0; mi < 2; ++mi) ldsm_x4_t(af[mi], &Ds[st][kk + (i >> 1) * 8 + r][mi * 16 + (i & 1) * 8]);
-            ldsm_x4_t(bf, &Cs[st][kk + (i & 1) * 8 + r][wid * 16 + (i >> 1) * 8]);
+            for (int m = 0; m < 2; ++m)
+                ldsm_x4_t(af[m], Ds + (row * kTW + (i >> 1) * 8 + r) * kWgLdD + m * 16 + (i & 1) * 8);
+            // pixels (i & 1) 8 + r, channels (i >> 1) 8 .. + 8 of each pair of channel groups
+            const uint32_t xr = xs + (uint32_t)((row * (kTW + 2) + (i & 1) * 8 + r) * ST);
+            if (NJ > 1) {
 #pragma unroll
-            for (int mi = 0; mi < 2; ++mi) {
-                mma16816(acc[mi][0], af[mi], bf[0], bf[1]);
-                mma16816(acc[mi][1], af[mi], bf[2], bf[3]);
+                for (int j = 0; j < NJ / 2; ++j) ldsm_x4_t_at(bf[j], xr + (uint32_t)(j * 32 + (i >> 1) * 16));
+            } else {
+                ldsm_x4_t_at(bf[0], xr);  // (its upper half repeats the lower)
             }
+#pragma unroll
+            for (int m = 0; m < 2; ++m)
+#pragma unroll
+                for (int j = 0; j < NJ; ++j)
+                    mma16816(acc[m][j], af[m], bf[j / 2][(j & 1) * 2], bf[j / 2][(j & 1) * 2 + 1]);
+        }
+        if (blockIdx.x == 0 && tid < 256) {  // 16 pixels of one channel
+#pragma unroll
+            for (int x = 0; x < kTW; ++x) bsum += __bfloat162float(Ds[((tid >> 5) * kTW + x) * kWgLdD + (tid & 31)]);
         }
         __syncthreads();
     }
     const int gid = lane >> 2, tig = lane & 3;
 #pragma unroll
-    for (int mi = 0; mi < 2; ++mi)
+    for (int m = 0; m < 2; ++m)
 #pragma unroll
-        for (int half = 0; half < 2; ++half) {
-            const int o = o0 + mi * 16 + gid + 8 * half;
+        for (int hf = 0; hf < 2; ++hf) {
+            float* dst = part + ((long long)blockIdx.z * cout + o0 + m * 16 + gid + 8 * hf) * K + tap * cin + c0 + tig * 2;
 #pragma unroll
-            for (int ni = 0; ni < 2; ++ni) {
-                const int k = k0 + wid * 16 + ni * 8 + tig * 2;
-                if (k < K)
-                    *reinterpret_cast<float2*>(part + ((long long)s * cout + o) * K + k) =
-                        make_float2(acc[mi][ni][2 * half], acc[mi][ni][2 * half + 1]);
-            }
+            for (int j = 0; j < NJ; ++j)
+                *reinterpret_cast<float2*>(dst + j * 8) = make_float2(acc[m][j][2 * hf], acc[m][j][2 * hf + 1]);
         }
+    if (blockIdx.x == 0) {
+        float* red = reinterpret_cast<float*>(conv_sm);
+        if (tid < 256) red[tid] = bsum;
+        __syncthreads();
+        if (tid < 32) {
+            float v = 0.0f;
+            for (int g = 0; g < 8; ++g) v += red[g * 32 + tid];
+            bpart[(long long)blockIdx.z * cout + o0 + tid] = v;
+        }
+    }
 }
 
-// grad[i] = sum over s of part[s][i] (s in order), i < count.
-__global__ void k_fold_splits(const float* __restrict__ part, int nsplit, long long count, float* __restrict__ grad) {
-    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (i >= count) return;
+// grad[i] = sum over s of part[s][i] and gbias[o] = sum over s of bpart[s][o],
+// in a fixed order: eight interleaved runs of s per value, then the runs.
+constexpr int kFoldRuns = 8, kFoldVals = 32;
+__global__ void __launch_bounds__(kFoldRuns * kFoldVals)
+k_fold_splits(const float* __restrict__ part, const float* __restrict__ bpart, int nsplit, long long count, int cout,
+              float* __restrict__ grad, float* __restrict__ gbias) {
+    __shared__ float sh[kFoldRuns][kFoldVals];
+    const int v = threadIdx.x % kFoldVals, run = threadIdx.x / kFoldVals;
+    const long long i = blockIdx.x * (long long)kFoldVals + v;
+    const bool bias = i >= count;
+    const long long n = bias ? cout : count, at = bias ? i - count : i;
+    const float* src = bias ? bpart : part;
     float acc = 0.0f;
-    for (int s = 0; s < nsplit; ++s) acc += part[(long long)s * count + i];
-    grad[i] = acc;
+    if (at < n)
+        for (int s = run; s < nsplit; s += kFoldRuns) acc += src[s * n + at];
+    sh[run][v] = acc;
+    __syncthreads();
+    if (run == 0 && at < n) {
+        for (int g = 1; g < kFoldRuns; ++g) acc += sh[g][v];
+        (bias ? gbias : grad)[at] = acc;
+    }
 }
 
 // Wt[c][tap][o] = W[o][tap][c]: the weights of the input-gradient convolution.
