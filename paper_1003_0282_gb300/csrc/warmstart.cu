@@ -144,30 +144,71 @@ __global__ void __launch_bounds__(256) k_ws_head(const bf16* x, const bf16* wt, 
     }
 }
 
-// Bilinear sample of canvas channel ch at normalised (rn, zn) in [0, 1]:
-// pixel centres at ((i + 1/2)/kW, (j + 1/2)/kH), clamped at the edges.
-__device__ float ws_sample(const float* cv, int ch, double rn, double zn) {
-    const double x = rn * kW - 0.5, y = zn * kH - 0.5;
-    const double xc = fmin(fmax(x, 0.0), kW - 1.0), yc = fmin(fmax(y, 0.0), kH - 1.0);
-    const int x0 = min(int(xc), kW - 2), y0 = min(int(yc), kH - 2);
-    const double fx = xc - x0, fy = yc - y0;
-    const float* p = cv + (long long)ch * kH * kW;
-    const double v00 = p[y0 * kW + x0], v01 = p[y0 * kW + x0 + 1], v10 = p[(y0 + 1) * kW + x0],
-                 v11 = p[(y0 + 1) * kW + x0 + 1];
-    return float((1 - fy) * ((1 - fx) * v00 + fx * v01) + fy * ((1 - fx) * v10 + fx * v11));
-}
-
-// Fields [5][nz][nr] (rho, u_r, u_z, u_theta, T) of one domain from its canvas.
-__global__ void k_ws_fields(const float* canvas, axlbm_ws_domain D, float* fields) {
-    const long long n = (long long)D.nr * D.nz;
-    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const int j = int(i % D.nr), k = int(i / D.nr);
+// Fields [5][nz][nr] (rho, u_r, u_z, u_theta, T) of every domain from its
+// canvas, bilinear at normalised (rn, zn) in [0, 1]: pixel centres at
+// ((i + 1/2)/kW, (j + 1/2)/kH), clamped at the edges.  A block takes kFieldRows
+// rows of up to kFieldCols columns of one domain; a thread walks down one
+// column and keeps its values interpolated along r at the two canvas rows
+// around it, which several domain rows share: FP64 instructions bound this
+// kernel (64.5 cycles a warp instruction and scheduler), and this takes about
+// 22 of them per node where sampling every node afresh took over a hundred
+// with its divisions.
+constexpr int kFieldCols = 128, kFieldRows = 32;
+struct FieldDom {
+    axlbm_ws_domain d;
+    long long out;  // first value of the domain's fields
+    int block0;     // first block
+};
+__global__ void __launch_bounds__(kFieldCols) k_ws_fields(const float* canvas, const FieldDom* doms, int n, float* fields) {
+    __shared__ double row_y[kFieldRows];
+    int lo = 0, hi = n - 1;  // the domain of this block
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (doms[mid].block0 <= (int)blockIdx.x) lo = mid;
+        else hi = mid - 1;
+    }
+    const FieldDom& F = doms[lo];
+    const axlbm_ws_domain& D = F.d;
+    const int cols = (D.nr + kFieldCols - 1) / kFieldCols, b = blockIdx.x - F.block0, rb = b / cols;
+    const int j = (b - rb * cols) * kFieldCols + threadIdx.x, k0 = rb * kFieldRows, k1 = min(k0 + kFieldRows, D.nz);
+    if (threadIdx.x < kFieldRows) {
+        const double zn = (D.z_first + (k0 + (int)threadIdx.x) - D.z_bottom) / D.height;
+        row_y[threadIdx.x] = fmin(fmax(zn * kH - 0.5, 0.0), kH - 1.0);
+    }
+    __syncthreads();
+    if (j >= D.nr) return;
     const double rn = (D.r_first + j) / D.r_wall;
-    const double zn = (D.z_first + k - D.z_bottom) / D.height;
-    fields[i] = float(D.rho0);
-    for (int f = 0; f < 3; ++f) fields[(1 + f) * n + i] = float(D.u_scale) * ws_sample(canvas, f, rn, zn);
-    fields[4 * n + i] = float(D.t_ref) + ws_sample(canvas, 3, rn, zn);
+    const double xc = fmin(fmax(rn * kW - 0.5, 0.0), kW - 1.0);
+    const int x0 = min(int(xc), kW - 2);
+    const double fx = xc - x0, gx = 1 - fx;
+    const float* cv = canvas + (long long)lo * 4 * kH * kW + x0;
+    const long long nn = (long long)D.nr * D.nz;
+    float* out = fields + F.out + j;
+    const float rho = float(D.rho0), us = float(D.u_scale), tr = float(D.t_ref);
+    auto along_r = [&](int y, int c) {
+        const float* p = cv + ((long long)c * kH + y) * kW;
+        return gx * p[0] + fx * p[1];
+    };
+    double h0[4], h1[4];
+    int have = -2;  // h0, h1 are canvas rows have, have + 1
+    for (int k = k0; k < k1; ++k) {
+        const double yc = row_y[k - k0];
+        const int y0 = min(int(yc), kH - 2);
+        const double fy = yc - y0, gy = 1 - fy;
+        if (y0 != have) {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                h0[c] = y0 == have + 1 ? h1[c] : along_r(y0, c);
+                h1[c] = along_r(y0 + 1, c);
+            }
+            have = y0;
+        }
+        const long long i = (long long)k * D.nr;
+        out[i] = rho;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) out[(1 + c) * nn + i] = us * float(gy * h0[c] + fy * h1[c]);
+        out[4 * nn + i] = tr + float(gy * h0[3] + fy * h1[3]);
+    }
 }
 
 // Canvas [4][kH][kW] of one domain from its moments [4][nz][nr] (u_r, u_z,
@@ -792,17 +833,31 @@ axlbm_status axlbm_ws_predict(axlbm_ws* w, const float* features, int32_t n, flo
 
 axlbm_status axlbm_ws_fields(axlbm_ws* w, const float* canvas, int32_t n, const axlbm_ws_domain* doms, float* fields) {
     if (!w || !canvas || !doms || !fields || n < 0) return wfail(w, AXLBM_EINVAL, "bad arguments");
-    size_t off = 0;
+    long long off = 0, blocks = 0;
+    std::vector<FieldDom> list(n);
     for (int d = 0; d < n; ++d) {
         const axlbm_ws_domain& D = doms[d];
         if (D.nr < 1 || D.nz < 1 || !(D.r_wall > 0.0) || !(D.height > 0.0))
             return wfail(w, AXLBM_EINVAL, "bad domain geometry");
-        const long long nn = (long long)D.nr * D.nz;
-        k_ws_fields<<<blocks_for(nn), 256, 0, w->stream>>>(canvas + (size_t)d * 4 * kH * kW, D, fields + off);
-        off += 5 * (size_t)nn;
+        list[d] = {D, off, (int)blocks};
+        off += 5 * (long long)D.nr * D.nz;
+        blocks += (long long)((D.nr + kFieldCols - 1) / kFieldCols) * ((D.nz + kFieldRows - 1) / kFieldRows);
     }
-    cudaError_t e = cudaGetLastError();
+    if (blocks > 0x7fffffffll) return wfail(w, AXLBM_EINVAL, "too many nodes in one call");
+    if (n == 0) return AXLBM_OK;
+    FieldDom* dev = nullptr;
+    cudaError_t e = cudaMalloc(&dev, n * sizeof(FieldDom));
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return wfail(w, AXLBM_ENOMEM, "domain list");
+    }
+    e = cudaMemcpyAsync(dev, list.data(), n * sizeof(FieldDom), cudaMemcpyHostToDevice, w->stream);
+    if (e == cudaSuccess) {
+        k_ws_fields<<<(unsigned)blocks, kFieldCols, 0, w->stream>>>(canvas, dev, n, fields);
+        e = cudaGetLastError();
+    }
     if (e == cudaSuccess) e = cudaStreamSynchronize(w->stream);
+    cudaFree(dev);
     if (e != cudaSuccess) return wfail(w, AXLBM_ECUDA, "resampling");
     return AXLBM_OK;
 }
