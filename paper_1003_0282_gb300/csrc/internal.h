@@ -70,6 +70,8 @@ struct CoefCore {
     R sv, se, seps, sq;
     R k_e6;         // s_e / (6 s_v) of Eq. 49
     R mrt_gam;      // 1 - s_v / 2 (Eq. 49: gamma = mrt_gam / r)
+    // 1 - s and 1 - s / 2 of the rates
+    R se1, se2, seps1, seps2, sq1, sq2, sv1, sv2;
 };
 
 // Collision coefficients plus the wall data of the boundary rules.

@@ -73,6 +73,46 @@ struct KArgs {
 // the sign of e_ar at a given radius.  R is double, float, or a pair of
 // floats (two nodes at the same radius); Sc is its scalar type.
 template <class R, bool SW, bool TH>
+struct Cell;
+
+// What the FP64 collision takes of a column: the terms in 1/r and the rates by
+// the sign of e_r ([0]: -1, [1]: 0, [2]: +1) in the combinations it uses.
+template <bool SW, bool TH>
+struct ColCoef {
+    double inv_r, rho0_r, mu_r2, fr_r2, gam, sg_r, sg_0;
+    double om1[3], ow[3][3], kw[3][3], kr[3][3];  // BGK: 1 - om, om w, (1 - om/2) w and that times rho0, by weight class
+    double go[3], go1[3], ho[3], ho1[3], ht[3];
+    __device__ __forceinline__ void set(double inv, const CoefCore<double>& C) {
+        inv_r = inv;
+        const double inv_r2 = inv * inv;
+        rho0_r = C.rho0 * inv;
+        mu_r2 = C.mu0 * inv_r2;
+        fr_r2 = -2.0 * C.mu0 * inv_r2;
+        gam = C.mrt_gam * inv;
+        sg_r = -2.0 * inv;
+        sg_0 = -C.nu * inv_r2;
+        const double W[3] = {4.0 / 9.0, 1.0 / 9.0, 1.0 / 36.0};
+#pragma unroll
+        for (int e = 0; e < 3; ++e) {
+            const double s = e - 1.0;
+            const double om = fma(s * C.c1, inv, C.c0);
+            om1[e] = 1.0 - om;
+#pragma unroll
+            for (int w = 0; w < 3; ++w) {
+                ow[e][w] = om * W[w];
+                kw[e][w] = (1.0 - 0.5 * om) * W[w];
+                kr[e][w] = kw[e][w] * C.rho0;
+            }
+            go[e] = fma(s * C.g1, inv, C.g0);
+            go1[e] = 1.0 - go[e];
+            ho[e] = fma(s * C.h1, inv, C.h0);
+            ho1[e] = 1.0 - ho[e];
+            ht[e] = -ho[e] * (C.t_ref * 0.25);
+        }
+    }
+};
+
+template <class R, bool SW, bool TH>
 struct Cell {
     using Sc = typename ScalarOf<R>::type;
     R d[9];  // f_a - w_a rho0
@@ -81,6 +121,12 @@ struct Cell {
     R rho, ur, uz, s0, ds0;
 
     __device__ __forceinline__ void collide(Sc inv_r, const CoefCore<Sc>& C, Sc az) {
+        if constexpr (std::is_same<R, D1>::value) {
+            ColCoef<SW, TH> k;
+            k.set(inv_r, C);
+            collide_d1(k, C, az);
+            return;
+        }
         const Sc W0 = Sc(4.0 / 9.0), W1 = Sc(1.0 / 9.0), W2 = Sc(1.0 / 36.0);
         const Sc half = Sc(0.5), one = Sc(1);
         // rates by the sign of e_r (Eq. 13) and their combinations
@@ -88,16 +134,9 @@ struct Cell {
         const Sc inv_r2 = inv_r * inv_r;
 
         // moments (Eqs. 14-17 with the half-force terms)
-        R sr, sz;
-        if constexpr (std::is_same<R, D1>::value) {  // sums that the MRT collision shares
-            ds0 = (d[0] + ((d[1] + d[3]) + (d[2] + d[4]))) + ((d[5] + d[6]) + (d[7] + d[8]));
-            sr = (d[1] - d[3]) + ((d[5] - d[6]) + (d[8] - d[7]));
-            sz = (d[2] - d[4]) + ((d[5] + d[6]) - (d[7] + d[8]));
-        } else {
-            ds0 = ((d[0] + d[1]) + (d[2] + d[3])) + ((d[4] + d[5]) + (d[6] + d[7])) + d[8];
-            sr = (d[1] - d[3]) + (d[5] - d[6]) + (d[8] - d[7]);
-            sz = (d[2] - d[4]) + (d[5] + d[6]) - (d[7] + d[8]);
-        }
+        ds0 = ((d[0] + d[1]) + (d[2] + d[3])) + ((d[4] + d[5]) + (d[6] + d[7])) + d[8];
+        const R sr = (d[1] - d[3]) + (d[5] - d[6]) + (d[8] - d[7]);
+        const R sz = (d[2] - d[4]) + (d[5] + d[6]) - (d[7] + d[8]);
         s0 = ds0 + R(C.rho0);
         R gsum = R(Sc(0)), dtemp = R(Sc(0));
         if (SW) gsum = (g[0] + g[1]) + (g[2] + g[3]);
@@ -118,8 +157,7 @@ struct Cell {
         const R inv_rho = den * inv_s0;
 
         if (C.mrt) {
-            if constexpr (std::is_same<R, D1>::value) collide_mrt_d1(urr, C, inv_r, drho, fr, fz);
-            else collide_mrt(inv_r, C, drho, fr, fz);
+            collide_mrt(inv_r, C, drho, fr, fz);
         } else {
         // equilibrium polynomials P_a
         const R ur2 = ur * ur, uz2 = uz * uz;
@@ -127,12 +165,12 @@ struct Cell {
         const R B = rho * R(Sc(3)), Cq = rho * R(Sc(4.5));
         const R Bur = B * ur, Buz = B * uz, Cuz2 = Cq * uz2;
         const R Cx = (Cq + Cq) * (ur * uz);
-        const R Ps = mad(Cq, ur2, A), Pz = A + Cuz2, Q = Ps + Cuz2;
+        const R Ps = A + Cq * ur2, Pz = A + Cuz2, Q = Ps + Cuz2;
         const R Qp = Q + Cx, Qm = Q - Cx, Bs = Bur + Buz, Bd = Bur - Buz;
         const R P[9] = {A, Ps + Bur, Pz + Buz, Ps - Bur, Pz - Buz, Qp + Bs, Qm - Bd, Qp - Bs, Qm + Bd};
         // source factors F_a
         const R fr3 = fr * inv_rho * R(Sc(3)), fz3 = fz * inv_rho * R(Sc(3));
-        const R base = fmaR(mad(ur, fr, uz * fz) * R(Sc(-3)), inv_rho, R(Sc(0)) - urr);
+        const R base = fmaR((ur * fr + uz * fz) * R(Sc(-3)), inv_rho, R(Sc(0)) - urr);
         const R F1 = base + fr3, F3 = base - fr3;
         const R F[9] = {base, F1, base + fz3, F3, base - fz3, F1 + fz3, F3 + fz3, F3 - fz3, F1 - fz3};
 #pragma unroll
@@ -182,7 +220,7 @@ struct Cell {
     // = rho0 (1, -2, 1, 0, ...).  Eq. 41 with the source -(u_r/r) m^eq + S'
     // of Eq. 51, the correction of Eqs. 49-50, then M^-1 = M^T diag(1/|row|^2).
     __device__ __forceinline__ void collide_mrt(Sc inv_r, const CoefCore<Sc>& C, R drho, R fr, R fz) {
-        const Sc one = Sc(1), half = Sc(0.5);
+        const Sc half = Sc(0.5);
         // moments of the deviations
         const R ax = (d[1] + d[2]) + (d[3] + d[4]);
         const R dg = (d[5] + d[6]) + (d[7] + d[8]);
@@ -221,14 +259,14 @@ struct Cell {
         const R ne8 = md8 - pxy_eq;
         // relaxation (Eq. 41); conserved moments with unit rate
         const R p0 = fmaR(S0, R(half), drho);                                      // rho + S0/2 - rho0
-        const R p1 = fmaR(ne1, R(one - C.se), fmaR(S1, R(one - half * C.se), r3u2 - (drho + drho)));
-        const R p2 = fmaR(ne2, R(one - C.seps), fmaR(S2, R(one - half * C.seps), drho - r3u2));
+        const R p1 = fmaR(ne1, R(C.se1), fmaR(S1, R(C.se2), r3u2 - (drho + drho)));
+        const R p2 = fmaR(ne2, R(C.seps1), fmaR(S2, R(C.seps2), drho - r3u2));
         const R p3 = fmaR(S3, R(half), ru);
-        const R p4 = fmaR(ne4, R(one - C.sq), fmaR(S4, R(one - half * C.sq), R(Sc(0)) - ru));
+        const R p4 = fmaR(ne4, R(C.sq1), fmaR(S4, R(C.sq2), R(Sc(0)) - ru));
         const R p5 = fmaR(S5, R(half), rz);
-        const R p6 = fmaR(ne6, R(one - C.sq), fmaR(S6, R(one - half * C.sq), R(Sc(0)) - rz));
-        const R p7 = fmaR(ne7, R(one - C.sv), fmaR(S7, R(one - half * C.sv), pxx_eq));
-        const R p8 = fmaR(ne8, R(one - C.sv), fmaR(S8, R(one - half * C.sv), pxy_eq));
+        const R p6 = fmaR(ne6, R(C.sq1), fmaR(S6, R(C.sq2), R(Sc(0)) - rz));
+        const R p7 = fmaR(ne7, R(C.sv1), fmaR(S7, R(C.sv2), pxx_eq));
+        const R p8 = fmaR(ne8, R(C.sv1), fmaR(S8, R(C.sv2), pxy_eq));
         // momentum correction (Eqs. 49-50), m^(1) = (m - m^eq) + S/2, gamma = (1 - s_v/2)/r
         const Sc gam = C.mrt_gam * inv_r;
         const R e1 = fmaR(S1, R(half), ne1);
@@ -256,64 +294,127 @@ struct Cell {
         d[8] = ((cd + dr) - dz) - a8;
     }
 
-    // The same in FP64, arranged for the fewest FP64 instructions (56 + 25 + 27
-    // for the relaxation, the way back and the moments; they are what bounds
-    // the FP64 kernels): moments share sums, S_4 = -S_3 and S_6 = -S_5, and
-    // the factors 1/|row|^2 ride on the fused multiply-adds of the way back.
-    __device__ __forceinline__ void collide_mrt_d1(R urr, const CoefCore<Sc>& C, Sc inv_r, R drho, R fr, R fz) {
-        const Sc one = Sc(1), half = Sc(0.5);
+    // The same collision in FP64 (the type D1), arranged for the fewest FP64
+    // instructions: GB300 issues one per scheduler in 64.5 cycles, and they are
+    // all that bounds the FP64 kernels.  Sums are shared between the moments
+    // and the MRT basis, S_4 = -S_3 and S_6 = -S_5, factors ride on fused
+    // multiply-adds, and what depends on the column alone comes in k.  About
+    // 112 per node for D2Q9 BGK, 155 for MRT with swirl; the form above takes
+    // 145 and 210.
+    __device__ __forceinline__ void collide_d1(const ColCoef<SW, TH>& k, const CoefCore<Sc>& C, Sc az) {
         const auto neg = [](R x) { return R(-x.v); };
+        const R half = R(Sc(0.5));
         const R s13 = d[1] + d[3], s24 = d[2] + d[4], s56 = d[5] + d[6], s78 = d[7] + d[8];
+        const R x13 = d[1] - d[3], x24 = d[2] - d[4];
         const R ax = s13 + s24, dg = s56 + s78;
-        const R md1 = fmaR(d[0], R(Sc(-4)), fmaR(dg, R(Sc(2)), neg(ax)));
-        const R md2 = fmaR(d[0], R(Sc(4)), fmaR(ax, R(Sc(-2)), dg));
-        const R md4 = fmaR(d[1] - d[3], R(Sc(-2)), (d[5] - d[6]) + (d[8] - d[7]));
-        const R md6 = fmaR(d[2] - d[4], R(Sc(-2)), s56 - s78);
-        const R md7 = s13 - s24;
-        const R md8 = (d[5] + d[7]) - (d[6] + d[8]);
-        const R ru = rho * ur, rz = rho * uz;
-        const R ur2 = ur * ur;
-        const R r3u2 = rho * (fmaR(uz, uz, ur2) * R(Sc(3)));
-        const R pxx_eq = rho * fmaR(neg(uz), uz, ur2), pxy_eq = ru * uz;
-        const R uF6 = fmaR(ur, fr, uz * fz) * R(Sc(6));
-        const R mu = neg(urr);
-        const R S1 = fmaR(mu, fmaR(rho, R(Sc(-2)), r3u2), uF6);
-        const R S2 = fmaR(mu, rho - r3u2, neg(uF6));
-        const R S3 = fmaR(mu, ru, fr), S5 = fmaR(mu, rz, fz);
-        const R dF = fmaR(ur, fr, neg(uz * fz));
-        const R S7 = fmaR(mu, pxx_eq, dF + dF);
-        const R S8 = fmaR(mu, pxy_eq, fmaR(ur, fz, uz * fr));
-        const R q1 = fmaR(drho, R(Sc(2)), neg(r3u2)), q2 = r3u2 - drho;  // m^eq of e and eps, sign reversed
-        const R ne1 = md1 + q1, ne2 = md2 + q2, ne4 = md4 + ru, ne6 = md6 + rz, ne7 = md7 - pxx_eq, ne8 = md8 - pxy_eq;
-        const R p0 = fmaR(mu * rho, R(half), drho);
-        const R p1 = fmaR(ne1, R(one - C.se), fmaR(S1, R(one - half * C.se), neg(q1)));
-        const R p2 = fmaR(ne2, R(one - C.seps), fmaR(S2, R(one - half * C.seps), neg(q2)));
-        const R p4 = fmaR(ne4, R(one - C.sq), fmaR(S3, R(half * C.sq - one), neg(ru)));
-        const R p6 = fmaR(ne6, R(one - C.sq), fmaR(S5, R(half * C.sq - one), neg(rz)));
-        const R p7 = fmaR(ne7, R(one - C.sv), fmaR(S7, R(one - half * C.sv), pxx_eq));
-        const R p8 = fmaR(ne8, R(one - C.sv), fmaR(S8, R(one - half * C.sv), pxy_eq));
-        const Sc gam = C.mrt_gam * inv_r;
-        const R e1 = fmaR(S1, R(half), ne1), pxx1 = fmaR(S7, R(half), ne7), pxy1 = fmaR(S8, R(half), ne8);
-        const R q3 = fmaR(fmaR(e1, R(C.k_e6), pxx1 * R(half)), R(-gam), fmaR(S3, R(half), ru));
-        const R q5 = fmaR(pxy1, R(-gam), fmaR(S5, R(half), rz));
-        const R P0 = p0 * R(Sc(1.0 / 9.0));
-        const R cx = fmaR(p1, R(Sc(-1.0 / 36.0)), fmaR(p2, R(Sc(-1.0 / 18.0)), P0));
-        const R cd = fmaR(p1, R(Sc(1.0 / 18.0)), fmaR(p2, R(Sc(1.0 / 36.0)), P0));
-        const R cxp = fmaR(p7, R(Sc(0.25)), cx), cxm = fmaR(p7, R(Sc(-0.25)), cx);
-        const R cdp = fmaR(p8, R(Sc(0.25)), cd), cdm = fmaR(p8, R(Sc(-0.25)), cd);
-        const R J = q3 - p4, K = q5 - p6;
-        const R M = fmaR(p4, R(half), q3), N = fmaR(p6, R(half), q5);
-        const R MpN = M + N, MmN = M - N;
-        const R sixth = R(Sc(1.0 / 6.0)), nsixth = R(Sc(-1.0 / 6.0));
-        d[0] = fmaR(p2 - p1, R(Sc(1.0 / 9.0)), P0);
-        d[1] = fmaR(J, sixth, cxp);
-        d[2] = fmaR(K, sixth, cxm);
-        d[3] = fmaR(J, nsixth, cxp);
-        d[4] = fmaR(K, nsixth, cxm);
-        d[5] = fmaR(MpN, sixth, cdp);
-        d[6] = fmaR(MmN, nsixth, cdm);
-        d[7] = fmaR(MpN, nsixth, cdp);
-        d[8] = fmaR(MmN, sixth, cdm);
+        const R dq_r = (d[5] - d[6]) + (d[8] - d[7]), dq_z = s56 - s78;
+        ds0 = d[0] + (ax + dg);
+        const R sr = x13 + dq_r, sz = x24 + dq_z;
+        s0 = ds0 + R(C.rho0);
+        R gsum = R(Sc(0)), dtemp = R(Sc(0)), fext_r = R(Sc(0));
+        if (SW) {
+            gsum = (g[0] + g[1]) + (g[2] + g[3]);
+            const R uth = gsum * R(C.inv_rho0);
+            fext_r = (uth * uth) * R(k.rho0_r);
+        }
+        if (TH) dtemp = (h[0] + h[1]) + (h[2] + h[3]);  // T - T_ref
+        const R fz = TH ? fmaR(dtemp, R(C.rho0 * C.gbeta), R(az)) : R(az);
+        const R inv_s0 = rcp(s0);
+        ur = (SW ? fmaR(fext_r, half, sr) : sr) * rcp(s0 + R(k.mu_r2));
+        uz = fmaR(fz, half, sz) * inv_s0;
+        const R urr = ur * R(k.inv_r);
+        const R den = fmaR(urr, half, R(Sc(1)));
+        const R inv_den = rcp(den);
+        rho = s0 * inv_den;
+        const R drho = fmaR(urr, R(Sc(-0.5) * C.rho0), ds0) * inv_den;
+        const R fr = SW ? fmaR(ur, R(k.fr_r2), fext_r) : ur * R(k.fr_r2);
+        if (C.mrt) {
+            const R md1 = fmaR(d[0], R(Sc(-4)), fmaR(dg, R(Sc(2)), neg(ax)));
+            const R md2 = fmaR(d[0], R(Sc(4)), fmaR(ax, R(Sc(-2)), dg));
+            const R md4 = fmaR(x13, R(Sc(-2)), dq_r), md6 = fmaR(x24, R(Sc(-2)), dq_z);
+            const R md7 = s13 - s24, md8 = (d[5] + d[7]) - (d[6] + d[8]);
+            const R ru = rho * ur, rz = rho * uz;
+            const R ur2 = ur * ur;
+            const R r3u2 = rho * (fmaR(uz, uz, ur2) * R(Sc(3)));
+            const R pxx_eq = rho * fmaR(neg(uz), uz, ur2), pxy_eq = ru * uz;
+            const R uzfz = uz * fz;
+            const R uF6 = fmaR(ur, fr, uzfz) * R(Sc(6)), dF = fmaR(ur, fr, neg(uzfz));
+            const R mu = neg(urr);
+            const R S1 = fmaR(mu, fmaR(rho, R(Sc(-2)), r3u2), uF6);
+            const R S2 = fmaR(mu, rho - r3u2, neg(uF6));
+            const R S3 = fmaR(mu, ru, fr), S5 = fmaR(mu, rz, fz);
+            const R S7 = fmaR(mu, pxx_eq, dF + dF);
+            const R S8 = fmaR(mu, pxy_eq, fmaR(ur, fz, uz * fr));
+            const R q1 = fmaR(drho, R(Sc(2)), neg(r3u2)), q2 = r3u2 - drho;  // m^eq of e and eps, sign reversed
+            const R ne1 = md1 + q1, ne2 = md2 + q2, ne4 = md4 + ru, ne6 = md6 + rz, ne7 = md7 - pxx_eq, ne8 = md8 - pxy_eq;
+            const R p0 = fmaR(mu * rho, half, drho);
+            const R p1 = fmaR(ne1, R(C.se1), fmaR(S1, R(C.se2), neg(q1)));
+            const R p2 = fmaR(ne2, R(C.seps1), fmaR(S2, R(C.seps2), neg(q2)));
+            const R p4 = fmaR(ne4, R(C.sq1), fmaR(S3, R(-C.sq2), neg(ru)));
+            const R p6 = fmaR(ne6, R(C.sq1), fmaR(S5, R(-C.sq2), neg(rz)));
+            const R p7 = fmaR(ne7, R(C.sv1), fmaR(S7, R(C.sv2), pxx_eq));
+            const R p8 = fmaR(ne8, R(C.sv1), fmaR(S8, R(C.sv2), pxy_eq));
+            const R e1 = fmaR(S1, half, ne1), pxx1 = fmaR(S7, half, ne7), pxy1 = fmaR(S8, half, ne8);
+            const R q3 = fmaR(fmaR(e1, R(C.k_e6), pxx1 * half), R(-k.gam), fmaR(S3, half, ru));
+            const R q5 = fmaR(pxy1, R(-k.gam), fmaR(S5, half, rz));
+            const R P0 = p0 * R(Sc(1.0 / 9.0));
+            const R cx = fmaR(p1, R(Sc(-1.0 / 36.0)), fmaR(p2, R(Sc(-1.0 / 18.0)), P0));
+            const R cd = fmaR(p1, R(Sc(1.0 / 18.0)), fmaR(p2, R(Sc(1.0 / 36.0)), P0));
+            const R cxp = fmaR(p7, R(Sc(0.25)), cx), cxm = fmaR(p7, R(Sc(-0.25)), cx);
+            const R cdp = fmaR(p8, R(Sc(0.25)), cd), cdm = fmaR(p8, R(Sc(-0.25)), cd);
+            const R J = q3 - p4, K = q5 - p6;
+            const R M = fmaR(p4, half, q3), N = fmaR(p6, half, q5);
+            const R MpN = M + N, MmN = M - N;
+            const R sixth = R(Sc(1.0 / 6.0)), nsixth = R(Sc(-1.0 / 6.0));
+            d[0] = fmaR(p2 - p1, R(Sc(1.0 / 9.0)), P0);
+            d[1] = fmaR(J, sixth, cxp);
+            d[2] = fmaR(K, sixth, cxm);
+            d[3] = fmaR(J, nsixth, cxp);
+            d[4] = fmaR(K, nsixth, cxm);
+            d[5] = fmaR(MpN, sixth, cdp);
+            d[6] = fmaR(MmN, nsixth, cdm);
+            d[7] = fmaR(MpN, nsixth, cdp);
+            d[8] = fmaR(MmN, sixth, cdm);
+        } else {
+            // d'_a = P_a (om w + kw F_a) + (kw rho0 F_a + (1 - om) d_a), kw = (1 - om/2) w
+            const R inv_rho3 = (den * inv_s0) * R(Sc(3));
+            const R uz2 = uz * uz;
+            const R A = fmaR(rho * R(Sc(-1.5)), fmaR(ur, ur, uz2), drho);
+            const R B = rho * R(Sc(3)), Cq = rho * R(Sc(4.5));
+            const R Cr = Cq * ur, Cuz2 = Cq * uz2, Cx = Cr * uz;
+            const R Bur = B * ur, Buz = B * uz;
+            const R Ps = fmaR(Cr, ur, A), Pz = A + Cuz2, Q = Ps + Cuz2;
+            const R Qp = fmaR(Cx, R(Sc(2)), Q), Qm = fmaR(Cx, R(Sc(-2)), Q), Bs = Bur + Buz, Bd = Bur - Buz;
+            const R P[9] = {A, Ps + Bur, Pz + Buz, Ps - Bur, Pz - Buz, Qp + Bs, Qm - Bd, Qp - Bs, Qm + Bd};
+            const R fr3 = fr * inv_rho3, fz3 = fz * inv_rho3;
+            const R base = fmaR(fmaR(ur, fr, uz * fz), neg(inv_rho3), neg(urr));
+            const R Fp = base + fr3, Fm = base - fr3;
+            const R F[9] = {base, Fp, base + fz3, Fm, base - fz3, Fp + fz3, Fm + fz3, Fm - fz3, Fp - fz3};
+#pragma unroll
+            for (int a = 0; a < 9; ++a) {
+                const int e = cr9(a) + 1, w = a == 0 ? 0 : (a <= 4 ? 1 : 2);
+                d[a] = fmaR(P[a], fmaR(F[a], R(k.kw[e][w]), R(k.ow[e][w])),
+                            fmaR(F[a], R(k.kr[e][w]), d[a] * R(k.om1[e])));
+            }
+        }
+        if (SW) {
+            const R g4 = gsum * R(Sc(0.25));
+            const R g2r = (g4 + g4) * ur, g2z = (g4 + g4) * uz;
+            const R geq[4] = {g4 + g2r, g4 + g2z, g4 - g2r, g4 - g2z};
+            const R sg = fmaR(ur, R(k.sg_r), R(k.sg_0));
+            const R m[3] = {sg + R(k.go[0]), sg + R(k.go[1]), sg + R(k.go[2])};
+#pragma unroll
+            for (int q = 0; q < 4; ++q) g[q] = fmaR(R(k.go1[cr4(q) + 1]), g[q], m[cr4(q) + 1] * geq[q]);
+        }
+        if (TH) {
+            const R h4 = (dtemp + R(C.t_ref)) * R(Sc(0.25));
+            const R h2r = (h4 + h4) * ur, h2z = (h4 + h4) * uz;
+            const R heq[4] = {h4 + h2r, h4 + h2z, h4 - h2r, h4 - h2z};
+            const R m[3] = {R(k.ho[0]) - urr, R(k.ho[1]) - urr, R(k.ho[2]) - urr};
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                h[q] = fmaR(R(k.ho1[cr4(q) + 1]), h[q], fmaR(m[cr4(q) + 1], heq[q], R(k.ht[cr4(q) + 1])));
+        }
     }
 };
 
@@ -1609,6 +1710,11 @@ Coef<R> make_coef(double tau_s, const axlbm_forcing& fo, const axlbm_boundary& b
     C.sq = R(sq);
     C.k_e6 = R(1.0 / 6.0);  // s_e / (6 s_v) with s_e = s_v
     C.mrt_gam = R(1.0 - 0.5 * sv);
+    const R one = R(1), half = R(0.5);
+    C.se1 = one - C.se, C.se2 = one - half * C.se;
+    C.seps1 = one - C.seps, C.seps2 = one - half * C.seps;
+    C.sq1 = one - C.sq, C.sq2 = one - half * C.sq;
+    C.sv1 = one - C.sv, C.sv2 = one - half * C.sv;
     return C;
 }
 

@@ -66,8 +66,7 @@ __device__ __forceinline__ F2 rcp(F2 x) {
 }
 
 // One FP64 value whose operations round as written: which products are fused
-// is stated in the collision (mad below), so that every kernel rounds a node
-// alike (the compiler fuses plain double expressions differently from kernel
+// is stated in the collision, so that every kernel rounds a node alike (the compiler fuses plain double expressions differently from kernel
 // to kernel).
 struct D1 {
     double v;
@@ -91,12 +90,6 @@ __device__ __forceinline__ D1 rcp(D1 x) {
     const double e = __fma_rn(-x.v, r, 1.0);
     return D1(__fma_rn(r, __fma_rn(e, e, e), r));
 }
-
-// a b + c where the FP32 types round the product (their form is fixed:
-// 16-bit storage would amplify another rounding) and FP64 fuses it.
-template <class R>
-__device__ __forceinline__ R mad(R a, R b, R c) { return a * b + c; }
-__device__ __forceinline__ D1 mad(D1 a, D1 b, D1 c) { return fmaR(a, b, c); }
 
 template <class R>
 struct ScalarOf {

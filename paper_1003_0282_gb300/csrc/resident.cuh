@@ -599,15 +599,32 @@ constexpr int kResSlabThreads = 384;
 // table, or -1 away from the tile's outline, where every slot is the CTA's own.
 template <class R>
 struct ResPair {
-    R inv_r;
+    float inv_r;
     int i, tab;
 };
+template <>
+struct ResPair<double> {
+    int col, i, tab;  // col: column of the tile
+};
+// Bytes of the pairs, so that what follows lies on an 8-byte boundary.
+template <class R>
+__host__ __device__ constexpr size_t res_pairs_bytes(int chunk, int max_ghost) {
+    const size_t b = (size_t)chunk * sizeof(ResPair<R>);
+    return b + (sizeof(R) == 8 ? (8 - (b + (size_t)max_ghost * 3 * sizeof(int)) % 8) % 8 : 0);
+}
 // A row of the slot table: where population (q, l) is pulled from in an odd
 // step (index into the values), then the links.
 template <class R, bool SW, bool TH>
 __host__ __device__ constexpr size_t res_row_bytes() {
     return Lanes<typename PairArith<R>::type>::n *
            (nplanes<SW, TH>() * sizeof(int) + ((SW ? 8 : 0) + (TH ? 12 : 0)) * sizeof(R));
+}
+
+// FP64: what the collision takes of each column of the tile, in shared memory
+// (recomputed per node it would be a tenth of the FP64 instructions).
+template <class R, bool SW, bool TH>
+__host__ __device__ constexpr size_t res_column_bytes(int w) {
+    return sizeof(R) == 8 ? (size_t)w * sizeof(ColCoef<SW, TH>) : 0;
 }
 
 // Several pairs per thread.
@@ -624,9 +641,10 @@ __device__ __forceinline__ void res_slab_cta(const ResDom<R, R>& D, Clock* clock
     const ResTile tile(D, nkp, blockIdx.x - D.cta0);
     const int tw = tile.w, n = tw * tile.h;
     const ResSlab<R> S(smem, gbase, max_ghost);
-    ResPair<R>* pairs = reinterpret_cast<ResPair<R>*>(S.rest + (sizeof(R) == 8 ? (max_ghost & 1) * 4 : 0));
-    R* tf = reinterpret_cast<R*>(pairs + chunk);  // [NF][NL][max_tab]: sg, cg, then sh, ch, ct, four each
-    int* tab = reinterpret_cast<int*>(tf + NF * NL * max_tab);  // [P][NL][max_tab]
+    ResPair<R>* pairs = reinterpret_cast<ResPair<R>*>(S.rest);
+    R* tf = reinterpret_cast<R*>(S.rest + res_pairs_bytes<R>(chunk, max_ghost));  // [NF][NL][max_tab]: sg, cg, then sh, ch, ct, four each
+    ColCoef<SW, TH>* columns = reinterpret_cast<ColCoef<SW, TH>*>(tf + NF * NL * max_tab);  // [w], FP64 only
+    int* tab = reinterpret_cast<int*>(reinterpret_cast<unsigned char*>(columns) + res_column_bytes<R, SW, TH>(D.w));  // [P][NL][max_tab]
     if (tid == 0) ghosts = bad = 0;
     __syncthreads();
     // pairs in order, those with a row of the table last (a warp's slots and words then lie side by side)
@@ -640,7 +658,8 @@ __device__ __forceinline__ void res_slab_cta(const ResDom<R, R>& D, Clock* clock
                 const unsigned m0 = __ballot_sync(0xffffffffu, i < n && !row), m1 = __ballot_sync(0xffffffffu, i < n && row);
                 if (pass && i < n) {
                     ResPair<R> r;
-                    r.inv_r = step_inv_radius<R>(G, tile.j0 + jl);
+                    if constexpr (sizeof(R) == 8) r.col = jl;
+                    else r.inv_r = step_inv_radius<R>(G, tile.j0 + jl);
                     r.i = i;
                     const int to = row ? at1 + __popc(m1 & ((1u << tid) - 1u)) : at0 + __popc(m0 & ((1u << tid) - 1u));
                     r.tab = row ? to - plain : -1;
@@ -699,6 +718,8 @@ __device__ __forceinline__ void res_slab_cta(const ResDom<R, R>& D, Clock* clock
             }
         }
     }
+    if constexpr (sizeof(R) == 8)
+        for (int jl = tid; jl < tw; jl += T) columns[jl].set(step_inv_radius<R>(G, tile.j0 + jl), C);
     for (int m = tid; m < PL * n; m += T) {  // the state, natural layout
         const int ql = m / n, i = m - ql * n, kl = i / tw, j = tile.j0 + i - kl * tw, k = NL * (tile.k0 + kl) + ql % NL;
         S.st[ql * chunk + i] = k < G.nz ? *slot(D.pop, G, ql / NL, j, k) : R(0);
@@ -740,7 +761,8 @@ __device__ __forceinline__ void res_slab_cta(const ResDom<R, R>& D, Clock* clock
             if (PAR == 0) res_load<RC, SW, TH, 0>(c, [&](int q, int l) { return mine[(q * NL + l) * chunk]; }, none);
             else if (r.tab < 0) res_load<RC, SW, TH, 1>(c, [&](int q, int l) { return mine[inside(q, l)]; }, none);
             else res_load<RC, SW, TH, 1>(c, [&](int q, int l) { return S.st[e[(q * NL + l) * max_tab]]; }, tl);
-            c.collide(r.inv_r, C, az);
+            if constexpr (sizeof(R) == 8) c.collide_d1(columns[r.col], C, az);
+            else c.collide(r.inv_r, C, az);
             if (PAR == 0) res_store<RC, SW, TH, 0>(c, [&](int q, int l, R v) { mine[(q * NL + l) * chunk] = v; }, none);
             else if (r.tab < 0) res_store<RC, SW, TH, 1>(c, [&](int q, int l, R v) { mine[inside(q, l)] = v; }, none);
             else res_store<RC, SW, TH, 1>(c, [&](int q, int l, R v) { S.st[e[(q * NL + l) * max_tab]] = v; }, tl);

@@ -201,7 +201,7 @@ cudaError_t res_build(Resident* r, const ResidentDomain* d, int n, int num_sms, 
                 // (a domain without h in a batch with it has fewer planes)
                 size_t need = h ? res_slab_smem<R, SW, TH>(y.chunk, y.max_ghost) : res_slab_smem<R, SW, false>(y.chunk, y.max_ghost);
                 if (!one)
-                    need += 8 + (size_t)y.chunk * sizeof(ResPair<R>) +
+                    need += res_pairs_bytes<R>(y.chunk, y.max_ghost) + res_column_bytes<R, SW, TH>(y.w) +
                             y.max_tab * (h ? res_row_bytes<R, SW, TH>() : res_row_bytes<R, SW, false>());
                 smem = std::max(smem, need);
             }
