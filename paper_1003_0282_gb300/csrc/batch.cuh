@@ -253,7 +253,8 @@ __device__ __forceinline__ uint32_t batch_tile_bytes(bool th) {
 // eg: some lane of the warp sits on a side column the bulk kernel updates
 // (odd steps; the other warps load and store without the side-column
 // selections -- only those sections exist twice, the collision once).
-template <class S, class R, class RC, bool SW, bool THD, int PAR, bool CHK, int TK, int TJ, bool WET>
+// Off: type of a node's byte offset in a plane (see k_bulk_batch).
+template <class S, class R, class RC, bool SW, bool THD, int PAR, bool CHK, int TK, int TJ, bool WET, class Off>
 __device__ __forceinline__ void batch_nodes(const BatchArgs<S, R>& A, const SlotDesc& D, const S* st, int k0, int j0,
                                             int jj, int rr, R inv_r, R az, const R* sp_old, RedR<R>& red, bool eg) {
     constexpr int NL = Lanes<RC>::n;
@@ -343,19 +344,21 @@ __device__ __forceinline__ void batch_nodes(const BatchArgs<S, R>& A, const Slot
 #pragma unroll
     for (int l = 0; l < NL; ++l) {
         if (!act[l]) continue;
+        const Off xb = ((Off)(k0 + rr + l * (TK / NL)) * (Off)A.pitch + (Off)(j0 + jj)) * (Off)sizeof(S);
+        auto at = [&](long long plane_off) { return reinterpret_cast<S*>(reinterpret_cast<char*>(A.pop + plane_off) + xb); };
         const long long x = (long long)(k0 + rr + l * (TK / NL)) * A.pitch + (j0 + jj);
         if (PAR == 0 && keep[l]) {
             // stored by the copy below, after the collided state is dead
         } else if (PAR == 0) {
 #pragma unroll
-            for (int a = 0; a < 9; ++a) Codec<S>::store(A.pop + opp9(a) * pl + x, Lanes<RC>::get(c.d[a], l));
+            for (int a = 0; a < 9; ++a) Codec<S>::store(at(opp9(a) * pl), Lanes<RC>::get(c.d[a], l));
             if (SW) {
 #pragma unroll
-                for (int q = 0; q < 4; ++q) Codec<S>::store(A.pop + (9 + opp4(q)) * pl + x, Lanes<RC>::get(c.g[q], l));
+                for (int q = 0; q < 4; ++q) Codec<S>::store(at((9 + opp4(q)) * pl), Lanes<RC>::get(c.g[q], l));
             }
             if (THD) {
 #pragma unroll
-                for (int q = 0; q < 4; ++q) Codec<S>::store(A.pop + (HP + opp4(q)) * pl + x, Lanes<RC>::get(c.h[q], l));
+                for (int q = 0; q < 4; ++q) Codec<S>::store(at((HP + opp4(q)) * pl), Lanes<RC>::get(c.h[q], l));
             }
         } else {
             auto store_node = [&](auto edge_tag) {
@@ -364,32 +367,32 @@ __device__ __forceinline__ void batch_nodes(const BatchArgs<S, R>& A, const Slot
 #pragma unroll
             for (int a = 0; a < 9; ++a) {
                 if (cr9(a) < 0 && edge == kEdgeAxis)
-                    Codec<S>::store(A.pop + axis_push_plane9(a) * pl + x + cz9(a) * A.pitch, Lanes<RC>::get(c.d[a], l));
+                    Codec<S>::store(at(axis_push_plane9(a) * pl + cz9(a) * A.pitch), Lanes<RC>::get(c.d[a], l));
                 else if (cr9(a) > 0 && edge == kEdgeWall)
-                    Codec<S>::store(A.pop + opp9(a) * pl + x, Lanes<RC>::get(c.d[a], l));
+                    Codec<S>::store(at(opp9(a) * pl), Lanes<RC>::get(c.d[a], l));
                 else
-                    Codec<S>::store(A.pop + a * pl + x + cz9(a) * A.pitch + cr9(a), Lanes<RC>::get(c.d[a], l));
+                    Codec<S>::store(at(a * pl + cz9(a) * A.pitch + cr9(a)), Lanes<RC>::get(c.d[a], l));
             }
             if (SW) {
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
                     if (q == 2 && edge == kEdgeAxis)
-                        Codec<S>::store(A.pop + 9 * pl + x, Lanes<RC>::get(gsend, l));
+                        Codec<S>::store(at(9 * pl), Lanes<RC>::get(gsend, l));
                     else if (q == 0 && edge == kEdgeWall)
-                        Codec<S>::store(A.pop + 11 * pl + x, Lanes<RC>::get(gsend, l));
+                        Codec<S>::store(at(11 * pl), Lanes<RC>::get(gsend, l));
                     else
-                        Codec<S>::store(A.pop + (9 + q) * pl + x + cz4(q) * A.pitch + cr4(q), Lanes<RC>::get(c.g[q], l));
+                        Codec<S>::store(at((9 + q) * pl + cz4(q) * A.pitch + cr4(q)), Lanes<RC>::get(c.g[q], l));
                 }
             }
             if (THD) {
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
                     if (q == 2 && edge == kEdgeAxis)
-                        Codec<S>::store(A.pop + HP * pl + x, Lanes<RC>::get(hsend, l));
+                        Codec<S>::store(at(HP * pl), Lanes<RC>::get(hsend, l));
                     else if (q == 0 && edge == kEdgeWall)
-                        Codec<S>::store(A.pop + (HP + 2) * pl + x, Lanes<RC>::get(hsend, l));
+                        Codec<S>::store(at((HP + 2) * pl), Lanes<RC>::get(hsend, l));
                     else
-                        Codec<S>::store(A.pop + (HP + q) * pl + x + cz4(q) * A.pitch + cr4(q), Lanes<RC>::get(c.h[q], l));
+                        Codec<S>::store(at((HP + q) * pl + cz4(q) * A.pitch + cr4(q)), Lanes<RC>::get(c.h[q], l));
                 }
             }
             };
@@ -436,7 +439,11 @@ __device__ __forceinline__ void batch_nodes(const BatchArgs<S, R>& A, const Slot
 // computing warp has released it; the computing warps only compute.  SW:
 // every domain carries g; TH: shelves may carry h (per-tile flag); WET: some
 // domain has a wet wall (its wall nodes keep their state in even steps).
-template <class S, class R, bool SW, bool TH, int PAR, bool CHK, int TK, int TJ, bool WET>
+// Off: a node's byte offset in a plane, 32 bits unless a plane has 4 GiB or
+// more (against 64 bits, sweep of 320 domains: FP16 even 0.2102 -> 0.2034 and
+// odd 0.2989 -> 0.2912 ms, FP32 odd 0.3196 -> 0.3154 ms: fewer instructions
+// per store).
+template <class S, class R, bool SW, bool TH, int PAR, bool CHK, int TK, int TJ, bool WET, class Off = unsigned>
 __global__ void __launch_bounds__(batch_nthreads<TK, TJ>() + 32, batch_min_blocks<TK, TJ>())
 k_bulk_batch(const __grid_constant__ CUtensorMap map, const BatchArgs<S, R> A) {
     constexpr int NS = batch_nstages<S, SW, TH, TK, TJ>();
@@ -563,10 +570,10 @@ k_bulk_batch(const __grid_constant__ CUtensorMap map, const BatchArgs<S, R> A) {
 #pragma unroll
                 for (int p = 0; p < NP; ++p) {
                     if (dth)
-                        batch_nodes<S, R, RC, SW, TH, PAR, CHK, TK, TJ, WET>(A, D, st, k0, j0, jj, rr0 + p * TPC, inv_r,
+                        batch_nodes<S, R, RC, SW, TH, PAR, CHK, TK, TJ, WET, Off>(A, D, st, k0, j0, jj, rr0 + p * TPC, inv_r,
                                                                               az, sp_old + 2 * p, red, eg);
                     else
-                        batch_nodes<S, R, RC, SW, false, PAR, CHK, TK, TJ, WET>(A, D, st, k0, j0, jj, rr0 + p * TPC,
+                        batch_nodes<S, R, RC, SW, false, PAR, CHK, TK, TJ, WET, Off>(A, D, st, k0, j0, jj, rr0 + p * TPC,
                                                                                  inv_r, az, sp_old + 2 * p, red, eg);
                 }
                 if (CHK)

@@ -73,10 +73,10 @@ KArgs<S, R> domain_args(axlbm_batch* b, int d) {
     return K;
 }
 
-template <class S, class R, bool TH, int PAR, bool CHK, int SH, bool WET>
+template <class S, class R, bool TH, int PAR, bool CHK, int SH, bool WET, class Off = unsigned>
 cudaError_t launch_bulk_batch(axlbm_batch* b, const BatchArgs<S, R>& A) {
     constexpr int TK = kShapeTK[SH], TJ = kShapeTJ[SH];
-    auto kern = k_bulk_batch<S, R, true, TH, PAR, CHK, TK, TJ, WET>;
+    auto kern = k_bulk_batch<S, R, true, TH, PAR, CHK, TK, TJ, WET, Off>;
     constexpr size_t smem = batch_smem_bytes<S, true, TH, TK, TJ>();
     int& grid = b->grid[SH][PAR][CHK ? 1 : 0];
     if (grid == 0) {
@@ -94,17 +94,20 @@ cudaError_t launch_bulk_batch(axlbm_batch* b, const BatchArgs<S, R>& A) {
     return cudaGetLastError();
 }
 
-template <class S, class R, bool TH, int PAR, bool CHK, bool WET>
+template <class S, class R, bool TH, int PAR, bool CHK, bool WET, class Off = unsigned>
 cudaError_t launch_bulk_batch_wet(axlbm_batch* b, const BatchArgs<S, R>& A) {
     if constexpr (sizeof(S) == 2) {
-        if (b->shape[PAR] == 2) return launch_bulk_batch<S, R, TH, PAR, CHK, 2, WET>(b, A);
+        if (b->shape[PAR] == 2) return launch_bulk_batch<S, R, TH, PAR, CHK, 2, WET, Off>(b, A);
     }
-    return b->shape[PAR] == 0 ? launch_bulk_batch<S, R, TH, PAR, CHK, 0, WET>(b, A)
-                              : launch_bulk_batch<S, R, TH, PAR, CHK, 1, WET>(b, A);
+    return b->shape[PAR] == 0 ? launch_bulk_batch<S, R, TH, PAR, CHK, 0, WET, Off>(b, A)
+                              : launch_bulk_batch<S, R, TH, PAR, CHK, 1, WET, Off>(b, A);
 }
 
 template <class S, class R, bool TH, int PAR, bool CHK>
 cudaError_t launch_bulk_batch_shape(axlbm_batch* b, const BatchArgs<S, R>& A) {
+    // a plane of 4 GiB or more: 64-bit offsets, in one kernel for every mix of domains
+    if ((unsigned long long)A.plane * sizeof(S) >= (1ull << 32))
+        return launch_bulk_batch_wet<S, R, true, PAR, CHK, PAR == 0, unsigned long long>(b, A);
     // wet walls matter only in even steps (odd steps leave the rings to the ring kernels)
     if constexpr (PAR == 0) {
         if (b->L.nnee > 0) return launch_bulk_batch_wet<S, R, TH, PAR, CHK, true>(b, A);
