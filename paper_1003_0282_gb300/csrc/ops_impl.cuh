@@ -1099,6 +1099,7 @@ k_bulk(const __grid_constant__ CUtensorMap map, const KArgs<S, R> A) {
                     (eg && PAR == 1 && G.side) ? (j == 0 ? kEdgeAxis : (j == G.nr - 1 ? kEdgeWall : kEdgeNone)) : kEdgeNone;
                 const S* own = A.pop + (long long)(k0 + rr) * G.pitch + j;
                 const int LOWN = (kTileK / NL) * (int)G.pitch;
+                S* const tile_pop = A.pop + (long long)k0 * G.pitch + j0;
                 auto load_node = [&](auto edge_tag) {
                 constexpr bool EDGE = decltype(edge_tag)::value;
                 const int edge = EDGE ? edge_rt : kEdgeNone;
@@ -1157,31 +1158,36 @@ k_bulk(const __grid_constant__ CUtensorMap map, const KArgs<S, R> A) {
                 for (int l = 0; l < NL; ++l) {
                     if (!act[l]) continue;
                     const long long x = (long long)kk[l] * G.pitch + j;
+                    // a plane-uniform base and the node's byte offset in the tile
+                    const unsigned xb = ((unsigned)(rr + l * (kTileK / NL)) * (unsigned)G.pitch + (unsigned)jj) * (unsigned)sizeof(S);
+                    auto at = [&](long long plane_off) {
+                        return reinterpret_cast<S*>(reinterpret_cast<char*>(tile_pop + plane_off) + xb);
+                    };
                     if (PAR == 0 && has_wet_wall(G) && on_wet_wall(G, j, kk[l])) {
                         // a wet-wall node holds its post-collision state and keeps it
                         const S* src = row + l * LROW;
 #pragma unroll
-                        for (int a = 0; a < 9; ++a) A.pop[opp9(a) * G.plane + x] = src[a * kTileK * BW];
+                        for (int a = 0; a < 9; ++a) *at(opp9(a) * G.plane) = src[a * kTileK * BW];
                         if (SW) {
 #pragma unroll
-                            for (int q = 0; q < 4; ++q) A.pop[(9 + opp4(q)) * G.plane + x] = src[(9 + q) * kTileK * BW];
+                            for (int q = 0; q < 4; ++q) *at((9 + opp4(q)) * G.plane) = src[(9 + q) * kTileK * BW];
                         }
                         if (TH) {
 #pragma unroll
-                            for (int q = 0; q < 4; ++q) A.pop[(HP + opp4(q)) * G.plane + x] = src[(HP + q) * kTileK * BW];
+                            for (int q = 0; q < 4; ++q) *at((HP + opp4(q)) * G.plane) = src[(HP + q) * kTileK * BW];
                         }
                     } else if (PAR == 0) {
 #pragma unroll
-                        for (int a = 0; a < 9; ++a) Codec<S>::store(A.pop + opp9(a) * G.plane + x, Lanes<RC>::get(c.d[a], l));
+                        for (int a = 0; a < 9; ++a) Codec<S>::store(at(opp9(a) * G.plane), Lanes<RC>::get(c.d[a], l));
                         if (SW) {
 #pragma unroll
                             for (int q = 0; q < 4; ++q)
-                                Codec<S>::store(A.pop + (9 + opp4(q)) * G.plane + x, Lanes<RC>::get(c.g[q], l));
+                                Codec<S>::store(at((9 + opp4(q)) * G.plane), Lanes<RC>::get(c.g[q], l));
                         }
                         if (TH) {
 #pragma unroll
                             for (int q = 0; q < 4; ++q)
-                                Codec<S>::store(A.pop + (HP + opp4(q)) * G.plane + x, Lanes<RC>::get(c.h[q], l));
+                                Codec<S>::store(at((HP + opp4(q)) * G.plane), Lanes<RC>::get(c.h[q], l));
                         }
                     } else {
                         auto store_node = [&](auto edge_tag) {
@@ -1190,23 +1196,23 @@ k_bulk(const __grid_constant__ CUtensorMap map, const KArgs<S, R> A) {
 #pragma unroll
                         for (int a = 0; a < 9; ++a) {
                             if (cr9(a) < 0 && edge == kEdgeAxis)
-                                Codec<S>::store(A.pop + axis_push_plane9(a) * G.plane + x + cz9(a) * G.pitch,
+                                Codec<S>::store(at(axis_push_plane9(a) * G.plane + cz9(a) * G.pitch),
                                                 Lanes<RC>::get(c.d[a], l));
                             else if (cr9(a) > 0 && edge == kEdgeWall)
-                                Codec<S>::store(A.pop + opp9(a) * G.plane + x, Lanes<RC>::get(c.d[a], l));
+                                Codec<S>::store(at(opp9(a) * G.plane), Lanes<RC>::get(c.d[a], l));
                             else
-                                Codec<S>::store(A.pop + a * G.plane + x + cz9(a) * G.pitch + cr9(a),
+                                Codec<S>::store(at(a * G.plane + cz9(a) * G.pitch + cr9(a)),
                                                 Lanes<RC>::get(c.d[a], l));
                         }
                         if (SW) {
 #pragma unroll
                             for (int q = 0; q < 4; ++q) {
                                 if (q == 2 && edge == kEdgeAxis)
-                                    Codec<S>::store(A.pop + 9 * G.plane + x, Lanes<RC>::get(gsend, l));
+                                    Codec<S>::store(at(9 * G.plane), Lanes<RC>::get(gsend, l));
                                 else if (q == 0 && edge == kEdgeWall)
-                                    Codec<S>::store(A.pop + 11 * G.plane + x, Lanes<RC>::get(gsend, l));
+                                    Codec<S>::store(at(11 * G.plane), Lanes<RC>::get(gsend, l));
                                 else
-                                    Codec<S>::store(A.pop + (9 + q) * G.plane + x + cz4(q) * G.pitch + cr4(q),
+                                    Codec<S>::store(at((9 + q) * G.plane + cz4(q) * G.pitch + cr4(q)),
                                                     Lanes<RC>::get(c.g[q], l));
                             }
                         }
@@ -1214,11 +1220,11 @@ k_bulk(const __grid_constant__ CUtensorMap map, const KArgs<S, R> A) {
 #pragma unroll
                             for (int q = 0; q < 4; ++q) {
                                 if (q == 2 && edge == kEdgeAxis)
-                                    Codec<S>::store(A.pop + HP * G.plane + x, Lanes<RC>::get(hsend, l));
+                                    Codec<S>::store(at(HP * G.plane), Lanes<RC>::get(hsend, l));
                                 else if (q == 0 && edge == kEdgeWall)
-                                    Codec<S>::store(A.pop + (HP + 2) * G.plane + x, Lanes<RC>::get(hsend, l));
+                                    Codec<S>::store(at((HP + 2) * G.plane), Lanes<RC>::get(hsend, l));
                                 else
-                                    Codec<S>::store(A.pop + (HP + q) * G.plane + x + cz4(q) * G.pitch + cr4(q),
+                                    Codec<S>::store(at((HP + q) * G.plane + cz4(q) * G.pitch + cr4(q)),
                                                     Lanes<RC>::get(c.h[q], l));
                             }
                         }
