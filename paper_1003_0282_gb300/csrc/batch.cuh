@@ -596,7 +596,7 @@ k_bulk_batch(const __grid_constant__ CUtensorMap map, const BatchArgs<S, R> A) {
     if (PAR == 0 && blockIdx.x == 0) {
         const long long t1 = A.clock->t + 1;
         for (int d = tid; d < A.ndom; d += blockDim.x) {
-            const double a = A.doms[d].az0 * cos(A.doms[d].omega_t * (double)t1);
+            const double a = force_at(A.doms[d].az0, A.doms[d].omega_t, t1);
             A.dom_az[2 * d + 1] = a;
             store_az16(A.dom_az16, d, 1, a);
         }
@@ -648,7 +648,7 @@ __global__ void __launch_bounds__(kRingThreads) k_ring_batch(const BatchArgs<S, 
     if (advance && blockIdx.x == 0) {
         const long long t1 = A.clock->t + 1;
         for (int d = threadIdx.x; d < A.ndom; d += blockDim.x) {
-            const double a = A.doms[d].az0 * cos(A.doms[d].omega_t * (double)t1);
+            const double a = force_at(A.doms[d].az0, A.doms[d].omega_t, t1);
             A.dom_az[2 * d] = a;
             store_az16(A.dom_az16, d, 0, a);
         }
@@ -661,7 +661,7 @@ __global__ void __launch_bounds__(kRingThreads) k_ring_batch(const BatchArgs<S, 
 // force a(t) for the even step, as the step kernels compute it.
 static __global__ void k_batch_set_time(const DomDesc* doms, int ndom, Clock* clock, double* az, double* az16, long long t) {
     for (int d = threadIdx.x; d < ndom; d += blockDim.x) {
-        const double a = doms[d].az0 * cos(doms[d].omega_t * (double)t);
+        const double a = force_at(doms[d].az0, doms[d].omega_t, t);
         az[2 * d] = a;
         store_az16(az16, d, 0, a);
     }

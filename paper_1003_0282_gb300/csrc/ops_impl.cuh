@@ -568,43 +568,43 @@ __device__ __forceinline__ S* site_slot(const KArgs<S, R>& A, int plane, int j, 
     return slot(A.pop, G, plane, j, k);
 }
 
+// The slot of population (er, ez) -- plane `own`, or `p[fr][fz]` where the
+// link is mirrored in r / in z -- that a link to or from site s uses, chosen
+// by selects: a node's loads (and stores) are then in flight together, where a
+// branch per population made them wait for one another.
+template <bool HALO, class S, class R>
+__device__ __forceinline__ S* link_slot(const KArgs<S, R>& A, const Site& s, int j, int k, int own, int p00, int p10,
+                                        int p01, int p11) {
+    const int mirrored = s.fz ? (s.fr ? p11 : p01) : (s.fr ? p10 : p00);
+    return site_slot<HALO>(A, s.solid ? own : mirrored, s.solid ? j : s.j, s.solid ? k : s.k);
+}
+
 // Pull the odd-step populations of node (j, k) with boundary rules.
 template <class S, class R, bool SW, bool TH, bool HALO = false>
 __device__ __forceinline__ void pull_odd(const KArgs<S, R>& A, int j, int k, Cell<R, SW, TH>& c) {
     const Geom& G = A.G;
 #pragma unroll
     for (int a = 0; a < 9; ++a) {
-        const Site s = classify(G, j, k, -cr9(a), -cz9(a));
-        if (s.solid) {
-            c.d[a] = Codec<S>::load(slot(A.pop, G, a, j, k));
-        } else {
-            const int b = idx9(s.fr ? -cr9(a) : cr9(a), s.fz ? -cz9(a) : cz9(a));
-            c.d[a] = Codec<S>::load(site_slot<HALO>(A, opp9(b), s.j, s.k));
-        }
+        const int x = cr9(a), z = cz9(a);
+        const Site s = classify(G, j, k, -x, -z);
+        c.d[a] = Codec<S>::load(link_slot<HALO>(A, s, j, k, a, opp9(a), opp9(idx9(-x, z)), opp9(idx9(x, -z)),
+                                                opp9(idx9(-x, -z))));
     }
-    if (SW) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const Site s = classify(G, j, k, -cr4(q), -cz4(q));
-            if (s.solid) {
-                c.g[q] = bounce_g(G, A.C, s.face, j, Codec<S>::load(slot(A.pop, G, A.g_plane + q, j, k)));
-            } else {
-                const int b = idx4(s.fr ? -cr4(q) : cr4(q), s.fz ? -cz4(q) : cz4(q));
-                const R v = Codec<S>::load(site_slot<HALO>(A, A.g_plane + opp4(b), s.j, s.k));
-                c.g[q] = s.fr ? -v : v;
-            }
+    for (int q = 0; q < 4; ++q) {
+        if (!SW && !TH) break;
+        const int x = cr4(q), z = cz4(q), p00 = opp4(q), p10 = opp4(idx4(-x, z)), p01 = opp4(idx4(x, -z)),
+                  p11 = opp4(idx4(-x, -z));
+        const Site s = classify(G, j, k, -x, -z);
+        if (SW) {
+            const int P = A.g_plane;
+            const R v = Codec<S>::load(link_slot<HALO>(A, s, j, k, P + q, P + p00, P + p10, P + p01, P + p11));
+            c.g[q] = s.solid ? bounce_g(G, A.C, s.face, j, v) : (s.fr ? -v : v);
         }
-    }
-    if (TH) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const Site s = classify(G, j, k, -cr4(q), -cz4(q));
-            if (s.solid) {
-                c.h[q] = bounce_h(A.C, s.face, R(Codec<S>::load(slot(A.pop, G, A.h_plane + q, j, k))));
-            } else {
-                const int b = idx4(s.fr ? -cr4(q) : cr4(q), s.fz ? -cz4(q) : cz4(q));
-                c.h[q] = Codec<S>::load(site_slot<HALO>(A, A.h_plane + opp4(b), s.j, s.k));
-            }
+        if (TH) {
+            const int P = A.h_plane;
+            const R v = Codec<S>::load(link_slot<HALO>(A, s, j, k, P + q, P + p00, P + p10, P + p01, P + p11));
+            c.h[q] = s.solid ? bounce_h(A.C, s.face, v) : v;
         }
     }
 }
@@ -613,44 +613,30 @@ __device__ __forceinline__ void pull_odd(const KArgs<S, R>& A, int j, int k, Cel
 template <class S, class R, bool SW, bool TH, bool HALO = false>
 __device__ __forceinline__ void push_odd(const KArgs<S, R>& A, int j, int k, const Cell<R, SW, TH>& c) {
     const Geom& G = A.G;
+    // (through the axis into the mirror column of a node-on-axis grid: the population leaves)
+    const bool mirror_col = G.inner == AXLBM_INNER_AXIS_NODE;
 #pragma unroll
     for (int a = 0; a < 9; ++a) {
-        const Site s = classify(G, j, k, cr9(a), cz9(a));
-        if (s.solid) {
-            Codec<S>::store(slot(A.pop, G, opp9(a), j, k), c.d[a]);
-        } else if (G.inner == AXLBM_INNER_AXIS_NODE && s.fr) {
-            // leaves through the axis into the mirror column
-        } else {
-            const int b = idx9(s.fr ? -cr9(a) : cr9(a), s.fz ? -cz9(a) : cz9(a));
-            Codec<S>::store(site_slot<HALO>(A, b, s.j, s.k), c.d[a]);
-        }
+        const int x = cr9(a), z = cz9(a);
+        const Site s = classify(G, j, k, x, z);
+        S* to = link_slot<HALO>(A, s, j, k, opp9(a), a, idx9(-x, z), idx9(x, -z), idx9(-x, -z));
+        if (s.solid || !(mirror_col && s.fr)) Codec<S>::store(to, c.d[a]);
     }
-    if (SW) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const Site s = classify(G, j, k, cr4(q), cz4(q));
-            if (s.solid) {
-                Codec<S>::store(slot(A.pop, G, A.g_plane + opp4(q), j, k), bounce_g(G, A.C, s.face, j, c.g[q]));
-            } else if (G.inner == AXLBM_INNER_AXIS_NODE && s.fr) {
-                // leaves through the axis into the mirror column
-            } else {
-                const int b = idx4(s.fr ? -cr4(q) : cr4(q), s.fz ? -cz4(q) : cz4(q));
-                Codec<S>::store(site_slot<HALO>(A, A.g_plane + b, s.j, s.k), s.fr ? -c.g[q] : c.g[q]);
-            }
+    for (int q = 0; q < 4; ++q) {
+        if (!SW && !TH) break;
+        const int x = cr4(q), z = cz4(q), p10 = idx4(-x, z), p01 = idx4(x, -z), p11 = idx4(-x, -z);
+        const Site s = classify(G, j, k, x, z);
+        const bool stays = s.solid || !(mirror_col && s.fr);
+        if (SW) {
+            const int P = A.g_plane;
+            S* to = link_slot<HALO>(A, s, j, k, P + opp4(q), P + q, P + p10, P + p01, P + p11);
+            if (stays) Codec<S>::store(to, s.solid ? bounce_g(G, A.C, s.face, j, c.g[q]) : (s.fr ? -c.g[q] : c.g[q]));
         }
-    }
-    if (TH) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const Site s = classify(G, j, k, cr4(q), cz4(q));
-            if (s.solid) {
-                Codec<S>::store(slot(A.pop, G, A.h_plane + opp4(q), j, k), bounce_h(A.C, s.face, c.h[q]));
-            } else if (G.inner == AXLBM_INNER_AXIS_NODE && s.fr) {
-                // leaves through the axis into the mirror column
-            } else {
-                const int b = idx4(s.fr ? -cr4(q) : cr4(q), s.fz ? -cz4(q) : cz4(q));
-                Codec<S>::store(site_slot<HALO>(A, A.h_plane + b, s.j, s.k), c.h[q]);
-            }
+        if (TH) {
+            const int P = A.h_plane;
+            S* to = link_slot<HALO>(A, s, j, k, P + opp4(q), P + q, P + p10, P + p01, P + p11);
+            if (stays) Codec<S>::store(to, s.solid ? bounce_h(A.C, s.face, c.h[q]) : c.h[q]);
         }
     }
 }
@@ -758,9 +744,15 @@ __device__ __forceinline__ void check_cell(const KArgs<S, R>& A, int j, int k, R
     red.bad += ok ? 0.0 : 1.0;
 }
 
+// a(t) = az0 cos(omega_t t); a steady force without the cosine, whose FP64
+// instructions take over a microsecond of one thread.
+__device__ __forceinline__ double force_at(double az0, double omega_t, long long t) {
+    return omega_t == 0.0 ? az0 : az0 * cos(omega_t * (double)t);
+}
+
 __device__ __forceinline__ void advance_clock(Clock* clk, int parity, double az0, double omega_t) {
     const long long t1 = clk->t + 1;
-    clk->a_z[1 - parity] = az0 * cos(omega_t * (double)t1);
+    clk->a_z[1 - parity] = force_at(az0, omega_t, t1);
     clk->t = t1;
 }
 

@@ -124,14 +124,14 @@ __host__ __device__ __forceinline__ void res_where(const Geom& G, int q, int j, 
 // a(t) in R, as the step kernels round it.
 template <class R>
 __device__ __forceinline__ R res_az(double az0, double omega_t, long long t) {
-    return R(az0 * cos(omega_t * (double)t));
+    return R(force_at(az0, omega_t, t));
 }
 
 // The force and the time level after the last step of a launch (an even
 // level; the odd entry holds the last step's force, as after single steps).
 template <class S, class R>
 __device__ __forceinline__ void res_finish(const ResDom<S, R>& D, long long t1) {
-    const double a0 = D.az0 * cos(D.omega_t * (double)t1), a1 = D.az0 * cos(D.omega_t * (double)(t1 - 1));
+    const double a0 = force_at(D.az0, D.omega_t, t1), a1 = force_at(D.az0, D.omega_t, t1 - 1);
     D.az[0] = a0;
     D.az[1] = a1;
     if (D.az16) {
