@@ -397,7 +397,12 @@ cudaError_t batch_capture_pairs(axlbm_batch* b, const BatchOps* ops, int pairs, 
     cudaStream_t caller = b->stream;
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaSuccess;
-    if (!b->cap) e = cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking);
+    if (!b->cap) {  // FP32: above the side stream (see batch_step_th), FP16: below it
+        int lo = 0, hi = 0;
+        e = cudaDeviceGetStreamPriorityRange(&lo, &hi);
+        if (e == cudaSuccess)
+            e = cudaStreamCreateWithPriority(&b->cap, cudaStreamNonBlocking, b->precision == AXLBM_FP32 ? hi : lo);
+    }
     if (e == cudaSuccess) e = cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return e;
     b->stream = b->cap;
@@ -670,7 +675,9 @@ axlbm_status axlbm_batch_create(const axlbm_domain* domains, int32_t n, int32_t 
     {
         int lo = 0, hi = 0;
         cudaError_t e = cudaDeviceGetStreamPriorityRange(&lo, &hi);
-        if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&b->side, cudaStreamNonBlocking, hi);
+        // (the graphs' bulk nodes are captured on a stream of their own priority, see batch_capture_pairs)
+        if (e == cudaSuccess)
+            e = cudaStreamCreateWithPriority(&b->side, cudaStreamNonBlocking, precision == AXLBM_FP32 ? lo : hi);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->join, cudaEventDisableTiming);
         if (e != cudaSuccess) st = bcuda(b, e, "side stream");

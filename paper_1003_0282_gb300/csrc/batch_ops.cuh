@@ -133,19 +133,16 @@ cudaError_t batch_step_th(axlbm_batch* b, int check, int residual, cudaEvent_t e
         }
         return e;
     }
-    // odd step: the interior (bulk) and the outer rings touch disjoint slots.
-    // With 16-bit storage the bulk kernel is bound by issue, not by HBM, so
-    // the rings run concurrently on the side stream (their small blocks use
-    // the SMs' leftover registers); with FP32 storage the bulk kernel needs
-    // all of HBM and the rings' scattered accesses would slow it, so they
-    // follow it on the same stream.
-    const bool overlap = sizeof(S) == 2;
-    cudaStream_t rs = overlap ? b->side : b->stream;
-    if (overlap) {
-        e = cudaEventRecord(b->fork, b->stream);
-        if (e == cudaSuccess) e = cudaStreamWaitEvent(b->side, b->fork, 0);
-        if (e != cudaSuccess) return e;
-    }
+    // odd step: the interior (bulk) and the outer rings touch disjoint slots, so
+    // the rings run on the side stream beside the bulk kernel.  With 16-bit
+    // storage they go first (that bulk kernel is bound by issue, and the rings'
+    // small blocks use the SMs' leftover registers).  With FP32 storage the
+    // bulk kernel needs all of HBM and every SM from the start, so there the
+    // rings have the lower priority and fill its tail.
+    cudaStream_t rs = b->side;
+    e = cudaEventRecord(b->fork, b->stream);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(b->side, b->fork, 0);
+    if (e != cudaSuccess) return e;
     e = check ? launch_bulk_batch_shape<S, R, TH, 1, true>(b, A) : launch_bulk_batch_shape<S, R, TH, 1, false>(b, A);
     if (ev1) cudaEventRecord(ev1, b->stream);
     if (e != cudaSuccess) return e;
@@ -153,15 +150,6 @@ cudaError_t batch_step_th(axlbm_batch* b, int check, int residual, cudaEvent_t e
     // the only one, also moves the force and the time level on)
     const int cold = b->L.nring_cold, hot = A.nring - cold;
     const bool two = TH && hot > 0 && cold > 0;
-    // with FP32 storage the two ring classes (disjoint domains) run side by
-    // side: the thermal one on the side stream, forked after the bulk kernel
-    cudaStream_t hs = rs;
-    if (!overlap && two) {
-        e = cudaEventRecord(b->fork, b->stream);
-        if (e == cudaSuccess) e = cudaStreamWaitEvent(b->side, b->fork, 0);
-        if (e != cudaSuccess) return e;
-        hs = b->side;
-    }
     *nl = 1;
     if (cold > 0 || !TH) {
         const int blocks = (cold + kRingThreads - 1) / kRingThreads;
@@ -171,15 +159,13 @@ cudaError_t batch_step_th(axlbm_batch* b, int check, int residual, cudaEvent_t e
     }
     if (TH && hot > 0) {
         const int blocks = (hot + kRingThreads - 1) / kRingThreads;
-        if (check) k_ring_batch<S, R, true, true, true><<<blocks, kRingThreads, 0, hs>>>(A, cold, A.nring, 1);
-        else k_ring_batch<S, R, true, true, false><<<blocks, kRingThreads, 0, hs>>>(A, cold, A.nring, 1);
+        if (check) k_ring_batch<S, R, true, true, true><<<blocks, kRingThreads, 0, rs>>>(A, cold, A.nring, 1);
+        else k_ring_batch<S, R, true, true, false><<<blocks, kRingThreads, 0, rs>>>(A, cold, A.nring, 1);
         *nl += 1;
     }
     e = cudaGetLastError();
-    if (overlap || hs != rs) {
-        if (e == cudaSuccess) e = cudaEventRecord(b->join, b->side);
-        if (e == cudaSuccess) e = cudaStreamWaitEvent(b->stream, b->join, 0);
-    }
+    if (e == cudaSuccess) e = cudaEventRecord(b->join, b->side);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(b->stream, b->join, 0);
     if (e == cudaSuccess && b->L.naxis > 0) {
         k_axis_mirror_batch<S, true, TH><<<b->L.naxis, kThreads, 0, b->stream>>>(
             A, reinterpret_cast<const int*>(b->mem + b->L.off_axis));
