@@ -465,7 +465,8 @@ axlbm_status axlbm_step(axlbm_handle* h, int64_t n) {
     const int tail = h->residual_lag == 2 ? 3 : 2;
     const bool odd_bulk = h->G.nr > 2 && h->G.nz > 2;
     const bool sized = h->bulk_grid[0][0] > 0 && (h->bulk_grid[1][0] > 0 || !odd_bulk);
-    if (h->use_graphs && !h->timing && (sized || h->res.on) && n - tail - h->parity >= 2 * kMinGraphPairs) {
+    const bool ready = h->res.on ? axl::resident_usable(h->res, h->stream) : sized;
+    if (h->use_graphs && !h->timing && ready && n - tail - h->parity >= 2 * kMinGraphPairs) {
         if (h->parity == 1) {
             int nl = 0;
             const cudaError_t e = ops->step(h, 0, 0, nullptr, nullptr, &nl);

@@ -483,7 +483,8 @@ axlbm_status batch_step_n(axlbm_batch* b, int64_t n) {
     // launches (a batch on the multi-step kernels needs none)
     const int tail = b->residual_lag == 2 ? 3 : 2;
     const bool sized = b->grid[b->shape[0]][0][0] > 0 && b->grid[b->shape[1]][1][0] > 0;
-    if (b->use_graphs && !b->timing && (sized || b->res.on) && n - tail - b->parity >= 2 * kMinGraphPairs) {
+    const bool ready = b->res.on ? axl::resident_usable(b->res, b->stream) : sized;
+    if (b->use_graphs && !b->timing && ready && n - tail - b->parity >= 2 * kMinGraphPairs) {
         if (b->parity == 1) {
             int nl = 0;
             const cudaError_t e = ops->step(b, 0, 0, nullptr, nullptr, &nl);

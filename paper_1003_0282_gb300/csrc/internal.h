@@ -120,6 +120,10 @@ extern const ResidentOps resident_fp64;
 
 constexpr int64_t kResMaxSteps = 1 << 16;  // steps of one launch, at most (even)
 
+// Whether a call on `stream` takes the multi-step launches.  A launch carries its time level and the base of its step
+// counters, so one that a caller captures could not be replayed: under capture the step kernels, which take both from
+// the device, run one by one.
+bool resident_usable(const Resident& r, cudaStream_t stream);
 cudaError_t resident_capture(Resident* r, Clock* clock, cudaStream_t cap);
 cudaError_t resident_launch(Resident* r, Clock* clock, int steps, long long t0, cudaStream_t stream);
 void resident_drop_graph(Resident* r);

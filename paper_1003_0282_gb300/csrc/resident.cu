@@ -37,6 +37,16 @@ struct ResArgs {
 
 }  // namespace
 
+bool resident_usable(const Resident& r, cudaStream_t stream) {
+    if (!r.on) return false;
+    cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(stream, &s) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return s == cudaStreamCaptureStatusNone;
+}
+
 cudaError_t resident_capture(Resident* r, Clock* clock, cudaStream_t cap) {
     ResArgs a(*r, clock, 2, 0);
     cudaLaunchConfig_t cfg = {};

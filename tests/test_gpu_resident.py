@@ -101,3 +101,42 @@ def test_small_batches(B, scale):
     for d in range(len(probs)):
         for x, y in zip(p0[d], p1[d]):
             assert (x is None and y is None) or np.array_equal(x, y), d
+
+
+@pytest.mark.parametrize("kind", ["domain", "batch"])
+def test_captured_calls_replay(B, kind):
+    """A call that the caller captures advances the state on every replay, as calls in between do."""
+    import torch
+
+    pb = problem(64, 48, "crystal") if kind == "domain" else None
+    probs = [problem(33, 40, "crystal"), problem(20, 31, "pipe", temperature=False)]
+    got = []
+    for captured in (True, False):
+        stream = torch.cuda.Stream()
+        with torch.cuda.stream(stream):
+            if kind == "domain":
+                sim = B.Domain(pb, "fp32", stream=stream)
+                st = seeded_state(pb, 3)
+                sim.set_populations(st.f, st.g, st.h, time=0)
+            else:
+                sim = B.Batch(probs, "fp32", stream=stream)
+                for d, p in enumerate(probs):
+                    st = seeded_state(p, 3 + d)
+                    sim.set_populations(d, st.f, st.g, st.h if p.temperature else None)
+            sim.step(20)
+            stream.synchronize()
+            if captured:
+                graph = torch.cuda.CUDAGraph()
+                with torch.cuda.graph(graph, stream=stream, capture_error_mode="thread_local"):
+                    sim.step(20)
+                for _ in range(3):
+                    graph.replay()
+            else:
+                for _ in range(3):
+                    sim.step(20)
+            stream.synchronize()
+            got.append([sim.get_populations()] if kind == "domain" else [sim.get_populations(d) for d in range(2)])
+            sim.close()
+    for x, y in zip(*got):
+        for u, v in zip(x, y):
+            assert (u is None and v is None) or np.array_equal(u, v)
