@@ -336,12 +336,14 @@ AXLBM_API axlbm_status axlbm_load(axlbm_handle* h, const void* buf, size_t bytes
  * and 1 pairs of an even and an odd step, on a stream of the library's own,
  * launched on the handle's stream) when enable != 0, the default, and while
  * kernel timing is off; enable = 0 launches every kernel directly.  Small
- * domains with FP32 or FP64 storage (up to 64 MB of populations) take one
+ * domains (FP32 and FP64 storage: up to 64 MB of populations; 16-bit storage:
+ * those whose state fits the SMs' shared memories as FP32 values) take one
  * graph of a single kernel that runs all the pairs of a call, with device
  * scratch of the library's own allocated at creation; where that cannot be
  * allocated, or the domain has wet walls, a Zou-He wall, a node on the axis or
- * cut faces, the step pairs are replayed.  The results are the same bit for
- * bit. */
+ * cut faces, the step pairs are replayed.  A call made while the caller
+ * captures the handle's stream launches such a domain's steps kernel by
+ * kernel.  The results are the same bit for bit. */
 AXLBM_API axlbm_status axlbm_use_graphs(axlbm_handle* h, int32_t enable);
 
 /* How many times the step graphs were captured and launched since creation
@@ -535,9 +537,9 @@ AXLBM_API axlbm_status axlbm_batch_tile_shape(const axlbm_batch* b, int32_t* row
  * axlbm_batch_step call) are replayed from CUDA graphs captured on first use
  * (8 and 1 pairs of an even and an odd step; recaptured after a tile shape
  * change) when enable != 0, the default, and while kernel timing is off;
- * enable = 0 launches every kernel directly.  Small FP32 batches (up to 64 MB
- * of populations, domains as axlbm_use_graphs lists them) take one graph of a
- * single kernel that runs all the pairs of a call.  The results are the same
+ * enable = 0 launches every kernel directly.  Small batches (as axlbm_use_graphs
+ * says of domains) take one graph of a single kernel that runs all the pairs of
+ * a call.  The results are the same
  * bit for bit.  The first capture synchronises nothing but takes a few ms. */
 AXLBM_API axlbm_status axlbm_batch_use_graphs(axlbm_batch* b, int32_t enable);
 

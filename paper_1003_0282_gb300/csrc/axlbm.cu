@@ -352,11 +352,14 @@ axlbm_status axlbm_create(const axlbm_grid* grid, double tau, const axlbm_forcin
             cudaFree(fields);
         }
     }
-    if (st == AXLBM_OK && (grid->precision == AXLBM_FP32 || grid->precision == AXLBM_FP64)) {
+    if (st == AXLBM_OK) {
         axl::Clock* clk = reinterpret_cast<axl::Clock*>(h->mem + L.off_clock);
         const axl::ResidentDomain d = {h->mem, h->G, tau, *forcing, *bc, grid->collision == AXLBM_MRT,
                                        grid->with_temperature, clk->a_z, nullptr};
-        const axl::ResidentOps& ro = grid->precision == AXLBM_FP32 ? axl::resident_fp32 : axl::resident_fp64;
+        const axl::ResidentOps& ro = grid->precision == AXLBM_FP32       ? axl::resident_fp32
+                                     : grid->precision == AXLBM_FP64     ? axl::resident_fp64
+                                     : grid->precision == AXLBM_FP16_DEV ? axl::resident_fp16
+                                                                         : axl::resident_bf16;
         e = ro.build(&h->res, &d, 1, grid->with_swirl != 0, grid->with_temperature != 0, h->num_sms, h->stream);
         if (e != cudaSuccess) st = cuda_fail(h, e, "multi-step launch");
     }

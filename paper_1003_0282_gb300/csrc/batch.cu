@@ -760,7 +760,7 @@ axlbm_status axlbm_batch_create(const axlbm_domain* domains, int32_t n, int32_t 
     if (st == AXLBM_OK) st = reset_rest(b);
     if (st == AXLBM_OK) st = tune(b);
     if (st == AXLBM_OK) st = reset_rest(b);
-    if (st == AXLBM_OK && precision == AXLBM_FP32) {
+    if (st == AXLBM_OK) {
         double* az = reinterpret_cast<double*>(b->mem + L.off_az);
         std::vector<axl::ResidentDomain> rd(n);
         for (int d = 0; d < n; ++d) {
@@ -784,7 +784,8 @@ axlbm_status axlbm_batch_create(const axlbm_domain* domains, int32_t n, int32_t 
             rd[d] = {b->mem, G, D.tau, D.forcing, D.boundary, D.grid.collision == AXLBM_MRT, D.grid.with_temperature,
                      az + 2 * d, az + 2 * n + 4 * d};
         }
-        const cudaError_t e = axl::resident_fp32.build(&b->res, rd.data(), n, true, b->thmax != 0, b->num_sms, b->stream);
+        const axl::ResidentOps& ro = precision == AXLBM_FP32 ? axl::resident_fp32 : axl::resident_fp16;
+        const cudaError_t e = ro.build(&b->res, rd.data(), n, true, b->thmax != 0, b->num_sms, b->stream);
         if (e != cudaSuccess) st = bcuda(b, e, "multi-step launch");
     }
     if (st == AXLBM_OK) {

@@ -117,6 +117,8 @@ struct ResidentOps {
 };
 extern const ResidentOps resident_fp32;
 extern const ResidentOps resident_fp64;
+extern const ResidentOps resident_fp16;
+extern const ResidentOps resident_bf16;
 
 constexpr int64_t kResMaxSteps = 1 << 16;  // steps of one launch, at most (even)
 

@@ -22,8 +22,11 @@
 //     domain and after every step waits only for the CTAs whose nodes its own
 //     exchange populations with (a step counter per CTA, polled with a bound).
 //
-// Arithmetic and storage are those of the step kernels (PairArith, Codec),
-// rounding included: a run here equals the same steps launched one by one.
+// Arithmetic and storage are those of the step kernels (PairArith, NodeArith,
+// Codec), rounding included: a run here equals the same steps launched one by
+// one.  With 16-bit storage (S) shared memory holds the FP32 value (R) of what
+// would be stored, rounded through S on every store, and the nodes that the
+// ring kernels update take their arithmetic in odd steps.
 #pragma once
 
 #include <cooperative_groups.h>
@@ -163,6 +166,71 @@ struct ResLinks {
     }
 };
 
+// v as storage S keeps it.
+template <class S, class R>
+__device__ __forceinline__ R res_keep(R v) {
+    if constexpr (std::is_same<S, R>::value) return v;
+    S t;
+    Codec<S>::store(&t, v);
+    return Codec<S>::load(&t);
+}
+
+// Lanes (bit l: row k0 + l) of a pair of column j that the ring kernels update
+// in odd steps with an arithmetic of their own, which is so with 16-bit
+// storage only: the outer ring, without the side columns where the bulk
+// kernels take them (Geom::side).
+template <class S, class R>
+__device__ __forceinline__ unsigned res_ring(const Geom& G, int j, int k0) {
+    if constexpr (std::is_same<S, R>::value) return 0;
+    const bool column = (j == 0 || j == G.nr - 1) && !(G.inner == AXLBM_INNER_AXIS && G.nr >= 3 && G.nz >= 3);
+    return (column || k0 == 0 || k0 == G.nz - 1 ? 1u : 0u) | (column || k0 + 1 == G.nz - 1 ? 2u : 0u);
+}
+
+// A node of the ring kernels.  Plain float expressions are fused by the
+// compiler within a basic block, and what it hoists out of a loop over steps is
+// no longer there to fuse: a call keeps the expressions as a ring kernel has
+// them, and with them the rounding.
+template <class R, bool SW, bool TH>
+__device__ __noinline__ void res_ring_collide(Cell<R, SW, TH>& s, R inv_r, const Coef<R>& C, R az) {
+    s.collide(inv_r, C, az);
+}
+
+// Collides a pair: the lanes of `ring` as the ring kernels do, at 1/r = inv_ring().
+template <class S, class RC, class R, bool SW, bool TH, class Inv>
+__device__ __forceinline__ void res_collide(Cell<RC, SW, TH>& c, R inv_r, const Coef<R>& C, R az, unsigned ring,
+                                            const Coef<R>& Cg, const Inv& inv_ring) {
+    if constexpr (!std::is_same<S, R>::value) {
+        if (ring) {
+            const Cell<RC, SW, TH> in = c;
+            if (ring != 3u) c.collide(inv_r, C, az);
+            const R inv = inv_ring();
+#pragma unroll 1
+            for (int l = 0; l < 2; ++l) {
+                if (!((ring >> l) & 1u)) continue;
+                Cell<R, SW, TH> s;
+                auto put = [&](RC& to, R v) { to = l ? RC(Lanes<RC>::get(to, 0), v) : RC(v, Lanes<RC>::get(to, 1)); };
+#pragma unroll
+                for (int a = 0; a < 9; ++a) s.d[a] = Lanes<RC>::get(in.d[a], l);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    if (SW) s.g[q] = Lanes<RC>::get(in.g[q], l);
+                    if (TH) s.h[q] = Lanes<RC>::get(in.h[q], l);
+                }
+                res_ring_collide(s, inv, Cg, az);
+#pragma unroll
+                for (int a = 0; a < 9; ++a) put(c.d[a], s.d[a]);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    if (SW) put(c.g[q], s.g[q]);
+                    if (TH) put(c.h[q], s.h[q]);
+                }
+            }
+            return;
+        }
+    }
+    c.collide(inv_r, C, az);
+}
+
 // Load / store the populations of a pair: at(q, l) is the value of plane-
 // ordered slot q of lane l; in odd steps links change g and h on the way, and
 // slot q takes the opposite population.
@@ -179,7 +247,7 @@ __device__ __forceinline__ void res_load(Cell<RC, SW, TH>& c, const At& at, cons
         if (TH && PAR) c.h[q] = L.h(q, c.h[q]);
     }
 }
-template <class RC, bool SW, bool TH, int PAR, class To, class Links>
+template <class S, class RC, bool SW, bool TH, int PAR, class To, class Links>
 __device__ __forceinline__ void res_store(const Cell<RC, SW, TH>& c, const To& to, const Links& L) {
     constexpr int NL = Lanes<RC>::n, HP = SW ? 13 : 9;
 #pragma unroll
@@ -189,7 +257,7 @@ __device__ __forceinline__ void res_store(const Cell<RC, SW, TH>& c, const To& t
         if (PAR && SW && q >= 9 && q < 13) x = L.g(m, x);
         if (PAR && TH && q >= HP) x = L.h(m, x);
 #pragma unroll
-        for (int l = 0; l < NL; ++l) to(q, l, Lanes<RC>::get(x, l));
+        for (int l = 0; l < NL; ++l) to(q, l, res_keep<S>(Lanes<RC>::get(x, l)));
     }
 }
 
@@ -250,13 +318,13 @@ __device__ __forceinline__ void res_dld(uint32_t a, double& v) {
 // the collision, barrier); the throughput of one scheduler for more pairs.
 // FP64: the FP64 pipe (64.5 cycles per warp instruction and scheduler,
 // whatever its active lanes).
-template <class R, bool SW, bool TH>
+template <class S, class R, bool SW, bool TH>
 __global__ void __launch_bounds__(kResThreads, 1)
-k_resident_cluster(const ResDom<R, R>* __restrict__ doms, Clock* clock, int nsteps, long long t0) {
+k_resident_cluster(const ResDom<S, R>* __restrict__ doms, Clock* clock, int nsteps, long long t0) {
     using RC = typename PairArith<R>::type;
     constexpr int NL = Lanes<RC>::n, P = nplanes<SW, TH>();
     extern __shared__ __align__(16) unsigned char res_smem[];
-    const ResDom<R, R>& D = doms[0];
+    const ResDom<S, R>& D = doms[0];
     const Geom& G = D.G;
     uint32_t nclust;
     asm("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(nclust));
@@ -278,7 +346,7 @@ k_resident_cluster(const ResDom<R, R>* __restrict__ doms, Clock* clock, int nste
 #pragma unroll
         for (int q = 0; q < P; ++q)
 #pragma unroll
-            for (int l = 0; l < NL; ++l) mine[(q * NL + l) * chunk] = k0 + l < G.nz ? *slot(D.pop, G, q, j, k0 + l) : R(0);
+            for (int l = 0; l < NL; ++l) mine[(q * NL + l) * chunk] = k0 + l < G.nz ? Codec<S>::load(slot(D.pop, G, q, j, k0 + l)) : R(0);
         res_links<RC, R, SW, TH>(G, C, j, k0, L, [&](int q, int l, int ql, int sp) {
             if (sp < 0) sp = p;
             const int sr = sp / chunk, si = sp - sr * chunk;
@@ -286,6 +354,7 @@ k_resident_cluster(const ResDom<R, R>* __restrict__ doms, Clock* clock, int nste
         });
     }
     const R inv_r = step_inv_radius<R>(G, j);
+    const unsigned ring = res_ring<S, R>(G, j, k0);
     auto meet = [&]() {
         if (ncta == 1) {
             __syncthreads();
@@ -306,7 +375,7 @@ k_resident_cluster(const ResDom<R, R>* __restrict__ doms, Clock* clock, int nste
             if ((s & 1) == 0) {  // even step: own slots, back into the opposite ones
                 res_load<RC, SW, TH, 0>(c, [&](int q, int l) { return mine[(q * NL + l) * chunk]; }, L);
                 c.collide(inv_r, C, az);
-                res_store<RC, SW, TH, 0>(c, [&](int q, int l, R v) { mine[(q * NL + l) * chunk] = v; }, L);
+                res_store<S, RC, SW, TH, 0>(c, [&](int q, int l, R v) { mine[(q * NL + l) * chunk] = v; }, L);
             } else {
                 R v[P][NL];
 #pragma unroll
@@ -314,8 +383,8 @@ k_resident_cluster(const ResDom<R, R>* __restrict__ doms, Clock* clock, int nste
 #pragma unroll
                     for (int l = 0; l < NL; ++l) res_dld(at[q][l], v[q][l]);
                 res_load<RC, SW, TH, 1>(c, [&](int q, int l) { return v[q][l]; }, L);
-                c.collide(inv_r, C, az);
-                res_store<RC, SW, TH, 1>(c, [&](int q, int l, R x) { res_dst(at[q][l], x); }, L);
+                res_collide<S>(c, inv_r, C, az, ring, D.C, [&]() { return inv_radius<R>(G, j); });
+                res_store<S, RC, SW, TH, 1>(c, [&](int q, int l, R x) { res_dst(at[q][l], x); }, L);
             }
         }
         meet();
@@ -325,7 +394,7 @@ k_resident_cluster(const ResDom<R, R>* __restrict__ doms, Clock* clock, int nste
         for (int l = 0; l < NL; ++l) {
             if (k0 + l >= G.nz) continue;
 #pragma unroll
-            for (int q = 0; q < P; ++q) *slot(D.pop, G, q, j, k0 + l) = mine[(q * NL + l) * chunk];
+            for (int q = 0; q < P; ++q) Codec<S>::store(slot(D.pop, G, q, j, k0 + l), mine[(q * NL + l) * chunk]);
         }
     }
     if (rank == 0 && tid == 0) {
@@ -479,8 +548,8 @@ __device__ __forceinline__ int res_new_ghost(bool remote, int* count) {
 // The common part of the kernels that keep the state in shared memory: loads
 // it, runs nsteps steps of update(par, force), each between the words of its
 // neighbours coming in and going out, and writes it back.
-template <class R, bool SW, bool TH, class Update>
-__device__ __forceinline__ void res_slab_run(const ResDom<R, R>& D, const ResSlab<R>& S, Clock* clock, int nsteps,
+template <class S_, class R, bool SW, bool TH, class Update>
+__device__ __forceinline__ void res_slab_run(const ResDom<S_, R>& D, const ResSlab<R>& S, Clock* clock, int nsteps,
                                              unsigned epoch, long long t0, int ng, int* bad, const Update& update) {
     constexpr int NL = Lanes<typename PairArith<R>::type>::n, PL = nplanes<SW, TH>() * NL;
     const Geom& G = D.G;
@@ -517,15 +586,15 @@ __device__ __forceinline__ void res_slab_run(const ResDom<R, R>& D, const ResSla
     const int n = tile.w * tile.h;
     for (int m = tid; m < PL * n; m += T) {
         const int ql = m / n, i = m - ql * n, kl = i / tile.w, j = tile.j0 + i - kl * tile.w, k = NL * (tile.k0 + kl) + ql % NL;
-        if (k < G.nz) *slot(D.pop, G, ql / NL, j, k) = S.st[ql * chunk + i];
+        if (k < G.nz) Codec<S_>::store(slot(D.pop, G, ql / NL, j, k), S.st[ql * chunk + i]);
     }
     if (rank == 0 && tid == 0) res_finish(D, t0 + nsteps);
     if (blockIdx.x == 0 && tid == 0) clock->t = t0 + nsteps;
 }
 
 // One pair per thread: addresses and links stay in registers.
-template <class R, bool SW, bool TH>
-__device__ __forceinline__ void res_one_cta(const ResDom<R, R>& D, Clock* clock, int nsteps, unsigned epoch, long long t0,
+template <class S_, class R, bool SW, bool TH>
+__device__ __forceinline__ void res_one_cta(const ResDom<S_, R>& D, Clock* clock, int nsteps, unsigned epoch, long long t0,
                                             unsigned char* smem) {
     using RC = typename PairArith<R>::type;
     constexpr int NL = Lanes<RC>::n, P = nplanes<SW, TH>();
@@ -557,23 +626,24 @@ __device__ __forceinline__ void res_one_cta(const ResDom<R, R>& D, Clock* clock,
                 S.even[g] = res_word<P * NL>(D, nkp, q * NL + l, j, kp);
                 S.odd[g] = res_word<P * NL>(D, nkp, ql, sp % nr, sp / nr);
             }
-            if (on) mine[(q * NL + l) * chunk] = k0 + l < G.nz ? *slot(D.pop, G, q, j, k0 + l) : R(0);
+            if (on) mine[(q * NL + l) * chunk] = k0 + l < G.nz ? Codec<S_>::load(slot(D.pop, G, q, j, k0 + l)) : R(0);
         });
     }
     __syncthreads();
     const R inv_r = step_inv_radius<R>(G, j);
-    res_slab_run<R, SW, TH>(D, S, clock, nsteps, epoch, t0, min(ghosts, max_ghost), &bad, [&](auto par_tag, R az) {
+    const unsigned ring = res_ring<S_, R>(G, j, k0);
+    res_slab_run<S_, R, SW, TH>(D, S, clock, nsteps, epoch, t0, min(ghosts, max_ghost), &bad, [&](auto par_tag, R az) {
         constexpr int PAR = decltype(par_tag)::value;
         if (!on) return;
         Cell<RC, SW, TH> c;
         if (PAR == 0) {
             res_load<RC, SW, TH, 0>(c, [&](int q, int l) { return mine[(q * NL + l) * chunk]; }, L);
             c.collide(inv_r, C, az);
-            res_store<RC, SW, TH, 0>(c, [&](int q, int l, R v) { mine[(q * NL + l) * chunk] = v; }, L);
+            res_store<S_, RC, SW, TH, 0>(c, [&](int q, int l, R v) { mine[(q * NL + l) * chunk] = v; }, L);
         } else {
             res_load<RC, SW, TH, 1>(c, [&](int q, int l) { return S.st[at[q][l]]; }, L);
-            c.collide(inv_r, C, az);
-            res_store<RC, SW, TH, 1>(c, [&](int q, int l, R v) { S.st[at[q][l]] = v; }, L);
+            res_collide<S_>(c, inv_r, C, az, ring, D.C, [&]() { return inv_radius<R>(G, j); });
+            res_store<S_, RC, SW, TH, 1>(c, [&](int q, int l, R v) { S.st[at[q][l]] = v; }, L);
         }
     });
 }
@@ -583,17 +653,20 @@ __device__ __forceinline__ void res_one_cta(const ResDom<R, R>& D, Clock* clock,
 //
 // What bounds it: the latency of a step -- the neighbours' words (a store and
 // a polled load of L2), one node's chain, two barriers.
-template <class R, bool SW, bool TH>
+template <class S, class R, bool SW, bool TH>
 __global__ void __launch_bounds__(kResThreads, 1)
-k_resident_one(const ResDom<R, R>* __restrict__ doms, const int* __restrict__ cta_dom, Clock* clock, int nsteps,
+k_resident_one(const ResDom<S, R>* __restrict__ doms, const int* __restrict__ cta_dom, Clock* clock, int nsteps,
                unsigned epoch, long long t0) {
     extern __shared__ __align__(16) unsigned char res_smem[];
-    const ResDom<R, R>& D = doms[cta_dom[blockIdx.x]];
-    if (TH && D.th) res_one_cta<R, SW, TH>(D, clock, nsteps, epoch, t0, res_smem);
-    else res_one_cta<R, SW, false>(D, clock, nsteps, epoch, t0, res_smem);
+    const ResDom<S, R>& D = doms[cta_dom[blockIdx.x]];
+    if (TH && D.th) res_one_cta<S, R, SW, TH>(D, clock, nsteps, epoch, t0, res_smem);
+    else res_one_cta<S, R, SW, false>(D, clock, nsteps, epoch, t0, res_smem);
 }
 
 constexpr int kResSlabThreads = 384;
+
+constexpr int kResRingShift = 28;  // a pair's index in the tile below, the lanes of res_ring above
+constexpr int kResPairMask = (1 << kResRingShift) - 1;
 
 // A pair of the kernel below: its index in the tile; tab: its row of the slot
 // table, or -1 away from the tile's outline, where every slot is the CTA's own.
@@ -628,8 +701,8 @@ __host__ __device__ constexpr size_t res_column_bytes(int w) {
 }
 
 // Several pairs per thread.
-template <class R, bool SW, bool TH>
-__device__ __forceinline__ void res_slab_cta(const ResDom<R, R>& D, Clock* clock, int nsteps, unsigned epoch, long long t0,
+template <class S_, class R, bool SW, bool TH>
+__device__ __forceinline__ void res_slab_cta(const ResDom<S_, R>& D, Clock* clock, int nsteps, unsigned epoch, long long t0,
                                              unsigned char* smem) {
     using RC = typename PairArith<R>::type;
     constexpr int NL = Lanes<RC>::n, P = nplanes<SW, TH>(), PL = P * NL, NF = (SW ? 8 : 0) + (TH ? 12 : 0);
@@ -660,7 +733,7 @@ __device__ __forceinline__ void res_slab_cta(const ResDom<R, R>& D, Clock* clock
                     ResPair<R> r;
                     if constexpr (sizeof(R) == 8) r.col = jl;
                     else r.inv_r = step_inv_radius<R>(G, tile.j0 + jl);
-                    r.i = i;
+                    r.i = i | (int)(res_ring<S_, R>(G, tile.j0 + jl, NL * (tile.k0 + kl)) << kResRingShift);
                     const int to = row ? at1 + __popc(m1 & ((1u << tid) - 1u)) : at0 + __popc(m0 & ((1u << tid) - 1u));
                     r.tab = row ? to - plain : -1;
                     pairs[to] = r;
@@ -682,7 +755,7 @@ __device__ __forceinline__ void res_slab_cta(const ResDom<R, R>& D, Clock* clock
         for (int w = tid >> 5; w < blocks * PL; w += T >> 5) {  // 32 pairs of one population and lane
             const int x = w / blocks, t = (w - x * blocks) * 32 + lane, q = x / NL, l = x - q * NL;
             const bool on = t < nt;
-            const int i = pairs[n0 + (on ? t : 0)].i, kl = i / tw, j = tile.j0 + i - kl * tw, kp = tile.k0 + kl, k = NL * kp + l;
+            const int i = pairs[n0 + (on ? t : 0)].i & kResPairMask, kl = i / tw, j = tile.j0 + i - kl * tw, kp = tile.k0 + kl, k = NL * kp + l;
             int ql = x, sp = kp * nr + j, how = 0;  // (a lane without a node keeps to itself)
             if (k < G.nz) res_where<NL>(G, q, j, k, ql, sp, how);
             const int here = tile.index(sp % nr, sp / nr);
@@ -722,7 +795,7 @@ __device__ __forceinline__ void res_slab_cta(const ResDom<R, R>& D, Clock* clock
         for (int jl = tid; jl < tw; jl += T) columns[jl].set(step_inv_radius<R>(G, tile.j0 + jl), C);
     for (int m = tid; m < PL * n; m += T) {  // the state, natural layout
         const int ql = m / n, i = m - ql * n, kl = i / tw, j = tile.j0 + i - kl * tw, k = NL * (tile.k0 + kl) + ql % NL;
-        S.st[ql * chunk + i] = k < G.nz ? *slot(D.pop, G, ql / NL, j, k) : R(0);
+        S.st[ql * chunk + i] = k < G.nz ? Codec<S_>::load(slot(D.pop, G, ql / NL, j, k)) : R(0);
     }
     __syncthreads();
     // links read from the table where they are used
@@ -738,11 +811,12 @@ __device__ __forceinline__ void res_slab_cta(const ResDom<R, R>& D, Clock* clock
             return fmaR(v, of(B + q), of(B + 4 + q)) + of(B + 8 + q);
         }
     };
-    res_slab_run<R, SW, TH>(D, S, clock, nsteps, epoch, t0, min(ghosts, max_ghost), &bad, [&](auto par_tag, R az) {
+    res_slab_run<S_, R, SW, TH>(D, S, clock, nsteps, epoch, t0, min(ghosts, max_ghost), &bad, [&](auto par_tag, R az) {
         constexpr int PAR = decltype(par_tag)::value;
         for (int m = tid; m < n; m += T) {
             const ResPair<R> r = pairs[m];
-            R* const mine = S.st + r.i;
+            const int i = std::is_same<S_, R>::value ? r.i : r.i & kResPairMask;
+            R* const mine = S.st + i;
             // index (from `mine`) of the slot of population q, lane l, in an odd step without a table row
             auto inside = [&](int q, int l) {
                 const int er = q < 9 ? cr9(q) : cr4((q - 9) & 3), ez = q < 9 ? cz9(q) : cz4((q - 9) & 3);
@@ -762,10 +836,13 @@ __device__ __forceinline__ void res_slab_cta(const ResDom<R, R>& D, Clock* clock
             else if (r.tab < 0) res_load<RC, SW, TH, 1>(c, [&](int q, int l) { return mine[inside(q, l)]; }, none);
             else res_load<RC, SW, TH, 1>(c, [&](int q, int l) { return S.st[e[(q * NL + l) * max_tab]]; }, tl);
             if constexpr (sizeof(R) == 8) c.collide_d1(columns[r.col], C, az);
-            else c.collide(r.inv_r, C, az);
-            if (PAR == 0) res_store<RC, SW, TH, 0>(c, [&](int q, int l, R v) { mine[(q * NL + l) * chunk] = v; }, none);
-            else if (r.tab < 0) res_store<RC, SW, TH, 1>(c, [&](int q, int l, R v) { mine[inside(q, l)] = v; }, none);
-            else res_store<RC, SW, TH, 1>(c, [&](int q, int l, R v) { S.st[e[(q * NL + l) * max_tab]] = v; }, tl);
+            else if (PAR == 0) c.collide(r.inv_r, C, az);
+            else
+                res_collide<S_>(c, r.inv_r, C, az, (unsigned)r.i >> kResRingShift, D.C,
+                                [&]() { return inv_radius<R>(G, tile.j0 + i % tw); });
+            if (PAR == 0) res_store<S_, RC, SW, TH, 0>(c, [&](int q, int l, R v) { mine[(q * NL + l) * chunk] = v; }, none);
+            else if (r.tab < 0) res_store<S_, RC, SW, TH, 1>(c, [&](int q, int l, R v) { mine[inside(q, l)] = v; }, none);
+            else res_store<S_, RC, SW, TH, 1>(c, [&](int q, int l, R v) { S.st[e[(q * NL + l) * max_tab]] = v; }, tl);
         }
     });
 }
@@ -773,14 +850,14 @@ __device__ __forceinline__ void res_slab_cta(const ResDom<R, R>& D, Clock* clock
 // Cooperative grid, one CTA per SM, several pairs per thread.
 //
 // What bounds it: instruction issue (FP32) or the FP64 pipe.
-template <class R, bool SW, bool TH>
+template <class S, class R, bool SW, bool TH>
 __global__ void __launch_bounds__(kResSlabThreads, 1)
-k_resident_slab(const ResDom<R, R>* __restrict__ doms, const int* __restrict__ cta_dom, Clock* clock, int nsteps,
+k_resident_slab(const ResDom<S, R>* __restrict__ doms, const int* __restrict__ cta_dom, Clock* clock, int nsteps,
                 unsigned epoch, long long t0) {
     extern __shared__ __align__(16) unsigned char res_smem[];
-    const ResDom<R, R>& D = doms[cta_dom[blockIdx.x]];
-    if (TH && D.th) res_slab_cta<R, SW, TH>(D, clock, nsteps, epoch, t0, res_smem);
-    else res_slab_cta<R, SW, false>(D, clock, nsteps, epoch, t0, res_smem);
+    const ResDom<S, R>& D = doms[cta_dom[blockIdx.x]];
+    if (TH && D.th) res_slab_cta<S, R, SW, TH>(D, clock, nsteps, epoch, t0, res_smem);
+    else res_slab_cta<S, R, SW, false>(D, clock, nsteps, epoch, t0, res_smem);
 }
 
 // ---------------------------------------------------------------------------- grid, state in L2

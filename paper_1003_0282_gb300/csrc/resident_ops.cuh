@@ -83,7 +83,7 @@ int res_lanes() { return std::is_same<R, float>::value ? 2 : 1; }
 
 template <class S, bool SW, bool TH>
 cudaError_t res_build(Resident* r, const ResidentDomain* d, int n, int num_sms, cudaStream_t stream) {
-    using R = S;
+    using R = typename std::conditional<std::is_same<S, double>::value, double, float>::type;
     const int nl = res_lanes<R>();
     size_t state = 0;
     long long pairs = 0;
@@ -134,8 +134,8 @@ cudaError_t res_build(Resident* r, const ResidentDomain* d, int n, int num_sms, 
         r->cluster = true;
         r->grid = c;
         r->threads = res_up32(chunk);
-        r->smem = kResAz * sizeof(R) + (size_t)nplanes<SW, TH>() * nl * chunk * sizeof(S);
-        auto kern = k_resident_cluster<R, SW, TH>;
+        r->smem = kResAz * sizeof(R) + (size_t)nplanes<SW, TH>() * nl * chunk * sizeof(R);
+        auto kern = k_resident_cluster<S, R, SW, TH>;
         // the attribute belongs to the kernel, not to this handle: always the largest a handle can ask for
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kResSmemMax);
         if (e != cudaSuccess) return e;
@@ -209,8 +209,8 @@ cudaError_t res_build(Resident* r, const ResidentDomain* d, int n, int num_sms, 
             r->smem = smem;
             const int iters = (chunk + kResSlabThreads - 1) / kResSlabThreads;
             r->threads = one ? kResThreads : std::max(kResThreads, res_up32((chunk + iters - 1) / iters));
-            const auto k1 = k_resident_one<R, SW, TH>;
-            const auto k2 = k_resident_slab<R, SW, TH>;
+            const auto k1 = k_resident_one<S, R, SW, TH>;
+            const auto k2 = k_resident_slab<S, R, SW, TH>;
             r->kernel = one ? reinterpret_cast<const void*>(k1) : reinterpret_cast<const void*>(k2);
             e = cudaFuncSetAttribute(r->kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kResSmemMax);
             if (e != cudaSuccess) return e;
@@ -221,28 +221,34 @@ cudaError_t res_build(Resident* r, const ResidentDomain* d, int n, int num_sms, 
             r->slab = true;
             break;
         }
-        auto kern = k_resident_grid<S, R, SW, TH>;
-        for (int per_sm = 2; per_sm >= 1 && !fits; --per_sm) {
-            const int most = per_sm * num_sms;
-            if (n > most) return cudaSuccess;
-            const int chunk = chunk_for(most);
-            place(chunk);
-            int ring = 0;
-            for (const ResDom<S, R>& y : doms)
-                for (int c = 0; c < y.ncta; ++c)
-                    ring = std::max(ring, res_ring_pairs(c * chunk, std::min((c + 1) * chunk, y.npairs), y.G.nr, y.G.nz, nl));
-            const int iters = (chunk + kResThreads - 1) / kResThreads;
-            r->slab = false;
-            r->kernel = reinterpret_cast<const void*>(kern);
-            r->threads = res_up32((chunk + iters - 1) / iters);
-            r->smem = res_grid_smem<R, SW, TH>(chunk, ring);
-            if (r->smem > (size_t)(per_sm == 2 ? kResSmemMax / 2 : kResSmemMax)) continue;
-            e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kResSmemMax);
-            if (e != cudaSuccess) return e;
-            int got = 0;
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&got, kern, r->threads, r->smem);
-            if (e != cudaSuccess) return e;
-            fits = (long long)got * num_sms >= r->grid;
+        // The state in L2.  Not with 16-bit storage: shared memory takes domains up
+        // to where a step kernel already has 300 k pairs to work on, and the step
+        // is then issue-bound in either form (512 x 768 x 100 steps, in shared
+        // memory: 1.39 -> 0.72 ms; 96 x 144 x 300: 2.58 -> 0.55 ms).
+        if constexpr (std::is_same<S, R>::value) {
+            auto kern = k_resident_grid<S, R, SW, TH>;
+            for (int per_sm = 2; per_sm >= 1 && !fits; --per_sm) {
+                const int most = per_sm * num_sms;
+                if (n > most) return cudaSuccess;
+                const int chunk = chunk_for(most);
+                place(chunk);
+                int ring = 0;
+                for (const ResDom<S, R>& y : doms)
+                    for (int c = 0; c < y.ncta; ++c)
+                        ring = std::max(ring, res_ring_pairs(c * chunk, std::min((c + 1) * chunk, y.npairs), y.G.nr, y.G.nz, nl));
+                const int iters = (chunk + kResThreads - 1) / kResThreads;
+                r->slab = false;
+                r->kernel = reinterpret_cast<const void*>(kern);
+                r->threads = res_up32((chunk + iters - 1) / iters);
+                r->smem = res_grid_smem<R, SW, TH>(chunk, ring);
+                if (r->smem > (size_t)(per_sm == 2 ? kResSmemMax / 2 : kResSmemMax)) continue;
+                e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kResSmemMax);
+                if (e != cudaSuccess) return e;
+                int got = 0;
+                e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&got, kern, r->threads, r->smem);
+                if (e != cudaSuccess) return e;
+                fits = (long long)got * num_sms >= r->grid;
+            }
         }
         if (!fits) return cudaSuccess;
     }

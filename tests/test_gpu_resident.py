@@ -140,3 +140,33 @@ def test_captured_calls_replay(B, kind):
     for x, y in zip(*got):
         for u, v in zip(x, y):
             assert (u is None and v is None) or np.array_equal(u, v)
+
+
+@pytest.mark.parametrize("shape", [(1, 1), (2, 5), (64, 4), (9, 255), (40, 60), (65, 64), (4099, 3), (199, 391)])
+@pytest.mark.parametrize("mix", ["pipe", "crystal", "annulus-mixed"])
+@pytest.mark.parametrize("swirl,temp,collision", [(True, True, "bgk"), (False, False, "bgk"), (True, False, "mrt"), (False, True, "mrt")])
+@pytest.mark.parametrize("precision", ["fp16", "bf16"])
+def test_16_bit_storage(B, shape, mix, swirl, temp, collision, precision):
+    """The outer ring keeps the ring kernels' own arithmetic; every store rounds to the storage type."""
+    both_ways(B, problem(*shape, mix, swirl=swirl, temperature=temp, collision=collision), precision, [11, 52])
+
+
+def test_small_fp16_batch(B):
+    probs = [problem(17, 29, "crystal"), problem(143, 208, "pipe", temperature=False),
+             problem(50, 63, "annulus-mixed", collision="mrt", tau=0.55), problem(1, 1, "closed")]
+    out = []
+    for graphs in (True, False):
+        batch = B.Batch(probs, "fp16")
+        batch.use_graphs(graphs)
+        for d, pb in enumerate(probs):
+            st = seeded_state(pb, 40 + d)
+            batch.set_populations(d, st.f, st.g, st.h if pb.temperature else None)
+        batch.step(1)
+        batch.step(24)
+        out.append(([batch.get_populations(d) for d in range(len(probs))], batch.residuals()))
+        batch.close()
+    (p0, r0), (p1, r1) = out
+    assert np.array_equal(r0, r1)
+    for x, y in zip(p0, p1):
+        for u, v in zip(x, y):
+            assert (u is None and v is None) or np.array_equal(u, v)
