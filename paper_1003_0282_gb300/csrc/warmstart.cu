@@ -151,8 +151,8 @@ __global__ void __launch_bounds__(256) k_ws_head(const bf16* x, const bf16* wt, 
 // column and keeps its values interpolated along r at the two canvas rows
 // around it, which several domain rows share: FP64 instructions bound this
 // kernel (64.5 cycles a warp instruction and scheduler), and this takes about
-// 22 of them per node where sampling every node afresh took over a hundred
-// with its divisions.
+// 12 of them per node and 16 per new canvas row, where sampling every node
+// afresh took over a hundred with its divisions.
 constexpr int kFieldCols = 128, kFieldRows = 32;
 struct FieldDom {
     axlbm_ws_domain d;
@@ -160,7 +160,8 @@ struct FieldDom {
     int block0;     // first block
 };
 __global__ void __launch_bounds__(kFieldCols) k_ws_fields(const float* canvas, const FieldDom* doms, int n, float* fields) {
-    __shared__ double row_y[kFieldRows];
+    __shared__ double row_f[kFieldRows], row_g[kFieldRows];  // weights of a row's two canvas rows, and the first of them
+    __shared__ int row_y[kFieldRows];
     int lo = 0, hi = n - 1;  // the domain of this block
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
@@ -173,7 +174,10 @@ __global__ void __launch_bounds__(kFieldCols) k_ws_fields(const float* canvas, c
     const int j = (b - rb * cols) * kFieldCols + threadIdx.x, k0 = rb * kFieldRows, k1 = min(k0 + kFieldRows, D.nz);
     if (threadIdx.x < kFieldRows) {
         const double zn = (D.z_first + (k0 + (int)threadIdx.x) - D.z_bottom) / D.height;
-        row_y[threadIdx.x] = fmin(fmax(zn * kH - 0.5, 0.0), kH - 1.0);
+        const double yc = fmin(fmax(zn * kH - 0.5, 0.0), kH - 1.0);
+        row_y[threadIdx.x] = min(int(yc), kH - 2);
+        row_f[threadIdx.x] = yc - row_y[threadIdx.x];
+        row_g[threadIdx.x] = 1 - row_f[threadIdx.x];
     }
     __syncthreads();
     if (j >= D.nr) return;
@@ -192,9 +196,8 @@ __global__ void __launch_bounds__(kFieldCols) k_ws_fields(const float* canvas, c
     double h0[4], h1[4];
     int have = -2;  // h0, h1 are canvas rows have, have + 1
     for (int k = k0; k < k1; ++k) {
-        const double yc = row_y[k - k0];
-        const int y0 = min(int(yc), kH - 2);
-        const double fy = yc - y0, gy = 1 - fy;
+        const int y0 = row_y[k - k0];
+        const double fy = row_f[k - k0], gy = row_g[k - k0];
         if (y0 != have) {
 #pragma unroll
             for (int c = 0; c < 4; ++c) {

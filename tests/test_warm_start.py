@@ -293,3 +293,15 @@ def test_training_script_initial_weights():
         off += n
     x = np.random.default_rng(6).normal(size=1000)
     assert np.array_equal(T.bf16_bits(x), WS.float_to_bf16(x))
+
+
+@pytest.mark.gpu
+def test_canvases_do_not_depend_on_the_pass(Bgpu):
+    """One, a few and many canvases a pass take different tilings of the convolutions; a canvas comes out the same."""
+    net = Bgpu.WarmStart(random_weights(6))
+    feats = np.random.default_rng(7).uniform(-1.0, 1.0, (37, 6)).astype(np.float32)
+    alone = [net.predict(feats[i:i + 1]).cpu().numpy() for i in (0, 2, 36)]
+    for n in (3, 12, 37):
+        got = net.predict(feats[:n]).cpu().numpy()
+        assert np.array_equal(got[0], alone[0][0]) and np.array_equal(got[2], alone[1][0])
+    assert np.array_equal(got[36], alone[2][0])
