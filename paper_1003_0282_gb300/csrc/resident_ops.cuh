@@ -192,7 +192,14 @@ cudaError_t res_build(Resident* r, const ResidentDomain* d, int n, int num_sms, 
             for (ResDom<S, R>& y : doms) {
                 const bool h = TH && y.th;
                 y.max_tab = y.max_ghost = 1;
+                bool inner_seen = false;
                 for (int c = 0; c < y.ncta; ++c) {
+                    // whole tiles away from the domain's outline are alike: the first one stands for all
+                    const int nkp = (y.G.nz + nl - 1) / nl;
+                    const ResTile T(y, nkp, c);
+                    const bool inner = T.j0 > 0 && T.k0 > 0 && T.j0 + T.w < y.G.nr && T.k0 + T.h < nkp && T.w == y.w && T.h == y.h;
+                    if (inner && inner_seen) continue;
+                    inner_seen |= inner;
                     int t, g;
                     res_tile_tables<Lanes<typename PairArith<R>::type>::n>(y, c, SW, h, &t, &g);
                     y.max_tab = std::max(y.max_tab, t);
