@@ -12,14 +12,18 @@
 // step is enough.  The boundary rules are the addresses of those slots and
 // are worked out once per launch, from classify() as the ring kernels use it.
 //
-// Two forms, chosen by resident_plan():
+// Three forms, chosen by res_build():
 //   k_resident_cluster  one thread-block cluster (up to 8 CTAs), one node
 //     pair per thread (FP64: one node), the state in shared memory for the
 //     whole launch; neighbours' slots are reached through distributed shared
 //     memory and a step ends with the cluster barrier.
-//   k_resident_grid     a cooperative grid over the whole chip, the state in
-//     global memory (L2); a CTA owns a contiguous range of node pairs of one
-//     domain and after every step waits only for the CTAs whose nodes its own
+//   k_resident_one, k_resident_slab  a cooperative grid, one CTA per SM, each
+//     with the state of a tile of one domain in shared memory (one pair, or
+//     several, per thread); populations that cross tiles travel through L2 as
+//     words of value and step that the reader polls with a bound.
+//   k_resident_grid     (FP32, FP64) a cooperative grid, the state in global
+//     memory (L2); a CTA owns a contiguous range of node pairs of one domain
+//     and after every step waits only for the CTAs whose nodes its own
 //     exchange populations with (a step counter per CTA, polled with a bound).
 //
 // Arithmetic and storage are those of the step kernels (PairArith, NodeArith,
