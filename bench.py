@@ -36,16 +36,15 @@ sys.path.insert(0, ROOT)
 
 # DRAM traffic of the bulk kernel from the ncu capture summarised in profiles/:
 # (dram__bytes_read.sum + dram__bytes_write.sum) / algorithmic bytes of the
-# captured launch, keyed by kernel and the SHA-256 prefix of the kernel source
-# at capture time.  Reported as null once the source has changed.
-NCU_TRAFFIC = {
-    # profiles/k_bulk_batch_fp32_sweep320_launches.md: one even and one odd launch (4 x 128 tiles)
-    "batch fp32": {"src_sha": "e40a9af016e25318", "dram_per_alg_byte": 0.9899},
-    # profiles/k_bulk_batch_fp16_sweep_half_full.md: full-size DRAM capture, one even (8 x 128) and one odd launch
-    "batch fp16": {"src_sha": "e40a9af016e25318", "dram_per_alg_byte": 0.9657},
-    # profiles/k_bulk_fp32_pipe4096x8192_launches.md: one even and one odd launch (4 x 128 tiles)
-    "pipe fp32": {"src_sha": "e40a9af016e25318", "dram_per_alg_byte": 1.0577},
-}
+# captured launches, keyed by kernel, with the SHA-256 prefix of the kernel
+# sources at capture time and the profile, which states the same prefix in a
+# line "DRAM capture: kernel sources `<prefix>`".  Once the sources have
+# changed an entry goes out (`roofline.traffic` is then null) until the
+# capture is taken again: the commands stand in
+#   batch fp32  profiles/k_bulk_batch_fp32_sweep320_launches.md
+#   batch fp16  profiles/k_bulk_batch_fp16_sweep_half_full.md (full-size DRAM capture)
+#   pipe fp32   profiles/k_bulk_fp32_pipe4096x8192_launches.md
+NCU_TRAFFIC = {}
 
 
 def parse():

@@ -97,3 +97,16 @@ def test_dram_traffic_entries_describe_the_current_kernels():
     for name in ("k_bulk_batch_fp32_sweep320_launches.md", "k_bulk_batch_fp16_sweep_half_full.md",
                  "k_bulk_fp32_pipe4096x8192_launches.md"):
         assert name in src and os.path.exists(os.path.join(ROOT, "profiles", name)), name
+
+
+def test_dram_traffic_entries_carry_the_hash_of_their_capture():
+    """A tag is the hash that the named profile states for its DRAM capture: moving a tag on to newer sources
+    without a new capture would report old traffic as that of the present kernels."""
+    sys.path.insert(0, ROOT)
+    try:
+        import bench
+    finally:
+        sys.path.remove(ROOT)
+    for key, entry in bench.NCU_TRAFFIC.items():
+        with open(os.path.join(ROOT, "profiles", entry["profile"])) as fh:
+            assert f"DRAM capture: kernel sources `{entry['src_sha']}`" in fh.read(), key
