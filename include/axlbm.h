@@ -343,7 +343,9 @@ AXLBM_API axlbm_status axlbm_load(axlbm_handle* h, const void* buf, size_t bytes
  * allocated, or the domain has wet walls, a Zou-He wall, a node on the axis or
  * cut faces, the step pairs are replayed.  A call made while the caller
  * captures the handle's stream launches such a domain's steps kernel by
- * kernel.  The results are the same bit for bit. */
+ * kernel; calls may follow replays of it (steps take the force's time level
+ * from the device; axlbm_time counts a captured call once, when it is made).
+ * The results are the same bit for bit. */
 AXLBM_API axlbm_status axlbm_use_graphs(axlbm_handle* h, int32_t enable);
 
 /* How many times the step graphs were captured and launched since creation

@@ -438,7 +438,7 @@ axlbm_status graph_pairs(axlbm_handle* h, const Ops* ops, int64_t pairs) {
         int64_t done;
         if (h->res.on) {
             done = pairs - p < axl::kResMaxSteps / 2 ? pairs - p : axl::kResMaxSteps / 2;
-            e = axl::resident_launch(&h->res, clk, (int)(2 * done), h->t + 2 * p, h->stream);
+            e = axl::resident_launch(&h->res, clk, (int)(2 * done), h->stream);
         } else {
             const bool many = pairs - p >= kGraphPairs;
             done = many ? kGraphPairs : 1;

@@ -439,7 +439,7 @@ axlbm_status batch_graph_pairs(axlbm_batch* b, const BatchOps* ops, int64_t pair
         }
         for (int64_t p = 0; p < pairs;) {
             const int64_t done = std::min(pairs - p, axl::kResMaxSteps / 2);
-            e = axl::resident_launch(&b->res, clk, (int)(2 * done), b->t + 2 * p, b->stream);
+            e = axl::resident_launch(&b->res, clk, (int)(2 * done), b->stream);
             if (e != cudaSuccess) return bcuda(b, e, "graph launch");
             p += done;
             b->graph_launches += 1;

@@ -93,8 +93,8 @@ struct Resident {
     int grid = 0, threads = 0;
     size_t smem = 0;
     const void* kernel = nullptr;
-    void* scratch = nullptr;  // descriptors, CTA map, step counters or words between CTAs
-    size_t off_map = 0, off_flags = 0;
+    void* scratch = nullptr;  // descriptors, CTA map, step counters or words between CTAs, count of CTAs with their time level
+    size_t off_map = 0, off_flags = 0, off_taken = 0;
     unsigned epoch = 0;       // steps launched so far: the step counters' base
     cudaGraph_t graph = nullptr;
     cudaGraphNode_t node = nullptr;
@@ -122,12 +122,12 @@ extern const ResidentOps resident_bf16;
 
 constexpr int64_t kResMaxSteps = 1 << 16;  // steps of one launch, at most (even)
 
-// Whether a call on `stream` takes the multi-step launches.  A launch carries its time level and the base of its step
-// counters, so one that a caller captures could not be replayed: under capture the step kernels, which take both from
-// the device, run one by one.
+// Whether a call on `stream` takes the multi-step launches.  A launch carries the base of its step counters, so one that
+// a caller captures could not be replayed: under capture the step kernels run one by one.  The time level comes from the
+// device in either form, so calls before, between and after replays agree on it.
 bool resident_usable(const Resident& r, cudaStream_t stream);
 cudaError_t resident_capture(Resident* r, Clock* clock, cudaStream_t cap);
-cudaError_t resident_launch(Resident* r, Clock* clock, int steps, long long t0, cudaStream_t stream);
+cudaError_t resident_launch(Resident* r, Clock* clock, int steps, cudaStream_t stream);
 void resident_drop_graph(Resident* r);
 void resident_free(Resident* r);
 

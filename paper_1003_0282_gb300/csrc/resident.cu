@@ -5,7 +5,7 @@ namespace axl {
 
 namespace {
 
-// The kernels' arguments for `steps` steps from level t0 (storage must outlive the use of `args`).
+// The kernels' arguments for `steps` steps (storage must outlive the use of `args`).
 struct ResArgs {
     const void* doms;
     const int* map;
@@ -13,9 +13,9 @@ struct ResArgs {
     Clock* clock;
     int steps;
     unsigned epoch;
-    long long t0;
+    unsigned* taken;
     void* args[7];
-    ResArgs(const Resident& r, Clock* clk, int steps_, long long t0_) {
+    ResArgs(const Resident& r, Clock* clk, int steps_) {
         char* m = static_cast<char*>(r.scratch);
         doms = m;
         map = reinterpret_cast<const int*>(m + r.off_map);
@@ -23,15 +23,17 @@ struct ResArgs {
         clock = clk;
         steps = steps_;
         epoch = r.epoch;
-        t0 = t0_;
+        taken = reinterpret_cast<unsigned*>(m + r.off_taken);
         int n = 0;
         args[n++] = &doms;
         if (!r.cluster) args[n++] = &map;
         if (!r.cluster && !r.slab) args[n++] = &flags;
         args[n++] = &clock;
         args[n++] = &steps;
-        if (!r.cluster) args[n++] = &epoch;
-        args[n++] = &t0;
+        if (!r.cluster) {
+            args[n++] = &epoch;
+            args[n++] = &taken;
+        }
     }
 };
 
@@ -48,7 +50,7 @@ bool resident_usable(const Resident& r, cudaStream_t stream) {
 }
 
 cudaError_t resident_capture(Resident* r, Clock* clock, cudaStream_t cap) {
-    ResArgs a(*r, clock, 2, 0);
+    ResArgs a(*r, clock, 2);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(r->grid);
     cfg.blockDim = dim3(r->threads);
@@ -78,8 +80,8 @@ cudaError_t resident_capture(Resident* r, Clock* clock, cudaStream_t cap) {
     return e;
 }
 
-cudaError_t resident_launch(Resident* r, Clock* clock, int steps, long long t0, cudaStream_t stream) {
-    ResArgs a(*r, clock, steps, t0);
+cudaError_t resident_launch(Resident* r, Clock* clock, int steps, cudaStream_t stream) {
+    ResArgs a(*r, clock, steps);
     cudaKernelNodeParams p = {};
     p.func = const_cast<void*>(r->kernel);
     p.gridDim = dim3(r->grid);

@@ -134,8 +134,22 @@ __device__ __forceinline__ R res_az(double az0, double omega_t, long long t) {
     return R(force_at(az0, omega_t, t));
 }
 
-// The force and the time level after the last step of a launch (an even
-// level; the odd entry holds the last step's force, as after single steps).
+// The time level a launch starts from.  The device clock alone knows it (a
+// replay of steps that the caller captured moves it on without the host).
+// A thread loads it when the kernel starts, so that its set-up hides the load.
+__device__ __forceinline__ long long res_start(const Clock* clock) {
+    return *reinterpret_cast<const volatile long long*>(&clock->t);
+}
+
+// A CTA of a grid has its time level t0 (one thread, behind the barrier that
+// shared it).  The last CTA to say so moves the clock on: nobody is left to
+// read it.  `taken` wraps to zero.
+__device__ __forceinline__ void res_taken(Clock* clock, unsigned* taken, long long t0, int nsteps) {
+    if (atomicInc(taken, gridDim.x - 1) == gridDim.x - 1) clock->t = t0 + nsteps;
+}
+
+// The force after the last step of a launch, at level t1 (an even level; the
+// odd entry holds the last step's force, as after single steps).
 template <class S, class R>
 __device__ __forceinline__ void res_finish(const ResDom<S, R>& D, long long t1) {
     const double a0 = force_at(D.az0, D.omega_t, t1), a1 = force_at(D.az0, D.omega_t, t1 - 1);
@@ -324,7 +338,7 @@ __device__ __forceinline__ void res_dld(uint32_t a, double& v) {
 // whatever its active lanes).
 template <class S, class R, bool SW, bool TH>
 __global__ void __launch_bounds__(kResThreads, 1)
-k_resident_cluster(const ResDom<S, R>* __restrict__ doms, Clock* clock, int nsteps, long long t0) {
+k_resident_cluster(const ResDom<S, R>* __restrict__ doms, Clock* clock, int nsteps) {
     using RC = typename PairArith<R>::type;
     constexpr int NL = Lanes<RC>::n, P = nplanes<SW, TH>();
     extern __shared__ __align__(16) unsigned char res_smem[];
@@ -336,6 +350,7 @@ k_resident_cluster(const ResDom<S, R>* __restrict__ doms, Clock* clock, int nste
         if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&clock->err, 1u);
         return;
     }
+    const long long t0 = res_start(clock);
     R* az_tab = reinterpret_cast<R*>(res_smem);
     R* st = az_tab + kResAz;
     const int tid = threadIdx.x, chunk = D.chunk, ncta = D.ncta, rank = blockIdx.x;
@@ -401,7 +416,7 @@ k_resident_cluster(const ResDom<S, R>* __restrict__ doms, Clock* clock, int nste
             for (int q = 0; q < P; ++q) Codec<S>::store(slot(D.pop, G, q, j, k0 + l), mine[(q * NL + l) * chunk]);
         }
     }
-    if (rank == 0 && tid == 0) {
+    if (rank == 0 && tid == 0) {  // (every CTA took its time level before the first meeting)
         res_finish(D, t0 + nsteps);
         clock->t = t0 + nsteps;
     }
@@ -554,7 +569,8 @@ __device__ __forceinline__ int res_new_ghost(bool remote, int* count) {
 // neighbours coming in and going out, and writes it back.
 template <class S_, class R, bool SW, bool TH, class Update>
 __device__ __forceinline__ void res_slab_run(const ResDom<S_, R>& D, const ResSlab<R>& S, Clock* clock, int nsteps,
-                                             unsigned epoch, long long t0, int ng, int* bad, const Update& update) {
+                                             unsigned epoch, unsigned* taken, long long t_start, int ng, int* bad,
+                                             const Update& update) {
     constexpr int NL = Lanes<typename PairArith<R>::type>::n, PL = nplanes<SW, TH>() * NL;
     const Geom& G = D.G;
     const int tid = threadIdx.x, T = blockDim.x, chunk = D.chunk;
@@ -571,7 +587,10 @@ __device__ __forceinline__ void res_slab_run(const ResDom<S_, R>& D, const ResSl
         __syncthreads();
         if (ng > 0) res_scatter<R, PAR>(S, mail, gbase, ng, epoch + (unsigned)s + 1u);
     };
+    __shared__ long long t0;
+    if (tid == 0) t0 = t_start;
     int stop = __syncthreads_or(*bad);
+    if (tid == 0) res_taken(clock, taken, t_start, nsteps);
     for (int s = 0; s < nsteps && !stop; s += 2) {
         if (s % kResAz == 0) {
             for (int i = tid; i < kResAz && s + i < nsteps; i += T) S.az[i] = res_az<R>(D.az0, D.omega_t, t0 + s + i);
@@ -593,16 +612,16 @@ __device__ __forceinline__ void res_slab_run(const ResDom<S_, R>& D, const ResSl
         if (k < G.nz) Codec<S_>::store(slot(D.pop, G, ql / NL, j, k), S.st[ql * chunk + i]);
     }
     if (rank == 0 && tid == 0) res_finish(D, t0 + nsteps);
-    if (blockIdx.x == 0 && tid == 0) clock->t = t0 + nsteps;
 }
 
 // One pair per thread: addresses and links stay in registers.
 template <class S_, class R, bool SW, bool TH>
-__device__ __forceinline__ void res_one_cta(const ResDom<S_, R>& D, Clock* clock, int nsteps, unsigned epoch, long long t0,
+__device__ __forceinline__ void res_one_cta(const ResDom<S_, R>& D, Clock* clock, int nsteps, unsigned epoch, unsigned* taken,
                                             unsigned char* smem) {
     using RC = typename PairArith<R>::type;
     constexpr int NL = Lanes<RC>::n, P = nplanes<SW, TH>();
     __shared__ int ghosts, bad;
+    const long long t_start = res_start(clock);
     const Geom& G = D.G;
     const Coef<R> C = D.C;
     const int tid = threadIdx.x, chunk = D.chunk, nr = G.nr, nkp = (G.nz + NL - 1) / NL;
@@ -636,7 +655,7 @@ __device__ __forceinline__ void res_one_cta(const ResDom<S_, R>& D, Clock* clock
     __syncthreads();
     const R inv_r = step_inv_radius<R>(G, j);
     const unsigned ring = res_ring<S_, R>(G, j, k0);
-    res_slab_run<S_, R, SW, TH>(D, S, clock, nsteps, epoch, t0, min(ghosts, max_ghost), &bad, [&](auto par_tag, R az) {
+    res_slab_run<S_, R, SW, TH>(D, S, clock, nsteps, epoch, taken, t_start, min(ghosts, max_ghost), &bad, [&](auto par_tag, R az) {
         constexpr int PAR = decltype(par_tag)::value;
         if (!on) return;
         Cell<RC, SW, TH> c;
@@ -660,11 +679,11 @@ __device__ __forceinline__ void res_one_cta(const ResDom<S_, R>& D, Clock* clock
 template <class S, class R, bool SW, bool TH>
 __global__ void __launch_bounds__(kResThreads, 1)
 k_resident_one(const ResDom<S, R>* __restrict__ doms, const int* __restrict__ cta_dom, Clock* clock, int nsteps,
-               unsigned epoch, long long t0) {
+               unsigned epoch, unsigned* taken) {
     extern __shared__ __align__(16) unsigned char res_smem[];
     const ResDom<S, R>& D = doms[cta_dom[blockIdx.x]];
-    if (TH && D.th) res_one_cta<S, R, SW, TH>(D, clock, nsteps, epoch, t0, res_smem);
-    else res_one_cta<S, R, SW, false>(D, clock, nsteps, epoch, t0, res_smem);
+    if (TH && D.th) res_one_cta<S, R, SW, TH>(D, clock, nsteps, epoch, taken, res_smem);
+    else res_one_cta<S, R, SW, false>(D, clock, nsteps, epoch, taken, res_smem);
 }
 
 constexpr int kResSlabThreads = 384;
@@ -706,11 +725,12 @@ __host__ __device__ constexpr size_t res_column_bytes(int w) {
 
 // Several pairs per thread.
 template <class S_, class R, bool SW, bool TH>
-__device__ __forceinline__ void res_slab_cta(const ResDom<S_, R>& D, Clock* clock, int nsteps, unsigned epoch, long long t0,
+__device__ __forceinline__ void res_slab_cta(const ResDom<S_, R>& D, Clock* clock, int nsteps, unsigned epoch, unsigned* taken,
                                              unsigned char* smem) {
     using RC = typename PairArith<R>::type;
     constexpr int NL = Lanes<RC>::n, P = nplanes<SW, TH>(), PL = P * NL, NF = (SW ? 8 : 0) + (TH ? 12 : 0);
     __shared__ int ghosts, bad, rows;
+    const long long t_start = res_start(clock);
     const Geom& G = D.G;
     const Coef<R> C = D.C;
     const int tid = threadIdx.x, T = blockDim.x, chunk = D.chunk, nr = G.nr, nkp = (G.nz + NL - 1) / NL;
@@ -815,7 +835,7 @@ __device__ __forceinline__ void res_slab_cta(const ResDom<S_, R>& D, Clock* cloc
             return fmaR(v, of(B + q), of(B + 4 + q)) + of(B + 8 + q);
         }
     };
-    res_slab_run<S_, R, SW, TH>(D, S, clock, nsteps, epoch, t0, min(ghosts, max_ghost), &bad, [&](auto par_tag, R az) {
+    res_slab_run<S_, R, SW, TH>(D, S, clock, nsteps, epoch, taken, t_start, min(ghosts, max_ghost), &bad, [&](auto par_tag, R az) {
         constexpr int PAR = decltype(par_tag)::value;
         for (int m = tid; m < n; m += T) {
             const ResPair<R> r = pairs[m];
@@ -857,11 +877,11 @@ __device__ __forceinline__ void res_slab_cta(const ResDom<S_, R>& D, Clock* cloc
 template <class S, class R, bool SW, bool TH>
 __global__ void __launch_bounds__(kResSlabThreads, 1)
 k_resident_slab(const ResDom<S, R>* __restrict__ doms, const int* __restrict__ cta_dom, Clock* clock, int nsteps,
-                unsigned epoch, long long t0) {
+                unsigned epoch, unsigned* taken) {
     extern __shared__ __align__(16) unsigned char res_smem[];
     const ResDom<S, R>& D = doms[cta_dom[blockIdx.x]];
-    if (TH && D.th) res_slab_cta<S, R, SW, TH>(D, clock, nsteps, epoch, t0, res_smem);
-    else res_slab_cta<S, R, SW, false>(D, clock, nsteps, epoch, t0, res_smem);
+    if (TH && D.th) res_slab_cta<S, R, SW, TH>(D, clock, nsteps, epoch, taken, res_smem);
+    else res_slab_cta<S, R, SW, false>(D, clock, nsteps, epoch, taken, res_smem);
 }
 
 // ---------------------------------------------------------------------------- grid, state in L2
@@ -988,10 +1008,12 @@ __device__ __forceinline__ void res_grid_step(const ResDom<S, R>& D, const Coef<
 // The work of one CTA: a contiguous range of pairs of domain D.
 template <class S, class R, bool SW, bool TH>
 __device__ __forceinline__ void res_grid_cta(const ResDom<S, R>& D, unsigned* flags, Clock* clock, int nsteps,
-                                             unsigned epoch, long long t0, unsigned char* smem) {
+                                             unsigned epoch, unsigned* taken, unsigned char* smem) {
     using RC = typename PairArith<R>::type;
     constexpr int NL = Lanes<RC>::n, P = nplanes<SW, TH>();
     __shared__ int n_ring, abort_flag;
+    __shared__ long long t0;
+    const long long t_start = res_start(clock);
     const Geom& G = D.G;
     const Coef<R> C = D.C;
     const int tid = threadIdx.x, chunk = D.chunk, nr = G.nr;
@@ -1010,7 +1032,9 @@ __device__ __forceinline__ void res_grid_cta(const ResDom<S, R>& D, unsigned* fl
         r.ring = j == 0 || j == nr - 1 || k == 0 || k + (two ? 1 : 0) == G.nz - 1 ? atomicAdd(&n_ring, 1) : -1;
         rec[i] = r;
     }
+    if (tid == 0) t0 = t_start;
     __syncthreads();
+    if (tid == 0) res_taken(clock, taken, t_start, nsteps);
     // outline table: the slots, and rho0 u_w / 2 where a g population meets a wall
     R* ring_cg = reinterpret_cast<R*>(rec + chunk);
     int* ring_at = reinterpret_cast<int*>(ring_cg + (SW ? n_ring * 4 * NL : 0));
@@ -1081,7 +1105,6 @@ __device__ __forceinline__ void res_grid_cta(const ResDom<S, R>& D, unsigned* fl
         return;
     }
     if (rank == 0 && tid == 0) res_finish(D, t0 + nsteps);
-    if (blockIdx.x == 0 && tid == 0) clock->t = t0 + nsteps;
 }
 
 // Cooperative grid; CTA b works for domain cta_dom[b].
@@ -1092,11 +1115,11 @@ __device__ __forceinline__ void res_grid_cta(const ResDom<S, R>& D, unsigned* fl
 template <class S, class R, bool SW, bool TH>
 __global__ void __launch_bounds__(kResThreads, 2)
 k_resident_grid(const ResDom<S, R>* __restrict__ doms, const int* __restrict__ cta_dom, unsigned* flags, Clock* clock,
-                int nsteps, unsigned epoch, long long t0) {
+                int nsteps, unsigned epoch, unsigned* taken) {
     extern __shared__ __align__(16) unsigned char res_smem[];
     const ResDom<S, R>& D = doms[cta_dom[blockIdx.x]];
-    if (TH && D.th) res_grid_cta<S, R, SW, true>(D, flags, clock, nsteps, epoch, t0, res_smem);
-    else res_grid_cta<S, R, SW, false>(D, flags, clock, nsteps, epoch, t0, res_smem);
+    if (TH && D.th) res_grid_cta<S, R, SW, true>(D, flags, clock, nsteps, epoch, taken, res_smem);
+    else res_grid_cta<S, R, SW, false>(D, flags, clock, nsteps, epoch, taken, res_smem);
 }
 
 }  // namespace axl

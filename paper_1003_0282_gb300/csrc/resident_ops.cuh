@@ -259,7 +259,7 @@ cudaError_t res_build(Resident* r, const ResidentDomain* d, int n, int num_sms, 
         }
         if (!fits) return cudaSuccess;
     }
-    // descriptors, CTA map, step counters: one allocation of the library's own
+    // descriptors, CTA map, step counters or words, count of CTAs with their time level: one allocation of the library's own
     const size_t b_doms = (n * sizeof(ResDom<S, R>) + 255) / 256 * 256;
     const size_t b_map = (cta_dom.size() * sizeof(int) + 255) / 256 * 256;
     auto words = [&](const ResDom<S, R>& y) {  // (whole 128-byte lines per domain)
@@ -271,13 +271,16 @@ cudaError_t res_build(Resident* r, const ResidentDomain* d, int n, int num_sms, 
         b_flags = 0;
         for (const ResDom<S, R>& y : doms) b_flags += words(y);
     }
-    if (cudaMalloc(&r->scratch, b_doms + b_map + b_flags) != cudaSuccess) {
+    b_flags = (b_flags + 127) / 128 * 128;
+    const size_t b_taken = 128;
+    if (cudaMalloc(&r->scratch, b_doms + b_map + b_flags + b_taken) != cudaSuccess) {
         cudaGetLastError();
         r->scratch = nullptr;
         return cudaSuccess;  // no room for it: the step kernels run
     }
     r->off_map = b_doms;
     r->off_flags = b_doms + b_map;
+    r->off_taken = r->off_flags + b_flags;
     char* m = static_cast<char*>(r->scratch);
     if (r->slab) {
         size_t off = r->off_flags;
@@ -289,7 +292,7 @@ cudaError_t res_build(Resident* r, const ResidentDomain* d, int n, int num_sms, 
     e = cudaMemcpyAsync(m, doms.data(), n * sizeof(ResDom<S, R>), cudaMemcpyHostToDevice, stream);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(m + r->off_map, cta_dom.data(), cta_dom.size() * sizeof(int), cudaMemcpyHostToDevice, stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(m + r->off_flags, 0, b_flags, stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(m + r->off_flags, 0, b_flags + b_taken, stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);  // the lists live on this stack
     r->epoch = 0;
     r->on = e == cudaSuccess;

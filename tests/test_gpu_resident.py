@@ -170,3 +170,61 @@ def test_small_fp16_batch(B):
     for x, y in zip(p0, p1):
         for u, v in zip(x, y):
             assert (u is None and v is None) or np.array_equal(u, v)
+
+
+# a cluster, one pair per thread, several pairs per thread, the state in L2, a batch
+REPLAYED = {
+    "cluster": ("fp32", [(64, 48)], {}),
+    "one": ("fp32", [(128, 192)], {}),
+    "slab": ("fp64", [(199, 391)], {}),
+    "l2": ("fp32", [(701, 809)], {"temperature": False}),
+    "batch": ("fp32", [(33, 40), (90, 61)], {}),
+}
+
+
+@pytest.mark.parametrize("kind", sorted(REPLAYED))
+def test_direct_calls_around_replays(B, kind):
+    """Direct calls before, between and after replays of a captured call continue from the level that the replays
+    reached: with an oscillating force a call that took its level from elsewhere would have the wrong phase."""
+    import torch
+
+    precision, shapes, extra = REPLAYED[kind]
+    probs = [problem(*s, "crystal", **extra) for s in shapes]
+    assert all(pb.omega_t != 0 and pb.az0 != 0 for pb in probs)
+    states = [seeded_state(pb, 3 + d) for d, pb in enumerate(probs)]
+    got = []
+    for captured in (True, False):
+        stream = torch.cuda.Stream()
+        with torch.cuda.stream(stream):
+            if kind == "batch":
+                sim = B.Batch(probs, precision, stream=stream)
+                for d, (pb, st) in enumerate(zip(probs, states)):
+                    sim.set_populations(d, st.f, st.g, st.h)
+            else:
+                pb, st = probs[0], states[0]
+                sim = B.Domain(pb, precision, stream=stream)
+                sim.set_populations(st.f, st.g, st.h if pb.temperature else None, time=0)
+            if not captured:
+                sim.use_graphs(False)
+            sim.step(20)
+            stream.synchronize()
+            if captured:
+                graph = torch.cuda.CUDAGraph()
+                with torch.cuda.graph(graph, stream=stream, capture_error_mode="thread_local"):
+                    sim.step(20)
+                again = graph.replay
+            else:
+                again = lambda: sim.step(20)
+            again()
+            again()
+            sim.step(20)
+            again()
+            sim.step(40)
+            sim.step(20)
+            stream.synchronize()
+            got.append([sim.get_populations(d) for d in range(len(probs))] if kind == "batch"
+                       else [sim.get_populations()])
+            sim.close()
+    for x, y in zip(*got):
+        for u, v in zip(x, y):
+            assert (u is None and v is None) or np.array_equal(u, v)
