@@ -159,21 +159,27 @@ struct FieldDom {
     long long out;  // first value of the domain's fields
     int block0;     // first block
 };
-__global__ void __launch_bounds__(kFieldCols) k_ws_fields(const float* canvas, const FieldDom* doms, int n, float* fields) {
+// The domains of a launch are kernel arguments (22 of the 32 KB there may be): a call needs no memory for its list.
+constexpr int kFieldDoms = 256;
+struct FieldDoms {
+    FieldDom d[kFieldDoms];
+};
+__global__ void __launch_bounds__(kFieldCols)
+k_ws_fields(const float* canvas, const __grid_constant__ FieldDoms doms, int n, float* fields) {
     __shared__ double row_f[kFieldRows], row_g[kFieldRows];  // weights of a row's two canvas rows, and the first of them
     __shared__ int row_y[kFieldRows];
     int lo = 0, hi = n - 1;  // the domain of this block
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
-        if (doms[mid].block0 <= (int)blockIdx.x) lo = mid;
+        if (doms.d[mid].block0 <= (int)blockIdx.x) lo = mid;
         else hi = mid - 1;
     }
-    const FieldDom& F = doms[lo];
+    const FieldDom& F = doms.d[lo];
     const axlbm_ws_domain& D = F.d;
-    const int cols = (D.nr + kFieldCols - 1) / kFieldCols, b = blockIdx.x - F.block0, rb = b / cols;
-    const int j = (b - rb * cols) * kFieldCols + threadIdx.x, k0 = rb * kFieldRows, k1 = min(k0 + kFieldRows, D.nz);
+    const int cols = (D.nr - 1) / kFieldCols + 1, b = blockIdx.x - F.block0, rb = b / cols;
+    const int j = (b - rb * cols) * kFieldCols + threadIdx.x, k0 = rb * kFieldRows, k1 = k0 + min(kFieldRows, D.nz - k0);
     if (threadIdx.x < kFieldRows) {
-        const double zn = (D.z_first + (k0 + (int)threadIdx.x) - D.z_bottom) / D.height;
+        const double zn = (D.z_first + ((double)k0 + threadIdx.x) - D.z_bottom) / D.height;
         const double yc = fmin(fmax(zn * kH - 0.5, 0.0), kH - 1.0);
         row_y[threadIdx.x] = min(int(yc), kH - 2);
         row_f[threadIdx.x] = yc - row_y[threadIdx.x];
@@ -836,31 +842,27 @@ axlbm_status axlbm_ws_predict(axlbm_ws* w, const float* features, int32_t n, flo
 
 axlbm_status axlbm_ws_fields(axlbm_ws* w, const float* canvas, int32_t n, const axlbm_ws_domain* doms, float* fields) {
     if (!w || !canvas || !doms || !fields || n < 0) return wfail(w, AXLBM_EINVAL, "bad arguments");
-    long long off = 0, blocks = 0;
-    std::vector<FieldDom> list(n);
-    for (int d = 0; d < n; ++d) {
-        const axlbm_ws_domain& D = doms[d];
-        if (D.nr < 1 || D.nz < 1 || !(D.r_wall > 0.0) || !(D.height > 0.0))
+    for (int d = 0; d < n; ++d)
+        if (doms[d].nr < 1 || doms[d].nz < 1 || !(doms[d].r_wall > 0.0) || !(doms[d].height > 0.0))
             return wfail(w, AXLBM_EINVAL, "bad domain geometry");
-        list[d] = {D, off, (int)blocks};
-        off += 5 * (long long)D.nr * D.nz;
-        blocks += (long long)((D.nr + kFieldCols - 1) / kFieldCols) * ((D.nz + kFieldRows - 1) / kFieldRows);
-    }
-    if (blocks > 0x7fffffffll) return wfail(w, AXLBM_EINVAL, "too many nodes in one call");
-    if (n == 0) return AXLBM_OK;
-    FieldDom* dev = nullptr;
-    cudaError_t e = cudaMalloc(&dev, n * sizeof(FieldDom));
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        return wfail(w, AXLBM_ENOMEM, "domain list");
-    }
-    e = cudaMemcpyAsync(dev, list.data(), n * sizeof(FieldDom), cudaMemcpyHostToDevice, w->stream);
-    if (e == cudaSuccess) {
-        k_ws_fields<<<(unsigned)blocks, kFieldCols, 0, w->stream>>>(canvas, dev, n, fields);
+    cudaError_t e = cudaSuccess;
+    long long off = 0;
+    for (int d0 = 0, m; d0 < n && e == cudaSuccess; d0 += m) {
+        FieldDoms list;
+        long long blocks = 0;
+        for (m = 0; m < kFieldDoms && d0 + m < n; ++m) {
+            const axlbm_ws_domain& D = doms[d0 + m];
+            const long long more = ((D.nr - 1) / kFieldCols + 1ll) * ((D.nz - 1) / kFieldRows + 1);
+            if (m > 0 && blocks + more > 0x7fffffffll) break;  // (a domain of more blocks than a grid holds 1.4 TB of fields)
+            list.d[m] = {D, off, (int)blocks};
+            off += 5 * (long long)D.nr * D.nz;
+            blocks += more;
+        }
+        if (blocks > 0x7fffffffll) return wfail(w, AXLBM_EINVAL, "too many nodes in one domain");
+        k_ws_fields<<<(unsigned)blocks, kFieldCols, 0, w->stream>>>(canvas + (size_t)d0 * 4 * kH * kW, list, m, fields);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(w->stream);
-    cudaFree(dev);
     if (e != cudaSuccess) return wfail(w, AXLBM_ECUDA, "resampling");
     return AXLBM_OK;
 }

@@ -305,3 +305,63 @@ def test_canvases_do_not_depend_on_the_pass(Bgpu):
         got = net.predict(feats[:n]).cpu().numpy()
         assert np.array_equal(got[0], alone[0][0]) and np.array_equal(got[2], alone[1][0])
     assert np.array_equal(got[36], alone[2][0])
+
+
+@pytest.mark.gpu
+def test_fields_refuse_a_bad_domain_before_anything_else(Bgpu):
+    """The call looks at the domains before it makes room for a list of them, so a count far beyond memory is refused at
+    the first bad domain like any other."""
+    import torch
+    net = Bgpu.WarmStart(random_weights(6))
+    buf = torch.zeros(16, device="cuda")
+    bad = Bgpu.axlbm_ws_domain(nr=0, nz=4, r_wall=1.0, height=1.0)
+    for n in (1, 2 ** 31 - 1):
+        assert Bgpu.lib().axlbm_ws_fields(net.handle, buf.data_ptr(), n, bad, buf.data_ptr()) == Bgpu.EINVAL
+
+
+@pytest.mark.gpu
+def test_fields_of_many_domains(Bgpu):
+    """More domains than one launch takes, of uneven size: each comes out as it does alone."""
+    import torch
+    net = Bgpu.WarmStart(random_weights(6))
+    rng = np.random.default_rng(8)
+    probs = [I.rotating_lid_cavity(nr=int(rng.integers(8, 150)), aspect=float(rng.uniform(0.5, 2.0)), re=100.0)
+             for _ in range(517)]
+    canvas = torch.tensor(rng.normal(size=(517, 4, 256, 128)), dtype=torch.float32, device="cuda")
+    got, off = net.fields(canvas, probs).cpu().numpy(), 0
+    for d, pb in enumerate(probs):
+        size = 5 * pb.nr * pb.nz
+        if d in (0, 255, 256, 511, 512, 516):
+            assert np.array_equal(got[off:off + size], net.fields(canvas[d:d + 1], [pb]).cpu().numpy()), d
+        off += size
+    assert off == got.size
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("nr,nz", [(2 ** 31 - 1, 1), (1, 2 ** 31 - 1)])
+def test_fields_of_the_longest_domain(Bgpu, nr, nz):
+    """Rows and columns counted in 32 bits up to their end (43 GB of fields)."""
+    import torch
+    if torch.cuda.mem_get_info()[0] < 60e9:
+        pytest.skip("needs 43 GB of device memory")
+    net = Bgpu.WarmStart(random_weights(6))
+    canvas = torch.tensor(np.random.default_rng(9).normal(size=(1, 4, 256, 128)), dtype=torch.float32, device="cuda")
+    n = nr * nz
+    dom = Bgpu.axlbm_ws_domain(nr=nr, nz=nz, r_first=0.5, r_wall=float(nr), z_first=0.5, z_bottom=0.0, height=float(nz),
+                               rho0=1.0, u_scale=1.0, t_ref=0.0)
+    out = torch.full((5, n), float("nan"), device="cuda")
+    assert Bgpu.lib().axlbm_ws_fields(net.handle, canvas.data_ptr(), 1, dom, out.data_ptr()) == Bgpu.OK
+    cv = canvas[0].cpu().numpy().astype(np.float64)
+    for i in (0, n // 3, n - 33, n - 32, n - 1):
+        x = min(max((0.5 + i % nr) / nr * 128 - 0.5, 0.0), 127.0)
+        y = min(max((0.5 + i // nr) / nz * 256 - 0.5, 0.0), 255.0)
+        x0, y0 = min(int(x), 126), min(int(y), 254)
+        fx, fy = x - x0, y - y0
+        want = (1 - fy) * ((1 - fx) * cv[:, y0, x0] + fx * cv[:, y0, x0 + 1]) + \
+            fy * ((1 - fx) * cv[:, y0 + 1, x0] + fx * cv[:, y0 + 1, x0 + 1])
+        # one rounding to FP32 of a value formed in FP64
+        assert np.all(np.abs(out[1:, i].cpu().numpy() - want) <= 2.0 ** -23 * np.abs(want) + 1e-12), i
+        assert float(out[0, i]) == 1.0
+    assert bool(torch.isfinite(out[4, -64:]).all())
+    del out
+    torch.cuda.empty_cache()
