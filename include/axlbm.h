@@ -415,6 +415,10 @@ AXLBM_API axlbm_status axlbm_selftest_bounded_wait(int64_t max_cycles, int32_t* 
  * arrays or n out of range. */
 AXLBM_API axlbm_status axlbm_selftest_rcp(const float* x, int64_t n, float* out);
 
+/* The same for the FP64 reciprocal of the collision: out[i] for n host values
+ * x[i] (host arrays). */
+AXLBM_API axlbm_status axlbm_selftest_rcp64(const double* x, int64_t n, double* out);
+
 /* ------------------------------------------------------------------ batches
  * Many independent domains of uneven size advanced together: every step is
  * one persistent launch over a packed tile list of all domains (plus one

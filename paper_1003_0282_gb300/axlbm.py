@@ -133,6 +133,7 @@ def lib() -> ctypes.CDLL:
         L.axlbm_selftest_bounded_wait.argtypes = [ctypes.c_int64, ctypes.POINTER(ctypes.c_int32),
                                                   ctypes.POINTER(ctypes.c_uint32)]
         L.axlbm_selftest_rcp.argtypes = [ctypes.c_void_p, ctypes.c_int64, ctypes.c_void_p]
+        L.axlbm_selftest_rcp64.argtypes = [ctypes.c_void_p, ctypes.c_int64, ctypes.c_void_p]
         L.axlbm_batch_set_tile_shape.argtypes = [H, ctypes.c_int32, ctypes.c_int32]
         L.axlbm_batch_set_tile_shapes.argtypes = [H, ctypes.POINTER(ctypes.c_int32), ctypes.POINTER(ctypes.c_int32)]
         L.axlbm_batch_tile_shapes.argtypes = [H, ctypes.POINTER(ctypes.c_int32), ctypes.POINTER(ctypes.c_int32)]
@@ -187,7 +188,7 @@ def lib() -> ctypes.CDLL:
                      "axlbm_destroy", "axlbm_kernel_timing", "axlbm_kernel_times", "axlbm_check_static",
                      "axlbm_use_graphs", "axlbm_graph_stats", "axlbm_set_residual_lag",
                      "axlbm_halo_bytes", "axlbm_halo_send", "axlbm_halo_recv",
-                     "axlbm_selftest_bounded_wait", "axlbm_selftest_rcp"):
+                     "axlbm_selftest_bounded_wait", "axlbm_selftest_rcp", "axlbm_selftest_rcp64"):
             getattr(L, name).restype = ctypes.c_int
         _lib = L
     return _lib
@@ -606,6 +607,14 @@ def axlbm_selftest_rcp(x) -> tuple:
     out = np.empty(2 * x.size, dtype=np.float32)
     _check(lib().axlbm_selftest_rcp(x.ctypes.data, x.size, out.ctypes.data), None)
     return out[:x.size], out[x.size:]
+
+
+def axlbm_selftest_rcp64(x) -> np.ndarray:
+    """The collision's FP64 reciprocal of x on the device."""
+    x = np.ascontiguousarray(x, dtype=np.float64)
+    out = np.empty_like(x)
+    _check(lib().axlbm_selftest_rcp64(x.ctypes.data, x.size, out.ctypes.data), None)
+    return out
 
 
 def axlbm_selftest_bounded_wait(max_cycles: int):

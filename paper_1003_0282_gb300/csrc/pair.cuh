@@ -46,7 +46,8 @@ __device__ __forceinline__ double fmaR(double a, double b, double c) { return fm
 // multiply-adds leave the result within one ulp of 1/x (faithful rounding)
 // for the normal arguments the collision takes (densities near rho0, radii
 // of at least 1/2), without the branches of the correctly rounded call.  The
-// scalar and the paired forms round alike, lane by lane.  FP64: a divide.
+// scalar and the paired forms round alike, lane by lane.  FP64 has two: D1's,
+// below, in the collision, and a divide for what is formed once per column.
 __device__ __forceinline__ float rcp_estimate(float x) {
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
@@ -80,8 +81,10 @@ __device__ __forceinline__ D1 fmaR(D1 a, D1 b, D1 c) { return D1(__fma_rn(a.v, b
 // Reciprocal in FP64: the hardware estimate (PTX rcp.approx.ftz.f64, about
 // 20 bits) refined by one step of Halley's third-order iteration for 1/x,
 // r' = r + r (e + e^2) with e = 1 - x r, which cubes the estimate's relative
-// error: three fused multiply-adds, within an ulp for the normal arguments the
-// collision takes, no branch.  A correctly rounded divide costs about three
+// error: three fused multiply-adds, no branch.  The estimate has 21 significant
+// bits, so e is exact, and the result is off by half an ulp and e^3 (2^-60
+// relative, 2^-7 ulp) at most, for the normal arguments the collision takes
+// (axlbm_selftest_rcp64).  A correctly rounded divide costs about three
 // times as many FP64 instructions, and FP64 instructions bound these kernels
 // (GB300 issues one per SM in 16 cycles).
 __device__ __forceinline__ D1 rcp(D1 x) {

@@ -45,6 +45,12 @@ __global__ void __launch_bounds__(256) k_rcp_selftest(const float* x, long long 
     }
 }
 
+// The collision's FP64 reciprocal.
+__global__ void __launch_bounds__(256) k_rcp64_selftest(const double* x, long long n, double* out) {
+    const long long i = blockIdx.x * 256ll + threadIdx.x;
+    if (i < n) out[i] = rcp(D1(x[i])).v;
+}
+
 axlbm_status selftest_fail(axlbm_status st, const char* msg) {
     set_handleless_error(msg);
     return st;
@@ -93,6 +99,25 @@ extern "C" AXLBM_API axlbm_status axlbm_selftest_rcp(const float* x, int64_t n, 
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaMemcpyAsync(out, dev + n, 2 * n * sizeof(float), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (dev) cudaFree(dev);
+    if (s) cudaStreamDestroy(s);
+    return e == cudaSuccess ? AXLBM_OK : selftest_fail(AXLBM_ECUDA, cudaGetErrorString(e));
+}
+
+extern "C" AXLBM_API axlbm_status axlbm_selftest_rcp64(const double* x, int64_t n, double* out) {
+    using namespace axl;
+    if (!x || !out || n < 1 || n > (1ll << 26)) return selftest_fail(AXLBM_EINVAL, "x and out are required, 1 <= n <= 2^26");
+    double* dev = nullptr;
+    cudaStream_t s = nullptr;
+    cudaError_t e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaMalloc(&dev, 2 * n * sizeof(double));
+    if (e == cudaSuccess) e = cudaMemcpyAsync(dev, x, n * sizeof(double), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) {
+        k_rcp64_selftest<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(dev, n, dev + n);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaMemcpyAsync(out, dev + n, n * sizeof(double), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (dev) cudaFree(dev);
     if (s) cudaStreamDestroy(s);

@@ -50,3 +50,25 @@ def test_reciprocal_rejects_bad_arguments(B):
     out = np.empty(2, dtype=np.float32)
     assert L.axlbm_selftest_rcp(None, 1, out.ctypes.data) == B.EINVAL
     assert L.axlbm_selftest_rcp(out.ctypes.data, 0, out.ctypes.data) == B.EINVAL
+
+
+def test_fp64_reciprocal_within_half_an_ulp_and_the_estimate(B):
+    """The FP64 collision's reciprocal: an estimate r with 1 - x r = e, |e| <= 2^-20, and one step that leaves e^3.
+    Off by half an ulp from the last rounding and e^3 <= 2^-60 relative (2^-7 ulp) before it."""
+    wide = np.longdouble
+    assert np.finfo(wide).eps < 2e-19  # more digits than FP64: 1/x to 2^-10 ulp at least
+    rng = np.random.default_rng(12)
+    x = np.concatenate([
+        np.exp(rng.uniform(np.log(1e-6), np.log(1e6), 200_000)),
+        rng.uniform(0.5, 2.0, 200_000),
+        np.arange(1, 20001) - 0.5, np.arange(1, 20001, dtype=float),
+        [1.0 + 2.0 ** -52, 1.0 - 2.0 ** -53, 2.0 - 2.0 ** -52],
+        -rng.uniform(0.5, 2.0, 1000),
+    ])
+    got = B.axlbm_selftest_rcp64(x)
+    exact = wide(1) / x.astype(wide)
+    ulp = np.spacing(np.abs(exact.astype(np.float64)))
+    err = np.abs(got.astype(wide) - exact) / ulp
+    assert err.max() <= 0.5 + 2.0 ** -7 + 2.0 ** -9, float(err.max())
+    p2 = np.concatenate([2.0 ** np.arange(-60, 61.0), -(2.0 ** np.arange(-60, 61.0))])
+    assert np.array_equal(B.axlbm_selftest_rcp64(p2), 1.0 / p2)
