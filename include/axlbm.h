@@ -352,6 +352,13 @@ AXLBM_API axlbm_status axlbm_use_graphs(axlbm_handle* h, int32_t enable);
  * (either pointer may be NULL). */
 AXLBM_API axlbm_status axlbm_graph_stats(const axlbm_handle* h, int64_t* captures, int64_t* launches);
 
+/* For tests: how the runs of plain steps of a domain go (see
+ * axlbm_use_graphs).  form: 0 pairs of step kernels; one launch for a run, the
+ * state 1 in the shared memory of one thread-block cluster, 2 and 3 in that of
+ * a grid with one and with several pairs of nodes per thread, 4 in L2.  ctas:
+ * the launch's thread blocks (0 for form 0).  Either pointer may be NULL. */
+AXLBM_API axlbm_status axlbm_selftest_step_form(const axlbm_handle* h, int32_t* form, int32_t* ctas);
+
 /* Device timing of the bulk update kernel (the kernel that moves almost all
  * bytes), for throughput and roofline reporting.  enable = 1 clears the
  * totals and starts recording a CUDA event pair around every bulk-kernel
@@ -552,6 +559,8 @@ AXLBM_API axlbm_status axlbm_batch_use_graphs(axlbm_batch* b, int32_t enable);
 /* How many times the step graphs were captured and launched since creation
  * (either pointer may be NULL). */
 AXLBM_API axlbm_status axlbm_batch_graph_stats(const axlbm_batch* b, int64_t* captures, int64_t* launches);
+/* axlbm_selftest_step_form of a batch. */
+AXLBM_API axlbm_status axlbm_selftest_batch_step_form(const axlbm_batch* b, int32_t* form, int32_t* ctas);
 
 /* Use the bulk tile shape rows x nodes in both steps of a pair from the next
  * step on, instead of the ones timed at creation (for profiling a given

@@ -107,6 +107,7 @@ def lib() -> ctypes.CDLL:
         L.axlbm_halo_recv.argtypes = [H, ctypes.c_int32, ctypes.c_void_p, ctypes.c_int32]
         L.axlbm_batch_set_residual_lag.argtypes = [H, ctypes.c_int32]
         L.axlbm_graph_stats.argtypes = [H, ctypes.POINTER(ctypes.c_int64), ctypes.POINTER(ctypes.c_int64)]
+        L.axlbm_selftest_step_form.argtypes = [H, ctypes.POINTER(ctypes.c_int32), ctypes.POINTER(ctypes.c_int32)]
         L.axlbm_kernel_times.argtypes = [H, ctypes.POINTER(ctypes.c_int64), dp, dp, ctypes.POINTER(ctypes.c_int64)]
         L.axlbm_check_static.argtypes = [ctypes.POINTER(axlbm_grid), ctypes.c_double,
                                          ctypes.POINTER(axlbm_forcing), ctypes.POINTER(axlbm_boundary),
@@ -149,6 +150,7 @@ def lib() -> ctypes.CDLL:
             getattr(L, pre + "load").restype = ctypes.c_int
         L.axlbm_batch_copy_domain.argtypes = [H, ctypes.c_int32, H, ctypes.c_int32]
         L.axlbm_batch_graph_stats.argtypes = [H, ctypes.POINTER(ctypes.c_int64), ctypes.POINTER(ctypes.c_int64)]
+        L.axlbm_selftest_batch_step_form.argtypes = [H, ctypes.POINTER(ctypes.c_int32), ctypes.POINTER(ctypes.c_int32)]
         L.axlbm_batch_kernel_timing.argtypes = [H, ctypes.c_int32]
         L.axlbm_batch_kernel_times.argtypes = [H, ctypes.POINTER(ctypes.c_int64), dp, dp, ctypes.POINTER(ctypes.c_int64)]
         L.axlbm_batch_kernel_times_by_parity.argtypes = [H, ctypes.POINTER(ctypes.c_int64), dp, dp]
@@ -188,7 +190,8 @@ def lib() -> ctypes.CDLL:
                      "axlbm_destroy", "axlbm_kernel_timing", "axlbm_kernel_times", "axlbm_check_static",
                      "axlbm_use_graphs", "axlbm_graph_stats", "axlbm_set_residual_lag",
                      "axlbm_halo_bytes", "axlbm_halo_send", "axlbm_halo_recv",
-                     "axlbm_selftest_bounded_wait", "axlbm_selftest_rcp", "axlbm_selftest_rcp64"):
+                     "axlbm_selftest_bounded_wait", "axlbm_selftest_rcp", "axlbm_selftest_rcp64",
+                     "axlbm_selftest_step_form", "axlbm_selftest_batch_step_form"):
             getattr(L, name).restype = ctypes.c_int
         _lib = L
     return _lib
@@ -384,6 +387,12 @@ class Domain:
         """(captures, launches) of the step graphs since creation."""
         c, n = ctypes.c_int64(), ctypes.c_int64()
         _check(lib().axlbm_graph_stats(self.handle, ctypes.byref(c), ctypes.byref(n)), self.handle)
+        return int(c.value), int(n.value)
+
+    def step_form(self):
+        """(form, thread blocks) of runs of plain steps, for tests: forms as in axlbm_selftest_step_form."""
+        c, n = ctypes.c_int32(), ctypes.c_int32()
+        _check(lib().axlbm_selftest_step_form(self.handle, ctypes.byref(c), ctypes.byref(n)), self.handle)
         return int(c.value), int(n.value)
 
     @property
@@ -706,6 +715,12 @@ class Batch:
         """(captures, launches) of the step graphs since creation."""
         c, n = ctypes.c_int64(), ctypes.c_int64()
         _bcheck(lib().axlbm_batch_graph_stats(self.handle, ctypes.byref(c), ctypes.byref(n)), self.handle)
+        return int(c.value), int(n.value)
+
+    def step_form(self):
+        """(form, thread blocks) of runs of plain steps, for tests: forms as in axlbm_selftest_step_form."""
+        c, n = ctypes.c_int32(), ctypes.c_int32()
+        _bcheck(lib().axlbm_selftest_batch_step_form(self.handle, ctypes.byref(c), ctypes.byref(n)), self.handle)
         return int(c.value), int(n.value)
 
     def residuals(self, allow_nonfinite: bool = False) -> np.ndarray:

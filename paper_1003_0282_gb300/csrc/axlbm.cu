@@ -541,6 +541,13 @@ axlbm_status axlbm_graph_stats(const axlbm_handle* h, int64_t* captures, int64_t
     return AXLBM_OK;
 }
 
+axlbm_status axlbm_selftest_step_form(const axlbm_handle* h, int32_t* form, int32_t* ctas) {
+    if (!h) return AXLBM_EINVAL;
+    if (form) *form = axl::resident_form(h->res);
+    if (ctas) *ctas = h->res.on ? h->res.grid : 0;
+    return AXLBM_OK;
+}
+
 axlbm_status axlbm_kernel_timing(axlbm_handle* h, int32_t enable) {
     if (!h) return fail(nullptr, AXLBM_EINVAL, "handle is NULL");
     if (enable) {

@@ -1277,6 +1277,13 @@ axlbm_status axlbm_batch_graph_stats(const axlbm_batch* b, int64_t* captures, in
     return AXLBM_OK;
 }
 
+axlbm_status axlbm_selftest_batch_step_form(const axlbm_batch* b, int32_t* form, int32_t* ctas) {
+    if (!b) return AXLBM_EINVAL;
+    if (form) *form = axl::resident_form(b->res);
+    if (ctas) *ctas = b->res.on ? b->res.grid : 0;
+    return AXLBM_OK;
+}
+
 axlbm_status axlbm_batch_kernel_timing(axlbm_batch* b, int32_t enable) {
     if (!b) return bfail(nullptr, AXLBM_EINVAL, "batch is NULL");
     if (enable) {

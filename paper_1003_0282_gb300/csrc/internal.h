@@ -89,6 +89,7 @@ struct Resident {
     bool on = false;
     bool cluster = false;  // one thread-block cluster, else a cooperative grid
     bool slab = false;     // a grid with the state in shared memory, else in L2
+    bool one = false;      // ... one pair per thread, else several
     bool sw = false, th = false;
     int grid = 0, threads = 0;
     size_t smem = 0;
@@ -128,6 +129,8 @@ constexpr int64_t kResMaxSteps = 1 << 16;  // steps of one launch, at most (even
 bool resident_usable(const Resident& r, cudaStream_t stream);
 cudaError_t resident_capture(Resident* r, Clock* clock, cudaStream_t cap);
 cudaError_t resident_launch(Resident* r, Clock* clock, int steps, cudaStream_t stream);
+// The form as axlbm_selftest_step_form numbers it.
+inline int resident_form(const Resident& r) { return !r.on ? 0 : (r.cluster ? 1 : (!r.slab ? 4 : (r.one ? 2 : 3))); }
 void resident_drop_graph(Resident* r);
 void resident_free(Resident* r);
 

@@ -226,6 +226,7 @@ cudaError_t res_build(Resident* r, const ResidentDomain* d, int n, int num_sms, 
             if (e != cudaSuccess) return e;
             fits = (long long)got * num_sms >= r->grid;
             r->slab = true;
+            r->one = one;
             break;
         }
         // The state in L2.  Not with 16-bit storage: shared memory takes domains up
