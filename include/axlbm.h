@@ -561,6 +561,10 @@ AXLBM_API axlbm_status axlbm_batch_use_graphs(axlbm_batch* b, int32_t enable);
 AXLBM_API axlbm_status axlbm_batch_graph_stats(const axlbm_batch* b, int64_t* captures, int64_t* launches);
 /* axlbm_selftest_step_form of a batch. */
 AXLBM_API axlbm_status axlbm_selftest_batch_step_form(const axlbm_batch* b, int32_t* form, int32_t* ctas);
+/* For tests: run the step kernels of batches whose planes reach 4 GiB (64-bit
+ * offsets) on this batch, from the next call on; enable = 0 goes back to the
+ * rule.  The results are the same bit for bit.  Synchronises. */
+AXLBM_API axlbm_status axlbm_selftest_batch_wide_offsets(axlbm_batch* b, int32_t enable);
 
 /* Use the bulk tile shape rows x nodes in both steps of a pair from the next
  * step on, instead of the ones timed at creation (for profiling a given

@@ -151,6 +151,7 @@ def lib() -> ctypes.CDLL:
         L.axlbm_batch_copy_domain.argtypes = [H, ctypes.c_int32, H, ctypes.c_int32]
         L.axlbm_batch_graph_stats.argtypes = [H, ctypes.POINTER(ctypes.c_int64), ctypes.POINTER(ctypes.c_int64)]
         L.axlbm_selftest_batch_step_form.argtypes = [H, ctypes.POINTER(ctypes.c_int32), ctypes.POINTER(ctypes.c_int32)]
+        L.axlbm_selftest_batch_wide_offsets.argtypes = [H, ctypes.c_int32]
         L.axlbm_batch_kernel_timing.argtypes = [H, ctypes.c_int32]
         L.axlbm_batch_kernel_times.argtypes = [H, ctypes.POINTER(ctypes.c_int64), dp, dp, ctypes.POINTER(ctypes.c_int64)]
         L.axlbm_batch_kernel_times_by_parity.argtypes = [H, ctypes.POINTER(ctypes.c_int64), dp, dp]
@@ -191,7 +192,7 @@ def lib() -> ctypes.CDLL:
                      "axlbm_use_graphs", "axlbm_graph_stats", "axlbm_set_residual_lag",
                      "axlbm_halo_bytes", "axlbm_halo_send", "axlbm_halo_recv",
                      "axlbm_selftest_bounded_wait", "axlbm_selftest_rcp", "axlbm_selftest_rcp64",
-                     "axlbm_selftest_step_form", "axlbm_selftest_batch_step_form"):
+                     "axlbm_selftest_step_form", "axlbm_selftest_batch_step_form", "axlbm_selftest_batch_wide_offsets"):
             getattr(L, name).restype = ctypes.c_int
         _lib = L
     return _lib
@@ -722,6 +723,10 @@ class Batch:
         c, n = ctypes.c_int32(), ctypes.c_int32()
         _bcheck(lib().axlbm_selftest_batch_step_form(self.handle, ctypes.byref(c), ctypes.byref(n)), self.handle)
         return int(c.value), int(n.value)
+
+    def wide_offsets(self, enable: bool) -> None:
+        """Step kernels with 64-bit offsets in a plane (those of planes of 4 GiB or more), for tests."""
+        _bcheck(lib().axlbm_selftest_batch_wide_offsets(self.handle, int(bool(enable))), self.handle)
 
     def residuals(self, allow_nonfinite: bool = False) -> np.ndarray:
         """[n][3]: residual (Eq. 57), mass, budget of each domain's last check step."""

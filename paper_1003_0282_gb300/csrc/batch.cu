@@ -757,6 +757,7 @@ axlbm_status axlbm_batch_create(const axlbm_domain* domains, int32_t n, int32_t 
             if (e != cudaSuccess) st = bcuda(b, e, "TMA descriptor");
         }
     }
+    b->wide = axl::batch_needs_wide(b->L, precision);
     if (st == AXLBM_OK) st = reset_rest(b);
     if (st == AXLBM_OK) st = tune(b);
     if (st == AXLBM_OK) st = reset_rest(b);
@@ -1282,6 +1283,15 @@ axlbm_status axlbm_selftest_batch_step_form(const axlbm_batch* b, int32_t* form,
     if (form) *form = axl::resident_form(b->res);
     if (ctas) *ctas = b->res.on ? b->res.grid : 0;
     return AXLBM_OK;
+}
+
+axlbm_status axlbm_selftest_batch_wide_offsets(axlbm_batch* b, int32_t enable) {
+    if (!b) return bfail(nullptr, AXLBM_EINVAL, "batch is NULL");
+    b->wide = enable != 0 || axl::batch_needs_wide(b->L, b->precision);
+    memset(b->grid, 0, sizeof b->grid);  // other kernels, to be sized on their first launch
+    cudaError_t e = cudaStreamSynchronize(b->stream);
+    batch_drop_graphs(b);
+    return e == cudaSuccess ? AXLBM_OK : bcuda(b, e, "wide offsets");
 }
 
 axlbm_status axlbm_batch_kernel_timing(axlbm_batch* b, int32_t enable) {

@@ -61,6 +61,7 @@ struct axlbm_batch {
     int shape[2];                     // tile shape of even and odd steps
     int grid[axl::kBatchShapes][2][2];  // persistent grid per (shape, parity, check)
     int num_sms;
+    bool wide;  // bulk kernels with 64-bit offsets in a plane
     int parity;
     int64_t t;
     bool speed_valid, have_check, last_residual_valid;
@@ -120,5 +121,10 @@ struct BatchOps {
 
 extern const BatchOps batch_ops_fp32;
 extern const BatchOps batch_ops_fp16;
+
+// Whether a plane of the batch's atlas is too large for 32-bit byte offsets.
+inline bool batch_needs_wide(const BatchLayout& L, int precision) {
+    return (unsigned long long)L.plane * (precision == AXLBM_FP32 ? 4 : 2) >= (1ull << 32);
+}
 
 }  // namespace axl

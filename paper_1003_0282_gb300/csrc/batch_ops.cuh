@@ -106,7 +106,7 @@ cudaError_t launch_bulk_batch_wet(axlbm_batch* b, const BatchArgs<S, R>& A) {
 template <class S, class R, bool TH, int PAR, bool CHK>
 cudaError_t launch_bulk_batch_shape(axlbm_batch* b, const BatchArgs<S, R>& A) {
     // a plane of 4 GiB or more: 64-bit offsets, in one kernel for every mix of domains
-    if ((unsigned long long)A.plane * sizeof(S) >= (1ull << 32))
+    if (b->wide)
         return launch_bulk_batch_wet<S, R, true, PAR, CHK, PAR == 0, unsigned long long>(b, A);
     // wet walls matter only in even steps (odd steps leave the rings to the ring kernels)
     if constexpr (PAR == 0) {
