@@ -58,6 +58,7 @@ struct axlbm_ws {
     cudaStream_t stream;
     __nv_bfloat16* w;  // all layers, packed as in include/axlbm.h
     std::vector<size_t> woff, boff;
+    int num_sms;
     int chunk;  // canvases that `act` holds
     Acts act;
     axlbm_ws_train* train;  // allocated by the first training call
@@ -248,19 +249,19 @@ unsigned blocks_for(long long n) { return (unsigned)((n + 255) / 256); }
 // of 32 WN channels, tiles of 16 x 16 pixels where those still give every SM
 // two blocks, else of 8 x 16 (the deep levels; wide outputs of the gradients).
 template <int MODE>
-cudaError_t launch_conv(cudaStream_t st, const axl::wsconv::ConvIn& in, int n, const bf16* wt, int cout, const bf16* bias,
+cudaError_t launch_conv(const axlbm_ws* w, const axl::wsconv::ConvIn& in, int n, const bf16* wt, int cout, const bf16* bias,
                         const axl::wsconv::ConvOut& to) {
     using namespace axl::wsconv;
     const int wn = cout % 96 == 0 ? 3 : (cout % 64 == 0 ? 2 : (cout % 160 == 0 ? 5 : (cout % 224 == 0 ? 7 : 1)));
     const long long px = (long long)n * in.h * in.w;
-    const bool tall = wn <= 3 && px / 256 * (cout / (32 * wn)) >= 2 * 148;
+    const bool tall = wn <= 3 && px / 256 * (cout / (32 * wn)) >= 2 * w->num_sms;
     auto go = [&](auto wn_tag, auto th_tag) -> cudaError_t {
         constexpr int WN = decltype(wn_tag)::value, TH = decltype(th_tag)::value;
         auto kern = k_conv3<WN, TH, MODE>;
         const size_t smem = conv_smem<WN, TH>(in.c0 + in.c1);
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)conv_smem<WN, TH>(224));
         if (e != cudaSuccess) return e;
-        kern<<<dim3((unsigned)(px / (TH * kTW)), (unsigned)(cout / (32 * WN))), 8 * WN * TH, smem, st>>>(in, wt, cout, bias, to);
+        kern<<<dim3((unsigned)(px / (TH * kTW)), (unsigned)(cout / (32 * WN))), 8 * WN * TH, smem, w->stream>>>(in, wt, cout, bias, to);
         return cudaGetLastError();
     };
     using std::integral_constant;
@@ -281,7 +282,7 @@ cudaError_t launch_conv(cudaStream_t st, const axl::wsconv::ConvIn& in, int n, c
 // 3x3 convolution of layer `layer` over n canvases, with bias, ReLU and BF16
 // output, and the output's 2x2 average in `pool` unless null (the forward pass).
 cudaError_t conv3(axlbm_ws* w, int layer, const axl::wsconv::ConvIn& in, int n, bf16* out, bf16* pool = nullptr) {
-    return launch_conv<0>(w->stream, in, n, w->w + w->woff[layer], kNet[layer].cout, w->w + w->boff[layer],
+    return launch_conv<0>(w, in, n, w->w + w->woff[layer], kNet[layer].cout, w->w + w->boff[layer],
                           {out, pool, nullptr, nullptr, 0, nullptr});
 }
 
@@ -580,7 +581,9 @@ struct axlbm_ws_train {
 namespace {
 
 constexpr int kLossBlocks = 1024;
-constexpr int kWgradBlocks = 4 * 148;  // blocks of a weight gradient, about (two waves of two blocks per SM)
+// Blocks of a weight gradient, about: just under two waves of two blocks on 152 SMs.  A number of its own and not the
+// device's, because the splits set the order of the sums.
+constexpr int kWgradBlocks = 592;
 
 // Splits of layer l's weight gradient over n canvases, and the pixel tiles of one.
 void wgrad_splits(int l, int n, int* nsplit, int* per, int* tiles);
@@ -717,7 +720,7 @@ cudaError_t conv_dgrad(axlbm_ws* w, int l, int n, const bf16* dy, const axl::wsc
     axlbm_ws_train* t = w->train;
     const Layer& L = kNet[l];
     k_transpose_taps<<<blocks_for((long long)L.cout * 9 * L.cin), 256, 0, w->stream>>>(w->w + w->woff[l], L.cout, L.cin, t->wtt);
-    return launch_conv<MODE>(w->stream, plain_in(dy, L.cout, layer_level(l)), n, t->wtt, L.cin, nullptr, to);
+    return launch_conv<MODE>(w, plain_in(dy, L.cout, layer_level(l)), n, t->wtt, L.cin, nullptr, to);
 }
 
 // Backward pass of the kept forward pass from t->dout, gradients into t->grad.
@@ -783,6 +786,10 @@ axlbm_status axlbm_ws_create(const uint16_t* weights, size_t count, void* cuda_s
     if (!w) return wfail(nullptr, AXLBM_ENOMEM, "host allocation failed");
     w->stream = static_cast<cudaStream_t>(cuda_stream);
     w->chunk = 8;  // (axlbm_ws_predict grows it)
+    int dev = 0;
+    w->num_sms = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&w->num_sms, cudaDevAttrMultiProcessorCount, dev);
+    if (w->num_sms < 1) w->num_sms = 1;
     size_t off = 0;
     for (const Layer& l : kNet) {
         w->woff.push_back(off);
