@@ -104,18 +104,19 @@ __host__ __device__ __forceinline__ ResSlot res_slot4(const Geom& G, int q, int 
 // g and h on their way through a slot, as the step kernels' boundary rules
 // round them, without a branch: g' = sg g + cg with sg = 1, -1 (axis, or off a
 // wall: cg = rho0 u_w / 2), h' = (sh h + ch) + ct with sh = -1, ch = -T_ref/2,
-// ct = T_w/2 off a wall of given temperature, else h.  (Zero may lose its sign.)
+// ct = T_w/2 off a wall of given temperature, else h.  What adds nothing is
+// -0, which leaves either zero as it is.
 template <class R>
 __device__ __forceinline__ void res_through_g(const Geom& G, const Coef<R>& C, int how, int j, R& sg, R& cg) {
     sg = how == 0 ? R(1) : R(-1);
-    cg = how >= 2 ? mul_rn(R(0.5) * C.rho0, wall_uth(G, C, how - 2, j)) : R(0);
+    cg = how >= 2 ? mul_rn(R(0.5) * C.rho0, wall_uth(G, C, how - 2, j)) : R(-0.0);
 }
 template <class R>
 __device__ __forceinline__ void res_through_h(const Coef<R>& C, int how, R& sh, R& ch, R& ct) {
     const bool dirichlet = how >= 2 && pick4(C.t_dir, how - 2);
     sh = dirichlet ? R(-1) : R(1);
-    ch = dirichlet ? R(-0.5) * C.t_ref : R(0);
-    ct = dirichlet ? R(0.5) * pick4(C.t_w, how - 2) : R(0);
+    ch = dirichlet ? R(-0.5) * C.t_ref : R(-0.0);
+    ct = dirichlet ? R(0.5) * pick4(C.t_w, how - 2) : R(-0.0);
 }
 
 // The slot of plane-ordered population q of node (j, k): plane-ordered slot
