@@ -552,8 +552,7 @@ AXLBM_API axlbm_status axlbm_batch_tile_shape(const axlbm_batch* b, int32_t* row
  * change) when enable != 0, the default, and while kernel timing is off;
  * enable = 0 launches every kernel directly.  Small batches (as axlbm_use_graphs
  * says of domains) take one graph of a single kernel that runs all the pairs of
- * a call.  The results are the same
- * bit for bit.  The first capture synchronises nothing but takes a few ms. */
+ * a call.  The results are the same bit for bit.  The first capture synchronises nothing but takes a few ms. */
 AXLBM_API axlbm_status axlbm_batch_use_graphs(axlbm_batch* b, int32_t enable);
 
 /* How many times the step graphs were captured and launched since creation
@@ -641,7 +640,11 @@ AXLBM_API size_t axlbm_ws_weight_count(void);
  * AXLBM_EINVAL if count != axlbm_ws_weight_count(); AXLBM_ENOMEM; AXLBM_ECUDA. */
 AXLBM_API axlbm_status axlbm_ws_create(const uint16_t* weights, size_t count, void* cuda_stream, axlbm_ws** out);
 /* Canvases of n feature vectors (host, [n][AXLBM_WS_FEATURES]) into the
- * caller's device array canvas [n][4][256][128] (FP32).  Synchronises. */
+ * caller's device array canvas [n][4][256][128] (FP32).  Synchronises.
+ * Passes of up to 32 canvases: a call with more canvases than an earlier one
+ * grows the activation buffers (0.13 GB for 8 at creation, 0.51 GB for 32) and
+ * keeps them until axlbm_ws_destroy; where that memory cannot be had, the
+ * passes stay as they were. */
 AXLBM_API axlbm_status axlbm_ws_predict(axlbm_ws* w, const float* features, int32_t n, float* canvas);
 /* Resample n canvases (device) onto n domains (host descriptions): fields
  * rho, u_r, u_z, u_theta, T of each domain, packed as [5][nz][nr] one domain
@@ -660,14 +663,14 @@ AXLBM_API axlbm_status axlbm_ws_to_canvas(axlbm_ws* w, const float* moments, int
                                           float* canvas);
 /* One training step of the network on n (1..16) canvases with the library's
  * kernels: forward pass keeping the activations, mean squared error against
- * target, backward pass (ReLU, pooling, upsampling and concatenation, im2col
- * and its adjoint; weight and input gradients as BF16 GEMMs with FP32
+ * target, backward pass (ReLU, pooling, upsampling and concatenation; weight
+ * and input gradients of the 3x3 convolutions with BF16 operands and FP32
  * accumulation), then Adam (lr, beta1, beta2, eps; no weight decay) on FP32
  * master weights, which start from the weights passed to axlbm_ws_create and
  * are rounded to BF16 for every later forward pass.
  *   features: device [n][AXLBM_WS_FEATURES]; target: device [n][4][256][128];
  *   loss: receives the mean squared error before the update (or NULL).
- * The first call allocates about 3 GB of training buffers.  Synchronises. */
+ * The first call allocates about 0.62 GB of training buffers.  Synchronises. */
 AXLBM_API axlbm_status axlbm_ws_train_step(axlbm_ws* w, const float* features, const float* target, int32_t n,
                                            float lr, float beta1, float beta2, float eps, double* loss);
 /* Mean squared error of the network on n canvases (device features and

@@ -440,9 +440,9 @@ __device__ __forceinline__ void batch_nodes(const BatchArgs<S, R>& A, const Slot
 // every domain carries g; TH: shelves may carry h (per-tile flag); WET: some
 // domain has a wet wall (its wall nodes keep their state in even steps).
 // Off: a node's byte offset in a plane, 32 bits unless a plane has 4 GiB or
-// more (against 64 bits, sweep of 320 domains: FP16 even 0.2102 -> 0.2034 and
-// odd 0.2989 -> 0.2912 ms, FP32 odd 0.3196 -> 0.3154 ms: fewer instructions
-// per store).
+// more: fewer instructions per store (ms a launch of the sweep of 320 domains,
+// 32 and 64 bits: FP16 even 0.2034 and 0.2102, odd 0.2912 and 0.2989; FP32 odd
+// 0.3154 and 0.3196).
 template <class S, class R, bool SW, bool TH, int PAR, bool CHK, int TK, int TJ, bool WET, class Off = unsigned>
 __global__ void __launch_bounds__(batch_nthreads<TK, TJ>() + 32, batch_min_blocks<TK, TJ>())
 k_bulk_batch(const __grid_constant__ CUtensorMap map, const BatchArgs<S, R> A) {

@@ -295,7 +295,8 @@ struct Cell {
     }
 
     // The same collision in FP64 (the type D1), arranged for the fewest FP64
-    // instructions: GB300 issues one per scheduler in 64.5 cycles, and they are
+    // instructions: an SM of GB300 takes 19 cycles for one of a warp (a warp
+    // alone on its SM waits 64 for each), and they are
     // all that bounds the FP64 kernels.  Sums are shared between the moments
     // and the MRT basis, S_4 = -S_3 and S_6 = -S_5, factors ride on fused
     // multiply-adds, and what depends on the column alone comes in k.  About

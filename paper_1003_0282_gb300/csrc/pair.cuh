@@ -67,8 +67,8 @@ __device__ __forceinline__ F2 rcp(F2 x) {
 }
 
 // One FP64 value whose operations round as written: which products are fused
-// is stated in the collision, so that every kernel rounds a node alike (the compiler fuses plain double expressions differently from kernel
-// to kernel).
+// is stated in the collision, so that every kernel rounds a node alike (the
+// compiler fuses plain double expressions differently from kernel to kernel).
 struct D1 {
     double v;
     __device__ __forceinline__ D1() {}
@@ -86,7 +86,7 @@ __device__ __forceinline__ D1 fmaR(D1 a, D1 b, D1 c) { return D1(__fma_rn(a.v, b
 // relative, 2^-7 ulp) at most, for the normal arguments the collision takes
 // (axlbm_selftest_rcp64).  A correctly rounded divide costs about three
 // times as many FP64 instructions, and FP64 instructions bound these kernels
-// (GB300 issues one per SM in 16 cycles).
+// (an SM of GB300 takes 19 cycles for one of a warp).
 __device__ __forceinline__ D1 rcp(D1 x) {
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x.v));

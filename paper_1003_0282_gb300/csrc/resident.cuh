@@ -335,8 +335,8 @@ __device__ __forceinline__ void res_dld(uint32_t a, double& v) {
 //
 // What bounds it: the latency of one step of one thread (slots, the chain of
 // the collision, barrier); the throughput of one scheduler for more pairs.
-// FP64: the FP64 pipe (64.5 cycles per warp instruction and scheduler,
-// whatever its active lanes).
+// FP64: the FP64 pipe, whatever a warp's active lanes (64 cycles per warp
+// instruction of a warp alone on its SM, 76 with one on each scheduler).
 template <class S, class R, bool SW, bool TH>
 __global__ void __launch_bounds__(kResThreads, 1)
 k_resident_cluster(const ResDom<S, R>* __restrict__ doms, Clock* clock, int nsteps) {
@@ -428,8 +428,8 @@ k_resident_cluster(const ResDom<S, R>* __restrict__ doms, Clock* clock, int nste
 // A population on its way between two CTAs: the value and the step it is for
 // in one 8-byte word (FP64: two halves, each with the step), written and read
 // with relaxed 8-byte accesses.  The reader polls the word itself, so a hop
-// costs one store and one load of L2 (470-850 cycles one way on GB300, the
-// larger figure between the dies) where a flag behind a release costs 2600.
+// costs one store and one load of L2 (590 to 1170 cycles one way on GB300,
+// median 1070) where a flag behind a release costs 1730 to 2500.
 // One word serves a slot in both directions: its owner and the node that uses
 // it in odd steps take turns.
 template <class R>

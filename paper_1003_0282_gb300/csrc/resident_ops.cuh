@@ -230,9 +230,9 @@ cudaError_t res_build(Resident* r, const ResidentDomain* d, int n, int num_sms, 
             break;
         }
         // The state in L2.  Not with 16-bit storage: shared memory takes domains up
-        // to where a step kernel already has 300 k pairs to work on, and the step
-        // is then issue-bound in either form (512 x 768 x 100 steps, in shared
-        // memory: 1.39 -> 0.72 ms; 96 x 144 x 300: 2.58 -> 0.55 ms).
+        // to where a step kernel already has 300 k pairs to work on (in shared
+        // memory and with the step kernels: 512 x 768, 100 steps: 0.72 and 1.39 ms;
+        // 96 x 144, 300 steps: 0.55 and 2.58 ms).
         if constexpr (std::is_same<S, R>::value) {
             auto kern = k_resident_grid<S, R, SW, TH>;
             for (int per_sm = 2; per_sm >= 1 && !fits; --per_sm) {

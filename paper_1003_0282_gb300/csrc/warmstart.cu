@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(256) k_ws_head(const bf16* x, const bf16* wt, 
 // rows of up to kFieldCols columns of one domain; a thread walks down one
 // column and keeps its values interpolated along r at the two canvas rows
 // around it, which several domain rows share: FP64 instructions bound this
-// kernel (64.5 cycles a warp instruction and scheduler), and this takes about
+// kernel (an SM takes 19 cycles for one of a warp), and this takes about
 // 12 of them per node and 16 per new canvas row, where sampling every node
 // afresh took over a hundred with its divisions.
 constexpr int kFieldCols = 128, kFieldRows = 32;

@@ -128,9 +128,9 @@ __device__ __forceinline__ uint4 relu_mask(uint4 v, uint4 a) {
 // The tile's input is read once (an implicit im2col gather reads it nine
 // times); the A operands of every tap are the same shared memory at a shifted
 // address.  A warp owns four rows of 16 pixels x 32 channels: 6 ldmatrix per
-// 16 mma, below the shared-memory rate at the full mma.sync rate (600 TFLOP/s
-// measured on GB300, against 57 reached by the gathering kernel).  Weights
-// stream through kWStages cp.async stages.  k ascends in steps of 16 into one
+// 16 mma, below the shared-memory rate at the full mma.sync rate (605 TFLOP/s
+// from registers, measured on GB300).  Weights stream through kWStages
+// cp.async stages.  k ascends in steps of 16 into one
 // accumulator per output, so sums round as in any other tiling.  mma.sync and
 // not tcgen05.mma: with the tile as unswizzled core matrices, a tap being a
 // descriptor shifted by 16-byte places, an instruction of 128 pixels took 200
