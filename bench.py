@@ -44,7 +44,14 @@ sys.path.insert(0, ROOT)
 #   batch fp32  profiles/k_bulk_batch_fp32_sweep320_launches.md
 #   batch fp16  profiles/k_bulk_batch_fp16_sweep_half_full.md (full-size DRAM capture)
 #   pipe fp32   profiles/k_bulk_fp32_pipe4096x8192_launches.md
-NCU_TRAFFIC = {}
+NCU_TRAFFIC = {
+    "batch fp32": {"src_sha": "b35846556b84531a", "dram_per_alg_byte": 0.9915,
+                   "profile": "k_bulk_batch_fp32_sweep320_launches.md"},
+    "batch fp16": {"src_sha": "b35846556b84531a", "dram_per_alg_byte": 0.9645,
+                   "profile": "k_bulk_batch_fp16_sweep_half_full.md"},
+    "pipe fp32": {"src_sha": "b35846556b84531a", "dram_per_alg_byte": 1.0555,
+                  "profile": "k_bulk_fp32_pipe4096x8192_launches.md"},
+}
 
 
 def parse():

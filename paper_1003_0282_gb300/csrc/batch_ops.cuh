@@ -135,7 +135,7 @@ cudaError_t batch_step_th(axlbm_batch* b, int check, int residual, cudaEvent_t e
     }
     // odd step: the interior (bulk) and the outer rings touch disjoint slots, so
     // the rings run on the side stream beside the bulk kernel.  With 16-bit
-    // storage they go first (that bulk kernel is bound by issue, and the rings'
+    // storage they go first (that bulk kernel leaves HBM half idle, and the rings'
     // small blocks use the SMs' leftover registers).  With FP32 storage the
     // bulk kernel needs all of HBM and every SM from the start, so there the
     // rings have the lower priority and fill its tail.

@@ -874,7 +874,9 @@ __device__ __forceinline__ void res_slab_cta(const ResDom<S_, R>& D, Clock* cloc
 
 // Cooperative grid, one CTA per SM, several pairs per thread.
 //
-// What bounds it: instruction issue (FP32) or the FP64 pipe.
+// What bounds it: FP32 latency at three warps a scheduler (words in, barrier,
+// update, barrier, words out in series; a third of the issue slots used); the
+// FP64 pipe.
 template <class S, class R, bool SW, bool TH>
 __global__ void __launch_bounds__(kResSlabThreads, 1)
 k_resident_slab(const ResDom<S, R>* __restrict__ doms, const int* __restrict__ cta_dom, Clock* clock, int nsteps,
@@ -1112,7 +1114,8 @@ __device__ __forceinline__ void res_grid_cta(const ResDom<S, R>& D, unsigned* fl
 //
 // What bounds it: for few pairs per CTA the latency of a step -- the slots
 // from L2, the collision's chain, a fence, a release store and the
-// neighbours' polls; for many, instruction issue (FP32) or the FP64 pipe.
+// neighbours' polls -- also for many in FP32, at three warps a scheduler (38 %
+// of the issue slots, 37 % of L2's rate at 512 x 1280); in FP64 the FP64 pipe.
 template <class S, class R, bool SW, bool TH>
 __global__ void __launch_bounds__(kResThreads, 2)
 k_resident_grid(const ResDom<S, R>* __restrict__ doms, const int* __restrict__ cta_dom, unsigned* flags, Clock* clock,

@@ -143,3 +143,59 @@ def test_zeros_keep_their_sign(B, shape, precision):
             dom.close()
         for u, v in zip(*got):
             assert np.array_equal(u.view(np.uint64), v.view(np.uint64))
+
+
+def test_streams_and_threads(B):
+    """Domains and a batch stepped by threads of their own, on streams of two priorities beside other work: each launch
+    needs all its blocks on the card at once, whatever else runs, and ends with what it gives alone."""
+    import threading
+
+    import torch
+    cases = [(problem(64, 48, "crystal"), "fp32"), (problem(128, 192, "crystal"), "fp32"),
+             (problem(199, 391, "annulus-mixed"), "fp32"), (problem(199, 391, "crystal"), "fp64"),
+             (problem(1001, 1201, "pipe", temperature=False, swirl=False), "fp32")]
+    states = [seeded_state(pb, 70 + i) for i, (pb, _) in enumerate(cases)]
+
+    def make(i, stream):
+        (pb, precision), st = cases[i], states[i]
+        with torch.cuda.stream(stream):
+            dom = B.Domain(pb, precision, stream=stream)
+            dom.set_populations(st.f, st.g if pb.swirl else None, st.h if pb.temperature else None, time=0)
+        return dom
+
+    want = []
+    for i in range(len(cases)):
+        dom = make(i, torch.cuda.Stream())
+        dom.use_graphs(False)
+        for _ in range(6):
+            dom.step(34)
+        want.append((dom.get_populations(), dom.residual()))
+        dom.close()
+    doms = [make(i, torch.cuda.Stream(priority=-(i % 2))) for i in range(len(cases))]
+    assert {d.step_form()[0] for d in doms} == {CLUSTER, ONE, SEVERAL, L2}
+    errors = []
+
+    def run(dom):
+        try:
+            torch.cuda.set_device(0)
+            for _ in range(6):
+                dom.step(34)
+        except Exception as e:  # noqa: BLE001 (reported below)
+            errors.append(e)
+
+    other = torch.cuda.Stream()
+    a = torch.randn(4096, 4096, device="cuda")
+    threads = [threading.Thread(target=run, args=(d,)) for d in doms]
+    for t in threads:
+        t.start()
+    with torch.cuda.stream(other):
+        for _ in range(20):
+            a = torch.tanh(a @ a)
+    for t in threads:
+        t.join()
+    assert not errors
+    for dom, (pops, residual) in zip(doms, want):
+        assert dom.residual() == residual
+        for u, v in zip(dom.get_populations(), pops):
+            assert (u is None and v is None) or np.array_equal(u, v)
+        dom.close()
